@@ -32,11 +32,12 @@ cg_status cg_im2col_bf16(const void* x, void* a, int n, int h, int w, int c, int
 /* The whole stem -- 7x7, stride 2, padding 3, 3 -> 64 channels, with its gate, batch norms and activation --
  * from the image: what cg_im2col_bf16 (k = 7, stride 2, pad 3) and cg_conv_forward of `h` over the patch matrix
  * compute, without the matrix.  `h`: that 1x1 layer (BF16, groups = 1, c_in = k_pad >= 147, c_out = 64, extents of
- * the output; its statistics count the call).  x [n,image_h,image_w,3] bf16, h' = (image_h - 1)/2 + 1 (w' alike);
- * w_base [64,k_pad]; bn, delta as for cg_conv_forward (no delta_high); y [n,h',w',64]; workspace:
- * cg_stem_workspace_bytes() of device scratch.  CG_ERR_UNSUPPORTED where the layer is not on tensor cores. */
+ * the output; its statistics count the call).  x [n,image_h,image_w,c] bf16 with c = 3 and n at most the handle's
+ * (the images behind the n-th keep what y held), h' = (image_h - 1)/2 + 1 (w' alike); w_base [64,k_pad]; bn, delta as
+ * for cg_conv_forward (no delta_high); y [n,h',w',64]; workspace: cg_stem_workspace_bytes() of device scratch.
+ * CG_ERR_INVALID_ARG for other extents, CG_ERR_UNSUPPORTED where the layer is not on tensor cores. */
 size_t cg_stem_workspace_bytes(void);
-cg_status cg_stem_forward(cg_conv_t h, const void* x, int image_h, int image_w, const void* w_base,
+cg_status cg_stem_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
                           const cg_bn_params* bn, const float* delta, void* y, void* workspace, void* cuda_stream);
 
 /* Every stride-th pixel: y[n,i,j,:] = x[n,i*stride,j*stride,:], y is [n,ceil(h/stride),

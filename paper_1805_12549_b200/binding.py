@@ -106,7 +106,7 @@ def lib():
         L.cg_stem_workspace_bytes.restype = C.c_size_t
         L.cg_stem_workspace_bytes.argtypes = []
         L.cg_stem_forward.restype = C.c_int
-        L.cg_stem_forward.argtypes = [C.c_void_p, C.c_void_p, i, i, C.c_void_p, C.POINTER(CgBnParams), C.c_void_p,
+        L.cg_stem_forward.argtypes = [C.c_void_p, C.c_void_p, i, i, i, i, C.c_void_p, C.POINTER(CgBnParams), C.c_void_p,
                                       C.c_void_p, C.c_void_p, C.c_void_p]
         L.cg_subsample_bf16.restype = C.c_int
         L.cg_subsample_bf16.argtypes = [C.c_void_p, C.c_void_p, i, i, i, i, i, C.c_void_p]
@@ -274,8 +274,9 @@ def cg_stem_workspace_bytes() -> int:
 
 
 def cg_stem_forward(h, x, w_base, bn: CgBnParams, delta, y, workspace, stream=None):
-    """x [n,h,w,3] -> y [n,h',w',64] (include/cgnet.h)."""
-    _check(lib().cg_stem_forward(h, _ptr(x), x.shape[1], x.shape[2], _ptr(w_base), C.byref(bn), _ptr(delta), _ptr(y),
+    """x [n,h,w,3] -> y [n,h',w',64], n at most the handle's (include/cgnet.h)."""
+    n, ih, iw, c = x.shape
+    _check(lib().cg_stem_forward(h, _ptr(x), n, ih, iw, c, _ptr(w_base), C.byref(bn), _ptr(delta), _ptr(y),
                                  _ptr(workspace), _stream_ptr(stream)), "cg_stem_forward")
 
 

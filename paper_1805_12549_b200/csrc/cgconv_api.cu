@@ -292,9 +292,10 @@ cg_status cg_conv_forward(cg_conv_t h, const void* x, const void* w_base, const 
 
 size_t cg_stem_workspace_bytes(void) { return cg::kStemWeightBytes; }
 
-cg_status cg_stem_forward(cg_conv_t h, const void* x, int image_h, int image_w, const void* w_base, const cg_bn_params* bn,
-                          const float* delta, void* y, void* workspace, void* cuda_stream) {
-  if (!h || !x || !w_base || !y || !workspace || image_h <= 0 || image_w <= 0) return CG_ERR_INVALID_ARG;
+cg_status cg_stem_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
+                          const cg_bn_params* bn, const float* delta, void* y, void* workspace, void* cuda_stream) {
+  if (!h || !x || !w_base || !y || !workspace || n <= 0 || image_h <= 0 || image_w <= 0 || c != 3) return CG_ERR_INVALID_ARG;
+  if (n > h->L.n) return CG_ERR_INVALID_ARG;               // y has room for the handle's batch; fewer images are fine
   const cg_status st = check_bn(h, bn, delta);
   if (st != CG_OK) return st;
   const cg::LayerDims& L = h->L;
@@ -308,7 +309,7 @@ cg_status cg_stem_forward(cg_conv_t h, const void* x, int image_h, int image_w, 
   int cur = -1;
   if (cudaGetDevice(&cur) != cudaSuccess) return CG_ERR_CUDA;
   if (cur != h->device) return CG_ERR_INVALID_ARG;
-  const int err = cg::launch_stem(x, L.n, image_h, image_w, w_base, L.c_in, *bn, delta, L.eps, L.relu, y, workspace,
+  const int err = cg::launch_stem(x, n, image_h, image_w, w_base, L.c_in, *bn, delta, L.eps, L.relu, y, workspace,
                                   h->counters, reinterpret_cast<cudaStream_t>(cuda_stream));
   return err == 0 ? CG_OK : CG_ERR_CUDA;
 }

@@ -85,3 +85,22 @@ def test_a_pass_without_hooks_matches_the_recorded_one(algo):
     per, _ = inst.stats()
     assert per["stem"].calls == 2 and all(st.device_status == 0 for st in per.values())
     inst.close()
+
+
+def test_a_short_batch_gives_its_own_logits_and_other_extents_are_refused():
+    import torch
+    from paper_1805_12549_b200 import binding as B, resnet18 as R
+    net = R.CgResNet18(image=33, classes=20)
+    net.set_density(1.0)
+    x = R.synthetic_images("stemshort", 4, 33)
+    inst = net.instance(3)
+    full = inst.forward(x[:3]).clone()
+    stem = inst.out["stem"].clone()
+    for k in (1, 2):
+        inst.out["stem"].fill_(3.0)
+        assert torch.equal(inst.forward(x[:k].clone())[:k], full[:k])
+        assert torch.equal(inst.out["stem"][:k], stem[:k]) and bool((inst.out["stem"][k:] == 3).all())
+    for bad in (x, torch.cat([x, x], -1)[:3, ..., :4].contiguous(), x[:3, ..., :2].contiguous(), x[:3, :31].contiguous()):
+        with pytest.raises(B.CgError):
+            inst.forward(bad)
+    inst.close()

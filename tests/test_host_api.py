@@ -54,6 +54,36 @@ def test_network_operators_reject_bad_arguments_before_any_launch():
     assert lib.cg_avgpool_bf16(odd, p, 1, 49, 16, None) == ALIGN
 
 
+def test_the_stem_is_told_the_images_and_channels_of_its_input(monkeypatch):
+    """The extents come from x itself: a short batch is that many images, another channel count is refused."""
+    import torch
+    seen = []
+
+    class Recorder:
+        def cg_stem_forward(self, *args):
+            seen.append(args)
+            return 0
+
+    monkeypatch.setattr(B, "_lib", Recorder())
+    monkeypatch.setattr(B, "_stream_ptr", lambda stream: None)
+    x = torch.zeros((3, 9, 11, 4), dtype=torch.bfloat16)
+    B.cg_stem_forward(C.c_void_p(16), x, x, B.CgBnParams(), x, x, x)
+    assert seen[0][2:6] == (3, 9, 11, 4)
+
+
+def test_the_stem_rejects_bad_arguments_before_any_launch():
+    lib = B.lib()
+    buf = (C.c_uint8 * 4096)()
+    p = C.c_void_p((C.addressof(buf) + 15) & ~15)
+    bn = C.byref(B.CgBnParams())
+    for h, x, n, ih, iw, c, w, y, ws in ((None, p, 1, 8, 8, 3, p, p, p), (p, None, 1, 8, 8, 3, p, p, p),
+                                         (p, p, 0, 8, 8, 3, p, p, p), (p, p, 1, 0, 8, 3, p, p, p),
+                                         (p, p, 1, 8, -1, 3, p, p, p), (p, p, 1, 8, 8, 4, p, p, p),
+                                         (p, p, 1, 8, 8, 1, p, p, p), (p, p, 1, 8, 8, 3, None, p, p),
+                                         (p, p, 1, 8, 8, 3, p, None, p), (p, p, 1, 8, 8, 3, p, p, None)):
+        assert lib.cg_stem_forward(h, x, n, ih, iw, c, w, bn, None, y, ws, None) == 1   # (the handle is not looked at)
+
+
 def test_status_strings():
     lib = B.lib()
     seen = {lib.cg_status_string(i) for i in range(8)}
