@@ -839,7 +839,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.wp = L.wo; P.hp = L.ho;
   if (k3 && L.stride == 1) {
     // a window: 128 positions and what the last tap reaches behind them, at most two loads of 256
-    const int need = 128 + 2 * (L.w + 2);
+    const int need = L.w <= 512 ? 128 + 2 * (L.w + 2) : 1 << 20;
     if (need <= 512) {
       P.mode = kTc4Window;
       P.wp = L.w + 1; P.hp = L.h + 1;
@@ -849,9 +849,11 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
       P.a_step = 8;
     }
   }
-  P.div_ip.set((uint32_t)(P.wp * P.hp)); P.div_wp.set((uint32_t)P.wp);
-  const long long positions = (long long)L.n * P.wp * P.hp;
-  if (positions > 0x7fffffffll - 65536 || (long long)P.wp * P.hp > 0x3fffffffll) return false;
+  // (the extent of an image first: the products below stay within their types)
+  const long long per_image = (long long)P.wp * P.hp;
+  if (per_image > 0x3fffffffll || L.n * per_image > 0x7fffffffll - 65536) return false;
+  const long long positions = L.n * per_image;
+  P.div_ip.set((uint32_t)per_image); P.div_wp.set((uint32_t)P.wp);
   const int tiles128 = (int)((positions + 127) / 128), tiles256 = (int)((positions + 255) / 256);
   const int tn64 = (L.c_out + 63) / 64, tn128 = (L.c_out + 127) / 128;
 

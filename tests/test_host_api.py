@@ -150,6 +150,27 @@ def test_tap_stacked_algo_eligibility_is_decided_on_the_host():
             assert B.lib().cg_conv_create(C.byref(h), C.byref(d)) == 5, kw   # CG_ERR_CUDA: eligible, no device
 
 
+BEYOND_32_BITS = [dict(h=65536, w=65536), dict(h=65536, w=65536, stride=2), dict(h=32768, w=131072), dict(h=1, w=2 ** 30),
+                  dict(n=2 ** 31 - 1, h=65536, w=65536), dict(n=2 ** 31 - 1, h=3, w=3),
+                  dict(h=65536, w=65536, kh=1, kw=1, pad=0, groups=1)]
+
+
+def test_extents_beyond_32_bits_return_a_status():
+    """Products of extents that leave 32 bits (one is a multiple of 2^32) must not end the process: a layer that no
+    tensor-core kernel can run goes to the direct kernels.  In a process of its own, without devices."""
+    import subprocess
+    import sys
+    base = dict(n=1, h=8, w=8, c_in=128, c_out=64, kh=3, kw=3, stride=1, pad=1, groups=4, requant_shift=8)
+    descs = [{**base, "in_dtype": t, "out_dtype": t, **kw} for t in (B.CG_F32, B.CG_BF16, B.CG_I8) for kw in BEYOND_32_BITS]
+    code = ("import ctypes as C\nfrom paper_1805_12549_b200 import binding as B\nh = C.c_void_p()\n"
+            "for d in %r:\n    print(B.lib().cg_conv_create(C.byref(h), C.byref(B.CgConvDesc(**d))), flush=True)" % (descs,))
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                       env={**os.environ, "CUDA_VISIBLE_DEVICES": ""})
+    got = r.stdout.split()
+    assert r.returncode == 0, (r.returncode, descs[min(len(got), len(descs) - 1)], r.stderr[-500:])
+    assert got == ["5"] * len(descs)                     # CG_ERR_CUDA: described, no device
+
+
 def test_null_handle_calls_are_safe():
     lib = B.lib()
     assert lib.cg_conv_workspace_bytes(None) == 0
