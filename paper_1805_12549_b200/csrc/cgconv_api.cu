@@ -45,7 +45,8 @@ cg_status check_desc(const cg_conv_desc* d) {
   if (d->kh <= 0 || d->kw <= 0 || d->stride <= 0 || d->pad < 0) return CG_ERR_INVALID_ARG;
   if (d->kh != d->kw) return CG_ERR_INVALID_ARG;
   if (d->groups <= 0 || d->c_in % d->groups != 0) return CG_ERR_INVALID_ARG;
-  if ((d->h + 2 * d->pad - d->kh) < 0 || (d->w + 2 * d->pad - d->kw) < 0) return CG_ERR_INVALID_ARG;
+  const long long span_h = d->h + 2ll * d->pad - d->kh, span_w = d->w + 2ll * d->pad - d->kw;
+  if (span_h < 0 || span_w < 0 || span_h > 0x7ffffffell || span_w > 0x7ffffffell) return CG_ERR_INVALID_ARG;
   if (d->in_dtype != CG_F32 && d->in_dtype != CG_BF16 && d->in_dtype != CG_I8) return CG_ERR_INVALID_ARG;
   if (d->out_dtype != d->in_dtype) return CG_ERR_INVALID_ARG;
   if (d->in_dtype == CG_I8 && (d->requant_shift < 1 || d->requant_shift > 31)) return CG_ERR_INVALID_ARG;
@@ -66,8 +67,8 @@ cg::LayerDims make_dims(const cg_conv_desc& d) {
   L.n = d.n; L.h = d.h; L.w = d.w; L.c_in = d.c_in; L.c_out = d.c_out;
   L.kh = d.kh; L.kw = d.kw; L.stride = d.stride; L.pad = d.pad;
   L.groups = d.groups; L.c_p = d.c_in / d.groups; L.c_r = d.c_in - L.c_p;
-  L.ho = (d.h + 2 * d.pad - d.kh) / d.stride + 1;
-  L.wo = (d.w + 2 * d.pad - d.kw) / d.stride + 1;
+  L.ho = (int)((d.h + 2ll * d.pad - d.kh) / d.stride + 1);
+  L.wo = (int)((d.w + 2ll * d.pad - d.kw) / d.stride + 1);
   L.m = (long long)d.n * L.ho * L.wo;
   L.words = (d.c_out + 31) / 32;
   L.eps = d.bn_eps; L.relu = d.relu ? 1 : 0; L.has_residual = d.has_residual ? 1 : 0;

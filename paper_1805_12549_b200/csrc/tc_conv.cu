@@ -1463,6 +1463,9 @@ bool tc_plan(const LayerDims& L_in, int in_dtype, int cond_mode, TcPlan* plan) {
   if (L.c_out % 64 != 0) return false;   // (int8: the last 128-channel tile may be half empty)
   const int xpad = s2 ? 1 : L.pad;                  // zero columns/rows shared between patch rows
   if (L.wo + xpad > kBM) return false;
+  // (rows of an image and of the batch in 32 bits; a larger input would not fit the memory of the GPU)
+  if ((long long)(L.ho + (long long)xpad) * (L.wo + xpad) > 0x3fffffffll) return false;
+  if (L.n * ((long long)L.ho + xpad) > 0x3fffffffll) return false;
   P.elem_bytes = eb;
   P.ck = ck;
   P.planes = s2 ? 4 : 1;

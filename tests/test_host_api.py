@@ -151,6 +151,7 @@ def test_tap_stacked_algo_eligibility_is_decided_on_the_host():
 
 
 BEYOND_32_BITS = [dict(h=65536, w=65536), dict(h=65536, w=65536, stride=2), dict(h=32768, w=131072), dict(h=1, w=2 ** 30),
+                  dict(h=2 ** 30, w=2), dict(h=2 ** 31 - 1, w=2), dict(h=2 ** 31 - 1, w=2 ** 31 - 1),
                   dict(n=2 ** 31 - 1, h=65536, w=65536), dict(n=2 ** 31 - 1, h=3, w=3),
                   dict(h=65536, w=65536, kh=1, kw=1, pad=0, groups=1)]
 
