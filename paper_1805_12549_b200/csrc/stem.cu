@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
       for (int i = 0; i < 2; ++i) {
         uint32_t p[2][8];
         const uint32_t tp = tmem + ((uint32_t)(quad * 32 + 16 * i) << 16) + (uint32_t)(s * 64 + c0);
+        __syncwarp();                                 // (the loads are .aligned; the rows of a ragged tile diverge)
         ptx::tmem_ld_frag16(tp, p[0]);
         ptx::tmem_ld_frag16(tp + 16, p[1]);
         ptx::tmem_ld_wait16(p[0], p[1]);

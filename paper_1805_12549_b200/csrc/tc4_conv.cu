@@ -471,6 +471,7 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
             for (int g = 0; g < 2; ++g) {                      // 16 columns at a time (registers)
               uint32_t p[8], r[8];
               const uint32_t t_p = t_lane + ((uint32_t)(16 * i) << 16) + (uint32_t)(stage * 2 * NT + c0 + 16 * g);
+              __syncwarp();                                    // (the loads are .aligned; what is before them diverges)
               ptx::tmem_ld_frag16(t_p, p);
               if (has_cond) {
                 ptx::tmem_ld_frag16(t_p + NT, r);
@@ -525,12 +526,13 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-              if (m[h] < 0) { bits &= ~(255u << (8 * (2 * i + h))); continue; }
               const long long at = (long long)m[h] * L.c_out + ch + q8;
-              if constexpr (I8) *(uint2*)((uint8_t*)prm.y + at) = make_uint2(out[h][0], out[h][1]);
+              if (m[h] < 0) bits &= ~(255u << (8 * (2 * i + h)));
+              else if constexpr (I8) *(uint2*)((uint8_t*)prm.y + at) = make_uint2(out[h][0], out[h][1]);
               else *(uint4*)((__nv_bfloat16*)prm.y + at) = make_uint4(out[h][0], out[h][1], out[h][2], out[h][3]);
             }
           }
+          __syncwarp();
           // the four lanes of a row group exchange bytes: lane q gets the mask word of row r4 + 8q
           bits = __byte_perm(bits, __shfl_xor_sync(0xffffffffu, bits, 1), sel1);
           bits = __byte_perm(bits, __shfl_xor_sync(0xffffffffu, bits, 2), sel2);
