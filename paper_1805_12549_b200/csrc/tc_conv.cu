@@ -1335,6 +1335,7 @@ tc_compact_cond_kernel(const __grid_constant__ CUtensorMap map_wc, const __grid_
 #pragma unroll
       for (int cb = 0; cb < kWords; ++cb) {
         uint32_t r[32];
+        __syncwarp();                                    // (the load is .aligned; rows behind the list's end skip the rest)
         ptx::tmem_ld32(t_lane + (uint32_t)(cb * 32), r);
         if (!rvalid) continue;
         const uint32_t word = rec[NT + cb];
@@ -1369,6 +1370,7 @@ tc_compact_cond_kernel(const __grid_constant__ CUtensorMap map_wc, const __grid_
     if (threadIdx.x == 192 && ok && items_done)
       atomicAdd(&prm.counters[CNT_EXEC_MACS], items_done * (unsigned long long)kBM * NT * taps * L.c_r);
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 1) ptx::tmem_dealloc(tmem, NT);
