@@ -244,8 +244,8 @@ direct_gated_conv_i8_kernel(LayerDims L, const int8_t* __restrict__ x,
 // for one pair of global loads per product: 156 us for the partial sums of four images of 56x56 (64 channels,
 // c_p = 16), here 17 us; it remains for channel counts that are not multiples of four, channel
 // grouping and the channel-wise gate.
-// fp32 operands are multiplied and added with separate roundings.  Products of bf16 values are exact in fp32
-// (16 significant bits), so the fused multiply-add gives the same sums.
+// Products and sums are rounded separately, for bf16 operands too: their products are exact in fp32 only inside its
+// normal range, so a fused multiply-add is another sum where one is below 2^-126 or beyond 2^128.
 
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
 template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -254,8 +254,7 @@ template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bf
   return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
                      __uint_as_float(v.y & 0xffff0000u));
 }
-__device__ __forceinline__ float mul_add(float a, float b, float c, float) { return __fadd_rn(c, __fmul_rn(a, b)); }
-__device__ __forceinline__ float mul_add(float a, float b, float c, __nv_bfloat16) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float mul_add(float a, float b, float c) { return __fadd_rn(c, __fmul_rn(a, b)); }
 
 template <int NTH, int TC, int PXT, int CH>
 struct DirectTile {
@@ -279,7 +278,7 @@ __global__ void __launch_bounds__(NTH, PXT == 4 ? 2 : 3)
 direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w_base, const T* __restrict__ w_cond,
                    cg_bn_params bn, const float* __restrict__ delta, const T* __restrict__ residual, T* __restrict__ y,
                    uint32_t* __restrict__ mask, float* __restrict__ p_out, int base_only,
-                   unsigned long long* __restrict__ counters, FastDiv div_base, FastDiv div_cond, FastDiv div_kw) {
+                   unsigned long long* __restrict__ counters, FastDiv div_base, FastDiv div_cond, FastDiv div_kw, uint64_t minus_zero) {
   using D = DirectTile<NTH, TC, PXT, CH>;
   constexpr int kStage = D::kStage;
   ptx::grid_launch_dependents();
@@ -358,6 +357,9 @@ direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w
     for (int i = 0; i < PXT; ++i)
 #pragma unroll
       for (int e = 0; e < CH; ++e) acc[i][e] = 0.f;
+    [[maybe_unused]] uint64_t a2[PXT][2];                    // CH = 4: the accumulators, two channels each
+#pragma unroll
+    for (int i = 0; i < PXT; ++i) a2[i][0] = a2[i][1] = 0;
     const int kt = L.kh * L.kw * cw, stages = (kt + kStage - 1) / kStage;
     put(b);
     __syncthreads();
@@ -383,15 +385,19 @@ direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w
         for (int i = 0; i < PXT; ++i) {
           if (!ok[h][i]) continue;
           if constexpr (CH == 1) {
-            acc[i][0] = mul_add(xv[h][i].x, wv[h][0].x, acc[i][0], T{}); acc[i][0] = mul_add(xv[h][i].y, wv[h][0].y, acc[i][0], T{});
-            acc[i][0] = mul_add(xv[h][i].z, wv[h][0].z, acc[i][0], T{}); acc[i][0] = mul_add(xv[h][i].w, wv[h][0].w, acc[i][0], T{});
+            acc[i][0] = mul_add(xv[h][i].x, wv[h][0].x, acc[i][0]); acc[i][0] = mul_add(xv[h][i].y, wv[h][0].y, acc[i][0]);
+            acc[i][0] = mul_add(xv[h][i].z, wv[h][0].z, acc[i][0]); acc[i][0] = mul_add(xv[h][i].w, wv[h][0].w, acc[i][0]);
           } else {
+            // Two channels per instruction, each rounded like the scalar operation.  The product is a*b + (-0), the
+            // same in every case; -0 is a kernel argument, because of a product and a sum that it knows the compiler
+            // makes one fused operation, .rn or not (its results differed from the definition's).
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float v = q == 0 ? xv[h][i].x : q == 1 ? xv[h][i].y : q == 2 ? xv[h][i].z : xv[h][i].w;
-            acc[i][0] = mul_add(v, wv[h][q].x, acc[i][0], T{}); acc[i][1] = mul_add(v, wv[h][q].y, acc[i][1], T{});
-            acc[i][2] = mul_add(v, wv[h][q].z, acc[i][2], T{}); acc[i][3] = mul_add(v, wv[h][q].w, acc[i][3], T{});
-          }
+            for (int q = 0; q < 4; ++q) {
+              const float v = q == 0 ? xv[h][i].x : q == 1 ? xv[h][i].y : q == 2 ? xv[h][i].z : xv[h][i].w;
+              const uint64_t vv = ptx::pack_f32x2(v, v);
+              a2[i][0] = ptx::add_f32x2(a2[i][0], ptx::fma_f32x2(vv, ptx::pack_f32x2(wv[h][q].x, wv[h][q].y), minus_zero));
+              a2[i][1] = ptx::add_f32x2(a2[i][1], ptx::fma_f32x2(vv, ptx::pack_f32x2(wv[h][q].z, wv[h][q].w), minus_zero));
+            }
           }
         }
       };
@@ -412,6 +418,13 @@ direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w
       b ^= 1;
       if (st + 1 < stages) put(b);
       __syncthreads();
+    }
+    if constexpr (CH == 4) {
+#pragma unroll
+      for (int i = 0; i < PXT; ++i) {
+        ptx::unpack_f32x2(a2[i][0], acc[i][0], acc[i][1]);
+        ptx::unpack_f32x2(a2[i][1], acc[i][2], acc[i][3]);
+      }
     }
   };
 
@@ -519,7 +532,7 @@ int launch_tile(const LayerDims& L, const void* x, const void* w_base, const voi
   cfg.attrs = attr; cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, direct_tile_kernel<T, NTH, TC, PXT, CH>, L, (const T*)x, (const T*)w_base, (const T*)w_cond,
                                            bn, delta, (const T*)residual, (T*)y, mask, (float*)p_out, base_only, counters,
-                                           div_base, div_cond, div_kw);
+                                           div_base, div_cond, div_kw, (uint64_t)0x8000000080000000ull);
   return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
 }
 

@@ -54,3 +54,31 @@ def test_taps_in_the_padding_are_left_out():
     np.testing.assert_array_equal(mask, ref.mask)
     np.testing.assert_array_equal(np.isfinite(y), np.isfinite(ref.y))
     g.close()
+
+
+SIZES_OF_PRODUCTS = [(O.Shape(2, 8, 8, 16, 16, groups=2), "one channel per thread"),
+                     (O.Shape(40, 15, 16, 16, 32, groups=2), "two pixels per thread"),
+                     (O.Shape(64, 20, 16, 8, 64, groups=2), "four pixels per thread")]
+
+
+@pytest.mark.parametrize("s,why", SIZES_OF_PRODUCTS, ids=[w for _, w in SIZES_OF_PRODUCTS])
+def test_bf16_products_outside_the_normal_range_are_rounded_by_themselves(s, why):
+    """Products below 2^-126 round to multiples of 2^-149 and products from 2^128 on are infinite before they are added:
+    a fused multiply-add would keep what the separate multiplication of the definition loses."""
+    c = K.make_float_case("tiny", s, "bf16", density=0.5, smooth=False)
+    c.x, c.wb, c.wc = (np.ldexp(a, -68).astype(np.float32) for a in (c.x, c.wb, c.wc))
+    c.x[0, 0, 0, :2] = np.float32(2.0) ** 64     # P = -2^127 + 2^128: infinite by itself
+    c.wb[5] = 0.0
+    c.wb[5, 1, 1, :2] = -np.float32(2.0) ** 63, np.float32(2.0) ** 64
+    ref = K.run_oracle(c)
+    assert np.isinf(ref.p[0, 0, 0, 5])
+    g = K.GpuCase(c, algo=1)
+    y, mask, st = g.run()
+    K.compare(c, ref, y, mask, st, exact=True)
+    import torch
+    from paper_1805_12549_b200 import binding as B
+    p = torch.empty((s.m, s.c_out), dtype=torch.float32, device="cuda")
+    B.cg_conv_partial_sums(g.conv.handle, g.x, g.wb, p)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(p.cpu().numpy().reshape(ref.p.shape), ref.p)
+    g.close()
