@@ -6,6 +6,7 @@
 // sum only if its own gate fired (Eq. 1), applies the path's batch norm and ReLU, and the
 // warp's ballot is the mask word.  Floating-point sums run in the order (r, s, c_in) with
 // separately rounded multiply and add, so results do not depend on the launch shape.
+#include <algorithm>
 #include <cstring>
 
 #include "common.cuh"
@@ -247,6 +248,20 @@ direct_gated_conv_i8_kernel(LayerDims L, const int8_t* __restrict__ x,
 // Products and sums are rounded separately, for bf16 operands too: their products are exact in fp32 only inside its
 // normal range, so a fused multiply-add is another sum where one is below 2^-126 or beyond 2^128.
 
+// The filter rows [r0, r0 + kh) and columns [s0, s0 + kw) that some output pixel meets inside the image; the others
+// meet padding only, and are not run through.  (All of them unless the image is smaller than the filter's reach: a
+// 3x3 layer on one pixel has one tap, 128 channels 23.2 us with all nine run through, 7x7 on 2x2 images 9 of 49.)
+struct TapBox {
+  int r0, s0, kh, kw;
+};
+TapBox tap_box(const LayerDims& L) {
+  auto first = [&](int out) { return (int)std::max(0ll, L.pad - (out - 1ll) * L.stride); };
+  auto end = [&](int k, int in) { return (int)std::min((long long)k, (long long)L.pad + in); };
+  TapBox b = {first(L.ho), first(L.wo), 0, 0};
+  b.kh = std::max(0, end(L.kh, L.h) - b.r0); b.kw = std::max(0, end(L.kw, L.w) - b.s0);   // (0: every sum is empty)
+  return b;
+}
+
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
 template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
 template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
@@ -273,14 +288,16 @@ struct DirectTile {
   };
 };
 
-template <typename T, int NTH, int TC, int PXT, int CH>
+// BOX: the taps of tap_box() only (an instance of its own: the index arithmetic of its weights costs the others 4 %)
+template <typename T, int NTH, int TC, int PXT, int CH, bool BOX>
 __global__ void __launch_bounds__(NTH, PXT == 4 ? 2 : 3)
 direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w_base, const T* __restrict__ w_cond,
                    cg_bn_params bn, const float* __restrict__ delta, const T* __restrict__ residual, T* __restrict__ y,
                    uint32_t* __restrict__ mask, float* __restrict__ p_out, int base_only,
-                   unsigned long long* __restrict__ counters, FastDiv div_base, FastDiv div_cond, FastDiv div_kw, uint64_t minus_zero) {
+                   unsigned long long* __restrict__ counters, FastDiv div_base, FastDiv div_cond, FastDiv div_kw, TapBox box, uint64_t minus_zero) {
   using D = DirectTile<NTH, TC, PXT, CH>;
   constexpr int kStage = D::kStage;
+  const TapBox taps = BOX ? box : TapBox{0, 0, L.kh, L.kw};
   ptx::grid_launch_dependents();
   extern __shared__ __align__(16) uint8_t dyn[];
   typename D::Buffers& S = *reinterpret_cast<typename D::Buffers*>(dyn);
@@ -311,14 +328,14 @@ direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w
 
   // stage of the sums over `cw` channels from c_lo on: K elements [k0, k0 + kStage) into registers ...
   auto fetch = [&](const T* w, const FastDiv& div, int c_lo, int cw, int k0) {
-    const int kt = L.kh * L.kw * cw;
+    const int kt = taps.kh * taps.kw * cw, w_row = L.kh * L.kw * cw;
     okr = 0;
 #pragma unroll
     for (int i = 0; i < kXUnits; ++i) {
       const int u = tid + NTH * i, k = k0 + u / D::TM * 4;
       xr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (have_pixel && u < kXTotal && k < kt) {
-        const int tap = (int)div.div(k), ci = k - tap * cw, r = (int)div_kw.div(tap), s = tap - r * L.kw;
+        const int tap = (int)div.div(k), ci = k - tap * cw, rr = (int)div_kw.div(tap), r = taps.r0 + rr, s = taps.s0 + tap - rr * taps.kw;
         if (h0 + r >= 0 && h0 + r < L.h && w0 + s >= 0 && w0 + s < L.w) {
           xr[i] = load4<T>(x + x_off + ((long long)r * L.w + s) * L.c_in + c_lo + ci);
           okr |= 1u << i;
@@ -329,7 +346,14 @@ direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w
     for (int i = 0; i < kWUnits; ++i) {
       const int u = tid + NTH * i, c = u % TC, k = k0 + u / TC * 4;
       wr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (u < kWTotal && k < kt && c0 + c < L.c_out) wr[i] = load4<T>(w + (long long)(c0 + c) * kt + k);
+      if (u < kWTotal && k < kt && c0 + c < L.c_out) {
+        int at = k;                                        // element of the channel's filter
+        if (BOX) {
+          const int tap = (int)div.div(k), rr = (int)div_kw.div(tap);
+          at = ((taps.r0 + rr) * L.kw + taps.s0 + tap - rr * taps.kw) * cw + k - tap * cw;
+        }
+        wr[i] = load4<T>(w + (long long)(c0 + c) * w_row + at);
+      }
     }
   };
   // ... and from there to shared memory
@@ -360,7 +384,7 @@ direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w
     [[maybe_unused]] uint64_t a2[PXT][2];                    // CH = 4: the accumulators, two channels each
 #pragma unroll
     for (int i = 0; i < PXT; ++i) a2[i][0] = a2[i][1] = 0;
-    const int kt = L.kh * L.kw * cw, stages = (kt + kStage - 1) / kStage;
+    const int kt = taps.kh * taps.kw * cw, stages = (kt + kStage - 1) / kStage;
     put(b);
     __syncthreads();
     for (int st = 0; st < stages; ++st) {
@@ -505,8 +529,8 @@ direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w
   }
 }
 
-template <typename T, int NTH, int TC, int PXT, int CH>
-int launch_tile(const LayerDims& L, const void* x, const void* w_base, const void* w_cond, const cg_bn_params& bn,
+template <typename T, int NTH, int TC, int PXT, int CH, bool BOX = false>
+int launch_tile(const LayerDims& L, const TapBox& taps, const void* x, const void* w_base, const void* w_cond, const cg_bn_params& bn,
                 const float* delta, const void* residual, void* y, uint32_t* mask, void* p_out, int base_only,
                 unsigned long long* counters, cudaStream_t stream) {
   using D = DirectTile<NTH, TC, PXT, CH>;
@@ -516,12 +540,12 @@ int launch_tile(const LayerDims& L, const void* x, const void* w_base, const voi
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
   if (smem > 48 * 1024 && !set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(direct_tile_kernel<T, NTH, TC, PXT, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(direct_tile_kernel<T, NTH, TC, PXT, CH, BOX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     set[dev] = true;
   }
   FastDiv div_base, div_cond, div_kw;
-  div_base.set((uint32_t)L.c_p); div_cond.set((uint32_t)(L.c_r > 0 ? L.c_r : 1)); div_kw.set((uint32_t)L.kw);
+  div_base.set((uint32_t)L.c_p); div_cond.set((uint32_t)(L.c_r > 0 ? L.c_r : 1)); div_kw.set((uint32_t)std::max(1, BOX ? taps.kw : L.kw));
   // a programmatic dependent launch, like the tensor-core kernels
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
@@ -530,9 +554,9 @@ int launch_tile(const LayerDims& L, const void* x, const void* w_base, const voi
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, direct_tile_kernel<T, NTH, TC, PXT, CH>, L, (const T*)x, (const T*)w_base, (const T*)w_cond,
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, direct_tile_kernel<T, NTH, TC, PXT, CH, BOX>, L, (const T*)x, (const T*)w_base, (const T*)w_cond,
                                            bn, delta, (const T*)residual, (T*)y, mask, (float*)p_out, base_only, counters,
-                                           div_base, div_cond, div_kw, (uint64_t)0x8000000080000000ull);
+                                           div_base, div_cond, div_kw, taps, (uint64_t)0x8000000080000000ull);
   return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
 }
 
@@ -547,10 +571,16 @@ template <typename T>
 int launch_tiles(const LayerDims& L, const void* x, const void* w_base, const void* w_cond, const cg_bn_params& bn,
                  const float* delta, const void* residual, void* y, uint32_t* mask, void* p_out, int base_only,
                  unsigned long long* counters, cudaStream_t stream) {
-#define CG_TILE(TC, PXT, CH) launch_tile<T, 256, TC, PXT, CH>(L, x, w_base, w_cond, bn, delta, residual, y, mask, p_out, base_only, counters, stream)
+#define CG_TILE(TC, PXT, CH, ...) launch_tile<T, 256, TC, PXT, CH, ##__VA_ARGS__>(L, taps, x, w_base, w_cond, bn, delta, residual, y, mask, p_out, base_only, counters, stream)
   const int tc = L.c_out <= 16 ? 16 : (L.c_out <= 32 ? 32 : 64);
   const long long outputs = L.m * ((L.c_out + tc - 1) / tc * tc);
   const int v = outputs >= 900000 ? 4 : (outputs >= 100000 ? 2 : 1);
+  const TapBox taps = tap_box(L);
+  // images smaller than the filter's reach (us with all taps and with the box, before them the kernel of one warp per
+  // output: fp32, one pixel x 128 23.2, 5.1, 9.2; 2x2 x 64, 7x7 58, 13.5, 41).  Large layers, where a product of this
+  // instance costs four times as much: a fifth of the taps and fewer (4000 x one pixel x 64 53, 13; with 3 of 9 taps
+  // 64 x 1x1000 x 32 71, 92)
+  if (taps.kh * taps.kw < L.kh * L.kw && (v == 1 || 5 * taps.kh * taps.kw <= L.kh * L.kw)) return CG_TILE(16, 1, 1, true);
   if (v == 1) return CG_TILE(16, 1, 1);
   if (tc == 16) return CG_TILE(16, 2, 4);
   if (tc == 32) return v == 4 ? CG_TILE(32, 4, 4) : CG_TILE(32, 2, 4);

@@ -21,6 +21,14 @@ SHAPES = [
     (O.Shape(70, 18, 16, 8, 64, groups=2), "four pixels per thread, 64 channels"),
     (O.Shape(2, 11, 9, 16, 16, 5, 5, 2, 2, groups=4), "5x5, stride 2"),
     (O.Shape(2, 7, 7, 16, 16, 1, 1, 1, 0, groups=1), "1x1, no conditional path"),
+    (O.Shape(3, 1, 1, 16, 40, groups=4), "one pixel: one tap of nine"),
+    (O.Shape(2, 1, 4, 64, 16, groups=2), "one row: three taps of nine"),
+    (O.Shape(2, 2, 3, 16, 16, 7, 7, 1, 3, groups=4), "15 taps of 49"),
+    (O.Shape(1, 3, 1, 16, 16, 5, 5, 2, 2, groups=2), "stride 2, taps from the first on"),
+    (O.Shape(1, 2, 9, 16, 16, 3, 3, 4, 2, groups=2), "stride 4, padding 2"),
+    (O.Shape(2, 1, 1, 16, 16, 3, 3, 20, 5, groups=2), "padding only"),
+    (O.Shape(1500, 1, 4, 8, 64, groups=2), "one row, two pixels per thread"),
+    (O.Shape(4000, 4, 1, 8, 64, groups=2), "one column, four pixels per thread"),
 ]
 
 
