@@ -59,7 +59,11 @@ typedef enum {
 
 /* How the tensor-core path treats the conditional path (Eq. 1, second case). */
 typedef enum {
-  CG_COND_AUTO = 0,
+  CG_COND_AUTO = 0,      /* by kernel: skip tiles without a firing gate (pixel- and channel-major); compute R
+                            for every row, but for column tiles whose thresholds are all +inf (window;
+                            tap-stacked: for every row).  A layer whose finite thresholds shut most of its
+                            128-pixel tiles is faster with CG_COND_SKIP_TILES: 512 channels, 4x4, batch 256,
+                            nothing fires: 19 us against 28 */
   CG_COND_DENSE = 1,     /* compute R for every row of every tile (gate density 1.0 behaviour)  */
   CG_COND_SKIP_TILES = 2,/* skip tiles (and column blocks) in which no gate fired               */
   CG_COND_COMPACT = 3    /* additionally gather only the pixel rows in which a gate fired       */
@@ -138,7 +142,8 @@ typedef struct {
   int64_t dense_macs;    /* multiplications of the ungated layer: outputs * k^2 * c_in         */
   int64_t gated_macs;    /* the method's count (Section 4): k^2*(c_p*outputs + c_r*active)     */
   int64_t executed_macs; /* multiplications the kernels really issued, at tile/row granularity */
-  int64_t tiles_total;   /* conditional-path tiles (row block x column block) considered       */
+  int64_t tiles_total;   /* conditional-path tiles (row block x column block) considered (none of
+                            the window kernel's column tiles whose thresholds are all +inf)    */
   int64_t tiles_skipped; /* ... of which skipped because no gate fired in them                 */
   int64_t rows_total;    /* pixel rows x column blocks considered                              */
   int64_t rows_active;   /* ... of which contained at least one firing gate                    */
@@ -165,7 +170,7 @@ typedef struct {
  *   tap-stacked kernel:   BF16, 3x3, stride 1, pad 1, c_in = c_out = 64, c_in/G a multiple of 16, image
  *                         width at most 128, no channel grouping, no channel-wise gate, no row compaction
  *                         (AUTO and TENSOR choose it when the width divides 32).
- *   window kernel (AUTO only): BF16 or I8, conditional path AUTO or DENSE (R is computed for every pixel), 3x3
+ *   window kernel (AUTO only): BF16 or I8, conditional path AUTO or DENSE (no tile waits for its gates), 3x3
  *                         with pad 1 and any stride up to 8, or 1x1 with groups = 1; c_in a multiple of 64
  *                         (I8: 128), c_out a multiple of 32, c_in/G equal to 16 or 32 (I8: 32 or 64) or a multiple
  *                         of 64 (128); no channel grouping, no channel-wise gate.

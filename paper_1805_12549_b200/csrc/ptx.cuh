@@ -361,6 +361,11 @@ __device__ __forceinline__ void stmatrix_x4_trans(uint32_t smem_addr, uint32_t r
                : "memory");
 }
 
+// One column for the warp's 32 lanes.
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t& r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r) : : "memory");
+}
 // N = 16 or 32 columns for the warp's 32 lanes, without waiting: several loads can be in flight.
 // Every use of the registers must come after tmem_ld_wait<N>() on the same array.
 template <int N>
@@ -521,6 +526,12 @@ __device__ __forceinline__ uint4 ld_cluster_16(uint32_t addr, uint32_t rank) {
       : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
       : "r"(addr), "r"(rank)
       : "memory");
+  return v;
+}
+
+__device__ __forceinline__ uint32_t ld_cluster_4(uint32_t addr, uint32_t rank) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(map_cluster(addr, rank)) : "memory");
   return v;
 }
 

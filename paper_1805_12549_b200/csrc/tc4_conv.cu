@@ -16,6 +16,11 @@
 // (N = 64) jobs deep, and both are computed for every pixel: a block of 128 pixels and 64 channels always
 // holds a firing gate at the densities in use, and waiting for the gate costs more than it saves.  So the
 // K loop is one run of MMAs per job and the epilogue one pass: d = (P >= t), y = f(BN1(P)) or f(BN2(P+R)).
+// Pairs look at the thresholds, though: the jobs of a column tile in which no gate can fire run the base rows only
+// (run_roles<BASE>; all thresholds +inf, us for all rows and for the base rows: 512@4x4 b256 28 and 14.6, 256@14x14 b64
+// 18.3 and 13.2, 512@7x7 b64 18.0 and 11.7).  That is a second copy of the role code, chosen by a look that a warp
+// takes while the block sets up: with row tables and bounds as variables of one copy, and a function call in its
+// epilogue, every layer took 0.5 to 1.5 us more.
 //
 // Jobs are 256 pixels of a CTA pair (cta_group::2): each SM holds half of a job's pixels and half of its
 // weights, which halves what an SM has to fetch from L2 and what an MMA reads of shared memory (one CTA's
@@ -44,6 +49,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "direct_point.cuh"
 #include "ptx.cuh"
 #include "tc4_conv.cuh"
 
@@ -70,6 +76,7 @@ struct Tc4Params {
   void* y;
   uint32_t* mask;
   unsigned long long* counters;
+  const __nv_bfloat16 *x, *w_cond;   // (read by infinite_sums only)
   Tc4Plan P;
 };
 
@@ -81,6 +88,7 @@ struct Shared4 {
   uint32_t tmem_base;
   uint32_t abort_flag;
   uint32_t active, rows_active;
+  uint32_t maybe_shut;   // no gate of the column tile could fire when the block started
 };
 static_assert(sizeof(Shared4) <= kOffConsts, "barrier block");
 
@@ -181,14 +189,54 @@ __device__ __forceinline__ int finish_q(int mul, long long off, int acc, int shi
   return (int)(q < lo ? lo : (q > 127 ? 127 : q));
 }
 
-template <int NT, bool I8, bool PAIR>
-__global__ void __launch_bounds__(kT4Threads, 1)
-tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wb,
-                      const __grid_constant__ CUtensorMap map_wc, const __grid_constant__ Tc4Params prm) {
-  extern __shared__ uint8_t smem_raw[];
+// Whether no gate of the column tile can fire: thresholds of +inf (or not a number); int8: beyond every sum.  (Finite
+// thresholds that no partial sum happens to reach are not looked for: the conditional rows would have to wait for the
+// base rows and the epilogue.)  Taken by a whole warp; reads past L1, so that it may run before the kernels in front
+// of this one are done.
+template <int NT, bool I8>
+__device__ __forceinline__ bool gates_shut(const Tc4Params& prm, int tile_n, int lane) {
+  bool open = false;
+#pragma unroll
+  for (int c = 0; c < NT; c += 32) {
+    const int ch = tile_n * NT + c + lane;
+    if (ch >= prm.L.c_out) continue;
+    if (I8) open = open || __ldcg(prm.bn.q_gate_thr + ch) <= prm.L.kh * prm.L.kw * prm.L.c_p * (128 * 128);
+    else open = open || __ldcg(prm.delta + ch) < __int_as_float(0x7f800000);
+  }
+  return !__any_sync(0xffffffffu, open);
+}
+
+// A tie fires, at +inf too: outputs whose partial sum of +inf meets a threshold of +inf, in a column tile without
+// conditional rows.  Lane by row (pixel m, or -1), 32 channels from ch on: R comes from its definition.
+__device__ __forceinline__ void infinite_sums(const Tc4Params& prm, uint32_t t_col, const float* t, const float* t2,
+                                           const float4* k, int ch, int m) {
+  const LayerDims& L = prm.L;
+  const int row = m / L.wo, n = row / L.ho;
+#pragma unroll 1
+  for (int col = 0; col < 32; ++col) {
+    uint32_t v;
+    __syncwarp();                                              // (also orders the lanes' stores to y)
+    ptx::tmem_ld1(t_col + (uint32_t)col, v);
+    const float p = __uint_as_float(v);
+    const int c = 8 * ((col >> 1) & 3) + 2 * (col >> 3) + (col & 1);   // (the weight tiles' row order)
+    if (m < 0 || !(p >= t[c]) || !(p <= t2[c])) continue;
+    const float sum = p + conv_point<__nv_bfloat16>(L, prm.x, prm.w_cond, n, row - n * L.ho, m - row * L.wo, ch + c, L.c_p, L.c_r);
+    const long long at = (long long)m * L.c_out + ch + c;
+    float o = fmaf(k[c].z, sum, k[c].w);
+    if (prm.residual) o += __bfloat162float(prm.residual[at]);
+    if (L.relu) o = fmaxf(o, 0.f);
+    ((__nv_bfloat16*)prm.y)[at] = __float2bfloat16_rn(o);
+  }
+  __syncwarp();
+}
+
+// What the warps of a block do (see the top of the file).  BASE: the jobs of a column tile whose gates cannot fire, which run
+// the base rows only.
+template <int NT, bool I8, bool PAIR, bool BASE>
+__device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtensorMap& map_wb, const CUtensorMap& map_wc,
+                                          const Tc4Params& prm, uint8_t* smem, int warp, int lane, int part, int tile_n,
+                                          int group, int groups, int jobs, uint32_t tmem) {
   constexpr bool SPLIT = !PAIR;
-  ptx::grid_launch_dependents();
-  uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
   const LayerDims& L = prm.L;
   const Tc4Plan& P = prm.P;
   Shared4* sh = (Shared4*)smem;
@@ -202,43 +250,11 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   constexpr int kAcc = 512 / (2 * NT);                         // accumulator pairs in TMEM
   constexpr int kTileRows = PAIR ? NT / 2 : NT;                // rows of a weight tile in this CTA
   constexpr uint32_t kTile = kTileRows * 128;
-
-  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const unsigned members = PAIR ? 2u : (unsigned)P.split;      // CTAs of a cluster
-  const int part = (int)(blockIdx.x % members);                // rank in the cluster
-  const int block = (int)(blockIdx.x / members), blocks = (int)(gridDim.x / members);
-  // jobs of this cluster: a fixed column tile, every `groups`-th pixel tile (split layers: one job)
-  const int tile_n = block % P.tiles_n, group = block / P.tiles_n, groups = blocks / P.tiles_n;
-  const int jobs = group < P.tiles_m ? (P.tiles_m - group + groups - 1) / groups : 0;
-  const int lo = SPLIT ? P.lo[part] : 0, hi = SPLIT ? P.lo[part + 1] : P.rows;
-  const bool has_cond = L.c_r > 0;
+  const int lo = SPLIT ? P.lo[part] : 0, hi = BASE ? P.base_rows : SPLIT ? P.lo[part + 1] : P.rows;
+  const bool has_cond = !BASE && L.c_r > 0;
+  const uint32_t table = ptx::smem_u32(smem + kOffRows);
   // first position of this CTA in job j
   auto job_pos = [&](int j) { return PAIR ? (group + j * groups) * 256 + part * 128 : (group + j * groups) * 128; };
-
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < P.na; ++i) { ptx::mbar_init(&sh->a_full[i], 1); ptx::mbar_init(&sh->a_empty[i], 1); }
-    for (int i = 0; i < P.nb; ++i) { ptx::mbar_init(&sh->b_full[i], 1); ptx::mbar_init(&sh->b_empty[i], 1); }
-    for (int i = 0; i < kAcc; ++i) {
-      ptx::mbar_init(&sh->acc_full[i], 1);
-      ptx::mbar_init(&sh->acc_empty[i], (PAIR ? 2 : 1) * NT / 8);   // warps per job, of both CTAs of a pair
-    }
-    ptx::mbar_init(&sh->turn[0], 1); ptx::mbar_init(&sh->turn[1], 1);
-    sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0;
-    ptx::fence_mbar_init();
-  }
-  if (threadIdx.x == 32 * 2) { ptx::prefetch_tensormap(&map_x); ptx::prefetch_tensormap(&map_wb); ptx::prefetch_tensormap(&map_wc); }
-  // (the row table moves to shared memory: an indexed read of a kernel parameter costs hundreds of cycles)
-  for (int i = (int)threadIdx.x - kEpiWarp0 * 32; i >= 0 && i < P.rows; i += kT4Threads)
-    ((uint4*)(smem + kOffRows))[i] = ((const uint4*)P.row)[i];
-  const uint32_t table = ptx::smem_u32(smem + kOffRows);
-  __syncwarp();
-  if (warp == 1) { if (PAIR) ptx::tmem_alloc_pair(&sh->tmem_base, 512); else ptx::tmem_alloc(&sh->tmem_base, 512); }
-  ptx::tc_fence_before();
-  if (PAIR) ptx::cluster_sync(); else __syncthreads();
-  ptx::tc_fence_after();
-  // everything above touched only this cluster's own state
-  ptx::grid_dependency_wait();
-  const uint32_t tmem = sh->tmem_base;
   // address of the leader's copy of a barrier, for copies and arrivals
   auto leader = [&](uint64_t* bar) { return PAIR ? ptx::map_cluster(ptx::smem_u32(bar), 0) : ptx::smem_u32(bar); };
   // (a pair's leader announces both CTAs' bytes; the other CTA's copies count on the leader's barrier: an
@@ -341,8 +357,8 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
         ptx::tc_fence_after();
         const uint32_t d_p = tmem + (uint32_t)(stage * 2 * NT);
         Cursor ca, cb;
-        ca.at((unsigned)j * (unsigned)P.a_per_job, (unsigned)P.na);
-        if (P.resident) cb = Cursor{0, 0}; else cb.at((unsigned)j * (unsigned)P.b_per_job, (unsigned)P.nb);
+        ca.at((unsigned)j * (unsigned)(BASE ? P.a_base : P.a_per_job), (unsigned)P.na);
+        if (P.resident) cb = Cursor{0, 0}; else cb.at((unsigned)j * (unsigned)(BASE ? P.b_base : P.b_per_job), (unsigned)P.nb);
         int sa = 0, sb_base = 0, sb_cond = 0;                  // slots in use
         bool a_seen = false, b_seen = false;                   // the next row's slots were full when last looked at
         const bool weights_here = P.resident && j >= 2;        // (this issuer has waited for every stage)
@@ -360,7 +376,7 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
             cb.next(P.nb);
           }
           if (!ok) break;
-          if (i == P.turn) ptx::mbar_arrive(&sh->turn[j & 1]);
+          if (i == (BASE ? P.turn_base : P.turn)) ptx::mbar_arrive(&sh->turn[j & 1]);
           if (i + 1 < hi) {
             // a look at the next row's barriers, whose answer arrives while this row's MMAs are issued
             a_seen = (next.flags & kRowANew) && ptx::mbar_test_wait(&sh->a_full[ca.slot], ca.par);
@@ -540,9 +556,14 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
           rows_active += bits != 0u ? 1u : 0u;
           const int m_word = __shfl_sync(0xffffffffu, own, r4 + q8);
           if (prm.mask && m_word >= 0) prm.mask[(long long)m_word * L.words + (ch >> 5)] = bits;
+          return bits;
         };
         if (ch < L.c_out) {                                    // (uniform over the warp)
-          if (I8) finish(std::false_type{}, std::false_type{});
+          if constexpr (BASE && !I8) {
+            const uint32_t fired = finish(std::true_type{}, std::true_type{});
+            if (__any_sync(0xffffffffu, fired != 0u))
+              infinite_sums(prm, t_lane + (uint32_t)(stage * 2 * NT + c0), s_t + c0, s_t2 + c0, s_k + c0, ch, own);
+          } else if (I8) finish(std::false_type{}, std::false_type{});
           else if (two_sided) finish(std::true_type{}, std::true_type{});
           else if (has_res) finish(std::false_type{}, std::true_type{});
           else finish(std::false_type{}, std::false_type{});
@@ -653,6 +674,79 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     rows_active = __reduce_add_sync(0xffffffffu, rows_active);
     if (lane == 0) { atomicAdd(&sh->active, active); atomicAdd(&sh->rows_active, rows_active); }
   }
+}
+
+template <int NT, bool I8, bool PAIR>
+__global__ void __launch_bounds__(kT4Threads, 1)
+tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wb,
+                      const __grid_constant__ CUtensorMap map_wc, const __grid_constant__ Tc4Params prm) {
+  extern __shared__ uint8_t smem_raw[];
+  constexpr bool SPLIT = !PAIR;
+  ptx::grid_launch_dependents();
+  uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
+  const LayerDims& L = prm.L;
+  const Tc4Plan& P = prm.P;
+  Shared4* sh = (Shared4*)smem;
+  constexpr int kAcc = 512 / (2 * NT);                         // accumulator pairs in TMEM
+
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const unsigned members = PAIR ? 2u : (unsigned)P.split;      // CTAs of a cluster
+  const int part = (int)(blockIdx.x % members);                // rank in the cluster
+  const int block = (int)(blockIdx.x / members), blocks = (int)(gridDim.x / members);
+  // jobs of this cluster: a fixed column tile, every `groups`-th pixel tile (split layers: one job)
+  const int tile_n = block % P.tiles_n, group = block / P.tiles_n, groups = blocks / P.tiles_n;
+  const int jobs = group < P.tiles_m ? (P.tiles_m - group + groups - 1) / groups : 0;
+  const bool has_cond = L.c_r > 0;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < P.na; ++i) { ptx::mbar_init(&sh->a_full[i], 1); ptx::mbar_init(&sh->a_empty[i], 1); }
+    for (int i = 0; i < P.nb; ++i) { ptx::mbar_init(&sh->b_full[i], 1); ptx::mbar_init(&sh->b_empty[i], 1); }
+    for (int i = 0; i < kAcc; ++i) {
+      ptx::mbar_init(&sh->acc_full[i], 1);
+      ptx::mbar_init(&sh->acc_empty[i], (PAIR ? 2 : 1) * NT / 8);   // warps per job, of both CTAs of a pair
+    }
+    ptx::mbar_init(&sh->turn[0], 1); ptx::mbar_init(&sh->turn[1], 1);
+    sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0;
+    ptx::fence_mbar_init();
+  }
+  if (threadIdx.x == 32 * 2) { ptx::prefetch_tensormap(&map_x); ptx::prefetch_tensormap(&map_wb); ptx::prefetch_tensormap(&map_wc); }
+  // (the row table moves to shared memory: an indexed read of a kernel parameter costs hundreds of cycles)
+  for (int i = (int)threadIdx.x - kEpiWarp0 * 32; i >= 0 && i < P.rows; i += kT4Threads)
+    ((uint4*)(smem + kOffRows))[i] = ((const uint4*)P.row)[i];
+  if (PAIR && P.base_rows && warp == kEpiWarp0 + kEpiWarps - 1) {
+    // a first look, which costs nothing here; an open gate stays open for this launch whatever is written meanwhile
+    const bool shut = gates_shut<NT, I8>(prm, tile_n, lane);
+    if (lane == 0) sh->maybe_shut = shut ? 1u : 0u;
+  }
+  __syncwarp();
+  if (warp == 1) { if (PAIR) ptx::tmem_alloc_pair(&sh->tmem_base, 512); else ptx::tmem_alloc(&sh->tmem_base, 512); }
+  ptx::tc_fence_before();
+  if (PAIR) ptx::cluster_sync(); else __syncthreads();
+  ptx::tc_fence_after();
+  // everything above touched only this cluster's own state
+  ptx::grid_dependency_wait();
+  const uint32_t tmem = sh->tmem_base;
+  bool shut = false;
+  if constexpr (PAIR) {
+    // both CTAs of a pair have to choose alike: only where both saw shut gates, each looks at what counts
+    if (P.base_rows && sh->maybe_shut && ptx::ld_cluster_4(ptx::smem_u32(&sh->maybe_shut), (uint32_t)(part ^ 1)))
+      shut = gates_shut<NT, I8>(prm, tile_n, lane);
+  }
+  if (shut) {
+    if constexpr (PAIR) {
+      // the base rows move together; another row may now be the last of its patch
+      const int i = (int)threadIdx.x;
+      if (i < P.rows && ((P.base_mask >> i) & 1ull)) {
+        uint4 row = ((const uint4*)P.row)[i];
+        row.w = (row.w & ~(uint32_t)kRowAFree) | ((row.w & kRowAFreeBase) ? (uint32_t)kRowAFree : 0u);
+        ((uint4*)(smem + kOffRows))[__popcll(P.base_mask & ((1ull << i) - 1ull))] = row;
+      }
+      __syncthreads();
+      run_roles<NT, I8, PAIR, true>(map_x, map_wb, map_wc, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
+    }
+  } else {
+    run_roles<NT, I8, PAIR, false>(map_x, map_wb, map_wc, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
+  }
   __syncwarp();
   if (SPLIT && warp < kEpiWarp0) ptx::cluster_sync();
   // ---------------------------------------------------------------- teardown
@@ -670,6 +764,11 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   if (threadIdx.x == 0 && !*(volatile uint32_t*)&sh->abort_flag) {
     if (sh->active) atomicAdd(&prm.counters[CNT_ACTIVE], (unsigned long long)sh->active);
     if (sh->rows_active) atomicAdd(&prm.counters[CNT_ROWS_ACTIVE], (unsigned long long)sh->rows_active);
+    if (shut && part == 0) {
+      // the jobs without conditional rows are taken from the totals below
+      atomicAdd(&prm.counters[CNT_TILES_TOTAL], 0ull - (unsigned long long)jobs);
+      atomicAdd(&prm.counters[CNT_EXEC_MACS], 0ull - (unsigned long long)jobs * 256ull * NT * (unsigned long long)(L.kh * L.kw) * L.c_r);
+    }
     if (blockIdx.x == 0) {
       const unsigned long long tiles = (unsigned long long)P.tiles_m * P.tiles_n;
       atomicAdd(&prm.counters[CNT_CALLS], 1ull);
@@ -814,6 +913,23 @@ void flag_rows(RawRow* st, int lo, int hi, int* a_count, int* b_count) {
   }
 }
 
+// The base rows of a pair's jobs, as the jobs of a column tile whose gates cannot fire run them.
+void plan_base(RawRow* raw, Tc4Plan* P) {
+  for (int i = 0; i < P->rows; ++i) {
+    Tc4Row& r = raw[i].r;
+    if (r.flags & kRowCond) continue;
+    int k = i + 1;
+    while (k < P->rows && (raw[k].r.flags & kRowCond)) ++k;
+    if (k == P->rows || raw[k].a_key != raw[i].a_key) r.flags |= kRowAFreeBase;
+    // (a patch that base rows use is taken by a base row, and their stages serve no other rows)
+    if (r.flags & kRowANew) ++P->a_base;
+    if (r.flags & kRowBNew) ++P->b_base;
+    if ((r.flags & kRowANew) || (!P->resident && (r.flags & kRowBNew))) P->turn_base = (uint16_t)P->base_rows;
+    P->base_mask |= 1ull << i;
+    ++P->base_rows;
+  }
+}
+
 template <int NT, bool I8, bool PAIR>
 const void* instance() { return (const void*)tc4_gated_conv_kernel<NT, I8, PAIR>; }
 
@@ -915,7 +1031,6 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     }
     if (s == 0) { P.a_per_job = a; P.b_per_job = b; }
   }
-  for (int i = 0; i < P.rows; ++i) P.row[i] = raw[i].r;
 
   // shared memory: resident weights if they leave room for three patch slots, else rings of both
   P.stage_bytes = 3 * (P.pair ? P.nt / 2 : P.nt) * 128;
@@ -937,8 +1052,11 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.na = (room - P.nb * P.stage_bytes) / P.slot_bytes;         // what is left goes to patches
   if (P.na > kMaxNA) P.na = kMaxNA;
   if (P.na < 1 || (P.na < 2 && max_a * jobs > 1)) return false;
-  for (int i = 0; i < P.rows; ++i)
+  if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) plan_base(raw, &P);
+  for (int i = 0; i < P.rows; ++i) {
+    P.row[i] = raw[i].r;
     if ((P.row[i].flags & kRowANew) || (!P.resident && (P.row[i].flags & kRowBNew))) P.turn = (uint16_t)i;
+  }
   P.off_b = kOffStages;
   P.off_a = kOffStages + (unsigned)(P.nb * P.stage_bytes);
   P.smem_bytes = kSmemBytes;
@@ -971,6 +1089,7 @@ int launch_tc4(const LayerDims& L, const Tc4Plan& P, Tc4Maps* maps, const void* 
   prm.L = L; prm.P = P; prm.bn = bn; prm.delta = delta;
   prm.residual = static_cast<const __nv_bfloat16*>(residual);
   prm.y = y; prm.mask = mask; prm.counters = counters;
+  prm.x = static_cast<const __nv_bfloat16*>(x); prm.w_cond = static_cast<const __nv_bfloat16*>(w_cond);
   const int which = (P.nt == 128 ? 1 : 0) | (P.i8 ? 2 : 0) | (P.pair ? 4 : 0);
   static const void* const kernels[8] = {
       instance<64, false, false>(), nullptr, instance<64, true, false>(), nullptr,

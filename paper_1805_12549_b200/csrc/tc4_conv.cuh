@@ -31,7 +31,8 @@ enum : uint8_t {
   kRowANew = 4, kRowAFree = 8,     // takes the next patch slot / is the last to read its slot
   kRowBNew = 16, kRowBFree = 32,   // the same for the weight stage
   kKindTaps = 64,   // (in `kind`) the first taps of the base path of a window, several per weight tile
-  kRowCond = 64     // the weights come from W_cond (else W_base)
+  kRowCond = 64,    // the weights come from W_cond (else W_base)
+  kRowAFreeBase = 128              // kRowAFree of a job that runs the base rows only
 };
 
 enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2 };
@@ -58,6 +59,10 @@ struct Tc4Plan {
   int a_per_job, b_per_job;        // patch slots and weight stages of a job
   uint16_t lo[kTc4MaxSplit + 1];   // rows [lo[s], lo[s+1]) belong to CTA s of a cluster
   uint16_t turn;                   // last row of a job that waits for a ring
+  uint16_t turn_base;
+  // jobs of a column tile whose gates cannot fire (pairs) run the base rows only
+  int base_rows, a_base, b_base;   // 0: all jobs run all rows
+  unsigned long long base_mask;    // which rows
   uint8_t p_mask, r_mask;          // which CTAs of a cluster add to P / to R
   unsigned off_b, off_a, smem_bytes;
   Tc4Row row[kTc4MaxRows];

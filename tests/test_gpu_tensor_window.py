@@ -105,3 +105,68 @@ def test_outputs_that_are_only_16_byte_aligned(n):
     torch.cuda.synchronize()
     assert torch.equal(y1, g.y) and float(buf[:off].abs().sum()) == 0 and float(buf[off + g.y.numel():].abs().sum()) == 0
     g.close()
+
+
+SHUT = [
+    (O.Shape(40, 56, 56, 64, 64, groups=4), "one base slice, resident weights"),
+    (O.Shape(40, 28, 28, 128, 128, groups=4), "two base slices"),
+    (O.Shape(256, 4, 4, 512, 512, groups=4), "base chunks"),
+    (O.Shape(70, 28, 28, 64, 128, stride=2, groups=4), "stride 2, one base slice"),
+    (O.Shape(60, 28, 28, 128, 256, stride=2, groups=4), "stride 2, two base slices"),
+    (O.Shape(21, 13, 19, 256, 192, groups=2), "half-empty channel tile"),
+    (O.Shape(48, 7, 7, 512, 512, groups=8), "one job per pair"),
+]
+
+
+@pytest.mark.parametrize("s,why", SHUT, ids=[w for _, w in SHUT])
+@pytest.mark.parametrize("how", ["all", "some", "residual", "band", "dense"])
+def test_column_tiles_whose_gates_cannot_fire(s, why, how):
+    c = K.make_float_case("winshut", s, "bf16", density=0.3, residual=how == "residual")
+    if how == "some":
+        c.delta[:(s.c_out + 1) // 2] = K.INF
+        c.delta[-1] = np.nan                     # (fires nowhere either)
+    else:
+        c.delta[:] = K.INF
+    if how == "band":
+        c.delta_high = np.full(s.c_out, 2.0, np.float32)
+    ref, st, _ = _run(c, cond_mode=1 if how == "dense" else 0)
+    if how != "some":
+        skips = how != "dense"
+        assert st.active == 0 and (st.executed_macs < st.dense_macs) == skips and (st.tiles_total == 0) == skips
+
+
+@pytest.mark.parametrize("s", [O.Shape(40, 28, 28, 128, 128, groups=4), O.Shape(60, 14, 14, 256, 256, groups=4),
+                               O.Shape(40, 28, 28, 256, 128, stride=2, groups=4)],
+                         ids=["one chunk", "two chunks", "stride 2"])
+def test_int8_thresholds_beyond_every_sum(s):
+    c = K.make_int8_case("winshut8", s, density=0.3)
+    top = 9 * s.c_p * 128 * 128                  # (the largest sum there is)
+    for thr, skips in ((top, False), (top + 1, True)):
+        c.bn["q_gate_thr"] = np.full(s.c_out, thr, np.int32)
+        _, st, _ = _run(c)
+        assert (st.executed_macs < st.dense_macs) == skips
+
+
+@pytest.mark.parametrize("residual", [False, True])
+def test_an_infinite_sum_meets_an_infinite_threshold(residual):
+    """A tie fires, at +inf too: those outputs are the full sum under its batch norm."""
+    s = O.Shape(40, 20, 20, 128, 128, groups=4)
+    c = K.make_float_case("winshutinf", s, "bf16", density=0.3, residual=residual)
+    c.delta[:] = K.INF
+    c.x[1, 7, 19, 3] = np.inf                    # P = +-inf around it
+    c.x[39, 19, 0, 5] = np.inf
+    c.x[39, 18, 1, 77] = -np.inf                 # R = +-inf there: P + R is infinite or not a number
+    c.x[2, 3, 4, 6] = np.nan
+    ref = K.run_oracle(c)
+    assert ref.active > 0 and np.isnan(ref.p).any()
+    g = K.GpuCase(c, algo=0)
+    assert g.conv.kernel_id == WINDOW
+    for with_mask in (True, False):
+        y, mask, st = g.run(with_mask=with_mask)
+        if with_mask:
+            np.testing.assert_array_equal(mask, ref.mask)
+        assert st.executed_macs < st.dense_macs and st.active == ref.active
+        fin = np.isfinite(ref.y)
+        np.testing.assert_array_equal(y[~fin], ref.y[~fin])
+        assert (np.abs(y[fin] - ref.y[fin]) <= K.BF16_ATOL + K.BF16_RTOL * np.abs(ref.y[fin])).all()
+    g.close()
