@@ -438,8 +438,8 @@ def run_network_block(args, peaks):
         "ms_gated_layers": round(sum(v for k, v in per_op.items() if k in gated_names), 4),
         "ms_other_operators": round(sum(v for k, v in per_op.items() if k not in gated_names), 4),
         "ms_per_operator": {k: round(v, 4) for k, v in per_op.items()},
-        "kernels": {s.name: KERNEL_NAMES[inst.convs[s.name].kernel_id]
-                    for s in net.specs},
+        "kernels": {s.name: "tcgen05 stem" if s.name == "stem" and inst.convs[s.name].uses_tensor_cores
+                    else KERNEL_NAMES[inst.convs[s.name].kernel_id] for s in net.specs},
     }
     inst.close()
     # batch-1 latency (the regime of the paper's accelerator, Table 4): the same network and

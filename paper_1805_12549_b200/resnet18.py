@@ -9,8 +9,8 @@ calls.
 
 Layers that are not gated (the 7x7 stem, the 1x1 shortcut convolutions, the classifier) run as
 layers with G = 1, where the base path is the whole convolution (Section 3.1 allows eta = 1).
-The stem is one operator (cg_stem_forward); passes that record or calibrate every layer compute it as
-a patch matrix (cg_im2col_bf16) followed by a 1x1 layer over it.
+The stem is one operator (cg_stem_forward); where its layer is not on tensor cores, and in passes that
+calibrate, it is a patch matrix (cg_im2col_bf16) followed by a 1x1 layer over it.
 
 Weights are random (Kaiming-normal); the batch-norm statistics, the gate statistics of Eq. 3 and
 the thresholds Delta come from a layer-by-layer calibration pass over a few images, which stands
@@ -235,11 +235,17 @@ class Instance:
 
     @property
     def patches(self):
-        """Patch matrix of the stem, for the passes that look at every layer's input."""
+        """Patch matrix of the stem, for the passes that compute it that way or record it."""
         if self._patches is None:
             hw = self.net.stem_hw
             self._patches = torch.empty((self.n, hw, hw, STEM_KPAD), dtype=torch.bfloat16, device="cuda")
         return self._patches
+
+    def _fused_stem(self, x):
+        s = self.net.specs[0]
+        y = self.out[s.name]
+        B.cg_stem_forward(self.convs[s.name].handle, x, s.wb, s.bn, s.delta, y, self.stem_ws)
+        return y
 
     def _conv(self, s, x, residual, before_conv, density, record):
         if before_conv is not None:
@@ -253,7 +259,8 @@ class Instance:
 
     def forward(self, x, before_conv=None, density=None, record=None, events=None):
         """x [n,image,image,3] bf16 -> logits [n,classes] bf16 (a view of an owned buffer).
-        `events`, a list, receives (operator name, start event, end event) per call."""
+        `events`, a list, receives (operator name, start event, end event) per call; `record`, a list, every
+        layer's (spec, input, residual, output, mask).  Both see the operators of a plain pass."""
         if before_conv is None and record is None and events is None:
             return self._forward(x)
         net = self.net
@@ -269,8 +276,16 @@ class Instance:
             return out
 
         go = lambda s, a, r=None: timed(s.name, lambda: self._conv(s, a, r, before_conv, density, record))
-        timed("stem.im2col", lambda: B.cg_im2col_bf16(x, self.patches, STEM_K, STEM_STRIDE, STEM_PAD))
-        a = go(net.specs[0], self.patches)
+        patch = lambda: B.cg_im2col_bf16(x, self.patches, STEM_K, STEM_STRIDE, STEM_PAD)   # noqa: E731
+        stem = net.specs[0]
+        if before_conv is None and self.convs[stem.name].uses_tensor_cores:
+            a = timed(stem.name, lambda: self._fused_stem(x))
+            if record is not None:                    # (the layer's input is the patch matrix)
+                patch()
+                record.append((stem, self.patches.clone(), None, a.clone(), None))
+        else:
+            timed("stem.im2col", patch)
+            a = go(stem, self.patches)
         timed("maxpool", lambda: B.cg_maxpool_bf16(a, self.pooled, 3, 2, 1))
         a = self.pooled
         for short, c1, c2, st in net.blocks:
@@ -298,12 +313,11 @@ class Instance:
             return y
 
         stem = net.specs[0]
-        a = out[stem.name]
         if convs[stem.name].uses_tensor_cores:
-            B.cg_stem_forward(convs[stem.name].handle, x, stem.wb, stem.bn, stem.delta, a, self.stem_ws)
+            a = self._fused_stem(x)
         else:
             B.cg_im2col_bf16(x, self.patches, STEM_K, STEM_STRIDE, STEM_PAD)
-            conv(stem, self.patches)
+            a = conv(stem, self.patches)
         B.cg_maxpool_bf16(a, self.pooled, 3, 2, 1)
         a = self.pooled
         for short, c1, c2, st in net.blocks:

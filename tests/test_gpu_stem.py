@@ -104,3 +104,27 @@ def test_a_short_batch_gives_its_own_logits_and_other_extents_are_refused():
         with pytest.raises(B.CgError):
             inst.forward(bad)
     inst.close()
+
+
+@pytest.mark.parametrize("algo", [0, 1], ids=["auto", "direct"])
+def test_events_and_records_are_those_of_a_plain_pass(algo):
+    import torch
+    from paper_1805_12549_b200 import resnet18 as R
+    net = R.CgResNet18(image=33, classes=20, algo=algo)
+    net.set_density(1.0)
+    x = R.synthetic_images("stemhooks", 2, 33)
+    inst = net.instance(2)
+    plain = inst.forward(x).clone()
+    stem = inst.out["stem"].clone()
+    events, record = [], []
+    assert torch.equal(inst.forward(x, events=events), plain)
+    assert torch.equal(inst.forward(x, record=record), plain)
+    torch.cuda.synchronize()
+    names = [name for name, _, _ in events]
+    assert names.count("stem") == 1 and ("stem.im2col" in names) == (algo == 1)
+    # one kernel per operator, the fused stem two
+    assert len(names) == inst.launches_per_forward() - (algo == 0)
+    spec, patches, _, y, _ = record[0]
+    assert spec.name == "stem" and patches.shape[-1] == spec.c_in and torch.equal(y, stem)
+    assert len(record) == len(net.specs)
+    inst.close()
