@@ -35,7 +35,7 @@ constexpr long long kWaitCycles = 2000000000ll;
 
 struct SharedS {
   uint64_t a_full[2], a_empty[2], acc_full[2], acc_empty[2], b_ready;
-  uint32_t tmem_base, abort_flag, active;
+  uint32_t tmem_base, abort_flag, active, rows_active;
   float t[64];
   float4 k[64];                                       // {a1, b1, a2, b2}
 };
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
       ptx::mbar_init(&sh->acc_full[i], 1); ptx::mbar_init(&sh->acc_empty[i], kEpiWarps);
     }
     ptx::mbar_init(&sh->b_ready, 2 * kGatherWarps);
-    sh->abort_flag = 0; sh->active = 0;
+    sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0;
     ptx::fence_mbar_init();
   }
   __syncwarp();
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
     float4 k[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) { t[e] = sh->t[c0 + q8 + e]; k[e] = sh->k[c0 + q8 + e]; }
-    uint32_t active = 0;
+    uint32_t active = 0, rows_active = 0;               // (rows: of all four lanes of a row, kept by every lane)
     bool ok = true;
     for (int j = 0; j < jobs && ok; ++j) {
       const int s = j & 1;
@@ -255,8 +255,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int row = quad * 32 + 16 * i + 8 * h + r4;
-          if (row >= cnt) continue;
-          uint32_t out[4];
+          uint32_t out[4], fired = 0;
 #pragma unroll
           for (int g = 0; g < 4; ++g) {
             float v[2];
@@ -265,14 +264,19 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
               const int c = 2 * g + e;
               const float pv = __uint_as_float(p[g >> 1][4 * (g & 1) + 2 * h + e]);
               const bool d = pv >= t[c];              // (a NaN sum does not fire)
-              active += d ? 1u : 0u;
+              fired += d ? 1u : 0u;
               v[e] = fmaf(d ? k[c].z : k[c].x, pv, d ? k[c].w : k[c].y);
             }
             if (P.relu) { v[0] = fmaxf(v[0], 0.f); v[1] = fmaxf(v[1], 0.f); }
             const __nv_bfloat162 b = __floats2bfloat162_rn(v[0], v[1]);
             out[g] = *reinterpret_cast<const uint32_t*>(&b);
           }
-          *(uint4*)(yp + (long long)row * 64) = make_uint4(out[0], out[1], out[2], out[3]);
+          if (row < cnt) *(uint4*)(yp + (long long)row * 64) = make_uint4(out[0], out[1], out[2], out[3]);
+          else fired = 0;
+          active += fired;
+          uint32_t on = __ballot_sync(0xffffffffu, fired != 0u);   // four lanes to a row
+          on |= on >> 1; on |= on >> 2;
+          rows_active += (uint32_t)__popc(on & 0x11111111u);
         }
       }
       ptx::tc_fence_before();
@@ -280,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
       if (lane == 0) ptx::mbar_arrive(&sh->acc_empty[s]);
     }
     active = __reduce_add_sync(0xffffffffu, active);
-    if (lane == 0) atomicAdd(&sh->active, active);
+    if (lane == 0) { atomicAdd(&sh->active, active); atomicAdd(&sh->rows_active, rows_active); }
   }
   __syncwarp();
   if (*(volatile uint32_t*)&sh->abort_flag) {
@@ -292,8 +296,10 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
   ptx::tc_fence_after();
   if (threadIdx.x == 0 && !*(volatile uint32_t*)&sh->abort_flag) {
     if (sh->active) atomicAdd(&P.counters[CNT_ACTIVE], (unsigned long long)sh->active);
+    if (sh->rows_active) atomicAdd(&P.counters[CNT_ROWS_ACTIVE], (unsigned long long)sh->rows_active);
     if (blockIdx.x == 0) {
       atomicAdd(&P.counters[CNT_CALLS], 1ull);
+      atomicAdd(&P.counters[CNT_ROWS_TOTAL], (unsigned long long)(P.jobs / P.segs) * P.wo * 2ull);
       atomicAdd(&P.counters[CNT_EXEC_MACS], (unsigned long long)P.jobs * 128ull * 64ull * 176ull);
     }
   }

@@ -50,6 +50,9 @@ def test_stem_matches_the_convolution(n, h, w, dv):
     assert (err[~near.reshape(ref.y.shape)] <= 0).all()
     assert st.calls == 1 and st.device_status == 0 and abs(st.active - ref.active) <= near.sum()
     assert c.s.m * 64 == st.outputs
+    # blocks of a pixel and 32 channels, as the 1x1 layer over the patch matrix counts them
+    words = ref.mask.reshape(-1, 2)
+    assert st.rows_total == words.size and abs(st.rows_active - np.count_nonzero(words)) <= near.sum()
 
 
 def test_pixels_that_are_not_finite_stay_where_they_are_used():
