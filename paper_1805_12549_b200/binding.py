@@ -265,6 +265,8 @@ def cg_conv_plan_string(h) -> str:
 def cg_im2col_bf16(x, a, k, stride, pad, stream=None):
     """x [n,h,w,c] -> a [n,h',w',k_pad] (include/cgnet.h)."""
     n, h, w, c = x.shape
+    if n * ((h + 2 * pad - k) // stride + 1) * ((w + 2 * pad - k) // stride + 1) * a.shape[-1] > a.numel():
+        raise ValueError(f"the patch matrix of {tuple(x.shape)} does not fit {tuple(a.shape)}")
     _check(lib().cg_im2col_bf16(_ptr(x), _ptr(a), n, h, w, c, k, stride, pad, a.shape[-1],
                                 _stream_ptr(stream)), "cg_im2col_bf16")
 

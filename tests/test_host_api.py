@@ -71,6 +71,29 @@ def test_the_stem_is_told_the_images_and_channels_of_its_input(monkeypatch):
     assert seen[0][2:6] == (3, 9, 11, 4)
 
 
+def test_a_patch_matrix_that_does_not_fit_is_refused(monkeypatch):
+    """A batch larger than the matrix was made for must not be written behind it."""
+    import torch
+    calls = []
+
+    class Recorder:
+        def cg_im2col_bf16(self, *args):
+            calls.append(args)
+            return 0
+
+    monkeypatch.setattr(B, "_lib", Recorder())
+    monkeypatch.setattr(B, "_stream_ptr", lambda stream: None)
+    a = torch.zeros((2, 5, 6, 152), dtype=torch.bfloat16)
+    x = torch.zeros((4, 9, 12, 3), dtype=torch.bfloat16)
+    for n in (1, 2):
+        B.cg_im2col_bf16(x[:n], a, 7, 2, 3)
+    assert len(calls) == 2
+    for bad in (x[:3], torch.zeros((2, 11, 12, 3), dtype=torch.bfloat16)):
+        with pytest.raises(ValueError):
+            B.cg_im2col_bf16(bad, a, 7, 2, 3)
+    assert len(calls) == 2
+
+
 def test_the_stem_rejects_bad_arguments_before_any_launch():
     lib = B.lib()
     buf = (C.c_uint8 * 4096)()
