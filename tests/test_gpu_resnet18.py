@@ -65,6 +65,34 @@ def test_subsample_maxpool_avgpool_match_their_definitions():
     assert np.abs(got - mean).max() <= 2.0 ** -8 * np.abs(mean).max() + 1e-6   # one bf16 rounding of an fp32 sum
 
 
+@pytest.mark.parametrize("k,stride,pad", [(2, 2, 0), (3, 1, 1), (3, 2, 1), (3, 2, 0), (3, 3, 1), (5, 2, 2)])
+@pytest.mark.parametrize("n,h,w,c", [(1, 1, 1, 8), (2, 1, 13, 16), (1, 9, 1, 8), (2, 2, 2, 8), (3, 7, 10, 40), (1, 33, 31, 64)])
+def test_maxpool_over_filters_and_sizes(k, stride, pad, n, h, w, c):
+    """The kernel for 3x3 windows of stride 2 and the general one, with NaN among the values: a NaN never wins, and a window
+    of NaN gives -inf."""
+    import torch
+    from paper_1805_12549_b200 import binding as B
+    ho, wo = (h + 2 * pad - k) // stride + 1, (w + 2 * pad - k) // stride + 1
+    if h + 2 * pad < k or w + 2 * pad < k:
+        pytest.skip("no window")
+    x = _rand_bf16(("pools", h, w, c), (n, h, w, c))
+    x[..., 1] = np.nan                                   # whole windows of NaN
+    x[0, 0, 0, 2] = np.nan
+    x[-1, -1, -1, 3] = -np.inf
+    x[..., 4] = -np.abs(x[..., 4])                       # padding must not win over negative values
+    xp = np.full((n, h + 2 * pad, w + 2 * pad, c), -np.inf, np.float32)
+    xp[:, pad:pad + h, pad:pad + w] = x
+    ref = np.full((n, ho, wo, c), -np.inf, np.float32)
+    for r in range(k):
+        for s in range(k):
+            ref = np.fmax(ref, xp[:, r:r + (ho - 1) * stride + 1:stride, s:s + (wo - 1) * stride + 1:stride])
+    buf = torch.full((n * ho * wo * c + 128,), 7.0, dtype=torch.bfloat16, device="cuda")
+    y = buf[64:-64].view(n, ho, wo, c)
+    B.cg_maxpool_bf16(_bf16_dev(x), y, k, stride, pad)
+    np.testing.assert_array_equal(_f32(y), ref)
+    assert bool((buf[:64] == 7).all()) and bool((buf[-64:] == 7).all())
+
+
 @pytest.fixture(scope="module")
 def network():
     import torch
