@@ -978,7 +978,10 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.split = 1;
   const int room = (int)(kSmemBytes - 1024 - kOffStages);
   RawRow raw[kTc4MaxRows];
-  if ((long long)tiles128 * tn64 * 2 <= sms) {
+  // (1x1 layers of up to three chunks have one row and nothing to share: as pairs they end without the exchange of
+  // sums, 28x28 x 64 -> 128, one image, 8.5 and 5.0 us)
+  const bool one_row = P.mode == kTc4Chunks && L.c_in <= 3 * ck;
+  if (!one_row && (long long)tiles128 * tn64 * 2 <= sms) {
     // Fewer jobs of 128 pixels and 64 channels than half the SMs: their K loops are shared, as far as all clusters
     // fit on the chip at once (measured with 148 SMs: 32 clusters of 4 do, 15 of 8 do and 16 do not, 9.2 against
     // 16.5 us for 4 x 7x7 x 512).  Eight CTAs need sixteen rows, or exactly eight: with 9 or 12 the exchange costs

@@ -47,6 +47,9 @@ SHAPES = [
     (O.Shape(9, 10, 11, 320, 128, 1, 1, 1, 0, groups=1), "1x1, ungated, five chunks"),
     (O.Shape(70, 10, 11, 64, 256, 1, 1, 1, 0, groups=1), "1x1, one chunk, pairs"),
     (O.Shape(128, 1, 1, 512, 1024, 1, 1, 1, 0, groups=1), "a classifier"),
+    (O.Shape(3, 9, 9, 64, 96, 1, 1, 1, 0, groups=1), "1x1, one chunk, two jobs"),
+    (O.Shape(1, 7, 5, 192, 64, 1, 1, 1, 0, groups=1), "1x1, three chunks, part of a job"),
+    (O.Shape(1, 17, 16, 256, 64, 1, 1, 1, 0, groups=1), "1x1, four chunks, K loop over a cluster"),
     (O.Shape(3, 10, 10, 512, 64, groups=8), "G = 8"),
 ]
 
@@ -84,6 +87,7 @@ INT8 = [
     (O.Shape(1, 7, 7, 512, 512, groups=4), "a whole base chunk, K loop over a cluster"),
     (O.Shape(4, 13, 6, 128, 64, groups=2), "c_out = 64"),
     (O.Shape(5, 28, 28, 128, 256, stride=2, groups=4), "stride 2"),
+    (O.Shape(2, 9, 7, 256, 64, 1, 1, 1, 0, groups=1), "1x1, two chunks"),
 ]
 
 
