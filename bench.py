@@ -8,7 +8,8 @@ One step = one forward pass of every gated 3x3 layer shape of the workload over 
 of synthetic activations (ReLU of box-smoothed Gaussian noise, bf16).  Prints ONE JSON line:
 the headline value on --workload, every layer at the target density and with all gates open
 (`speedup_vs_density1` against `flop_reduction`), and, at one GPU, extra blocks for the ImageNet
-shapes, G = 8, a density sweep, cross-channel correlated inputs and the int8 layers.
+shapes, G = 8, a density sweep, cross-channel correlated inputs and the int8 layers.  The line has
+the extra blocks in short; the whole record goes to standard error, or to --details FILE.
 Under torchrun each rank runs the same layers on its own batch (weak scaling, no collective
 on the data path); the time is the max over ranks.
 """
@@ -348,6 +349,26 @@ EXTRA_BLOCKS = [
 ]
 
 
+LAYER_KEYS = ("layer", "us", "density", "kernel", "roof_frac", "speedup_vs_density1")
+NETWORK_KEYS = ("workload", "batch", "ms_per_forward", "images_per_s", "ms_per_forward_density1", "flop_reduction",
+                "batch1_latency_ms")
+
+
+def headline(out):
+    """The printed line: the record with its layers and extra blocks in short, so that it stays under 3000 characters
+    (programs that keep only the end of the output have to find all of it)."""
+    line = dict(out)
+    line["layers"] = [{k: rec[k] for k in LAYER_KEYS if k in rec} for rec in out["layers"]]
+    line["blocks"] = []
+    for b in out["blocks"]:
+        if "densities" in b:
+            line["blocks"].append({**{k: b[k] for k in ("workload", "groups", "rho", "dtype")},
+                                   "us_all_layers": {d: e["us_all_layers"] for d, e in b["densities"].items()}})
+        else:
+            line["blocks"].append({k: b[k] for k in NETWORK_KEYS if k in b})
+    return json.dumps(line, separators=(",", ":"))
+
+
 def run_block(block, args, peaks, rank):
     from paper_1805_12549_b200 import synth
     if block["workload"] == "imagenet":
@@ -616,7 +637,13 @@ def run_ours(args):
             "speedup_vs_density1": speedup,
             "roofline": roof, "cpu_baseline": cpu, "layers": per_layer, "blocks": blocks,
         }
-        print(json.dumps(out))
+        details = json.dumps(out)
+        if args.details:
+            with open(args.details, "w") as f:
+                f.write(details + "\n")
+        else:
+            print(details, file=sys.stderr)
+        print(headline(out))
     if world > 1:
         dist.destroy_process_group()
 
@@ -720,6 +747,8 @@ def main():
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--no-extra", action="store_true",
                     help="skip the extra blocks (ImageNet shapes, G = 8, density sweep, int8)")
+    ap.add_argument("--details", default=None, metavar="FILE",
+                    help="write the whole record (every layer of every block) to FILE; default: standard error")
     ap.add_argument("--layers", default=None,
                     help="comma-separated layer names to keep (e.g. c64@56,c256@14)")
     ap.add_argument("--no-graph", action="store_true",
