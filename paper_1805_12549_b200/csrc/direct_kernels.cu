@@ -243,7 +243,7 @@ direct_gated_conv_i8_kernel(LayerDims L, const int8_t* __restrict__ x,
 // x CH channels.  A run of kStage K elements (tap-major, then channel) is gathered per stage: four consecutive
 // channels of a tap per load, converted to fp32, two stages in flight.  The warp-per-output kernel above waits
 // for one pair of global loads per product: 156 us for the partial sums of four images of 56x56 (64 channels,
-// c_p = 16), here 17 us; it remains for channel counts that are not multiples of four, channel
+// c_p = 16), here 18.7; counters there: shared-memory reads 58 % of their rate, issue slots 48 %, DRAM 1 %.  It remains for channel counts that are not multiples of four, channel
 // grouping and the channel-wise gate.
 // Products and sums are rounded separately, for bf16 operands too: their products are exact in fp32 only inside its
 // normal range, so a fused multiply-add is another sum where one is below 2^-126 or beyond 2^128.
@@ -562,11 +562,11 @@ int launch_tile(const LayerDims& L, const TapBox& taps, const void* x, const voi
 
 // Large layers: the layer's channels (at most 64) per block, four channels and two or four pixels per thread.  Small
 // ones wait for the chain of additions of one output: one output per thread, 16 channels x 16 pixels per block, so
-// that a product costs few instructions and the blocks spread over the SMs (four channels per thread there: fp32
-// 2 x 8x8 x 16 9.6 us, 5x5 x 64 28.5; one: 5.4, 13.4).  Measured, us with two / four pixels per thread: 201 thousand
-// outputs (56x56 x 64, partial sums) 14.1 / 15.1, 803 thousand (4 x 56x56 x 64) 17.3 / 21.1, a million (16 x 32x32
-// x 64, fp32 layer) 123 / 87; with one output per thread against two pixels: 20 thousand (9x9 x 256) 9.7 / 19.0,
-// 130 thousand (3 x 13x13 x 256) 19.6 / 20.3 (four channels per thread).
+// that a product costs few instructions and the blocks spread over the SMs.  Measured, us of the bf16 partial sums /
+// the fp32 layer with every gate open, for one output, two and four pixels per thread: 100 thousand outputs (4 x 7x7 x
+// 512) 44 78 115 / 170 278 395; 201 thousand (56x56 x 64) 13.2 14.8 16.2 / 45 57 54; 401 thousand (2 x 56x56 x 64)
+// 24.5 17.7 19.2 / 83 66 70; 803 thousand (4 x 56x56 x 64) 44 18.5 22.1 / 161 74 84; a million (16 x 32x32 x 64)
+// 56 29 22 / 203 102 84; 1.6 million (8 x 56x56 x 64) 84 35 36 / 308 144 130.
 template <typename T>
 int launch_tiles(const LayerDims& L, const void* x, const void* w_base, const void* w_cond, const cg_bn_params& bn,
                  const float* delta, const void* residual, void* y, uint32_t* mask, void* p_out, int base_only,
@@ -574,7 +574,7 @@ int launch_tiles(const LayerDims& L, const void* x, const void* w_base, const vo
 #define CG_TILE(TC, PXT, CH, ...) launch_tile<T, 256, TC, PXT, CH, ##__VA_ARGS__>(L, taps, x, w_base, w_cond, bn, delta, residual, y, mask, p_out, base_only, counters, stream)
   const int tc = L.c_out <= 16 ? 16 : (L.c_out <= 32 ? 32 : 64);
   const long long outputs = L.m * ((L.c_out + tc - 1) / tc * tc);
-  const int v = outputs >= 900000 ? 4 : (outputs >= 100000 ? 2 : 1);
+  const int v = outputs >= 900000 ? 4 : (outputs >= 250000 ? 2 : 1);
   const TapBox taps = tap_box(L);
   // images smaller than the filter's reach (us with all taps and with the box, before them the kernel of one warp per
   // output: fp32, one pixel x 128 23.2, 5.1, 9.2; 2x2 x 64, 7x7 58, 13.5, 41).  Large layers, where a product of this

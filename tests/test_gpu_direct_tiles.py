@@ -14,9 +14,11 @@ SHAPES = [
     (O.Shape(3, 9, 7, 32, 32, groups=4), "32 channels"),
     (O.Shape(2, 6, 6, 48, 40, groups=4), "c_out = 40"),
     (O.Shape(1, 5, 4, 64, 100, groups=4), "two channel blocks, the second ragged"),
-    (O.Shape(16, 20, 21, 16, 16, groups=4), "two pixels per thread, 16 channels"),
+    (O.Shape(16, 20, 21, 16, 16, groups=4), "100 thousand outputs"),
+    (O.Shape(40, 20, 21, 16, 16, groups=4), "two pixels per thread, 16 channels"),
     (O.Shape(40, 15, 16, 16, 32, groups=4), "two pixels per thread, 32 channels"),
-    (O.Shape(64, 20, 16, 8, 24, groups=2), "four pixels per thread, 32 channels"),
+    (O.Shape(64, 20, 16, 8, 24, groups=2), "two pixels per thread, 24 channels"),
+    (O.Shape(100, 20, 16, 8, 24, groups=2), "four pixels per thread, 32 channels"),
     (O.Shape(40, 16, 15, 8, 64, groups=2), "two pixels per thread, 64 channels"),
     (O.Shape(70, 18, 16, 8, 64, groups=2), "four pixels per thread, 64 channels"),
     (O.Shape(2, 11, 9, 16, 16, 5, 5, 2, 2, groups=4), "5x5, stride 2"),
