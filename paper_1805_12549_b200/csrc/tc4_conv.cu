@@ -38,12 +38,14 @@
 // one per slot, and copies issued from divergent code, every streamed layer waited for its weights (512 channels,
 // 4x4, batch 256: 67 us).
 //
-// Measured (us on the device, batch as named, G = 4, against the other kernels' best): 128@16x16 b256 22.2 (34.3),
-// 256@8x8 b256 23.3 (34.1), 512@4x4 b256 27.6 (43.6), 64@56x56 b64 with residual 24.6 (50.1), 128->256 stride 2 at
-// 28x28 b64 15.7 (27.4), int8 128@28x28 b64 17.3 (32.7); layers of one image 6 to 8 (12 to 24).  What bounds it
-// now: the serial work of a row of the K loop (barriers, table, commits: 400 to 700 cycles beside 9 to 12 MMAs of
-// 64) and whole rounds of jobs; the counters show the tensor pipe 35 % active, L2 16 % and DRAM 7 % busy on
-// 128@16x16, and neither resident weights nor fewer, larger copies made it faster.
+// Measured (us per pass among others, batch as named, G = 4; in brackets the other kernels' best, timed alike):
+// 128@16x16 b256 24.3 (34.2), 256@8x8 b256 23.8 (34.0), 512@4x4 b256 28.1 (43.7), 64@56x56 b64 with residual 26.6 (50.1),
+// 128->256 stride 2 at 28x28 b64 16.3 (27.4), int8 128@28x28 b64 17.5 (32.6); on the device, one image: 128@28x28 8.2
+// (19.5), 512@7x7 8.1 (23.2).  What bounds it now (cycles that its roles wait, per launch, in a copy with clock reads):
+// nobody waits for copies.  512@4x4 takes what its MMAs take in two rounds of jobs (36,900 cycles), 256@8x8 27,600 of
+// 32,400; elsewhere the issuers' rows are the longer chain: 930 to 1,490 cycles of a row's issue, table entry, barriers
+// and commits beside 9 or 12 MMAs of 64, 33,000 of 38,500 cycles at 128@16x16.  Neither resident weights nor fewer,
+// larger copies made it faster.
 // Every mbarrier wait is bounded; on expiry the CTA records CG_ERR_DEVICE_TIMEOUT with the id of the wait
 // and leaves.
 #include <cstring>
@@ -983,10 +985,12 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   const bool one_row = P.mode == kTc4Chunks && L.c_in <= 3 * ck;
   if (!one_row && (long long)tiles128 * tn64 * 2 <= sms) {
     // Fewer jobs of 128 pixels and 64 channels than half the SMs: their K loops are shared, as far as all clusters
-    // fit on the chip at once (measured with 148 SMs: 32 clusters of 4 do, 15 of 8 do and 16 do not, 9.2 against
-    // 16.5 us for 4 x 7x7 x 512).  Eight CTAs need sixteen rows, or exactly eight: with 9 or 12 the exchange costs
-    // what the shorter loops save (14x14 x 256 7.5 us with 4 and 8; 28x28 x 128, 8 rows, 8.0 and 7.8; 9x9 x 128 7.0
-    // and 6.5; 56x56 x 64, 4 rows, 7.7 with 2 CTAs and 7.2 with 4).
+    // are on the chip at once.  Measured with 148 SMs: 32 clusters of 4 are, 15 of 8 are and 16 are not (9.2 against
+    // 16.5 us for 4 x 7x7 x 512); the lines are 32 of 4 and 13 of 8, short of the measured 15 because how many clusters
+    // of 8 fit depends on how the SMs are spread over the chip's processing clusters, which differs from chip to chip.
+    // Eight CTAs need sixteen rows, or exactly eight: with 9 or 12 the exchange costs what the shorter loops save (14x14 x
+    // 256 7.5 us with 4 and 8; 28x28 x 128, 8 rows, 8.0 and 7.8; 9x9 x 128 7.0 and 6.5; 56x56 x 64, 4 rows, 7.7 with 2
+    // CTAs and 7.2 with 4).
     P.nt = 64; P.tiles_m = tiles128; P.tiles_n = tn64;
     P.rows = raw_rows(L, P, raw);
     if (P.rows > kTc4MaxRows) return false;
