@@ -986,8 +986,8 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   if (!one_row && (long long)tiles128 * tn64 * 2 <= sms) {
     // Fewer jobs of 128 pixels and 64 channels than half the SMs: their K loops are shared, as far as all clusters
     // are on the chip at once.  Measured with 148 SMs: 32 clusters of 4 are, 15 of 8 are and 16 are not (9.2 against
-    // 16.5 us for 4 x 7x7 x 512); the lines are 32 of 4 and 13 of 8, short of the measured 15 because how many clusters
-    // of 8 fit depends on how the SMs are spread over the chip's processing clusters, which differs from chip to chip.
+    // 16.5 us for 4 x 7x7 x 512).  14 and 15 clusters of 8 gain nothing over 4 (4 x 7x7 x 512 -> 448 9.2 and 9.4 us, 6 x 7x7
+    // x 512 -> 320 9.4 and 9.3), so the line of 8 lies at 13, clear of the edge.
     // Eight CTAs need sixteen rows, or exactly eight: with 9 or 12 the exchange costs what the shorter loops save (14x14 x
     // 256 7.5 us with 4 and 8; 28x28 x 128, 8 rows, 8.0 and 7.8; 9x9 x 128 7.0 and 6.5; 56x56 x 64, 4 rows, 7.7 with 2
     // CTAs and 7.2 with 4).

@@ -151,10 +151,13 @@ def test_int8_thresholds_beyond_every_sum(s):
         assert (st.executed_macs < st.dense_macs) == skips
 
 
-@pytest.mark.parametrize("residual", [False, True])
-def test_an_infinite_sum_meets_an_infinite_threshold(residual):
+@pytest.mark.parametrize("s,residual", [(O.Shape(40, 20, 20, 128, 128, groups=4), False),
+                                        (O.Shape(40, 20, 20, 128, 128, groups=4), True),
+                                        (O.Shape(40, 20, 20, 128, 192, groups=2), False),
+                                        (O.Shape(40, 20, 20, 128, 256, stride=2, groups=4), True)],
+                         ids=["128 channels", "residual", "64 channels per tile", "stride 2"])
+def test_an_infinite_sum_meets_an_infinite_threshold(s, residual):
     """A tie fires, at +inf too: those outputs are the full sum under its batch norm."""
-    s = O.Shape(40, 20, 20, 128, 128, groups=4)
     c = K.make_float_case("winshutinf", s, "bf16", density=0.3, residual=residual)
     c.delta[:] = K.INF
     c.x[1, 7, 19, 3] = np.inf                    # P = +-inf around it
