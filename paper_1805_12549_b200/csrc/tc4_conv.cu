@@ -28,13 +28,13 @@
 // loop of a 128-pixel job over the 2, 4 or 8 CTAs of a cluster: each leaves its sums in shared memory, and
 // every CTA adds up and finishes 1/split of the rows.
 //
-// Warp roles (640 threads): 0 = patch producer, 2 = weight producer, 1 and 3 = MMA issuers of even and odd
-// jobs (the next job's MMAs are issued while the first issuer waits for its copies), 4-19 = epilogue (TMEM
+// Warp roles (640 threads): 0 = patch producer, 2 = weight producer, 1 = MMA issuer, 4-19 = epilogue (TMEM
 // lane quadrant x 32 channels).  The epilogue keeps out of shared memory, whose bandwidth the MMAs' operands
 // take: it reads TMEM in the fragment layout, keeps the constants of its channels in registers and writes
-// 16-byte pieces, four lanes to a 64-byte run.  The K loop is a table of filter rows (three taps, up to 12
-// MMAs, one weight stage): with one entry per tap an issuer spent 940 cycles on four MMAs, most of it between
-// them.  The copies of a pair's second CTA count on its leader's barriers without an arrival of their own: with
+// 16-byte pieces, four lanes to a 64-byte run.  The K loop goes by filter rows (three taps, up to 12 MMAs, one weight
+// stage), written out for the kinds of rows a layer has (issue_jobs): a row then costs its issuer 170 cycles beside its MMAs.
+// As a table of row kinds it took 570 to 1,000, two issuers in turns, more than the MMAs: 128@16x16 b256 23.6 us for 20.0
+// now, 128@28x28 b128 31.8 for 26.1, 64@56x56 b128 37.8 for 35.2 (graphs of 20 calls).  The copies of a pair's second CTA count on its leader's barriers without an arrival of their own: with
 // one per slot, and copies issued from divergent code, every streamed layer waited for its weights (512 channels,
 // 4x4, batch 256: 67 us).
 //
@@ -86,7 +86,6 @@ struct Shared4 {
   uint64_t a_full[kMaxNA], a_empty[kMaxNA];
   uint64_t b_full[kMaxNB], b_empty[kMaxNB];
   uint64_t acc_full[4], acc_empty[4];
-  uint64_t turn[2];      // by job parity: the job's issuer has seen everything it takes from the rings
   uint32_t tmem_base;
   uint32_t abort_flag;
   uint32_t active, rows_active;
@@ -133,7 +132,7 @@ struct Cursor {
   __device__ __forceinline__ void at(unsigned i, unsigned n) { const unsigned q = i / n; slot = (int)(i - q * n); par = q & 1u; }
 };
 
-// The MMAs of one row: up to three tiles of NKS K slices.
+// The MMAs of one row of the table: up to three tiles of NKS K slices.
 template <bool PAIR, bool I8, int NKS>
 __device__ __forceinline__ void issue_row(int tiles, uint32_t d, uint32_t hi, uint32_t a, uint32_t a_step, uint32_t b0,
                                           uint32_t b1, uint32_t b2, uint32_t idesc, uint32_t acc) {
@@ -148,18 +147,19 @@ __device__ __forceinline__ void issue_row(int tiles, uint32_t d, uint32_t hi, ui
   }
 }
 
-// The base path of a window's first chunk where it has KP = 1 or 2 of the four slices: its first T taps, 4/KP of
-// them per weight tile.
-template <bool PAIR, bool I8, int KP, int T>
-__device__ __forceinline__ void issue_taps(uint32_t d, uint32_t hi, uint32_t a, uint32_t row_lo, uint32_t b, uint32_t tile,
-                                           uint32_t idesc, uint32_t acc) {
+// The taps [T0, T1) of a chunk, K slices [K0, K0 + NK) of each: PER taps of NK slices share a weight tile, B0 is the first
+// tile of the stage.  Tap t reads the patch at (t / 3 - R0) * row_lo + (t % 3) * step.
+template <bool PAIR, bool I8, int T0, int T1, int R0, int K0, int NK, int PER, int B0>
+__device__ __forceinline__ void issue_taps(uint32_t d, uint32_t hi, uint32_t a, uint32_t row_lo, uint32_t step, uint32_t b,
+                                           uint32_t tile, uint32_t idesc, uint32_t acc) {
 #pragma unroll
-  for (int t = 0; t < T; ++t) {
-    const uint32_t a_t = a + (uint32_t)(t / 3) * row_lo + (uint32_t)(t % 3) * 8u;
-    const uint32_t b_t = b + (uint32_t)(t / (4 / KP)) * tile + (uint32_t)((t % (4 / KP)) * KP) * 2u;
+  for (int t = T0; t < T1; ++t) {
+    const uint32_t a_t = a + (uint32_t)(t / 3 - R0) * row_lo + (uint32_t)(t % 3) * step + 2u * K0;
+    const uint32_t b_t = b + (uint32_t)(t / PER - B0) * tile + (uint32_t)((t % PER) * NK) * 2u;
 #pragma unroll
-    for (int k = 0; k < KP; ++k)
-      ptx::umma<PAIR, I8>(d, ((uint64_t)hi << 32) | (a_t + 2u * k), ((uint64_t)hi << 32) | (b_t + 2u * k), idesc, t == 0 && k == 0 ? acc : 1u);
+    for (int k = 0; k < NK; ++k)
+      ptx::umma<PAIR, I8>(d, ((uint64_t)hi << 32) | (a_t + 2u * k), ((uint64_t)hi << 32) | (b_t + 2u * k), idesc,
+                          t == T0 && k == 0 ? acc : 1u);
   }
 }
 
@@ -230,6 +230,147 @@ __device__ __forceinline__ void infinite_sums(const Tc4Params& prm, uint32_t t_c
     ((__nv_bfloat16*)prm.y)[at] = __float2bfloat16_rn(o);
   }
   __syncwarp();
+}
+
+// A ring of slots as the issuer walks it: operand address (16-byte units) and the phase parity of the "full" barrier.
+struct IssueRing {
+  int slot;
+  uint32_t par, at;
+  __device__ __forceinline__ void next(int n, uint32_t size, uint32_t first) {
+    at += size;
+    if (++slot == n) { slot = 0; par ^= 1u; at = first; }
+  }
+};
+
+// The MMAs of all jobs of a pair, taken by one lane of its first CTA.  MODE and KP (slices of the first chunk that belong to
+// the base path; 4: the base path is whole chunks) are constants, so that a filter row is one look at its weights' barrier,
+// its MMAs and a commit: walked from a table of row kinds, a row's loads, tests and branches took 700 cycles beside the 576 of
+// nine MMAs of 64, two issuers taking turns.
+template <int NT, bool I8, bool BASE, int MODE, int KP>
+__device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, uint32_t a0, uint32_t b0, uint32_t tmem, int jobs) {
+  constexpr int kAcc = 512 / (2 * NT);
+  constexpr uint32_t kTileU = (uint32_t)(NT / 2) * 8u;         // a weight tile, 16-byte units
+  constexpr bool kWin = MODE == kTc4Window;
+  const Tc4Plan& P = prm.P;
+  const uint32_t idesc = I8 ? ptx::idesc_s8(256, NT) : ptx::idesc_bf16(256, NT);
+  const uint32_t hi = (uint32_t)(ptx::smem_desc(0, 1024, 2) >> 32);
+  const uint32_t a_size = (uint32_t)P.slot_bytes >> 4, b_size = (uint32_t)P.stage_bytes >> 4;
+  const uint32_t row_lo = kWin ? (uint32_t)P.wp * 8u : 0u;
+  constexpr uint32_t kStep = kWin ? 8u : 1024u;                // from tap to tap of a filter row
+  const int na = P.na, nb = P.nb;
+  const bool resident = P.resident != 0;
+  const int ck = I8 ? 128 : 64;
+  const int chunks = BASE ? (prm.L.c_p + ck - 1) / ck : prm.L.c_in / ck, base_chunks = KP == 4 ? prm.L.c_p / ck : 0;
+  IssueRing a{0, 0u, a0}, b{0, 0u, b0};
+  bool ok = true, a_seen = false, b_seen = false;
+  bool new_b = true;                                           // weights are waited for (resident ones: by the first job)
+  uint32_t a_at = 0, b_at = 0;
+  int a_slot = 0, b_slot = 0;
+  auto take_a = [&]() {
+    if (!a_seen) ok = ok && wait4_one(sh, prm.counters, &sh->a_full[a.slot], a.par, 4);
+    a_at = a.at; a_slot = a.slot;
+    a.next(na, a_size, a0);
+    a_seen = false;
+  };
+  auto take_b = [&]() {
+    if (new_b && !b_seen) ok = ok && wait4_one(sh, prm.counters, &sh->b_full[b.slot], b.par, 5);
+    b_at = b.at; b_slot = b.slot;
+    b.next(nb, b_size, b0);
+    // a look at the next stage's barrier, whose answer arrives while this one's MMAs are issued
+    b_seen = new_b && ptx::mbar_test_wait(&sh->b_full[b.slot], b.par);
+  };
+  auto look_a = [&]() { a_seen = ptx::mbar_test_wait(&sh->a_full[a.slot], a.par); };
+  auto free_a = [&]() { ptx::umma_commit_pair(&sh->a_empty[a_slot]); };
+  auto free_b = [&](int slot) { if (!resident) ptx::umma_commit_pair(&sh->b_empty[slot]); };
+  for (int j = 0; j < jobs; ++j) {
+    const int stage = j % kAcc;
+    ok = wait4_one(sh, prm.counters, &sh->acc_empty[stage], ((j / kAcc) & 1) ^ 1, 3);
+    if (!ok) return;
+    ptx::tc_fence_after();
+    const uint32_t d_p = tmem + (uint32_t)(stage * 2 * NT), d_r = d_p + NT;
+    if (resident) { b = IssueRing{0, 0u, b0}; new_b = j == 0; b_seen = false; }
+    for (int q = 0; q < chunks; ++q) {
+      if constexpr (MODE == kTc4Chunks) {
+        // up to three chunks of a 1x1 layer per slot
+        take_a(); take_b();
+        if (!ok) return;
+        look_a();
+        const int tiles = chunks - q < 3 ? chunks - q : 3;
+        const uint32_t acc = q ? 1u : 0u;
+        issue_taps<true, I8, 0, 1, 0, 0, 4, 1, 0>(d_p, hi, a_at, 0, kStep, b_at, kTileU, idesc, acc);
+        if (tiles > 1) issue_taps<true, I8, 1, 2, 0, 0, 4, 1, 0>(d_p, hi, a_at, 0, kStep, b_at, kTileU, idesc, 1u);
+        if (tiles > 2) issue_taps<true, I8, 2, 3, 0, 0, 4, 1, 0>(d_p, hi, a_at, 0, kStep, b_at, kTileU, idesc, 1u);
+        q += 2;
+        free_b(b_slot);
+        free_a();
+      } else if (KP < 4 && q == 0) {
+        // the first chunk holds the base channels (KP slices of every tap, several taps per weight tile) and the first
+        // conditional ones
+        constexpr int kPer = 4 / (KP < 4 ? KP : 1), kCond = 4 - KP > 0 ? 4 - KP : 1, kFirst = KP < 4 ? KP : 0;
+        uint32_t base_at = 0;
+        int base_slot = 0;
+        if (kWin) take_a();
+        take_b();
+        base_at = b_at; base_slot = b_slot;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          if (!kWin) take_a();
+          if (!ok) return;
+          if (kWin) {
+            if (r == 0) {
+              if (KP == 1) issue_taps<true, I8, 0, 9, 0, 0, 1, 4, 0>(d_p, hi, a_at, row_lo, kStep, base_at, kTileU, idesc, 0u);
+              else issue_taps<true, I8, 0, 6, 0, 0, 2, 2, 0>(d_p, hi, a_at, row_lo, kStep, base_at, kTileU, idesc, 0u);
+              free_b(base_slot);
+            }
+          } else {
+            if (KP == 1) {
+              if (r == 0) issue_taps<true, I8, 0, 3, 0, 0, 1, 4, 0>(d_p, hi, a_at, 0, kStep, base_at, kTileU, idesc, 0u);
+              if (r == 1) issue_taps<true, I8, 3, 6, 1, 0, 1, 4, 0>(d_p, hi, a_at, 0, kStep, base_at, kTileU, idesc, 1u);
+              if (r == 2) issue_taps<true, I8, 6, 9, 2, 0, 1, 4, 0>(d_p, hi, a_at, 0, kStep, base_at, kTileU, idesc, 1u);
+              if (r == 2) free_b(base_slot);
+            } else {
+              if (r == 0) issue_taps<true, I8, 0, 3, 0, 0, 2, 2, 0>(d_p, hi, a_at, 0, kStep, base_at, kTileU, idesc, 0u);
+              if (r == 1) issue_taps<true, I8, 3, 6, 1, 0, 2, 2, 0>(d_p, hi, a_at, 0, kStep, base_at, kTileU, idesc, 1u);
+              if (r == 1) free_b(base_slot);
+            }
+          }
+          if (KP == 2 && r == 2) {                             // the last three taps have a stage of their own
+            take_b();
+            if (!ok) return;
+            issue_taps<true, I8, 6, 9, kWin ? 0 : 2, 0, 2, 2, 3>(d_p, hi, a_at, row_lo, kStep, b_at, kTileU, idesc, 1u);
+            free_b(b_slot);
+          }
+          if (!BASE) {
+            take_b();
+            if (!ok) return;
+            if (!kWin || r == 2) look_a();
+            issue_taps<true, I8, 0, 3, 0, kFirst, kCond, 1, 0>(d_r, hi, a_at + (uint32_t)r * row_lo, 0, kStep, b_at, kTileU,
+                                                              idesc, r ? 1u : 0u);
+            free_b(b_slot);
+          }
+          if (!kWin || r == 2) free_a();
+        }
+      } else {
+        if (kWin) take_a();
+        const uint32_t d = q < base_chunks ? d_p : d_r;
+        uint32_t acc = q == 0 || (KP == 4 && q == base_chunks) ? 0u : 1u;
+#pragma unroll 1
+        for (int r = 0; r < 3; ++r) {
+          if (!kWin) take_a();
+          take_b();
+          if (!ok) return;
+          if (!kWin || r == 2) look_a();
+          issue_taps<true, I8, 0, 3, 0, 0, 4, 1, 0>(d, hi, a_at, 0, kStep, b_at, kTileU, idesc, acc);
+          acc = 1u;
+          free_b(b_slot);
+          if (!kWin) free_a();
+          else a_at += row_lo;
+        }
+        if (kWin) free_a();
+      }
+    }
+    ptx::umma_commit_pair(&sh->acc_full[stage]);
+  }
 }
 
 // What the warps of a block do (see the top of the file).  BASE: the jobs of a column tile whose gates cannot fire, which run
@@ -338,72 +479,73 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
       }
     }
     __syncwarp();
-  } else if (warp == 1 || warp == 3) {
-    // ============================================================ MMA issuers (even / odd jobs)
+  } else if (warp == 1) {
+    // ============================================================ MMA issuer
     // (One lane picked by elect.sync runs the loop: an MMA then takes under 40 cycles to issue, against 50
     // predicated or in a branch on the lane.  A pair's MMAs are issued by its first CTA.)
-    if ((!PAIR || part == 0) && ptx::elect_one()) {
-      const uint32_t idesc = I8 ? ptx::idesc_s8(PAIR ? 256 : 128, NT) : ptx::idesc_bf16(PAIR ? 256 : 128, NT);
-      const uint32_t hi_w = (uint32_t)(ptx::smem_desc(0, 1024, 2) >> 32);
-      const uint32_t a0 = (ptx::smem_u32(s_a) >> 4) | 0x10000u, b0 = (ptx::smem_u32(s_b) >> 4) | 0x10000u;
-      const uint32_t a_size = (uint32_t)P.slot_bytes >> 4, b_size = (uint32_t)P.stage_bytes >> 4, a_step = (uint32_t)P.a_step, row_lo = (uint32_t)P.wp * 8u;
-      auto commit = [&](uint64_t* bar) { if (PAIR) ptx::umma_commit_pair(bar); else ptx::umma_commit(bar); };
-      bool ok = true;
-      for (int j = warp == 1 ? 0 : 1; j < jobs && ok; j += 2) {
-        const int stage = j % kAcc;
-        ok = wait4_one(sh, prm.counters, &sh->acc_empty[stage], ((j / kAcc) & 1) ^ 1, 3);
-        // The rings are walked by one issuer at a time: a slot's barrier tells two successive uses apart,
-        // no more, so job j waits on it only when every use of the jobs before has been seen.
-        if (j > 0) ok = ok && wait4_one(sh, prm.counters, &sh->turn[(j - 1) & 1], ((j - 1) >> 1) & 1, 8);
-        if (!ok) break;
-        ptx::tc_fence_after();
-        const uint32_t d_p = tmem + (uint32_t)(stage * 2 * NT);
-        Cursor ca, cb;
-        ca.at((unsigned)j * (unsigned)(BASE ? P.a_base : P.a_per_job), (unsigned)P.na);
-        if (P.resident) cb = Cursor{0, 0}; else cb.at((unsigned)j * (unsigned)(BASE ? P.b_base : P.b_per_job), (unsigned)P.nb);
-        int sa = 0, sb_base = 0, sb_cond = 0;                  // slots in use
-        bool a_seen = false, b_seen = false;                   // the next row's slots were full when last looked at
-        const bool weights_here = P.resident && j >= 2;        // (this issuer has waited for every stage)
-        Tc4Row next = row_at(table, lo);
-        for (int i = lo; i < hi; ++i) {
-          const Tc4Row s = next;
-          if (i + 1 < hi) next = row_at(table, i + 1);
-          if (s.flags & kRowANew) {
-            if (!a_seen) ok = wait4_one(sh, prm.counters, &sh->a_full[ca.slot], ca.par, 4);
-            sa = ca.slot; ca.next(P.na);
-          }
-          if (s.flags & kRowBNew) {
-            if (!b_seen && !weights_here) ok = ok && wait4_one(sh, prm.counters, &sh->b_full[cb.slot], cb.par, 5);
-            if (s.flags & kRowCond) sb_cond = cb.slot; else sb_base = cb.slot;
-            cb.next(P.nb);
-          }
-          if (!ok) break;
-          if (i == (BASE ? P.turn_base : P.turn)) ptx::mbar_arrive(&sh->turn[j & 1]);
-          if (i + 1 < hi) {
-            // a look at the next row's barriers, whose answer arrives while this row's MMAs are issued
-            a_seen = (next.flags & kRowANew) && ptx::mbar_test_wait(&sh->a_full[ca.slot], ca.par);
-            b_seen = (next.flags & kRowBNew) && !weights_here && ptx::mbar_test_wait(&sh->b_full[cb.slot], cb.par);
-          }
-          const int sb = (s.flags & kRowCond) ? sb_cond : sb_base;
-          const uint32_t a = a0 + (uint32_t)sa * a_size + s.a_off, b = b0 + (uint32_t)sb * b_size;
-          const uint32_t d = d_p + ((s.flags & kRowR) ? (uint32_t)NT : 0u), acc = (s.flags & kRowInit) ? 0u : 1u;
-          const int tiles = ((s.kind >> 4) & 3) + 1, nks = (s.kind & 3) + 1;
-          const uint32_t b1 = b + s.b_off[0], b2 = b + s.b_off[1], b3 = b + s.b_off[2];
-          if (s.kind & kKindTaps) {
-            if (nks == 1) issue_taps<PAIR, I8, 1, 9>(d, hi_w, a, row_lo, b, kTile >> 4, idesc, acc);
-            else issue_taps<PAIR, I8, 2, 6>(d, hi_w, a, row_lo, b, kTile >> 4, idesc, acc);
-          } else if (nks == 4) issue_row<PAIR, I8, 4>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
-          else if (nks == 3) issue_row<PAIR, I8, 3>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
-          else if (nks == 2) issue_row<PAIR, I8, 2>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
-          else issue_row<PAIR, I8, 1>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
-          if ((s.flags & kRowBFree) && !P.resident) commit(&sh->b_empty[sb]);
-          if (s.flags & kRowAFree) commit(&sh->a_empty[sa]);
+    const uint32_t a0 = (ptx::smem_u32(s_a) >> 4) | 0x10000u, b0 = (ptx::smem_u32(s_b) >> 4) | 0x10000u;
+    if constexpr (PAIR) {
+      if (part == 0 && ptx::elect_one()) {
+        const int kp = L.c_p % (I8 ? 128 : 64) == 0 ? 4 : L.c_p / (I8 ? 32 : 16);
+        if (P.mode == kTc4Window) {
+          if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Window, 4>(prm, sh, a0, b0, tmem, jobs);
+          else if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window, 2>(prm, sh, a0, b0, tmem, jobs);
+          else issue_jobs<NT, I8, BASE, kTc4Window, 1>(prm, sh, a0, b0, tmem, jobs);
+        } else if (P.mode == kTc4Taps) {
+          if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Taps, 4>(prm, sh, a0, b0, tmem, jobs);
+          else if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Taps, 2>(prm, sh, a0, b0, tmem, jobs);
+          else issue_jobs<NT, I8, BASE, kTc4Taps, 1>(prm, sh, a0, b0, tmem, jobs);
+        } else if (!BASE) {
+          issue_jobs<NT, I8, BASE, kTc4Chunks, 4>(prm, sh, a0, b0, tmem, jobs);
         }
-        if (ok) commit(&sh->acc_full[stage]);
       }
+    } else if (jobs > 0 && ptx::elect_one()) {
+      // a CTA of a cluster: its rows of the table
+      const uint32_t idesc = I8 ? ptx::idesc_s8(128, NT) : ptx::idesc_bf16(128, NT);
+      const uint32_t hi_w = (uint32_t)(ptx::smem_desc(0, 1024, 2) >> 32);
+      const uint32_t a_size = (uint32_t)P.slot_bytes >> 4, b_size = (uint32_t)P.stage_bytes >> 4, a_step = (uint32_t)P.a_step, row_lo = (uint32_t)P.wp * 8u;
+      bool ok = true;
+      Cursor ca{0, 0}, cb{0, 0};
+      int sa = 0, sb_base = 0, sb_cond = 0;                    // slots in use
+      bool a_seen = false, b_seen = false;                     // the next row's slots were full when last looked at
+      Tc4Row next = row_at(table, lo);
+      for (int i = lo; i < hi; ++i) {
+        const Tc4Row s = next;
+        if (i + 1 < hi) next = row_at(table, i + 1);
+        if (s.flags & kRowANew) {
+          if (!a_seen) ok = wait4_one(sh, prm.counters, &sh->a_full[ca.slot], ca.par, 4);
+          sa = ca.slot; ca.next(P.na);
+        }
+        if (s.flags & kRowBNew) {
+          if (!b_seen) ok = ok && wait4_one(sh, prm.counters, &sh->b_full[cb.slot], cb.par, 5);
+          if (s.flags & kRowCond) sb_cond = cb.slot; else sb_base = cb.slot;
+          cb.next(P.nb);
+        }
+        if (!ok) break;
+        if (i + 1 < hi) {
+          // a look at the next row's barriers, whose answer arrives while this row's MMAs are issued
+          a_seen = (next.flags & kRowANew) && ptx::mbar_test_wait(&sh->a_full[ca.slot], ca.par);
+          b_seen = (next.flags & kRowBNew) && ptx::mbar_test_wait(&sh->b_full[cb.slot], cb.par);
+        }
+        const int sb = (s.flags & kRowCond) ? sb_cond : sb_base;
+        const uint32_t a = a0 + (uint32_t)sa * a_size + s.a_off, b = b0 + (uint32_t)sb * b_size;
+        const uint32_t d = tmem + ((s.flags & kRowR) ? (uint32_t)NT : 0u), acc = (s.flags & kRowInit) ? 0u : 1u;
+        const int tiles = ((s.kind >> 4) & 3) + 1, nks = (s.kind & 3) + 1;
+        const uint32_t b1 = b + s.b_off[0], b2 = b + s.b_off[1], b3 = b + s.b_off[2];
+        if (s.kind & kKindTaps) {
+          if (nks == 1) issue_taps<PAIR, I8, 0, 9, 0, 0, 1, 4, 0>(d, hi_w, a, row_lo, 8u, b, kTile >> 4, idesc, acc);
+          else issue_taps<PAIR, I8, 0, 6, 0, 0, 2, 2, 0>(d, hi_w, a, row_lo, 8u, b, kTile >> 4, idesc, acc);
+        } else if (nks == 4) issue_row<PAIR, I8, 4>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
+        else if (nks == 3) issue_row<PAIR, I8, 3>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
+        else if (nks == 2) issue_row<PAIR, I8, 2>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
+        else issue_row<PAIR, I8, 1>(tiles, d, hi_w, a, a_step, b1, b2, b3, idesc, acc);
+        if (s.flags & kRowBFree) ptx::umma_commit(&sh->b_empty[sb]);
+        if (s.flags & kRowAFree) ptx::umma_commit(&sh->a_empty[sa]);
+      }
+      if (ok) ptx::umma_commit(&sh->acc_full[0]);
     }
     __syncwarp();
-  } else {
+  } else if (warp >= kEpiWarp0) {
     // ============================================================ epilogue
     const int et = (int)threadIdx.x - kEpiWarp0 * 32;
     for (int c = et; c < NT; c += kEpiThreads) {
@@ -707,7 +849,6 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
       ptx::mbar_init(&sh->acc_full[i], 1);
       ptx::mbar_init(&sh->acc_empty[i], (PAIR ? 2 : 1) * NT / 8);   // warps per job, of both CTAs of a pair
     }
-    ptx::mbar_init(&sh->turn[0], 1); ptx::mbar_init(&sh->turn[1], 1);
     sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0;
     ptx::fence_mbar_init();
   }
@@ -923,10 +1064,6 @@ void plan_base(RawRow* raw, Tc4Plan* P) {
     int k = i + 1;
     while (k < P->rows && (raw[k].r.flags & kRowCond)) ++k;
     if (k == P->rows || raw[k].a_key != raw[i].a_key) r.flags |= kRowAFreeBase;
-    // (a patch that base rows use is taken by a base row, and their stages serve no other rows)
-    if (r.flags & kRowANew) ++P->a_base;
-    if (r.flags & kRowBNew) ++P->b_base;
-    if ((r.flags & kRowANew) || (!P->resident && (r.flags & kRowBNew))) P->turn_base = (uint16_t)P->base_rows;
     P->base_mask |= 1ull << i;
     ++P->base_rows;
   }
@@ -1036,7 +1173,6 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
       if (raw[i].r.flags & kRowR) P.r_mask |= (uint8_t)(1 << s);
       else P.p_mask |= (uint8_t)(1 << s);
     }
-    if (s == 0) { P.a_per_job = a; P.b_per_job = b; }
   }
 
   // shared memory: resident weights if they leave room for three patch slots, else rings of both
@@ -1062,7 +1198,6 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) plan_base(raw, &P);
   for (int i = 0; i < P.rows; ++i) {
     P.row[i] = raw[i].r;
-    if ((P.row[i].flags & kRowANew) || (!P.resident && (P.row[i].flags & kRowBNew))) P.turn = (uint16_t)i;
   }
   P.off_b = kOffStages;
   P.off_a = kOffStages + (unsigned)(P.nb * P.stage_bytes);

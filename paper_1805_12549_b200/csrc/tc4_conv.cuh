@@ -56,12 +56,9 @@ struct Tc4Plan {
   int split;             // 1, 2, 4 or 8
   int grid;
   int rows;              // entries of row[] in use
-  int a_per_job, b_per_job;        // patch slots and weight stages of a job
   uint16_t lo[kTc4MaxSplit + 1];   // rows [lo[s], lo[s+1]) belong to CTA s of a cluster
-  uint16_t turn;                   // last row of a job that waits for a ring
-  uint16_t turn_base;
   // jobs of a column tile whose gates cannot fire (pairs) run the base rows only
-  int base_rows, a_base, b_base;   // 0: all jobs run all rows
+  int base_rows;                   // 0: all jobs run all rows
   unsigned long long base_mask;    // which rows
   uint8_t p_mask, r_mask;          // which CTAs of a cluster add to P / to R
   unsigned off_b, off_a, smem_bytes;
