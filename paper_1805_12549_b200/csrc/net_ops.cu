@@ -8,6 +8,7 @@
 
 #include "cgnet.h"
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace {
 
@@ -22,11 +23,20 @@ inline int grid_for(long long items, int cap = 148 * 16) {
   return (int)g;
 }
 
+// Every operator is a dependent launch: its blocks are scheduled while the kernel in front ends, and wait here for it.
+// (Its input is then not read-only for the kernel's whole life: it must not go through the non-coherent load path, so no
+// __ldg and no __restrict__ on it.)
+__device__ __forceinline__ void dependent_start() {
+  cg::ptx::grid_launch_dependents();
+  cg::ptx::grid_dependency_wait();
+}
+
 // One thread per group of eight consecutive columns of the patch matrix.
-__global__ void __launch_bounds__(kBlock) im2col_kernel(const __nv_bfloat16* __restrict__ x,
+__global__ void __launch_bounds__(kBlock) im2col_kernel(const __nv_bfloat16* x,
                                                         __nv_bfloat16* __restrict__ a, int n, int h, int w,
                                                         int c, int k, int stride, int pad, int ho, int wo,
                                                         int k_pad) {
+  dependent_start();
   const int vecs = k_pad >> 3;
   const long long total = (long long)n * ho * wo * vecs;
   const int kkc = k * k * c;
@@ -57,10 +67,11 @@ __global__ void __launch_bounds__(kBlock) im2col_kernel(const __nv_bfloat16* __r
 // multiplications), one block per output row: the k input rows the output row reads are staged
 // in shared memory once, then every thread gathers 16-byte vectors of the patch matrix from it.
 template <int K, int C, int STRIDE>
-__global__ void __launch_bounds__(kBlock) im2col_rows_kernel(const __nv_bfloat16* __restrict__ x,
+__global__ void __launch_bounds__(kBlock) im2col_rows_kernel(const __nv_bfloat16* x,
                                                              __nv_bfloat16* __restrict__ a, int n, int h, int w,
                                                              int pad, int ho, int wo, int k_pad) {
   extern __shared__ __nv_bfloat16 rows[];               // [K][(w + 2*pad) * C], zero where outside the image
+  dependent_start();
   const int row_len = (w + 2 * pad) * C;
   const int vecs = k_pad >> 3;
   constexpr int kkc = K * K * C;
@@ -91,9 +102,10 @@ __global__ void __launch_bounds__(kBlock) im2col_rows_kernel(const __nv_bfloat16
   }
 }
 
-__global__ void __launch_bounds__(kBlock) subsample_kernel(const uint4* __restrict__ x, uint4* __restrict__ y,
+__global__ void __launch_bounds__(kBlock) subsample_kernel(const uint4* x, uint4* __restrict__ y,
                                                            int n, int h, int w, int cv, int stride, int ho,
                                                            int wo) {
+  dependent_start();
   const long long total = (long long)n * ho * wo * cv;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -112,9 +124,10 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   return *reinterpret_cast<const uint32_t*>(&r);
 }
 
-__global__ void __launch_bounds__(kBlock) maxpool_kernel(const uint4* __restrict__ x, uint4* __restrict__ y,
+__global__ void __launch_bounds__(kBlock) maxpool_kernel(const uint4* x, uint4* __restrict__ y,
                                                          int n, int h, int w, int cv, int k, int stride, int pad,
                                                          int ho, int wo) {
+  dependent_start();
   const long long total = (long long)n * ho * wo * cv;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -143,9 +156,10 @@ __global__ void __launch_bounds__(kBlock) maxpool_kernel(const uint4* __restrict
 // The 3x3, stride-2, padding-1 pooling of a ResNet, for up to 2^31 outputs: one output vector per thread, its
 // nine loads in flight together, indices by multiplications.  The general kernel spent its time on 64-bit divisions
 // and one load after the other: 128 x 112x112 x 64 (256 MB) 73 us, here 42.
-__global__ void __launch_bounds__(kBlock) maxpool3_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, unsigned total,
+__global__ void __launch_bounds__(kBlock) maxpool3_kernel(const uint4* x, uint4* __restrict__ y, unsigned total,
                                                           int h, int w, int cv, int ho, int wo, cg::FastDiv div_cv,
                                                           cg::FastDiv div_wo, cg::FastDiv div_ho) {
+  dependent_start();
   const unsigned i = blockIdx.x * kBlock + threadIdx.x;
   if (i >= total) return;
   const unsigned m = div_cv.div(i), v = i - m * (unsigned)cv;
@@ -159,7 +173,7 @@ __global__ void __launch_bounds__(kBlock) maxpool3_kernel(const uint4* __restric
     for (int s = 0; s < 3; ++s) {
       const int yy = (int)ii * 2 + r - 1, xx = (int)j * 2 + s - 1;
       t[r * 3 + s] = make_uint4(ninf, ninf, ninf, ninf);
-      if (yy >= 0 && yy < h && xx >= 0 && xx < w) t[r * 3 + s] = __ldg(x + (((long long)img * h + yy) * w + xx) * cv + v);
+      if (yy >= 0 && yy < h && xx >= 0 && xx < w) t[r * 3 + s] = x[(((long long)img * h + yy) * w + xx) * cv + v];
     }
   uint4 best = t[0];
 #pragma unroll
@@ -173,20 +187,30 @@ __global__ void __launch_bounds__(kBlock) maxpool3_kernel(const uint4* __restric
   y[i] = best;
 }
 
-// One thread per (image, group of eight channels): fp32 sums over the pixels in order.
-__global__ void __launch_bounds__(kBlock) avgpool_kernel(const uint4* __restrict__ x, uint4* __restrict__ y,
-                                                         int n, int hw, int cv) {
+// One thread per (image, group of eight channels): fp32 sums over the pixels in order, eight pixels' loads in flight (with
+// one or two, the 49 pixels of a 7x7 image are a chain of L2 reads).  64 threads to a block: a batch's few threads then
+// reach more SMs.
+constexpr int kAvgBlock = 64, kAvgLoads = 8;
+__global__ void __launch_bounds__(kAvgBlock) avgpool_kernel(const uint4* x, uint4* __restrict__ y, int n, int hw, int cv) {
+  dependent_start();
   const int total = n * cv;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const int v = i % cv, img = i / cv;
+    const uint4* src = x + (long long)img * hw * cv + v;
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    for (int p = 0; p < hw; ++p) {
-      const uint4 t = x[((long long)img * hw + p) * cv + v];
-      const __nv_bfloat16* tb = reinterpret_cast<const __nv_bfloat16*>(&t);
+    for (int p = 0; p < hw; p += kAvgLoads) {
+      uint4 t[kAvgLoads];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += __bfloat162float(tb[e]);
+      for (int k = 0; k < kAvgLoads; ++k) t[k] = p + k < hw ? src[(long long)(p + k) * cv] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int k = 0; k < kAvgLoads; ++k) {
+        if (p + k >= hw) break;
+        const __nv_bfloat16* tb = reinterpret_cast<const __nv_bfloat16*>(&t[k]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] += __bfloat162float(tb[e]);
+      }
     }
     __align__(16) __nv_bfloat16 out[8];
     const float inv = 1.0f / (float)hw;
@@ -196,7 +220,21 @@ __global__ void __launch_bounds__(kBlock) avgpool_kernel(const uint4* __restrict
   }
 }
 
-cg_status launched() { return cudaGetLastError() == cudaSuccess ? CG_OK : CG_ERR_CUDA; }
+template <typename... Args>
+cg_status launch(void (*kernel)(Args...), unsigned blocks, int threads, size_t smem, void* stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = static_cast<cudaStream_t>(stream);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? CG_OK : CG_ERR_CUDA;
+}
 
 }  // namespace
 
@@ -212,13 +250,11 @@ cg_status cg_im2col_bf16(const void* x, void* a, int n, int h, int w, int c, int
   const size_t stage = (size_t)k * (w + 2 * pad) * c * sizeof(__nv_bfloat16);
   if (k == 7 && c == 3 && stride == 2 && stage <= 48 * 1024) {   // the ResNet stem
     const int blocks = n * ho < 148 * 8 ? n * ho : 148 * 8;
-    im2col_rows_kernel<7, 3, 2><<<blocks, kBlock, stage, static_cast<cudaStream_t>(cuda_stream)>>>(
-        static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(a), n, h, w, pad, ho, wo, k_pad);
-    return launched();
+    return launch(im2col_rows_kernel<7, 3, 2>, (unsigned)blocks, kBlock, stage, cuda_stream,
+                  static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(a), n, h, w, pad, ho, wo, k_pad);
   }
-  im2col_kernel<<<grid_for(items), kBlock, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(a), n, h, w, c, k, stride, pad, ho, wo, k_pad);
-  return launched();
+  return launch(im2col_kernel, (unsigned)grid_for(items), kBlock, 0, cuda_stream, static_cast<const __nv_bfloat16*>(x),
+                static_cast<__nv_bfloat16*>(a), n, h, w, c, k, stride, pad, ho, wo, k_pad);
 }
 
 cg_status cg_subsample_bf16(const void* x, void* y, int n, int h, int w, int c, int stride, void* cuda_stream) {
@@ -226,9 +262,8 @@ cg_status cg_subsample_bf16(const void* x, void* y, int n, int h, int w, int c, 
   if (!aligned16(x) || !aligned16(y)) return CG_ERR_ALIGNMENT;
   const int ho = (h + stride - 1) / stride, wo = (w + stride - 1) / stride;
   const long long items = (long long)n * ho * wo * (c >> 3);
-  subsample_kernel<<<grid_for(items), kBlock, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      static_cast<const uint4*>(x), static_cast<uint4*>(y), n, h, w, c >> 3, stride, ho, wo);
-  return launched();
+  return launch(subsample_kernel, (unsigned)grid_for(items), kBlock, 0, cuda_stream, static_cast<const uint4*>(x),
+                static_cast<uint4*>(y), n, h, w, c >> 3, stride, ho, wo);
 }
 
 cg_status cg_maxpool_bf16(const void* x, void* y, int n, int h, int w, int c, int k, int stride, int pad,
@@ -241,21 +276,19 @@ cg_status cg_maxpool_bf16(const void* x, void* y, int n, int h, int w, int c, in
   if (k == 3 && stride == 2 && pad == 1 && items < (1ll << 31) - kBlock) {
     cg::FastDiv div_cv, div_wo, div_ho;
     div_cv.set((uint32_t)(c >> 3)); div_wo.set((uint32_t)wo); div_ho.set((uint32_t)ho);
-    maxpool3_kernel<<<(unsigned)((items + kBlock - 1) / kBlock), kBlock, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        static_cast<const uint4*>(x), static_cast<uint4*>(y), (unsigned)items, h, w, c >> 3, ho, wo, div_cv, div_wo, div_ho);
-    return launched();
+    return launch(maxpool3_kernel, (unsigned)((items + kBlock - 1) / kBlock), kBlock, 0, cuda_stream, static_cast<const uint4*>(x),
+                  static_cast<uint4*>(y), (unsigned)items, h, w, c >> 3, ho, wo, div_cv, div_wo, div_ho);
   }
-  maxpool_kernel<<<grid_for(items), kBlock, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      static_cast<const uint4*>(x), static_cast<uint4*>(y), n, h, w, c >> 3, k, stride, pad, ho, wo);
-  return launched();
+  return launch(maxpool_kernel, (unsigned)grid_for(items), kBlock, 0, cuda_stream, static_cast<const uint4*>(x),
+                static_cast<uint4*>(y), n, h, w, c >> 3, k, stride, pad, ho, wo);
 }
 
 cg_status cg_avgpool_bf16(const void* x, void* y, int n, int hw, int c, void* cuda_stream) {
   if (!x || !y || n <= 0 || hw <= 0 || c <= 0 || (c & 7)) return CG_ERR_INVALID_ARG;
   if (!aligned16(x) || !aligned16(y)) return CG_ERR_ALIGNMENT;
-  avgpool_kernel<<<grid_for((long long)n * (c >> 3)), kBlock, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      static_cast<const uint4*>(x), static_cast<uint4*>(y), n, hw, c >> 3);
-  return launched();
+  const long long groups = ((long long)n * (c >> 3) + kAvgBlock - 1) / kAvgBlock;
+  return launch(avgpool_kernel, (unsigned)(groups < 148 * 16 ? groups : 148 * 16), kAvgBlock, 0, cuda_stream,
+                static_cast<const uint4*>(x), static_cast<uint4*>(y), n, hw, c >> 3);
 }
 
 }  // extern "C"

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
 #pragma unroll
     for (int i = 0; i < (int)(kBTile / 16) / (2 * kGatherWarps * 32); ++i) {
       const int id = gt + (2 * i + group) * kGatherWarps * 32;
-      s_b[id] = __ldg(P.weights + id);
+      s_b[id] = P.weights[id];
     }
     ptx::fence_proxy_async();
     __syncwarp();
@@ -175,9 +175,9 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
         const bool in = r < 7 && q < words && yy >= 0 && yy < P.h && e >= 0 && e < w3;
         const unsigned short* p = P.x + (in ? ((long long)img * P.h + yy) * w3 + e : 0);
         if (EVEN) {
-          v[i] = __ldg((const uint32_t*)p);           // (rows of an even number of elements: whole words)
+          v[i] = *(const uint32_t*)p;           // (rows of an even number of elements: whole words)
         } else {
-          const uint32_t a = __ldg(p), b = in && e + 1 < w3 ? __ldg(p + 1) : 0;
+          const uint32_t a = *p, b = in && e + 1 < w3 ? p[1] : 0;
           v[i] = a | b << 16;
         }
         valid |= in ? 1u << i : 0u;
