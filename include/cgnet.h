@@ -40,6 +40,13 @@ size_t cg_stem_workspace_bytes(void);
 cg_status cg_stem_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
                           const cg_bn_params* bn, const float* delta, void* y, void* workspace, void* cuda_stream);
 
+/* cg_stem_forward and cg_maxpool_bf16 (k = 3, stride 2, pad 1) behind it in one kernel: y as there, pooled
+ * [n,(h' - 1)/2 + 1,(w' - 1)/2 + 1,64].  Even image widths (else CG_ERR_INVALID_ARG); no workspace.
+ * cg_stem_pool_pays: 1 where it is the faster way for n images of these extents, else 0. */
+int cg_stem_pool_pays(int n, int image_h, int image_w);
+cg_status cg_stem_pool_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
+                               const cg_bn_params* bn, const float* delta, void* y, void* pooled, void* cuda_stream);
+
 /* Every stride-th pixel: y[n,i,j,:] = x[n,i*stride,j*stride,:], y is [n,ceil(h/stride),
  * ceil(w/stride),c].  Input of the 1x1 stride-2 shortcut convolutions.  c a multiple of 8. */
 cg_status cg_subsample_bf16(const void* x, void* y, int n, int h, int w, int c, int stride,

@@ -27,7 +27,8 @@ EXPORTS = ("cg_conv_create", "cg_conv_workspace_bytes", "cg_conv_forward",
            "cg_conv_stats", "cg_conv_launches_per_forward", "cg_conv_uses_tensor_cores",
            "cg_conv_kernel_id", "cg_conv_plan_string", "cg_conv_destroy", "cg_status_string", "cg_conv_forward_static")
 # include/cgnet.h: the ungated operators of a whole network
-NET_EXPORTS = ("cg_stem_workspace_bytes", "cg_stem_forward", "cg_im2col_bf16", "cg_subsample_bf16", "cg_maxpool_bf16", "cg_avgpool_bf16")
+NET_EXPORTS = ("cg_stem_workspace_bytes", "cg_stem_forward", "cg_stem_pool_pays", "cg_stem_pool_forward",
+               "cg_im2col_bf16", "cg_subsample_bf16", "cg_maxpool_bf16", "cg_avgpool_bf16")
 
 
 class CgConvDesc(C.Structure):
@@ -108,6 +109,10 @@ def lib():
         L.cg_stem_forward.restype = C.c_int
         L.cg_stem_forward.argtypes = [C.c_void_p, C.c_void_p, i, i, i, i, C.c_void_p, C.POINTER(CgBnParams), C.c_void_p,
                                       C.c_void_p, C.c_void_p, C.c_void_p]
+        L.cg_stem_pool_pays.restype = C.c_int
+        L.cg_stem_pool_pays.argtypes = [i, i, i]
+        L.cg_stem_pool_forward.restype = C.c_int
+        L.cg_stem_pool_forward.argtypes = L.cg_stem_forward.argtypes
         L.cg_subsample_bf16.restype = C.c_int
         L.cg_subsample_bf16.argtypes = [C.c_void_p, C.c_void_p, i, i, i, i, i, C.c_void_p]
         L.cg_maxpool_bf16.restype = C.c_int
@@ -280,6 +285,17 @@ def cg_stem_forward(h, x, w_base, bn: CgBnParams, delta, y, workspace, stream=No
     n, ih, iw, c = x.shape
     _check(lib().cg_stem_forward(h, _ptr(x), n, ih, iw, c, _ptr(w_base), C.byref(bn), _ptr(delta), _ptr(y),
                                  _ptr(workspace), _stream_ptr(stream)), "cg_stem_forward")
+
+
+def cg_stem_pool_pays(n, image_h, image_w) -> bool:
+    return bool(lib().cg_stem_pool_pays(n, image_h, image_w))
+
+
+def cg_stem_pool_forward(h, x, w_base, bn: CgBnParams, delta, y, pooled, stream=None):
+    """x [n,h,w,3] -> y [n,h',w',64] and its 3x3 stride-2 maxima, n at most the handle's (include/cgnet.h)."""
+    n, ih, iw, c = x.shape
+    _check(lib().cg_stem_pool_forward(h, _ptr(x), n, ih, iw, c, _ptr(w_base), C.byref(bn), _ptr(delta), _ptr(y),
+                                      _ptr(pooled), _stream_ptr(stream)), "cg_stem_pool_forward")
 
 
 def cg_subsample_bf16(x, y, stride, stream=None):

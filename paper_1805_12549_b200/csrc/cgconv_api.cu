@@ -93,6 +93,27 @@ cg_status check_bn(const cg_conv_s* h, const cg_bn_params* bn, const float* delt
   return CG_OK;
 }
 
+// What both stem operators ask of a call; `other` is the workspace or the pooled output.
+cg_status check_stem(const cg_conv_s* h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
+                     const cg_bn_params* bn, const float* delta, const void* y, const void* other) {
+  if (!h || !x || !w_base || !y || n <= 0 || image_h <= 0 || image_w <= 0 || c != 3) return CG_ERR_INVALID_ARG;
+  if (n > h->L.n) return CG_ERR_INVALID_ARG;               // y has room for the handle's batch; fewer images are fine
+  const cg_status st = check_bn(h, bn, delta);
+  if (st != CG_OK) return st;
+  const cg::LayerDims& L = h->L;
+  // the handle describes the 1x1 layer over the patch matrix of the same convolution
+  if (h->desc.in_dtype != CG_BF16 || L.kh != 1 || L.kw != 1 || L.stride != 1 || L.pad != 0 || L.groups != 1 || L.c_out != 64 ||
+      L.c_in < 147 || L.has_residual || L.channel_tau > 0.f || bn->delta_high)
+    return CG_ERR_INVALID_ARG;
+  if ((image_h - 1) / 2 + 1 != L.ho || (image_w - 1) / 2 + 1 != L.wo) return CG_ERR_INVALID_ARG;
+  if (!aligned(x, 16) || !aligned(w_base, 16) || !aligned(y, 16) || !aligned(other, 16)) return CG_ERR_ALIGNMENT;
+  if (!h->use_tc) return CG_ERR_UNSUPPORTED;
+  int cur = -1;
+  if (cudaGetDevice(&cur) != cudaSuccess) return CG_ERR_CUDA;
+  if (cur != h->device) return CG_ERR_INVALID_ARG;
+  return CG_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -295,23 +316,27 @@ size_t cg_stem_workspace_bytes(void) { return cg::kStemWeightBytes; }
 
 cg_status cg_stem_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
                           const cg_bn_params* bn, const float* delta, void* y, void* workspace, void* cuda_stream) {
-  if (!h || !x || !w_base || !y || !workspace || n <= 0 || image_h <= 0 || image_w <= 0 || c != 3) return CG_ERR_INVALID_ARG;
-  if (n > h->L.n) return CG_ERR_INVALID_ARG;               // y has room for the handle's batch; fewer images are fine
-  const cg_status st = check_bn(h, bn, delta);
+  if (!workspace) return CG_ERR_INVALID_ARG;
+  const cg_status st = check_stem(h, x, n, image_h, image_w, c, w_base, bn, delta, y, workspace);
   if (st != CG_OK) return st;
   const cg::LayerDims& L = h->L;
-  // the handle describes the 1x1 layer over the patch matrix of the same convolution
-  if (h->desc.in_dtype != CG_BF16 || L.kh != 1 || L.kw != 1 || L.stride != 1 || L.pad != 0 || L.groups != 1 || L.c_out != 64 ||
-      L.c_in < 147 || L.has_residual || L.channel_tau > 0.f || bn->delta_high)
-    return CG_ERR_INVALID_ARG;
-  if ((image_h - 1) / 2 + 1 != L.ho || (image_w - 1) / 2 + 1 != L.wo) return CG_ERR_INVALID_ARG;
-  if (!aligned(x, 16) || !aligned(w_base, 16) || !aligned(y, 16) || !aligned(workspace, 16)) return CG_ERR_ALIGNMENT;
-  if (!h->use_tc) return CG_ERR_UNSUPPORTED;
-  int cur = -1;
-  if (cudaGetDevice(&cur) != cudaSuccess) return CG_ERR_CUDA;
-  if (cur != h->device) return CG_ERR_INVALID_ARG;
   const int err = cg::launch_stem(x, n, image_h, image_w, w_base, L.c_in, *bn, delta, L.eps, L.relu, y, workspace,
                                   h->counters, reinterpret_cast<cudaStream_t>(cuda_stream));
+  return err == 0 ? CG_OK : CG_ERR_CUDA;
+}
+
+int cg_stem_pool_pays(int n, int image_h, int image_w) {
+  return n > 0 && image_h > 0 && image_w > 0 && cg::stem_pool_pays(n, image_h, image_w) ? 1 : 0;
+}
+
+cg_status cg_stem_pool_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
+                               const cg_bn_params* bn, const float* delta, void* y, void* pooled, void* cuda_stream) {
+  if (!pooled || (image_w & 1)) return CG_ERR_INVALID_ARG;
+  const cg_status st = check_stem(h, x, n, image_h, image_w, c, w_base, bn, delta, y, pooled);
+  if (st != CG_OK) return st;
+  const cg::LayerDims& L = h->L;
+  const int err = cg::launch_stem_pool(x, n, image_h, image_w, w_base, L.c_in, *bn, delta, L.eps, L.relu, y, pooled,
+                                       h->counters, reinterpret_cast<cudaStream_t>(cuda_stream));
   return err == 0 ? CG_OK : CG_ERR_CUDA;
 }
 

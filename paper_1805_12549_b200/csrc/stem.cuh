@@ -13,4 +13,12 @@ int launch_stem(const void* x, int n, int h, int w, const void* w_base, int k_pa
                 const float* delta, float eps, int relu, void* y, void* ws, unsigned long long* counters,
                 cudaStream_t stream);
 
+// The stem and the 3x3 stride-2 max pooling behind it in one launch (stem_pool.cu): y as above, pooled [n,hp,wp,64].
+// Even image widths only.
+int launch_stem_pool(const void* x, int n, int h, int w, const void* w_base, int k_pad, const cg_bn_params& bn,
+                     const float* delta, float eps, int relu, void* y, void* pooled, unsigned long long* counters,
+                     cudaStream_t stream);
+// Whether that is faster than launch_stem and a pooling kernel.
+bool stem_pool_pays(int n, int h, int w);
+
 }  // namespace cg

@@ -9,8 +9,9 @@ calls.
 
 Layers that are not gated (the 7x7 stem, the 1x1 shortcut convolutions, the classifier) run as
 layers with G = 1, where the base path is the whole convolution (Section 3.1 allows eta = 1).
-The stem is one operator (cg_stem_forward); where its layer is not on tensor cores, and in passes that
-calibrate, it is a patch matrix (cg_im2col_bf16) followed by a 1x1 layer over it.
+The stem is one operator (cg_stem_forward; for batches that fill the device cg_stem_pool_forward, which does the
+pooling too); where its layer is not on tensor cores, and in passes that calibrate, it is a patch matrix
+(cg_im2col_bf16) followed by a 1x1 layer over it.
 
 Weights are random (Kaiming-normal); the batch-norm statistics, the gate statistics of Eq. 3 and
 the thresholds Delta come from a layer-by-layer calibration pass over a few images, which stands
@@ -232,6 +233,7 @@ class Instance:
         self.sub = {sh.name: torch.empty((n, sh.h, sh.h, sh.c_in), **bf) for sh, _, _, _ in net.blocks if sh}
         self.avg = torch.empty((n, 1, 1, net.fc.c_in), **bf)
         self.launches = None
+        self.stem_pools = self.convs["stem"].uses_tensor_cores and B.cg_stem_pool_pays(n, net.image, net.image)
 
     @property
     def patches(self):
@@ -242,9 +244,13 @@ class Instance:
         return self._patches
 
     def _fused_stem(self, x):
+        """The stem and, where one kernel does both, the pooling behind it."""
         s = self.net.specs[0]
         y = self.out[s.name]
-        B.cg_stem_forward(self.convs[s.name].handle, x, s.wb, s.bn, s.delta, y, self.stem_ws)
+        if self.stem_pools:
+            B.cg_stem_pool_forward(self.convs[s.name].handle, x, s.wb, s.bn, s.delta, y, self.pooled)
+        else:
+            B.cg_stem_forward(self.convs[s.name].handle, x, s.wb, s.bn, s.delta, y, self.stem_ws)
         return y
 
     def _conv(self, s, x, residual, before_conv, density, record):
@@ -278,7 +284,8 @@ class Instance:
         go = lambda s, a, r=None: timed(s.name, lambda: self._conv(s, a, r, before_conv, density, record))
         patch = lambda: B.cg_im2col_bf16(x, self.patches, STEM_K, STEM_STRIDE, STEM_PAD)   # noqa: E731
         stem = net.specs[0]
-        if before_conv is None and self.convs[stem.name].uses_tensor_cores:
+        fused = before_conv is None and self.convs[stem.name].uses_tensor_cores
+        if fused:
             a = timed(stem.name, lambda: self._fused_stem(x))
             if record is not None:                    # (the layer's input is the patch matrix)
                 patch()
@@ -286,7 +293,8 @@ class Instance:
         else:
             timed("stem.im2col", patch)
             a = go(stem, self.patches)
-        timed("maxpool", lambda: B.cg_maxpool_bf16(a, self.pooled, 3, 2, 1))
+        if not (fused and self.stem_pools):
+            timed("maxpool", lambda: B.cg_maxpool_bf16(a, self.pooled, 3, 2, 1))
         a = self.pooled
         for short, c1, c2, st in net.blocks:
             identity = a
@@ -318,7 +326,8 @@ class Instance:
         else:
             B.cg_im2col_bf16(x, self.patches, STEM_K, STEM_STRIDE, STEM_PAD)
             a = conv(stem, self.patches)
-        B.cg_maxpool_bf16(a, self.pooled, 3, 2, 1)
+        if not self.stem_pools:
+            B.cg_maxpool_bf16(a, self.pooled, 3, 2, 1)
         a = self.pooled
         for short, c1, c2, st in net.blocks:
             identity = a
@@ -335,7 +344,7 @@ class Instance:
     def launches_per_forward(self):
         """Kernels one forward pass launches: those of every layer plus the glue operators."""
         n = sum(B.cg_conv_launches_per_forward(c.handle) for c in self.convs.values())
-        return n + 3 + sum(1 for sh, _, _, st in self.net.blocks if sh is not None and st != 1)
+        return n + (1 if self.stem_pools else 3) + sum(1 for sh, _, _, st in self.net.blocks if sh is not None and st != 1)
 
     def stats(self):
         """Per-layer counters since the last call, and the network's FLOP summary (multiplications

@@ -131,3 +131,77 @@ def test_events_and_records_are_those_of_a_plain_pass(algo):
     assert spec.name == "stem" and patches.shape[-1] == spec.c_in and torch.equal(y, stem)
     assert len(record) == len(net.specs)
     inst.close()
+
+
+POOL_SIZES = [(1, 2, 2), (3, 5, 6), (1, 7, 10), (5, 33, 30), (1, 12, 300), (2, 9, 224), (3, 18, 226), (13, 40, 112), (6, 224, 224)]
+
+
+@pytest.mark.parametrize("n,h,w", POOL_SIZES)
+@pytest.mark.parametrize("dv,relu", [(K.INF, True), (K.INF, False), (0.0, True)])
+def test_stem_and_pooling_in_one_kernel(n, h, w, dv, relu):
+    """Strips that end inside a group, a second column tile, odd output extents, several items per block: y against the
+    oracle, the maxima against the pooling kernel over that y, bit by bit (with pixels that are not finite)."""
+    import torch
+    from paper_1805_12549_b200 import binding as B
+    key = ("stempool", n, h, w)
+    x = synth.bf16_round(synth.rng(key, "x").standard_normal((n, h, w, 3), dtype=np.float32))
+    if dv == K.INF and h > 4:
+        x[0, h // 2, w // 2, 1] = np.inf
+        x[n - 1, h - 1, w - 1, 2] = np.nan
+    wt, _ = synth.kaiming_weights(key, 64, 7, 7, 3, 1)
+    wt = synth.bf16_round(wt)
+    bn, delta = synth.bn_params(key, 64), np.full(64, dv, np.float32)
+    ref = O.gated_conv(O.Shape(n, h, w, 3, 64, 7, 7, 2, 3, 1, 1e-5, int(relu)), x, wt, np.zeros((64, 7, 7, 0), np.float32), bn, delta,
+                       None, out_bf16=True)
+    dev = lambda a: torch.from_numpy(synth.bf16_bits(np.ascontiguousarray(a, np.float32)).view(np.int16)).cuda().view(torch.bfloat16)  # noqa: E731
+    ho, wo = (h - 1) // 2 + 1, (w - 1) // 2 + 1
+    hp, wp = (ho - 1) // 2 + 1, (wo - 1) // 2 + 1
+    conv = B.GatedConv(n + 1, ho, wo, 192, 64, k=1, pad=0, groups=1, relu=relu)      # (a handle for more images)
+    wflat = np.zeros((64, 192), np.float32)
+    wflat[:, :147] = wt.reshape(64, -1)
+    params = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in bn.items() if v is not None}
+    guard = [torch.full((n * a * b * 64 + 4096,), 7.0, dtype=torch.bfloat16, device="cuda") for a, b in ((ho, wo), (hp, wp))]
+    y, pooled = guard[0][2048:-2048].view(n, ho, wo, 64), guard[1][2048:-2048].view(n, hp, wp, 64)
+    B.cg_stem_pool_forward(conv.handle, dev(x), dev(wflat), B.make_bn(params), torch.from_numpy(delta).cuda(), y, pooled)
+    st = conv.stats()
+    conv.close()
+    assert all(bool((g[:2048] == 7).all()) and bool((g[-2048:] == 7).all()) for g in guard)
+    with np.errstate(invalid="ignore"):
+        near = np.abs((ref.p.reshape(-1, 64) - bn["mean_base"]) / np.sqrt(bn["var_base"] + 1e-5) - delta) < K.NEAR_TIE
+    finite = np.isfinite(ref.p)
+    out = y.float().cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        err = np.abs(out.astype(np.float64) - ref.y) - K.BF16_ATOL - K.BF16_RTOL * np.abs(ref.y)
+    assert (err[finite.reshape(ref.y.shape) & ~near.reshape(ref.y.shape)] <= 0).all()
+    assert st.calls == 1 and st.device_status == 0 and abs(st.active - ref.active) <= near.sum()
+    assert st.rows_total == (n * ho * wo) * 2 and abs(st.rows_active - np.count_nonzero(ref.mask)) <= near.sum()
+    want = torch.empty_like(pooled)
+    B.cg_maxpool_bf16(y.contiguous(), want, 3, 2, 1)
+    assert torch.equal(pooled.view(torch.int16), want.view(torch.int16))
+
+
+def test_a_network_of_a_large_batch_pools_in_the_stem():
+    """The same logits and stem activations as the two kernels, with the operators and launches that a pass then has."""
+    import torch
+    from paper_1805_12549_b200 import binding as B, resnet18 as R
+    assert B.cg_stem_pool_pays(8, 224, 224) and not B.cg_stem_pool_pays(1, 224, 224) and not B.cg_stem_pool_pays(500, 224, 223)
+    net = R.CgResNet18(image=224, classes=20)
+    net.set_density(1.0)
+    x = R.synthetic_images("stempoolnet", 8, 224)
+    inst = net.instance(8)
+    assert inst.stem_pools
+    a = inst.forward(x).clone()
+    stem, pooled = inst.out["stem"].clone(), inst.pooled.clone()
+    events, record = [], []
+    assert torch.equal(inst.forward(x, events=events), a) and torch.equal(inst.forward(x, record=record), a)
+    names = [name for name, _, _ in events]
+    assert "maxpool" not in names and len(names) == inst.launches_per_forward()
+    assert torch.equal(record[0][3], stem) and len(record) == len(net.specs)
+    inst.stem_pools = False
+    b = inst.forward(x)
+    torch.cuda.synchronize()
+    # (another order of fp32 sums: some outputs differ by a bf16 rounding)
+    for u, v in ((inst.out["stem"], stem), (inst.pooled, pooled)):
+        assert float((u.float() - v.float()).norm()) <= 1e-3 * float(v.float().norm())
+    assert float((a.float() - b.float()).norm()) <= 3e-2 * float(b.float().norm())
+    inst.close()
