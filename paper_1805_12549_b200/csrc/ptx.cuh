@@ -454,6 +454,18 @@ __device__ __forceinline__ uint4 ld_shared_16(uint32_t addr) {
   asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
   return v;
 }
+// Global loads of what a kernel in front of this one may have written (after grid_dependency_wait; the non-coherent path of
+// __ldg is for memory that nothing writes while the kernel lives, its time before the wait included).
+__device__ __forceinline__ uint4 ld_global_16(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint2 ld_global_8(const void* p) {
+  uint2 v;
+  asm volatile("ld.global.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
 // shared::cluster address of this CTA's shared-memory address `addr` in CTA `rank` of the cluster.
 __device__ __forceinline__ uint32_t map_cluster(uint32_t addr, uint32_t rank) {
   uint32_t ra;
@@ -514,20 +526,21 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// 16 bytes at this CTA's shared-memory address `addr`, read from CTA `rank` of the cluster.
-__device__ __forceinline__ uint4 ld_cluster_16(uint32_t addr, uint32_t rank) {
-  uint4 v;
-  asm volatile(
-      "{\n"
-      " .reg .b32 ra;\n"
-      " mapa.shared::cluster.u32 ra, %4, %5;\n"
-      " ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [ra];\n"
-      "}"
-      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-      : "r"(addr), "r"(rank)
-      : "memory");
-  return v;
+// The same, ordering nothing: it does not wait for the threads' stores.
+__device__ __forceinline__ void cluster_sync_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
+// Copy from this CTA's shared memory to a shared::cluster address, counted on the barrier at shared::cluster address `bar`;
+// both 16-byte aligned, whole 16 bytes.  What generic stores wrote there is the copy's behind fence_proxy_async.
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src),
+               "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// Waits until this thread's copies have read their source.
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t ld_cluster_4(uint32_t addr, uint32_t rank) {
   uint32_t v;

@@ -25,8 +25,8 @@
 // Jobs are 256 pixels of a CTA pair (cta_group::2): each SM holds half of a job's pixels and half of its
 // weights, which halves what an SM has to fetch from L2 and what an MMA reads of shared memory (one CTA's
 // 128 x 128 MMA takes the whole 128 bytes per clock).  Layers with fewer jobs than SMs instead split the K
-// loop of a 128-pixel job over the 2, 4 or 8 CTAs of a cluster: each leaves its sums in shared memory, and
-// every CTA adds up and finishes 1/split of the rows.
+// loop of a 128-pixel job over the 2, 4 or 8 CTAs of a cluster: every CTA finishes 1/split of the rows, and is sent the
+// others' sums of those by bulk copies between the CTAs' shared memories.
 //
 // Warp roles (640 threads): 0 = patch producer, 2 = weight producer, 1 = MMA issuer, 4-19 = epilogue (TMEM
 // lane quadrant x 32 channels).  The epilogue keeps out of shared memory, whose bandwidth the MMAs' operands
@@ -61,6 +61,7 @@ namespace {
 
 constexpr int kT4Threads = 640;
 constexpr int kEpiWarp0 = 4, kEpiWarps = 16, kEpiThreads = kEpiWarps * 32;
+constexpr unsigned kSumPitch = (64 + 4) * 4;           // a row of partial sums on its way to the CTA that finishes it
 constexpr int kMaxNA = 8, kMaxNB = 16;
 constexpr int kSpinLimit = 1 << 21;
 constexpr long long kWaitCycles = 2000000000ll;
@@ -86,9 +87,11 @@ struct Shared4 {
   uint64_t a_full[kMaxNA], a_empty[kMaxNA];
   uint64_t b_full[kMaxNB], b_empty[kMaxNB];
   uint64_t acc_full[4], acc_empty[4];
+  uint64_t sums;         // the cluster's sums of this CTA's rows have arrived
   uint32_t tmem_base;
   uint32_t abort_flag;
   uint32_t active, rows_active;
+  uint32_t epi_done;     // epilogue warps that have added theirs
   uint32_t maybe_shut;   // no gate of the column tile could fire when the block started
 };
 static_assert(sizeof(Shared4) <= kOffConsts, "barrier block");
@@ -129,7 +132,6 @@ struct Cursor {
   int slot;
   uint32_t par;
   __device__ __forceinline__ void next(int n) { if (++slot == n) { slot = 0; par ^= 1u; } }
-  __device__ __forceinline__ void at(unsigned i, unsigned n) { const unsigned q = i / n; slot = (int)(i - q * n); par = q & 1u; }
 };
 
 // The MMAs of one row of the table: up to three tiles of NKS K slices.
@@ -306,12 +308,11 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
       } else if (KP < 4 && q == 0) {
         // the first chunk holds the base channels (KP slices of every tap, several taps per weight tile) and the first
         // conditional ones
-        constexpr int kPer = 4 / (KP < 4 ? KP : 1), kCond = 4 - KP > 0 ? 4 - KP : 1, kFirst = KP < 4 ? KP : 0;
-        uint32_t base_at = 0;
-        int base_slot = 0;
+        constexpr int kCond = 4 - KP > 0 ? 4 - KP : 1, kFirst = KP < 4 ? KP : 0;
         if (kWin) take_a();
         take_b();
-        base_at = b_at; base_slot = b_slot;
+        const uint32_t base_at = b_at;
+        const int base_slot = b_slot;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
           if (!kWin) take_a();
@@ -623,7 +624,7 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
               m[h] = __shfl_sync(0xffffffffu, own, r4 + 16 * i + 8 * h);
               if (kRes) {
                 res[h] = make_uint4(0u, 0u, 0u, 0u);
-                if (has_res && m[h] >= 0) res[h] = __ldg((const uint4*)(prm.residual + (long long)m[h] * L.c_out + ch + q8));
+                if (has_res && m[h] >= 0) res[h] = ptx::ld_global_16(prm.residual + (long long)m[h] * L.c_out + ch + q8);
               }
             }
             uint32_t out[2][4];
@@ -720,8 +721,29 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
           else ptx::mbar_arrive(&sh->acc_empty[stage]);
         }
       }
-    } else if (jobs > 0) {
-      // this CTA's share of the sums goes to shared memory (the rings are idle once every MMA is done)
+    }
+    if constexpr (SPLIT) {
+      // rows [part * rows, (part + 1) * rows) of the job are this CTA's to finish: four channels per thread
+      constexpr int kLanes = NT / 4;                           // threads per row
+      const int rows = 128 / P.split;
+      const uint32_t block = (uint32_t)rows * kSumPitch;       // a CTA's sums of those rows, of one path
+      struct Item { long long at; int m; uint2 res; bool valid; };
+      auto item = [&](int u) {
+        Item t;
+        const int lr = u / kLanes, cc = (u % kLanes) * 4;
+        const uint32_t pos = (uint32_t)(group * 128 + part * rows + lr);
+        const uint32_t n0 = P.div_ip.div(pos), rem = pos - n0 * (uint32_t)(P.wp * P.hp);
+        const uint32_t h0 = P.div_wp.div(rem), w0 = rem - h0 * (uint32_t)P.wp;
+        const int ch = tile_n * NT + cc;
+        t.valid = u < rows * kLanes && jobs > 0 && (int)n0 < L.n && (int)h0 < L.ho && (int)w0 < L.wo && ch < L.c_out;
+        t.m = t.valid ? (int)((n0 * L.ho + h0) * L.wo + w0) : 0;
+        t.at = (long long)t.m * L.c_out + ch;
+        t.res = make_uint2(0u, 0u);
+        if (!I8 && prm.residual && t.valid) t.res = ptx::ld_global_8(prm.residual + t.at);
+        return t;
+      };
+      Item next = item(et);                                    // (a residual is on its way while the sums are waited for)
+      // This CTA's share of the sums goes to shared memory (the rings are idle once every MMA is done) ...
       ok = wait4(sh, prm.counters, &sh->acc_full[0], 0, 7);
       if (ok) {
         ptx::tc_fence_after();
@@ -731,46 +753,51 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
           ptx::tmem_ld_nowait<32>(t_lane + (uint32_t)(path * NT + c0), v);
           ptx::tmem_ld_wait<32>(v);
           // (columns 2i, 2i+1 are channels 8*(i%4) + 2*(i/4), + 1 of the block: the weight tiles' row order)
-          uint2* dst = (uint2*)(smem + kOffStages + ((size_t)path * 128 + row) * (NT + 4) * 4 + c0 * 4);
+          uint2* dst = (uint2*)(smem + kOffStages + ((unsigned)path * 128u + (unsigned)row) * kSumPitch + (unsigned)c0 * 4u);
 #pragma unroll
           for (int i = 0; i < 16; ++i) dst[(i & 3) * 4 + (i >> 2)] = make_uint2(v[2 * i], v[2 * i + 1]);
         }
         ptx::tc_fence_before();
+        ptx::fence_proxy_async();
       }
-    }
-    if (SPLIT) {
+      // ... and from there, one copy per path, to the CTAs that finish its rows.  (Read by them through distributed shared
+      // memory, 16 bytes a thread, they took 3,500 of a layer's 10,000 cycles, in flight together or not.)
+      ok = !ptx::named_bar_or(3, kEpiThreads, !ok);
+      if (P.sums_late) ptx::cluster_sync();                    // (their room is part of the rings: no MMA reads those any more)
+      const int turn = warp - kEpiWarp0 + 1;                   // (one destination a warp, another one first in every CTA: all
+      if (ok && turn <= P.split && lane < 2) {                 // sending to the first and then to the second took three times as long)
+        const int to = (part + turn) & (P.split - 1), mine = lane ? P.r_mask : P.p_mask;
+        if ((mine >> part) & 1) {
+          const int slot = (lane ? __popc(P.p_mask) : 0) + __popc(mine & ((1 << part) - 1));
+          ptx::bulk_copy_cluster(ptx::map_cluster(ptx::smem_u32(smem) + P.off_sums + (uint32_t)slot * block, (uint32_t)to),
+                                 ptx::smem_u32(smem) + kOffStages + (uint32_t)lane * 128u * kSumPitch + (uint32_t)to * block, block,
+                                 ptx::map_cluster(ptx::smem_u32(&sh->sums), (uint32_t)to));
+          ptx::bulk_commit();
+        }
+      }
       __syncwarp();
-      ptx::cluster_sync();
-      // rows part, part + split, ...: four channels per thread, the partial sums of the CTAs in order
-      constexpr int kLanes = NT / 4;                           // threads per row
-      const int rows = 128 / P.split;
-      for (int u = et; u < rows * kLanes; u += kEpiThreads) {
-        const int lr = u / kLanes, cc = (u % kLanes) * 4;
-        const int rrow = part + lr * P.split;
-        const int pos = group * 128 + rrow;
-        const int ip = P.wp * P.hp, n0 = pos / ip, rem = pos - n0 * ip, h0 = rem / P.wp, w0 = rem - h0 * P.wp;
-        const int ch = tile_n * NT + cc;
-        const bool valid = jobs > 0 && n0 < L.n && h0 < L.ho && w0 < L.wo && ch < L.c_out;
-        const long long m = ((long long)n0 * L.ho + h0) * L.wo + w0;
+      ok = ok && wait4(sh, prm.counters, &sh->sums, 0, 9);
+      const int p_slots = __popc(P.p_mask), slots = p_slots + __popc(P.r_mask);
+      for (int u = et; ok && u < rows * kLanes; u += kEpiThreads) {
+        const Item t = next;
+        const int lr = u / kLanes, cc = (u % kLanes) * 4, ch = tile_n * NT + cc;
         uint32_t w = 0;
-        if (valid) {
-          float pf[4] = {0.f, 0.f, 0.f, 0.f}, rf[4] = {0.f, 0.f, 0.f, 0.f};
-          int pi[4] = {0, 0, 0, 0}, ri[4] = {0, 0, 0, 0};
-          const uint32_t off = ptx::smem_u32(smem + kOffStages) + (uint32_t)(rrow * (NT + 4) + cc) * 4u;
-#pragma unroll
-          for (int peer = 0; peer < kTc4MaxSplit; ++peer) {
-            if (peer >= P.split) break;
-            if ((P.p_mask >> peer) & 1) {
-              const uint4 v = ptx::ld_cluster_16(off, (uint32_t)peer);
-              if (I8) { pi[0] += (int)v.x; pi[1] += (int)v.y; pi[2] += (int)v.z; pi[3] += (int)v.w; }
-              else { pf[0] += __uint_as_float(v.x); pf[1] += __uint_as_float(v.y); pf[2] += __uint_as_float(v.z); pf[3] += __uint_as_float(v.w); }
-            }
-            if ((P.r_mask >> peer) & 1) {
-              const uint4 v = ptx::ld_cluster_16(off + 128u * (NT + 4) * 4u, (uint32_t)peer);
-              if (I8) { ri[0] += (int)v.x; ri[1] += (int)v.y; ri[2] += (int)v.z; ri[3] += (int)v.w; }
-              else { rf[0] += __uint_as_float(v.x); rf[1] += __uint_as_float(v.y); rf[2] += __uint_as_float(v.z); rf[3] += __uint_as_float(v.w); }
-            }
+        float pf[4] = {0.f, 0.f, 0.f, 0.f}, rf[4] = {0.f, 0.f, 0.f, 0.f};
+        int pi[4] = {0, 0, 0, 0}, ri[4] = {0, 0, 0, 0};
+        const uint32_t off = ptx::smem_u32(smem) + P.off_sums + (uint32_t)lr * kSumPitch + (uint32_t)cc * 4u;
+        // the partial sums of the CTAs in order
+        for (int k = 0; k < slots; ++k) {
+          const uint4 v = ptx::ld_shared_16(off + (uint32_t)k * block);
+          if (k < p_slots) {
+            if (I8) { pi[0] += (int)v.x; pi[1] += (int)v.y; pi[2] += (int)v.z; pi[3] += (int)v.w; }
+            else { pf[0] += __uint_as_float(v.x); pf[1] += __uint_as_float(v.y); pf[2] += __uint_as_float(v.z); pf[3] += __uint_as_float(v.w); }
+          } else {
+            if (I8) { ri[0] += (int)v.x; ri[1] += (int)v.y; ri[2] += (int)v.z; ri[3] += (int)v.w; }
+            else { rf[0] += __uint_as_float(v.x); rf[1] += __uint_as_float(v.y); rf[2] += __uint_as_float(v.z); rf[3] += __uint_as_float(v.w); }
           }
+        }
+        if (u + kEpiThreads < rows * kLanes) next = item(u + kEpiThreads);
+        if (t.valid) {
           if (I8) {
             uint32_t v = 0;
 #pragma unroll
@@ -781,7 +808,7 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
               const longlong2 o = s_o[cc + e];
               v |= ((uint32_t)finish_q(d ? k.z : k.y, d ? o.y : o.x, pi[e] + (d ? ri[e] : 0), L.shift, lo_q) & 255u) << (8 * e);
             }
-            *(uint32_t*)((uint8_t*)prm.y + m * L.c_out + ch) = v;
+            *(uint32_t*)((uint8_t*)prm.y + t.at) = v;
           } else {
             float v[4];
 #pragma unroll
@@ -793,13 +820,12 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
               v[e] = d ? full : base;
             }
             if (prm.residual) {
-              const uint2 x = __ldg((const uint2*)(prm.residual + m * L.c_out + ch));
-              v[0] += __uint_as_float(x.x << 16); v[1] += __uint_as_float(x.x & 0xffff0000u);
-              v[2] += __uint_as_float(x.y << 16); v[3] += __uint_as_float(x.y & 0xffff0000u);
+              v[0] += __uint_as_float(t.res.x << 16); v[1] += __uint_as_float(t.res.x & 0xffff0000u);
+              v[2] += __uint_as_float(t.res.y << 16); v[3] += __uint_as_float(t.res.y & 0xffff0000u);
             }
             uint2 o = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
             if (L.relu) o = make_uint2(relu_bf16x2(o.x), relu_bf16x2(o.y));
-            *(uint2*)((__nv_bfloat16*)prm.y + m * L.c_out + ch) = o;
+            *(uint2*)((__nv_bfloat16*)prm.y + t.at) = o;
           }
         }
         // eight neighbouring threads hold the 32 channels of a mask word
@@ -807,16 +833,26 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
         w |= __shfl_xor_sync(0xffffffffu, w, 1);
         w |= __shfl_xor_sync(0xffffffffu, w, 2);
         w |= __shfl_xor_sync(0xffffffffu, w, 4);
-        if (valid && (lane & 7) == 0) {
+        if (t.valid && (lane & 7) == 0) {
           active += (uint32_t)__popc(w);
           rows_active += w != 0u ? 1u : 0u;
-          if (prm.mask) prm.mask[m * L.words + (ch >> 5)] = w;
+          if (prm.mask) prm.mask[(long long)t.m * L.words + (ch >> 5)] = w;
         }
       }
+      if (warp - kEpiWarp0 < P.split) ptx::bulk_wait_read();   // (the copies have left this CTA's shared memory)
     }
     active = __reduce_add_sync(0xffffffffu, active);
     rows_active = __reduce_add_sync(0xffffffffu, rows_active);
-    if (lane == 0) { atomicAdd(&sh->active, active); atomicAdd(&sh->rows_active, rows_active); }
+    if (lane == 0) {
+      // the last warp sends the block's counts on their way, ahead of the cluster's last barrier
+      atomicAdd(&sh->active, active); atomicAdd(&sh->rows_active, rows_active);
+      __threadfence_block();
+      if (atomicAdd(&sh->epi_done, 1u) == (uint32_t)kEpiWarps - 1u && !*(volatile uint32_t*)&sh->abort_flag) {
+        const uint32_t all = atomicAdd(&sh->active, 0u), all_rows = atomicAdd(&sh->rows_active, 0u);
+        if (all) atomicAdd(&prm.counters[CNT_ACTIVE], (unsigned long long)all);
+        if (all_rows) atomicAdd(&prm.counters[CNT_ROWS_ACTIVE], (unsigned long long)all_rows);
+      }
+    }
   }
 }
 
@@ -831,7 +867,8 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   const LayerDims& L = prm.L;
   const Tc4Plan& P = prm.P;
   Shared4* sh = (Shared4*)smem;
-  constexpr int kAcc = 512 / (2 * NT);                         // accumulator pairs in TMEM
+  constexpr uint32_t kCols = PAIR ? 512 : 2 * NT;              // TMEM columns
+  constexpr int kAcc = (int)kCols / (2 * NT);                  // accumulator pairs in them
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const unsigned members = PAIR ? 2u : (unsigned)P.split;      // CTAs of a cluster
@@ -842,14 +879,20 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   const int jobs = group < P.tiles_m ? (P.tiles_m - group + groups - 1) / groups : 0;
   const bool has_cond = L.c_r > 0;
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < P.na; ++i) { ptx::mbar_init(&sh->a_full[i], 1); ptx::mbar_init(&sh->a_empty[i], 1); }
-    for (int i = 0; i < P.nb; ++i) { ptx::mbar_init(&sh->b_full[i], 1); ptx::mbar_init(&sh->b_empty[i], 1); }
-    for (int i = 0; i < kAcc; ++i) {
-      ptx::mbar_init(&sh->acc_full[i], 1);
-      ptx::mbar_init(&sh->acc_empty[i], (PAIR ? 2 : 1) * NT / 8);   // warps per job, of both CTAs of a pair
+  if (warp == 0) {
+    // (one barrier of a kind per lane: fifty in a row by one thread are a third of the set-up)
+    if (lane < P.na) { ptx::mbar_init(&sh->a_full[lane], 1); ptx::mbar_init(&sh->a_empty[lane], 1); }
+    if (lane < P.nb) { ptx::mbar_init(&sh->b_full[lane], 1); ptx::mbar_init(&sh->b_empty[lane], 1); }
+    if (lane < kAcc) {
+      ptx::mbar_init(&sh->acc_full[lane], 1);
+      ptx::mbar_init(&sh->acc_empty[lane], (PAIR ? 2 : 1) * NT / 8);   // warps per job, of both CTAs of a pair
     }
-    sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0;
+    if (SPLIT && lane == 0) {
+      // what the cluster sends here: P and R of this CTA's rows from every CTA that has some
+      ptx::mbar_init(&sh->sums, 1);
+      ptx::mbar_expect_tx(&sh->sums, (uint32_t)(__popc(P.p_mask) + __popc(P.r_mask)) * (128u / (unsigned)P.split) * kSumPitch);
+    }
+    if (lane == 0) { sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0; sh->epi_done = 0; }
     ptx::fence_mbar_init();
   }
   if (threadIdx.x == 32 * 2) { ptx::prefetch_tensormap(&map_x); ptx::prefetch_tensormap(&map_wb); ptx::prefetch_tensormap(&map_wc); }
@@ -862,9 +905,9 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     if (lane == 0) sh->maybe_shut = shut ? 1u : 0u;
   }
   __syncwarp();
-  if (warp == 1) { if (PAIR) ptx::tmem_alloc_pair(&sh->tmem_base, 512); else ptx::tmem_alloc(&sh->tmem_base, 512); }
+  if (warp == 1) { if (PAIR) ptx::tmem_alloc_pair(&sh->tmem_base, kCols); else ptx::tmem_alloc(&sh->tmem_base, kCols); }
   ptx::tc_fence_before();
-  if (PAIR) ptx::cluster_sync(); else __syncthreads();
+  ptx::cluster_sync();
   ptx::tc_fence_after();
   // everything above touched only this cluster's own state
   ptx::grid_dependency_wait();
@@ -891,7 +934,7 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     run_roles<NT, I8, PAIR, false>(map_x, map_wb, map_wc, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
   }
   __syncwarp();
-  if (SPLIT && warp < kEpiWarp0) ptx::cluster_sync();
+  if (SPLIT && P.sums_late && warp < kEpiWarp0) ptx::cluster_sync();
   // ---------------------------------------------------------------- teardown
   if (*(volatile uint32_t*)&sh->abort_flag) {
     // a wait gave up somewhere: let copies and MMAs that are still in flight finish (they take
@@ -901,12 +944,11 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
   __syncwarp();
   ptx::tc_fence_before();
-  // no CTA leaves while a peer may still use its shared memory or TMEM
-  ptx::cluster_sync();
+  // No CTA leaves while a peer may still use its shared memory or TMEM.  (A cluster's CTA has waited for all that is sent to it
+  // and sent on, and its stores to global memory need not be waited for.)
+  if (PAIR) ptx::cluster_sync(); else ptx::cluster_sync_relaxed();
   ptx::tc_fence_after();
   if (threadIdx.x == 0 && !*(volatile uint32_t*)&sh->abort_flag) {
-    if (sh->active) atomicAdd(&prm.counters[CNT_ACTIVE], (unsigned long long)sh->active);
-    if (sh->rows_active) atomicAdd(&prm.counters[CNT_ROWS_ACTIVE], (unsigned long long)sh->rows_active);
     if (shut && part == 0) {
       // the jobs without conditional rows are taken from the totals below
       atomicAdd(&prm.counters[CNT_TILES_TOTAL], 0ull - (unsigned long long)jobs);
@@ -922,7 +964,7 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
   if (warp == 1) {
     __syncwarp();
-    if (PAIR) ptx::tmem_dealloc_pair(tmem, 512); else ptx::tmem_dealloc(tmem, 512);
+    if (PAIR) ptx::tmem_dealloc_pair(tmem, kCols); else ptx::tmem_dealloc(tmem, kCols);
   }
 }
 
@@ -1115,7 +1157,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   const int tn64 = (L.c_out + 63) / 64, tn128 = (L.c_out + 127) / 128;
 
   P.split = 1;
-  const int room = (int)(kSmemBytes - 1024 - kOffStages);
+  int room = (int)(kSmemBytes - 1024 - kOffStages);
   RawRow raw[kTc4MaxRows];
   // (1x1 layers of up to three chunks have one row and nothing to share: as pairs they end without the exchange of
   // sums, 28x28 x 64 -> 128, one image, 8.5 and 5.0 us)
@@ -1175,8 +1217,16 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     }
   }
 
-  // shared memory: resident weights if they leave room for three patch slots, else rings of both
   P.stage_bytes = 3 * (P.pair ? P.nt / 2 : P.nt) * 128;
+  // a cluster's CTA: room for the sums that are sent to it, and for its own behind the rings' start
+  const unsigned sums_bytes = P.pair ? 0u : (unsigned)(__builtin_popcount(P.p_mask) + __builtin_popcount(P.r_mask)) * (128u / (unsigned)P.split) * kSumPitch;
+  // (within the rings' room, and one cluster barrier later, where the job's patches would not all fit beside it: tap by tap
+  // 256->512 at 14x14, one image, 8.1 us beside the rings)
+  const int slots_wanted = max_a < kMaxNA ? max_a : kMaxNA, stages_wanted = max_b < 3 ? max_b : 3;
+  P.sums_late = !P.pair && P.mode == kTc4Taps && room - (int)sums_bytes < slots_wanted * P.slot_bytes + stages_wanted * P.stage_bytes;
+  if (!P.sums_late) room -= (int)sums_bytes;
+
+  // shared memory: resident weights if they leave room for three patch slots, else rings of both
   const int clusters = P.grid / (P.pair ? 2 : P.split);
   const int jobs = P.pair ? (P.tiles_m + clusters / P.tiles_n - 1) / (clusters / P.tiles_n) : 1;
   if (max_b <= kMaxNB && jobs > 1 && room - max_b * P.stage_bytes >= 3 * P.slot_bytes) {
@@ -1187,6 +1237,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     int na = P.mode == kTc4Window ? 3 : 2;
     if (na > max_a * jobs) na = max_a * jobs;
     while (na > 2 && room - na * P.slot_bytes < 4 * P.stage_bytes) --na;
+    if (!P.pair && na > 1 && room - na * P.slot_bytes < 3 * P.stage_bytes) --na;
     P.nb = (room - na * P.slot_bytes) / P.stage_bytes;
     if (P.nb < 3) return false;
     if (P.nb > kMaxNB) P.nb = kMaxNB;
@@ -1194,7 +1245,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   }
   P.na = (room - P.nb * P.stage_bytes) / P.slot_bytes;         // what is left goes to patches
   if (P.na > kMaxNA) P.na = kMaxNA;
-  if (P.na < 1 || (P.na < 2 && max_a * jobs > 1)) return false;
+  if (P.na < 1 || (P.pair && P.na < 2 && max_a * jobs > 1)) return false;
   if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) plan_base(raw, &P);
   for (int i = 0; i < P.rows; ++i) {
     P.row[i] = raw[i].r;
@@ -1202,6 +1253,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.off_b = kOffStages;
   P.off_a = kOffStages + (unsigned)(P.nb * P.stage_bytes);
   P.smem_bytes = kSmemBytes;
+  if (!P.pair) P.off_sums = P.sums_late ? kOffStages + 2u * 128u * kSumPitch : kSmemBytes - 1024 - sums_bytes;
   P.valid = 1;
   *plan = P;
   return true;

@@ -61,7 +61,8 @@ struct Tc4Plan {
   int base_rows;                   // 0: all jobs run all rows
   unsigned long long base_mask;    // which rows
   uint8_t p_mask, r_mask;          // which CTAs of a cluster add to P / to R
-  unsigned off_b, off_a, smem_bytes;
+  int sums_late;         // the sums that a cluster exchanges lie within the rings
+  unsigned off_b, off_a, off_sums, smem_bytes;
   Tc4Row row[kTc4MaxRows];
 };
 
