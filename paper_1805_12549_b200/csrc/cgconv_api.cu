@@ -247,7 +247,7 @@ int cg_conv_plan_string(cg_conv_t h, char* buf, size_t len) {
                          "weights (%d stages), %d patch slots of %d bytes, grid %d",
                          P.tiles_m, P.pair ? 256 : 128, P.tiles_n, P.nt,
                          P.mode == cg::kTc4Window ? "one patch for all taps" : (P.mode == cg::kTc4Taps ? "one patch per tap" : "1x1"),
-                         P.rows, P.split, P.resident ? "resident" : "streamed", P.nb, P.na, P.slot_bytes, P.grid);
+                         P.rows, P.split, P.packed ? "packed" : P.resident ? "resident" : "streamed", P.nb, P.na, P.slot_bytes, P.grid);
   }
   if (h->use_tc) {
     const cg::TcPlan& P = h->plan;

@@ -165,6 +165,20 @@ __device__ __forceinline__ void issue_taps(uint32_t d, uint32_t hi, uint32_t a, 
   }
 }
 
+// The same with the weights' K slices packed (Tc4Plan::packed): a tap has PT conditional slices, of which the patch's chunk takes
+// NK from FIRST on, beside its own slices from K0 on.  Filter row R; `a` is its first tap.
+template <bool I8, int R, int PT, int FIRST, int K0, int NK>
+__device__ __forceinline__ void issue_packed(uint32_t d, uint32_t hi, uint32_t a, uint32_t b, uint32_t tile, uint32_t idesc, uint32_t acc) {
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+      const int s = (3 * R + t) * PT + FIRST + k;
+      ptx::umma<true, I8>(d, ((uint64_t)hi << 32) | (a + 8u * t + 2u * (K0 + k)),
+                          ((uint64_t)hi << 32) | (b + (uint32_t)(s / 4) * tile + (uint32_t)(s % 4) * 2u), idesc, t == 0 && k == 0 ? acc : 1u);
+    }
+}
+
 // One row of the table in shared memory.
 __device__ __forceinline__ Tc4Row row_at(uint32_t table, int i) {
   const uint4 v = ptx::ld_shared_16(table + (uint32_t)i * 16u);
@@ -248,7 +262,8 @@ struct IssueRing {
 // the base path; 4: the base path is whole chunks) are constants, so that a filter row is one look at its weights' barrier,
 // its MMAs and a commit: walked from a table of row kinds, a row's loads, tests and branches took 700 cycles beside the 576 of
 // nine MMAs of 64, two issuers taking turns.
-template <int NT, bool I8, bool BASE, int MODE, int KP>
+// CH: chunks of a layer with packed weights, else 0.
+template <int NT, bool I8, bool BASE, int MODE, int KP, int CH = 0>
 __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, uint32_t a0, uint32_t b0, uint32_t tmem, int jobs) {
   constexpr int kAcc = 512 / (2 * NT);
   constexpr uint32_t kTileU = (uint32_t)(NT / 2) * 8u;         // a weight tile, 16-byte units
@@ -265,6 +280,7 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
   const int chunks = BASE ? (prm.L.c_p + ck - 1) / ck : prm.L.c_in / ck, base_chunks = KP == 4 ? prm.L.c_p / ck : 0;
   IssueRing a{0, 0u, a0}, b{0, 0u, b0};
   bool ok = true, a_seen = false, b_seen = false;
+  int tiles_seen = 0;                                          // (packed weights)
   bool new_b = true;                                           // weights are waited for (resident ones: by the first job)
   uint32_t a_at = 0, b_at = 0;
   int a_slot = 0, b_slot = 0;
@@ -281,6 +297,10 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
     // a look at the next stage's barrier, whose answer arrives while this one's MMAs are issued
     b_seen = new_b && ptx::mbar_test_wait(&sh->b_full[b.slot], b.par);
   };
+  auto need_tile = [&](int tile) {
+    for (; ok && tiles_seen <= tile; tiles_seen += 3)
+      ok = wait4_one(sh, prm.counters, &sh->b_full[tiles_seen / 3], 0, 5);
+  };
   auto look_a = [&]() { a_seen = ptx::mbar_test_wait(&sh->a_full[a.slot], a.par); };
   auto free_a = [&]() { ptx::umma_commit_pair(&sh->a_empty[a_slot]); };
   auto free_b = [&](int slot) { if (!resident) ptx::umma_commit_pair(&sh->b_empty[slot]); };
@@ -291,7 +311,33 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
     ptx::tc_fence_after();
     const uint32_t d_p = tmem + (uint32_t)(stage * 2 * NT), d_r = d_p + NT;
     if (resident) { b = IssueRing{0, 0u, b0}; new_b = j == 0; b_seen = false; }
-    for (int q = 0; q < chunks; ++q) {
+    if constexpr (CH > 0) {
+      static_assert(CH == 0 || CH == 2, "two chunks");
+      constexpr int PT = 8 - KP;                               // conditional slices of a tap
+      const uint32_t bc = b0 + (uint32_t)P.tiles_base * kTileU;
+      take_a();
+      need_tile(P.tiles_base - 1);
+      if (!ok) return;
+      issue_taps<true, I8, 0, 9, 0, 0, KP, 4 / KP, 0>(d_p, hi, a_at, row_lo, kStep, b0, kTileU, idesc, 0u);
+      if (!BASE) {
+        auto upto = [&](int last) { need_tile(P.tiles_base + last / 4); return ok; };
+        if (!upto(2 * PT + 3 - KP)) return;
+        issue_packed<I8, 0, PT, 0, KP, 4 - KP>(d_r, hi, a_at, bc, kTileU, idesc, 0u);
+        if (!upto(5 * PT + 3 - KP)) return;
+        issue_packed<I8, 1, PT, 0, KP, 4 - KP>(d_r, hi, a_at + row_lo, bc, kTileU, idesc, 1u);
+        if (!upto(8 * PT + 3 - KP)) return;
+        look_a();
+        issue_packed<I8, 2, PT, 0, KP, 4 - KP>(d_r, hi, a_at + 2u * row_lo, bc, kTileU, idesc, 1u);
+        free_a();
+        take_a();
+        if (!upto(9 * PT - 1)) return;
+        issue_packed<I8, 0, PT, 4 - KP, 0, 4>(d_r, hi, a_at, bc, kTileU, idesc, 1u);
+        issue_packed<I8, 1, PT, 4 - KP, 0, 4>(d_r, hi, a_at + row_lo, bc, kTileU, idesc, 1u);
+        look_a();
+        issue_packed<I8, 2, PT, 4 - KP, 0, 4>(d_r, hi, a_at + 2u * row_lo, bc, kTileU, idesc, 1u);
+      }
+      free_a();
+    } else for (int q = 0; q < chunks; ++q) {
       if constexpr (MODE == kTc4Chunks) {
         // up to three chunks of a 1x1 layer per slot
         take_a(); take_b();
@@ -452,11 +498,26 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
     __syncwarp();
   } else if (warp == 2) {
     // ============================================================ weight producer
-    if (ptx::elect_one()) {
+    const int row0 = tile_n * (NT / 32) + (PAIR ? part * (NT / 64) : 0);   // blocks of 32 channels
+    if (PAIR && P.packed) {
+      if (jobs > 0 && ptx::elect_one()) {
+        const int total = P.tiles_base + (BASE ? 0 : P.tiles_cond);
+        for (int t = 0; t < total; t += 3) {
+          const int tiles = min(3, total - t);
+          const uint32_t bar = leader(&sh->b_full[t / 3]);
+          expect(&sh->b_full[t / 3], (uint32_t)tiles * kTile);
+          for (int k = t; k < t + tiles; ++k) {
+            const bool cond = k >= P.tiles_base;
+            const int tile = cond ? (int)P.order[k - P.tiles_base] : k;
+            ptx::tma_load_5d<PAIR>(s_b + (size_t)(tile + (cond ? P.tiles_base : 0)) * kTile, cond ? &map_wc : &map_wb, bar,
+                                   tile * (I8 ? 128 : 64), 0, 0, 0, row0);
+          }
+        }
+      }
+    } else if (ptx::elect_one()) {
       Cursor c{0, 0};
       bool ok = true, seen = false;
       const int rounds = P.resident ? (jobs > 0 ? 1 : 0) : jobs;
-      const int row0 = tile_n * (NT / 32) + (PAIR ? part * (NT / 64) : 0);   // blocks of 32 channels
       for (int j = 0; j < rounds && ok; ++j) {
         Tc4Row next = row_at(table, lo);
         for (int i = lo; i < hi; ++i) {
@@ -489,7 +550,10 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
       if (part == 0 && ptx::elect_one()) {
         const int kp = L.c_p % (I8 ? 128 : 64) == 0 ? 4 : L.c_p / (I8 ? 32 : 16);
         if (P.mode == kTc4Window) {
-          if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Window, 4>(prm, sh, a0, b0, tmem, jobs);
+          if (P.packed && NT == 128) {
+            if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window, 2, 2>(prm, sh, a0, b0, tmem, jobs);
+            else issue_jobs<NT, I8, BASE, kTc4Window, 1, 2>(prm, sh, a0, b0, tmem, jobs);
+          } else if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Window, 4>(prm, sh, a0, b0, tmem, jobs);
           else if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window, 2>(prm, sh, a0, b0, tmem, jobs);
           else issue_jobs<NT, I8, BASE, kTc4Window, 1>(prm, sh, a0, b0, tmem, jobs);
         } else if (P.mode == kTc4Taps) {
@@ -1229,7 +1293,26 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   // shared memory: resident weights if they leave room for three patch slots, else rings of both
   const int clusters = P.grid / (P.pair ? 2 : P.split);
   const int jobs = P.pair ? (P.tiles_m + clusters / P.tiles_n - 1) / (clusters / P.tiles_n) : 1;
-  if (max_b <= kMaxNB && jobs > 1 && room - max_b * P.stage_bytes >= 3 * P.slot_bytes) {
+  // 128 channels with a base path of less than a chunk, 128 to a job: whole tiles per tap and chunk are half empty and do not
+  // fit, packed to 64 K elements each they do.  Streamed, they come to 240 KB a job and CTA, 83 bytes a cycle with what a
+  // pair's MMAs fetch of each other's weights: 5,300 cycles a job, 4,600 of MMAs.
+  const int tile_bytes = (P.pair ? P.nt / 2 : P.nt) * 128;
+  const int tb = (9 * L.c_p + ck - 1) / ck, tc = (9 * L.c_r + ck - 1) / ck;
+  if (P.pair && P.mode == kTc4Window && P.nt == 128 && L.c_in == 2 * ck && L.c_p < ck && L.c_r > 0 &&
+      room - (tb + tc) * tile_bytes >= 2 * P.slot_bytes) {
+    P.packed = 1; P.resident = 1;
+    P.tiles_base = tb; P.tiles_cond = tc; P.tiles_first = tc;
+    P.nb = (tb + tc + 2) / 3;
+    // the conditional tiles in the order in which the taps take them
+    const int per_tap = L.c_r / slice;
+    bool in[kTc4MaxTiles] = {};
+    int n = 0;
+    for (int i = 0; i < 9; ++i) {
+      const int t = i;
+      for (int k = t * per_tap; k < (t + 1) * per_tap; ++k)
+        if (!in[k / 4]) { in[k / 4] = true; P.order[n++] = (uint8_t)(k / 4); }
+    }
+  } else if (max_b <= kMaxNB && jobs > 1 && room - max_b * P.stage_bytes >= 3 * P.slot_bytes) {
     P.resident = 1;
     P.nb = max_b;
   } else {
@@ -1243,7 +1326,8 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     if (P.nb > kMaxNB) P.nb = kMaxNB;
     if (P.nb > max_b * jobs) P.nb = max_b * jobs;
   }
-  P.na = (room - P.nb * P.stage_bytes) / P.slot_bytes;         // what is left goes to patches
+  const int weights = P.packed ? (tb + tc) * tile_bytes : P.nb * P.stage_bytes;
+  P.na = (room - weights) / P.slot_bytes;                      // what is left goes to patches
   if (P.na > kMaxNA) P.na = kMaxNA;
   if (P.na < 1 || (P.pair && P.na < 2 && max_a * jobs > 1)) return false;
   if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) plan_base(raw, &P);
@@ -1251,7 +1335,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     P.row[i] = raw[i].r;
   }
   P.off_b = kOffStages;
-  P.off_a = kOffStages + (unsigned)(P.nb * P.stage_bytes);
+  P.off_a = kOffStages + (unsigned)(P.packed ? weights : P.nb * P.stage_bytes);
   P.smem_bytes = kSmemBytes;
   if (!P.pair) P.off_sums = P.sums_late ? kOffStages + 2u * 128u * kSumPitch : kSmemBytes - 1024 - sums_bytes;
   P.valid = 1;

@@ -36,6 +36,7 @@ enum : uint8_t {
 };
 
 enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2 };
+constexpr int kTc4MaxTiles = 32;
 
 struct Tc4Plan {
   int valid;
@@ -52,6 +53,9 @@ struct Tc4Plan {
   int na, nb;            // ring depths: patch slots, weight stages
   int stage_bytes;       // weight stage of one CTA
   int resident;          // the weights of a column tile stay in shared memory
+  int packed, tiles_base, tiles_cond;   // ... as tiles of consecutive K elements of W_base and of W_cond, three to a barrier
+  int tiles_first;       // W_cond's tiles come in this order; so many serve the first patch of a stride-2 window
+  uint8_t order[kTc4MaxTiles];
   int tiles_m, tiles_n;  // jobs
   int split;             // 1, 2, 4 or 8
   int grid;
