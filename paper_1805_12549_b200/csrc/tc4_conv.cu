@@ -179,6 +179,30 @@ __device__ __forceinline__ void issue_packed(uint32_t d, uint32_t hi, uint32_t a
     }
 }
 
+// Stride-2 windows: the filter taps by parity patch (kTc4Window2): patch 0 serves taps 0, 2, 6, 8, patch 1 taps 1, 7, patch 2
+// taps 3, 5, patch 3 tap 4.
+constexpr unsigned long long kTapOrder = 0x453718620ull;       // a nibble each
+__host__ __device__ constexpr int tap_at(int i) { return (int)((kTapOrder >> (4 * i)) & 15); }
+constexpr int kParityTaps[5] = {0, 4, 6, 8, 9};                // where the taps of patch p start in that order
+
+// The taps [I0, I1) of that order, all of patch PP: NK slices of each from K0 on.  Their weights: PT slices a tap from FIRST on,
+// packed (PT > 0), or a stage of three tiles in the same order (PT = 0).
+template <bool I8, int PP, int I0, int I1, int PT, int FIRST, int K0, int NK>
+__device__ __forceinline__ void issue_parity(uint32_t d, uint32_t hi, uint32_t a, uint32_t row_lo, uint32_t b, uint32_t tile,
+                                             uint32_t idesc, uint32_t acc) {
+#pragma unroll
+  for (int i = I0; i < I1; ++i) {
+    const int j = i - kParityTaps[PP];                         // (the patch's second column, row: one position further)
+    const uint32_t a_t = a + (PP == 0 ? (j & 1) * 8u + (j >> 1) * row_lo : PP == 1 ? j * row_lo : PP == 2 ? j * 8u : 0u);
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+      const int s = tap_at(i) * PT + FIRST + k;
+      const uint32_t b_t = PT > 0 ? b + (uint32_t)(s / 4) * tile + (uint32_t)(s % 4) * 2u : b + (uint32_t)(i % 3) * tile + 2u * k;
+      ptx::umma<true, I8>(d, ((uint64_t)hi << 32) | (a_t + 2u * (K0 + k)), ((uint64_t)hi << 32) | b_t, idesc, i == I0 && k == 0 ? acc : 1u);
+    }
+  }
+}
+
 // One row of the table in shared memory.
 __device__ __forceinline__ Tc4Row row_at(uint32_t table, int i) {
   const uint4 v = ptx::ld_shared_16(table + (uint32_t)i * 16u);
@@ -267,7 +291,7 @@ template <int NT, bool I8, bool BASE, int MODE, int KP, int CH = 0>
 __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, uint32_t a0, uint32_t b0, uint32_t tmem, int jobs) {
   constexpr int kAcc = 512 / (2 * NT);
   constexpr uint32_t kTileU = (uint32_t)(NT / 2) * 8u;         // a weight tile, 16-byte units
-  constexpr bool kWin = MODE == kTc4Window;
+  constexpr bool kWin = MODE == kTc4Window || MODE == kTc4Window2;
   const Tc4Plan& P = prm.P;
   const uint32_t idesc = I8 ? ptx::idesc_s8(256, NT) : ptx::idesc_bf16(256, NT);
   const uint32_t hi = (uint32_t)(ptx::smem_desc(0, 1024, 2) >> 32);
@@ -311,7 +335,61 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
     ptx::tc_fence_after();
     const uint32_t d_p = tmem + (uint32_t)(stage * 2 * NT), d_r = d_p + NT;
     if (resident) { b = IssueRing{0, 0u, b0}; new_b = j == 0; b_seen = false; }
-    if constexpr (CH > 0) {
+    if constexpr (MODE == kTc4Window2 && CH > 0) {
+      constexpr int PT = 4 * CH - KP;                          // conditional slices of a tap
+      const uint32_t bc = b0 + (uint32_t)P.tiles_base * kTileU;
+      auto chunk = [&](auto second) {
+        constexpr int Q = decltype(second)::value, FIRST = Q ? 4 - KP : 0, K0 = Q ? 0 : KP, NK = Q ? 4 : 4 - KP;
+        auto patch = [&](auto which) {
+          constexpr int PP = decltype(which)::value, I0 = kParityTaps[PP], I1 = kParityTaps[PP + 1];
+          take_a();
+          if (Q == 0) need_tile(BASE ? P.tiles_base - 1 : P.tiles_base - 1 + (PP == 0 ? P.tiles_first : P.tiles_cond));
+          if (!ok) return;
+          look_a();
+          if (Q == 0) issue_parity<I8, PP, I0, I1, KP, 0, 0, KP>(d_p, hi, a_at, row_lo, b0, kTileU, idesc, PP ? 1u : 0u);
+          if (!BASE) issue_parity<I8, PP, I0, I1, PT, FIRST, K0, NK>(d_r, hi, a_at, row_lo, bc, kTileU, idesc, Q || PP ? 1u : 0u);
+          free_a();
+        };
+        patch(std::integral_constant<int, 0>{});
+        if (ok) patch(std::integral_constant<int, 1>{});
+        if (ok) patch(std::integral_constant<int, 2>{});
+        if (ok) patch(std::integral_constant<int, 3>{});
+      };
+      chunk(std::integral_constant<int, 0>{});
+      if (ok && CH == 2 && !BASE) chunk(std::integral_constant<int, 1>{});
+      if (!ok) return;
+    } else if constexpr (MODE == kTc4Window2) {
+#pragma unroll 1
+      for (int q = 0; q < chunks; ++q) {
+        const uint32_t d = q < base_chunks ? d_p : d_r, acc = q == 0 || q == base_chunks ? 0u : 1u;
+        take_a(); take_b();
+        if (!ok) return;
+        issue_parity<I8, 0, 0, 3, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, acc);
+        free_b(b_slot);
+        take_b();
+        if (!ok) return;
+        look_a();
+        issue_parity<I8, 0, 3, 4, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
+        free_a();
+        take_a();
+        if (!ok) return;
+        look_a();
+        issue_parity<I8, 1, 4, 6, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
+        free_b(b_slot);
+        free_a();
+        take_a(); take_b();
+        if (!ok) return;
+        look_a();
+        issue_parity<I8, 2, 6, 8, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
+        free_a();
+        take_a();
+        if (!ok) return;
+        look_a();
+        issue_parity<I8, 3, 8, 9, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
+        free_b(b_slot);
+        free_a();
+      }
+    } else if constexpr (CH > 0) {
       static_assert(CH == 0 || CH == 2, "two chunks");
       constexpr int PT = 8 - KP;                               // conditional slices of a tap
       const uint32_t bc = b0 + (uint32_t)P.tiles_base * kTileU;
@@ -466,6 +544,23 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
         const int n0 = pos / ip, rem = pos - n0 * ip, h0 = rem / P.wp, w0 = rem - h0 * P.wp;
         const int pos1 = pos + P.patch_rows;                   // start of a window's second load
         const int n1 = pos1 / ip, rem1 = pos1 - n1 * ip, h1 = rem1 / P.wp, w1 = rem1 - h1 * P.wp;
+        if (PAIR && P.mode == kTc4Window2) {
+          // four patches per chunk, the pixels of odd or even rows and columns
+          const int ck = I8 ? 128 : 64, patches = 4 * (BASE ? (L.c_p + ck - 1) / ck : L.c_in / ck);
+          for (int i = 0; i < patches && ok; ++i) {
+            if (!seen) ok = wait4_one(sh, prm.counters, &sh->a_empty[c.slot], c.par ^ 1u, 1);
+            if (!ok) break;
+            uint8_t* dst = s_a + (size_t)c.slot * P.slot_bytes;
+            uint64_t* full = &sh->a_full[c.slot];
+            c.next(P.na);
+            seen = ptx::mbar_test_wait(&sh->a_empty[c.slot], c.par ^ 1u);
+            const uint32_t bar = leader(full);
+            expect(full, (uint32_t)P.patch_rows * 128u);
+            ptx::tma_load_im2col_4d<PAIR>(dst, &map_x, bar, (i >> 2) * ck, w0 * 2 - 1, h0 * 2 - 1, n0, (uint16_t)(i & 1),
+                                          (uint16_t)((i >> 1) & 1));
+          }
+          continue;
+        }
         Tc4Row next = row_at(table, lo);
         for (int i = lo; i < hi; ++i) {
           const Tc4Row s = next;
@@ -514,6 +609,31 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
           }
         }
       }
+    } else if (PAIR && P.mode == kTc4Window2) {
+      // stages of three taps in the order of the parity patches
+      if (ptx::elect_one()) {
+        Cursor c{0, 0};
+        bool ok = true, seen = false;
+        const int ck = I8 ? 128 : 64, base_chunks = L.c_p / ck, stages = 3 * (BASE ? base_chunks : L.c_in / ck);
+        const int rounds = P.resident ? (jobs > 0 ? 1 : 0) : jobs;
+        for (int j = 0; j < rounds && ok; ++j) {
+          for (int i = 0; i < stages; ++i) {
+            if (!seen) ok = wait4_one(sh, prm.counters, &sh->b_empty[c.slot], c.par ^ 1u, 2);
+            if (!ok) break;
+            uint8_t* dst = s_b + (size_t)c.slot * P.stage_bytes;
+            uint64_t* full = &sh->b_full[c.slot];
+            c.next(P.nb);
+            seen = ptx::mbar_test_wait(&sh->b_empty[c.slot], c.par ^ 1u);
+            const uint32_t bar = leader(full);
+            const int q = i / 3, first = (i - 3 * q) * 3;
+            const bool cond = q >= base_chunks;
+            const int per_tap = cond ? L.c_r : L.c_p, k0 = (cond ? q - base_chunks : q) * ck;
+            expect(full, 3u * kTile);
+            for (int k = 0; k < 3; ++k)
+              ptx::tma_load_5d<PAIR>(dst + k * kTile, cond ? &map_wc : &map_wb, bar, tap_at(first + k) * per_tap + k0, 0, 0, 0, row0);
+          }
+        }
+      }
     } else if (ptx::elect_one()) {
       Cursor c{0, 0};
       bool ok = true, seen = false;
@@ -556,6 +676,15 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
           } else if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Window, 4>(prm, sh, a0, b0, tmem, jobs);
           else if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window, 2>(prm, sh, a0, b0, tmem, jobs);
           else issue_jobs<NT, I8, BASE, kTc4Window, 1>(prm, sh, a0, b0, tmem, jobs);
+        } else if (P.mode == kTc4Window2) {
+          if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Window2, 4>(prm, sh, a0, b0, tmem, jobs);
+          else if (L.c_in == (I8 ? 256 : 128)) {
+            if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window2, 2, 2>(prm, sh, a0, b0, tmem, jobs);
+            else issue_jobs<NT, I8, BASE, kTc4Window2, 1, 2>(prm, sh, a0, b0, tmem, jobs);
+          } else {
+            if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window2, 2, 1>(prm, sh, a0, b0, tmem, jobs);
+            else issue_jobs<NT, I8, BASE, kTc4Window2, 1, 1>(prm, sh, a0, b0, tmem, jobs);
+          }
         } else if (P.mode == kTc4Taps) {
           if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Taps, 4>(prm, sh, a0, b0, tmem, jobs);
           else if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Taps, 2>(prm, sh, a0, b0, tmem, jobs);
@@ -1056,9 +1185,9 @@ bool encode_x(CUtensorMap* map, const void* base, const LayerDims& L, const Tc4P
   const cuuint64_t str[3] = {L.c_in * eb, (cuuint64_t)L.w * L.c_in * eb, (cuuint64_t)L.h * L.w * L.c_in * eb};
   const int lower[2] = {-L.pad, -L.pad};
   // window mode: the box ends at the image's last column and row; else at the last filter position
-  const int up = P.mode == kTc4Window ? 0 : L.pad - (L.kw - 1);
+  const int up = P.mode == kTc4Window || P.mode == kTc4Window2 ? 0 : L.pad - (L.kw - 1);
   const int upper[2] = {up, up};
-  const cuuint32_t st = P.mode == kTc4Taps ? (cuuint32_t)L.stride : 1u;
+  const cuuint32_t st = P.mode == kTc4Taps || P.mode == kTc4Window2 ? (cuuint32_t)L.stride : 1u;
   const cuuint32_t es[4] = {1, st, st, 1};
   return fn(map, P.i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
             str, lower, upper, (cuuint32_t)(128 / eb), (cuuint32_t)P.patch_rows, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -1175,6 +1304,25 @@ void plan_base(RawRow* raw, Tc4Plan* P) {
   }
 }
 
+// Stride-2 layers of pairs: windows over the four lattices of odd and even rows and columns, of pitch w' + 1 and h' + 1 (an odd
+// lattice starts in the padding; an even one ends there).  Tap by tap the pixels of a job were copied nine times: 128->256
+// channels at 28x28, 650 KB a job and CTA, 9,000 cycles of copies for 4,600 of MMAs.
+bool plan_window2(const LayerDims& L, Tc4Plan* P) {
+  const int eb = P->i8 ? 1 : 2, ck = 128 / eb;
+  const int rows = (128 + L.wo + 2 + 7) / 8 * 8;
+  if (L.w % 2 || L.h % 2 || rows > 256) return false;
+  if ((long long)L.n * (L.wo + 1) * (L.ho + 1) > 0x7fffffffll - 65536) return false;
+  if (L.c_p % ck != 0) {
+    // a base path of less than a chunk: with packed weights that stay in shared memory
+    const int tiles = (9 * L.c_p + ck - 1) / ck + (9 * L.c_r + ck - 1) / ck;
+    if (L.c_in > 2 * ck || (int)(kSmemBytes - 1024 - kOffStages) - tiles * (L.c_out <= 64 || P->i8 ? 4096 : 8192) < 3 * rows * 128) return false;
+  }
+  P->mode = kTc4Window2;
+  P->wp = L.wo + 1; P->hp = L.ho + 1;
+  P->loads = 1; P->patch_rows = rows; P->slot_bytes = (rows * 128 + 1023) / 1024 * 1024; P->a_step = 8;
+  return true;
+}
+
 template <int NT, bool I8, bool PAIR>
 const void* instance() { return (const void*)tc4_gated_conv_kernel<NT, I8, PAIR>; }
 
@@ -1217,7 +1365,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   if (per_image > 0x3fffffffll || L.n * per_image > 0x7fffffffll - 65536) return false;
   const long long positions = L.n * per_image;
   P.div_ip.set((uint32_t)per_image); P.div_wp.set((uint32_t)P.wp);
-  const int tiles128 = (int)((positions + 127) / 128), tiles256 = (int)((positions + 255) / 256);
+  const int tiles128 = (int)((positions + 127) / 128);
   const int tn64 = (L.c_out + 63) / 64, tn128 = (L.c_out + 127) / 128;
 
   P.split = 1;
@@ -1259,11 +1407,25 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     // b256: 3 rounds of 64 36.1 us, 2 rounds of 128 27.6; 128->256 stride 2: 19.0 and 15.7).  int8: 64 (the requantisation constants of 128 do not fit the epilogue's registers).
     P.pair = 1;
     const int pairs = sms / 2;
+    int tiles256 = (int)((positions + 255) / 256);
     auto rounds = [&](int tn) { return tn > pairs ? 1e30 : (double)((tiles256 + pairs / tn - 1) / (pairs / tn)); };
+    if (k3 && L.stride == 2 && plan_window2(L, &P)) {
+      // a third of the patch bytes, and up to a third more positions: not where that makes more than half as many rounds again
+      const double taps = rounds(tn128);
+      const long long padded = (long long)L.n * P.wp * P.hp;
+      const int before = tiles256;
+      tiles256 = (int)((padded + 255) / 256);
+      if (rounds(tn128) > 1.5 * taps) {
+        tiles256 = before;
+        P.mode = kTc4Taps; P.wp = L.wo; P.hp = L.ho; P.patch_rows = 128; P.slot_bytes = 3 * 128 * 128; P.a_step = 1024;
+      }
+      P.div_ip.set((uint32_t)(P.wp * P.hp)); P.div_wp.set((uint32_t)P.wp);
+    }
     P.nt = (P.i8 || L.c_out <= 64 || rounds(tn64) * 0.85 < rounds(tn128)) ? 64 : 128;
     P.tiles_m = tiles256; P.tiles_n = P.nt == 64 ? tn64 : tn128;
     if (P.tiles_n > pairs) return false;
-    P.rows = raw_rows(L, P, raw);
+    if (P.mode == kTc4Window2) P.rows = 0;                     // (walked without a table)
+    else P.rows = raw_rows(L, P, raw);
     if (P.rows > kTc4MaxRows) return false;
     const int groups = pairs / P.tiles_n;
     P.grid = (groups < P.tiles_m ? groups : P.tiles_m) * P.tiles_n * 2;
@@ -1290,6 +1452,8 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.sums_late = !P.pair && P.mode == kTc4Taps && room - (int)sums_bytes < slots_wanted * P.slot_bytes + stages_wanted * P.stage_bytes;
   if (!P.sums_late) room -= (int)sums_bytes;
 
+  if (P.mode == kTc4Window2) { max_a = 4 * (L.c_in / ck); max_b = 3 * (L.c_in / ck); }
+
   // shared memory: resident weights if they leave room for three patch slots, else rings of both
   const int clusters = P.grid / (P.pair ? 2 : P.split);
   const int jobs = P.pair ? (P.tiles_m + clusters / P.tiles_n - 1) / (clusters / P.tiles_n) : 1;
@@ -1298,8 +1462,9 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   // pair's MMAs fetch of each other's weights: 5,300 cycles a job, 4,600 of MMAs.
   const int tile_bytes = (P.pair ? P.nt / 2 : P.nt) * 128;
   const int tb = (9 * L.c_p + ck - 1) / ck, tc = (9 * L.c_r + ck - 1) / ck;
-  if (P.pair && P.mode == kTc4Window && P.nt == 128 && L.c_in == 2 * ck && L.c_p < ck && L.c_r > 0 &&
-      room - (tb + tc) * tile_bytes >= 2 * P.slot_bytes) {
+  if (P.mode == kTc4Window2 ? L.c_p % ck != 0
+                            : P.pair && P.mode == kTc4Window && P.nt == 128 && L.c_in == 2 * ck && L.c_p < ck && L.c_r > 0 &&
+                                  room - (tb + tc) * tile_bytes >= 2 * P.slot_bytes) {
     P.packed = 1; P.resident = 1;
     P.tiles_base = tb; P.tiles_cond = tc; P.tiles_first = tc;
     P.nb = (tb + tc + 2) / 3;
@@ -1308,16 +1473,17 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     bool in[kTc4MaxTiles] = {};
     int n = 0;
     for (int i = 0; i < 9; ++i) {
-      const int t = i;
+      const int t = P.mode == kTc4Window2 ? tap_at(i) : i;
       for (int k = t * per_tap; k < (t + 1) * per_tap; ++k)
         if (!in[k / 4]) { in[k / 4] = true; P.order[n++] = (uint8_t)(k / 4); }
+      if (i == 3 && P.mode == kTc4Window2) P.tiles_first = n;
     }
   } else if (max_b <= kMaxNB && jobs > 1 && room - max_b * P.stage_bytes >= 3 * P.slot_bytes) {
     P.resident = 1;
     P.nb = max_b;
   } else {
     // (three weight stages at least: a base stage stays while conditional ones pass)
-    int na = P.mode == kTc4Window ? 3 : 2;
+    int na = P.mode == kTc4Window || P.mode == kTc4Window2 ? 3 : 2;
     if (na > max_a * jobs) na = max_a * jobs;
     while (na > 2 && room - na * P.slot_bytes < 4 * P.stage_bytes) --na;
     if (!P.pair && na > 1 && room - na * P.slot_bytes < 3 * P.stage_bytes) --na;
@@ -1330,7 +1496,10 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.na = (room - weights) / P.slot_bytes;                      // what is left goes to patches
   if (P.na > kMaxNA) P.na = kMaxNA;
   if (P.na < 1 || (P.pair && P.na < 2 && max_a * jobs > 1)) return false;
-  if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) plan_base(raw, &P);
+  if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) {
+    if (P.mode == kTc4Window2) P.base_rows = 1;
+    else plan_base(raw, &P);
+  }
   for (int i = 0; i < P.rows; ++i) {
     P.row[i] = raw[i].r;
   }

@@ -35,7 +35,7 @@ enum : uint8_t {
   kRowAFreeBase = 128              // kRowAFree of a job that runs the base rows only
 };
 
-enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2 };
+enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2, kTc4Window2 = 3 };
 constexpr int kTc4MaxTiles = 32;
 
 struct Tc4Plan {
@@ -43,7 +43,7 @@ struct Tc4Plan {
   int i8;
   int pair;              // 1: CTA pairs (256 pixels per job); 0: `split` CTAs share the K loop of a 128-pixel job
   int nt;                // output channels per job: 64 or 128
-  int mode;              // kTc4Window, kTc4Taps, kTc4Chunks: what a patch slot holds
+  int mode;              // kTc4Window, kTc4Taps, kTc4Chunks, kTc4Window2: what a patch slot holds
   int wp, hp;            // pitch of the stacked pixel space: window mode w + pad, h + pad; else w', h'
   FastDiv div_ip, div_wp;   // by wp * hp and by wp
   int patch_rows;        // pixels per patch load

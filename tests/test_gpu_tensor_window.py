@@ -177,3 +177,41 @@ def test_an_infinite_sum_meets_an_infinite_threshold(s, residual):
         np.testing.assert_array_equal(y[~fin], ref.y[~fin])
         assert (np.abs(y[fin] - ref.y[fin]) <= K.BF16_ATOL + K.BF16_RTOL * np.abs(ref.y[fin])).all()
     g.close()
+
+
+# K loops of pairs: packed weights and stride-2 windows, with the plan that the shape has to take.
+K_LOOPS = [
+    (O.Shape(40, 28, 28, 128, 128, groups=8), "one patch for all taps", "packed", "G = 8: one base slice"),
+    (O.Shape(60, 13, 15, 128, 256, groups=4), "one patch for all taps", "packed", "odd extents, two column tiles"),
+    (O.Shape(70, 28, 28, 64, 128, stride=2, groups=2), "four patches", "packed", "one chunk, two base slices"),
+    (O.Shape(30, 28, 28, 128, 256, stride=2, groups=8), "four patches", "packed", "two chunks, one base slice"),
+    (O.Shape(70, 30, 26, 64, 64, stride=2, groups=4), "four patches", "packed", "64 columns to a job"),
+    (O.Shape(40, 14, 14, 256, 512, stride=2, groups=4), "four patches", "streamed", "a base chunk, streamed"),
+    (O.Shape(150, 28, 28, 128, 64, stride=2, groups=2), "four patches", "resident", "a base chunk, resident"),
+    (O.Shape(40, 28, 28, 128, 128, stride=2, groups=1), "four patches", "streamed", "ungated"),
+    (O.Shape(600, 4, 4, 128, 256, stride=2, groups=4), "four patches", "packed", "four output pixels per image"),
+    (O.Shape(3000, 2, 2, 128, 256, stride=2, groups=4), "one patch per tap", "streamed", "too much padding for a window"),
+    (O.Shape(80, 13, 15, 128, 256, stride=2, groups=4), "one patch per tap", "streamed", "odd extents"),
+    (O.Shape(60, 28, 28, 256, 256, stride=2, groups=8), "one patch per tap", "streamed", "too many chunks to pack"),
+]
+
+
+@pytest.mark.parametrize("s,patch,weights,why", K_LOOPS, ids=[k[3] for k in K_LOOPS])
+@pytest.mark.parametrize("how", ["density", "some shut", "all shut"])
+def test_k_loops_of_pairs(s, patch, weights, why, how):
+    c = K.make_float_case("winkloop", s, "bf16", density=0.3, calib_images=4)
+    if how != "density":
+        c.delta[:s.c_out if how == "all shut" else (s.c_out + 1) // 2] = K.INF
+    ref, st, _ = _run(c)
+    g = K.GpuCase(c, algo=0)
+    plan = g.conv.plan
+    g.close()
+    assert patch in plan and (weights in plan or s.groups == 1), plan
+    assert how != "all shut" or s.c_r == 0 or (st.active == 0 and st.executed_macs < st.dense_macs)
+
+
+@pytest.mark.parametrize("s", [O.Shape(60, 28, 28, 128, 256, stride=2, groups=4), O.Shape(40, 28, 28, 256, 128, stride=2, groups=4),
+                               O.Shape(40, 28, 28, 256, 128, stride=2, groups=8), O.Shape(40, 28, 28, 256, 128, stride=2, groups=2)],
+                         ids=["one chunk", "two base slices", "one base slice", "a base chunk"])
+def test_int8_stride_2_windows(s):
+    _run(K.make_int8_case("wini8s2", s, density=0.3))
