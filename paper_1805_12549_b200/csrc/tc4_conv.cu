@@ -909,10 +909,8 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
         // the sums have been read: the accumulators go back to the issuers
         ptx::tc_fence_before();
         __syncwarp();
-        if (lane == 0) {
-          if (PAIR) ptx::mbar_arrive_cluster_relaxed(leader(&sh->acc_empty[stage]));
-          else ptx::mbar_arrive(&sh->acc_empty[stage]);
-        }
+        // (not behind the last jobs: nobody waits for them, and the block may be gone)
+        if (lane == 0 && j + kAcc < jobs) ptx::mbar_arrive_cluster_relaxed(leader(&sh->acc_empty[stage]));
       }
     }
     if constexpr (SPLIT) {
@@ -1137,9 +1135,9 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
   __syncwarp();
   ptx::tc_fence_before();
-  // No CTA leaves while a peer may still use its shared memory or TMEM.  (A cluster's CTA has waited for all that is sent to it
-  // and sent on, and its stores to global memory need not be waited for.)
-  if (PAIR) ptx::cluster_sync(); else ptx::cluster_sync_relaxed();
+  // No CTA leaves while a peer may still use its shared memory or TMEM.  (A CTA has waited for all that is sent to it and that
+  // it sends, and its stores to global memory need not be waited for.)
+  ptx::cluster_sync_relaxed();
   ptx::tc_fence_after();
   if (threadIdx.x == 0 && !*(volatile uint32_t*)&sh->abort_flag) {
     if (shut && part == 0) {
