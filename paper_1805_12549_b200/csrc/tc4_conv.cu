@@ -83,6 +83,11 @@ struct Tc4Params {
   Tc4Plan P;
 };
 
+// The weights' tensor maps; HALF: a layer whose last round is in halves (Tc4Plan::half_job) has maps for those, too.  (An
+// instance of the kernel of its own: the choice between the maps, operand starts and instruction descriptors costs others 1 to 5 %.)
+template <bool HALF> struct WeightMaps { CUtensorMap wb, wc; };
+template <> struct WeightMaps<true> { CUtensorMap wb, wc, half_wb, half_wc; };
+
 struct Shared4 {
   uint64_t a_full[kMaxNA], a_empty[kMaxNA];
   uint64_t b_full[kMaxNB], b_empty[kMaxNB];
@@ -287,13 +292,14 @@ struct IssueRing {
 // its MMAs and a commit: walked from a table of row kinds, a row's loads, tests and branches took 700 cycles beside the 576 of
 // nine MMAs of 64, two issuers taking turns.
 // CH: chunks of a layer with packed weights, else 0.
-template <int NT, bool I8, bool BASE, int MODE, int KP, int CH = 0>
-__device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, uint32_t a0, uint32_t b0, uint32_t tmem, int jobs) {
+template <int NT, bool I8, bool BASE, bool HALF, int MODE, int KP, int CH = 0>
+__device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, uint32_t a0, uint32_t b0, uint32_t tmem, int group,
+                                           int jobs) {
   constexpr int kAcc = 512 / (2 * NT);
   constexpr uint32_t kTileU = (uint32_t)(NT / 2) * 8u;         // a weight tile, 16-byte units
   constexpr bool kWin = MODE == kTc4Window || MODE == kTc4Window2;
   const Tc4Plan& P = prm.P;
-  const uint32_t idesc = I8 ? ptx::idesc_s8(256, NT) : ptx::idesc_bf16(256, NT);
+  uint32_t idesc = I8 ? ptx::idesc_s8(256, NT) : ptx::idesc_bf16(256, NT);
   const uint32_t hi = (uint32_t)(ptx::smem_desc(0, 1024, 2) >> 32);
   const uint32_t a_size = (uint32_t)P.slot_bytes >> 4, b_size = (uint32_t)P.stage_bytes >> 4;
   const uint32_t row_lo = kWin ? (uint32_t)P.wp * 8u : 0u;
@@ -334,6 +340,10 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
     if (!ok) return;
     ptx::tc_fence_after();
     const uint32_t d_p = tmem + (uint32_t)(stage * 2 * NT), d_r = d_p + NT;
+    if (HALF && j == P.half_job) {                             // 64 of the columns: half of the rows of every weight tile
+      idesc = I8 ? ptx::idesc_s8(256, 64) : ptx::idesc_bf16(256, 64);
+      if (resident) b0 += (uint32_t)(group & 1) * (kTileU / 2u);
+    }
     if (resident) { b = IssueRing{0, 0u, b0}; new_b = j == 0; b_seen = false; }
     if constexpr (MODE == kTc4Window2 && CH > 0) {
       constexpr int PT = 4 * CH - KP;                          // conditional slices of a tap
@@ -500,11 +510,11 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
 
 // What the warps of a block do (see the top of the file).  BASE: the jobs of a column tile whose gates cannot fire, which run
 // the base rows only.
-template <int NT, bool I8, bool PAIR, bool BASE>
-__device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtensorMap& map_wb, const CUtensorMap& map_wc,
-                                          const Tc4Params& prm, uint8_t* smem, int warp, int lane, int part, int tile_n,
+template <int NT, bool I8, bool PAIR, bool HALF, bool BASE>
+__device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const WeightMaps<HALF>& maps, const Tc4Params& prm, uint8_t* smem, int warp, int lane, int part, int tile_n,
                                           int group, int groups, int jobs, uint32_t tmem) {
   constexpr bool SPLIT = !PAIR;
+  const CUtensorMap &map_wb = maps.wb, &map_wc = maps.wc;
   const LayerDims& L = prm.L;
   const Tc4Plan& P = prm.P;
   Shared4* sh = (Shared4*)smem;
@@ -522,7 +532,10 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
   const bool has_cond = !BASE && L.c_r > 0;
   const uint32_t table = ptx::smem_u32(smem + kOffRows);
   // first position of this CTA in job j
-  auto job_pos = [&](int j) { return PAIR ? (group + j * groups) * 256 + part * 128 : (group + j * groups) * 128; };
+  auto job_pos = [&](int j) {
+    if (!PAIR) return group * 128;
+    return ((HALF && j == P.half_job ? group >> 1 : group) + j * groups) * 256 + part * 128;
+  };
   // address of the leader's copy of a barrier, for copies and arrivals
   auto leader = [&](uint64_t* bar) { return PAIR ? ptx::map_cluster(ptx::smem_u32(bar), 0) : ptx::smem_u32(bar); };
   // (a pair's leader announces both CTAs' bytes; the other CTA's copies count on the leader's barrier: an
@@ -628,9 +641,12 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
             const int q = i / 3, first = (i - 3 * q) * 3;
             const bool cond = q >= base_chunks;
             const int per_tap = cond ? L.c_r : L.c_p, k0 = (cond ? q - base_chunks : q) * ck;
-            expect(full, 3u * kTile);
+            const bool half = HALF && j == P.half_job && !P.resident;
+            const CUtensorMap* map = cond ? &map_wc : &map_wb;
+            if constexpr (HALF) map = half ? (cond ? &maps.half_wc : &maps.half_wb) : map;
+            expect(full, half ? 3u * kTile / 2u : 3u * kTile);
             for (int k = 0; k < 3; ++k)
-              ptx::tma_load_5d<PAIR>(dst + k * kTile, cond ? &map_wc : &map_wb, bar, tap_at(first + k) * per_tap + k0, 0, 0, 0, row0);
+              ptx::tma_load_5d<PAIR>(dst + k * kTile, map, bar, tap_at(first + k) * per_tap + k0, 0, 0, 0, row0 + (half ? group & 1 : 0));
           }
         }
       }
@@ -652,11 +668,14 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
           seen = ptx::mbar_test_wait(&sh->b_empty[c.slot], c.par ^ 1u);
           const int tiles = s.tap_row >> 4, bx = (int)s.bx, bstep = (int)s.bstep;
           const uint32_t bar = leader(full);
+          const bool half = HALF && j == P.half_job && !P.resident;
           const CUtensorMap* map = (s.flags & kRowCond) ? &map_wc : &map_wb;
-          expect(full, (uint32_t)tiles * kTile);
-          ptx::tma_load_5d<PAIR>(dst, map, bar, bx, 0, 0, 0, row0);
-          if (tiles > 1) ptx::tma_load_5d<PAIR>(dst + kTile, map, bar, bx + bstep, 0, 0, 0, row0);
-          if (tiles > 2) ptx::tma_load_5d<PAIR>(dst + 2 * kTile, map, bar, bx + 2 * bstep, 0, 0, 0, row0);
+          if constexpr (HALF) map = half ? ((s.flags & kRowCond) ? &maps.half_wc : &maps.half_wb) : map;
+          const int rows = row0 + (half ? group & 1 : 0);
+          expect(full, (uint32_t)tiles * (half ? kTile / 2u : kTile));
+          ptx::tma_load_5d<PAIR>(dst, map, bar, bx, 0, 0, 0, rows);
+          if (tiles > 1) ptx::tma_load_5d<PAIR>(dst + kTile, map, bar, bx + bstep, 0, 0, 0, rows);
+          if (tiles > 2) ptx::tma_load_5d<PAIR>(dst + 2 * kTile, map, bar, bx + 2 * bstep, 0, 0, 0, rows);
         }
       }
     }
@@ -671,26 +690,26 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
         const int kp = L.c_p % (I8 ? 128 : 64) == 0 ? 4 : L.c_p / (I8 ? 32 : 16);
         if (P.mode == kTc4Window) {
           if (P.packed && NT == 128) {
-            if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window, 2, 2>(prm, sh, a0, b0, tmem, jobs);
-            else issue_jobs<NT, I8, BASE, kTc4Window, 1, 2>(prm, sh, a0, b0, tmem, jobs);
-          } else if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Window, 4>(prm, sh, a0, b0, tmem, jobs);
-          else if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window, 2>(prm, sh, a0, b0, tmem, jobs);
-          else issue_jobs<NT, I8, BASE, kTc4Window, 1>(prm, sh, a0, b0, tmem, jobs);
+            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Window, 2, 2>(prm, sh, a0, b0, tmem, group, jobs);
+            else issue_jobs<NT, I8, BASE, HALF, kTc4Window, 1, 2>(prm, sh, a0, b0, tmem, group, jobs);
+          } else if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Window, 4>(prm, sh, a0, b0, tmem, group, jobs);
+          else if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Window, 2>(prm, sh, a0, b0, tmem, group, jobs);
+          else issue_jobs<NT, I8, BASE, HALF, kTc4Window, 1>(prm, sh, a0, b0, tmem, group, jobs);
         } else if (P.mode == kTc4Window2) {
-          if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Window2, 4>(prm, sh, a0, b0, tmem, jobs);
+          if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 4>(prm, sh, a0, b0, tmem, group, jobs);
           else if (L.c_in == (I8 ? 256 : 128)) {
-            if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window2, 2, 2>(prm, sh, a0, b0, tmem, jobs);
-            else issue_jobs<NT, I8, BASE, kTc4Window2, 1, 2>(prm, sh, a0, b0, tmem, jobs);
+            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 2, 2>(prm, sh, a0, b0, tmem, group, jobs);
+            else issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 1, 2>(prm, sh, a0, b0, tmem, group, jobs);
           } else {
-            if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Window2, 2, 1>(prm, sh, a0, b0, tmem, jobs);
-            else issue_jobs<NT, I8, BASE, kTc4Window2, 1, 1>(prm, sh, a0, b0, tmem, jobs);
+            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 2, 1>(prm, sh, a0, b0, tmem, group, jobs);
+            else issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 1, 1>(prm, sh, a0, b0, tmem, group, jobs);
           }
         } else if (P.mode == kTc4Taps) {
-          if (kp == 4) issue_jobs<NT, I8, BASE, kTc4Taps, 4>(prm, sh, a0, b0, tmem, jobs);
-          else if (kp == 2) issue_jobs<NT, I8, BASE, kTc4Taps, 2>(prm, sh, a0, b0, tmem, jobs);
-          else issue_jobs<NT, I8, BASE, kTc4Taps, 1>(prm, sh, a0, b0, tmem, jobs);
+          if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Taps, 4>(prm, sh, a0, b0, tmem, group, jobs);
+          else if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Taps, 2>(prm, sh, a0, b0, tmem, group, jobs);
+          else issue_jobs<NT, I8, BASE, HALF, kTc4Taps, 1>(prm, sh, a0, b0, tmem, group, jobs);
         } else if (!BASE) {
-          issue_jobs<NT, I8, BASE, kTc4Chunks, 4>(prm, sh, a0, b0, tmem, jobs);
+          issue_jobs<NT, I8, BASE, HALF, kTc4Chunks, 4>(prm, sh, a0, b0, tmem, group, jobs);
         }
       }
     } else if (jobs > 0 && ptx::elect_one()) {
@@ -794,6 +813,9 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
       const bool has_res = !I8 && prm.residual != nullptr;
       for (int j = NT == 128 ? 0 : eg >> 1; j < jobs && ok; j += NT == 128 ? 1 : 2) {
         const int stage = j % kAcc;
+        // (a half job's columns are the even or the odd blocks of 32 channels: warps of the others only wait)
+        const bool half = HALF && j == P.half_job, mine = !half || (eg & 1) == (group & 1);
+        const uint32_t t_col = t_lane + (uint32_t)(stage * 2 * NT + (half ? (eg >> 1) * 32 : c0));
         const uint32_t pos = (uint32_t)(job_pos(j) + row);
         const uint32_t n0 = P.div_ip.div(pos), rem = pos - n0 * (uint32_t)(P.wp * P.hp);
         const uint32_t h0 = P.div_wp.div(rem), w0 = rem - h0 * (uint32_t)P.wp;
@@ -824,7 +846,7 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
 #pragma unroll
             for (int g = 0; g < 2; ++g) {                      // 16 columns at a time (registers)
               uint32_t p[8], r[8];
-              const uint32_t t_p = t_lane + ((uint32_t)(16 * i) << 16) + (uint32_t)(stage * 2 * NT + c0 + 16 * g);
+              const uint32_t t_p = t_col + ((uint32_t)(16 * i) << 16) + (uint32_t)(16 * g);
               __syncwarp();                                    // (the loads are .aligned; what is before them diverges)
               ptx::tmem_ld_frag16(t_p, p);
               if (has_cond) {
@@ -896,11 +918,11 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
           if (prm.mask && m_word >= 0) prm.mask[(long long)m_word * L.words + (ch >> 5)] = bits;
           return bits;
         };
-        if (ch < L.c_out) {                                    // (uniform over the warp)
+        if (ch < L.c_out && mine) {                            // (uniform over the warp)
           if constexpr (BASE && !I8) {
             const uint32_t fired = finish(std::true_type{}, std::true_type{});
             if (__any_sync(0xffffffffu, fired != 0u))
-              infinite_sums(prm, t_lane + (uint32_t)(stage * 2 * NT + c0), s_t + c0, s_t2 + c0, s_k + c0, ch, own);
+              infinite_sums(prm, t_col, s_t + c0, s_t2 + c0, s_k + c0, ch, own);
           } else if (I8) finish(std::false_type{}, std::false_type{});
           else if (two_sided) finish(std::true_type{}, std::true_type{});
           else if (has_res) finish(std::false_type{}, std::true_type{});
@@ -1047,10 +1069,10 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const CUtens
   }
 }
 
-template <int NT, bool I8, bool PAIR>
+template <int NT, bool I8, bool PAIR, bool HALF>
 __global__ void __launch_bounds__(kT4Threads, 1)
-tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_wb,
-                      const __grid_constant__ CUtensorMap map_wc, const __grid_constant__ Tc4Params prm) {
+tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ WeightMaps<HALF> maps,
+                      const __grid_constant__ Tc4Params prm) {
   extern __shared__ uint8_t smem_raw[];
   constexpr bool SPLIT = !PAIR;
   ptx::grid_launch_dependents();
@@ -1067,7 +1089,8 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   const int block = (int)(blockIdx.x / members), blocks = (int)(gridDim.x / members);
   // jobs of this cluster: a fixed column tile, every `groups`-th pixel tile (split layers: one job)
   const int tile_n = block % P.tiles_n, group = block / P.tiles_n, groups = blocks / P.tiles_n;
-  const int jobs = group < P.tiles_m ? (P.tiles_m - group + groups - 1) / groups : 0;
+  const int jobs = HALF ? P.half_job + (group < 2 * P.half_tiles ? 1 : 0)
+                   : group < P.tiles_m ? (P.tiles_m - group + groups - 1) / groups : 0;
   const bool has_cond = L.c_r > 0;
 
   if (warp == 0) {
@@ -1086,7 +1109,7 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     if (lane == 0) { sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0; sh->epi_done = 0; }
     ptx::fence_mbar_init();
   }
-  if (threadIdx.x == 32 * 2) { ptx::prefetch_tensormap(&map_x); ptx::prefetch_tensormap(&map_wb); ptx::prefetch_tensormap(&map_wc); }
+  if (threadIdx.x == 32 * 2) { ptx::prefetch_tensormap(&map_x); ptx::prefetch_tensormap(&maps.wb); ptx::prefetch_tensormap(&maps.wc); }
   // (the row table moves to shared memory: an indexed read of a kernel parameter costs hundreds of cycles)
   for (int i = (int)threadIdx.x - kEpiWarp0 * 32; i >= 0 && i < P.rows; i += kT4Threads)
     ((uint4*)(smem + kOffRows))[i] = ((const uint4*)P.row)[i];
@@ -1119,10 +1142,10 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
         ((uint4*)(smem + kOffRows))[__popcll(P.base_mask & ((1ull << i) - 1ull))] = row;
       }
       __syncthreads();
-      run_roles<NT, I8, PAIR, true>(map_x, map_wb, map_wc, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
+      run_roles<NT, I8, PAIR, HALF, true>(map_x, maps, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
     }
   } else {
-    run_roles<NT, I8, PAIR, false>(map_x, map_wb, map_wc, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
+    run_roles<NT, I8, PAIR, HALF, false>(map_x, maps, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
   }
   __syncwarp();
   if (SPLIT && P.sums_late && warp < kEpiWarp0) ptx::cluster_sync();
@@ -1141,9 +1164,10 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   ptx::tc_fence_after();
   if (threadIdx.x == 0 && !*(volatile uint32_t*)&sh->abort_flag) {
     if (shut && part == 0) {
-      // the jobs without conditional rows are taken from the totals below
-      atomicAdd(&prm.counters[CNT_TILES_TOTAL], 0ull - (unsigned long long)jobs);
-      atomicAdd(&prm.counters[CNT_EXEC_MACS], 0ull - (unsigned long long)jobs * 256ull * NT * (unsigned long long)(L.kh * L.kw) * L.c_r);
+      // the jobs without conditional rows are taken from the totals below (the two halves of a job as one)
+      const int halves = HALF && jobs > P.half_job ? 1 : 0, tiles = jobs - (halves & group & 1);
+      atomicAdd(&prm.counters[CNT_TILES_TOTAL], 0ull - (unsigned long long)tiles);
+      atomicAdd(&prm.counters[CNT_EXEC_MACS], 0ull - (unsigned long long)(jobs * NT - halves * (NT / 2)) * 256ull * (unsigned long long)(L.kh * L.kw) * L.c_r);
     }
     if (blockIdx.x == 0) {
       const unsigned long long tiles = (unsigned long long)P.tiles_m * P.tiles_n;
@@ -1195,13 +1219,14 @@ bool encode_x(CUtensorMap* map, const void* base, const LayerDims& L, const Tc4P
 // Weight tiles [output channel][K], the channels of each block of 32 in the order 8*(i%4) + 2*(i/4), + 1 for
 // i = 0..15: accumulator columns 8k + 2q and + 1 are then channels 8q + 2k and + 1, so that the eight columns
 // a thread gets of a block in the accumulator-fragment layout are eight consecutive channels.
-bool encode_w(CUtensorMap* map, const void* base, const Tc4Plan& P, int c_out, int k_total) {
+// `blocks` of 32 channels to a copy.
+bool encode_w(CUtensorMap* map, const void* base, const Tc4Plan& P, int c_out, int k_total, int blocks) {
   static const EncodeTiledFn fn = (EncodeTiledFn)driver_fn("cuTensorMapEncodeTiled");
   if (!fn) return false;
   const cuuint64_t eb = P.i8 ? 1 : 2, pitch = (cuuint64_t)k_total * eb;
   const cuuint64_t dims[5] = {(cuuint64_t)k_total, 2, 4, 4, (cuuint64_t)c_out / 32};
   const cuuint64_t str[4] = {pitch, 8 * pitch, 2 * pitch, 32 * pitch};
-  const cuuint32_t box[5] = {(cuuint32_t)(128 / eb), 2, 4, 4, (cuuint32_t)(P.pair ? P.nt / 64 : P.nt / 32)};
+  const cuuint32_t box[5] = {(cuuint32_t)(128 / eb), 2, 4, 4, (cuuint32_t)blocks};
   const cuuint32_t es[5] = {1, 1, 1, 1, 1};
   return fn(map, P.i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims,
             str, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1321,8 +1346,8 @@ bool plan_window2(const LayerDims& L, Tc4Plan* P) {
   return true;
 }
 
-template <int NT, bool I8, bool PAIR>
-const void* instance() { return (const void*)tc4_gated_conv_kernel<NT, I8, PAIR>; }
+template <int NT, bool I8, bool PAIR, bool HALF = false>
+const void* instance() { return (const void*)tc4_gated_conv_kernel<NT, I8, PAIR, HALF>; }
 
 }  // namespace
 
@@ -1332,6 +1357,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   std::memset(&P, 0, sizeof(P));
   if (in_dtype != CG_BF16 && in_dtype != CG_I8) return false;
   P.i8 = in_dtype == CG_I8;
+  P.half_job = kNoHalfJob;
   const int eb = P.i8 ? 1 : 2, ck = 128 / eb, slice = 32 / eb;
   if (cond_mode == CG_COND_SKIP_TILES || cond_mode == CG_COND_COMPACT) return false;   // R is computed everywhere
   if (L.channel_tau > 0.f || (L.grouping && L.groups > 1)) return false;
@@ -1426,6 +1452,10 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     else P.rows = raw_rows(L, P, raw);
     if (P.rows > kTc4MaxRows) return false;
     const int groups = pairs / P.tiles_n;
+    // A last round that less than half of the pairs take part in: its jobs as two of 64 columns each, which take two thirds
+    // of the time (43 cycles an MMA for 64).
+    const int left = P.tiles_m % groups;
+    if (P.nt == 128 && P.tiles_m > groups && left > 0 && 2 * left <= groups) { P.half_job = P.tiles_m / groups; P.half_tiles = left; }
     P.grid = (groups < P.tiles_m ? groups : P.tiles_m) * P.tiles_n * 2;
     P.lo[1] = (uint16_t)P.rows;
   }
@@ -1525,9 +1555,13 @@ int launch_tc4(const LayerDims& L, const Tc4Plan& P, Tc4Maps* maps, const void* 
     ms->key[0] = nullptr;
     const int taps = L.kh * L.kw;
     if (!encode_x(&ms->x, x, L, P)) return (int)cudaErrorInvalidValue;
-    if (!encode_w(&ms->wb, w_base, P, L.c_out, taps * L.c_p)) return (int)cudaErrorInvalidValue;
-    if (L.c_r > 0) { if (!encode_w(&ms->wc, w_cond, P, L.c_out, taps * L.c_r)) return (int)cudaErrorInvalidValue; }
-    else ms->wc = ms->wb;
+    const int blocks = P.pair ? P.nt / 64 : P.nt / 32;
+    const bool halves = P.half_job < kNoHalfJob;
+    if (!encode_w(&ms->wb, w_base, P, L.c_out, taps * L.c_p, blocks)) return (int)cudaErrorInvalidValue;
+    ms->wc = ms->half_wb = ms->half_wc = ms->wb;
+    if (L.c_r > 0 && !encode_w(&ms->wc, w_cond, P, L.c_out, taps * L.c_r, blocks)) return (int)cudaErrorInvalidValue;
+    if (halves && !encode_w(&ms->half_wb, w_base, P, L.c_out, taps * L.c_p, blocks / 2)) return (int)cudaErrorInvalidValue;
+    if (halves && L.c_r > 0 && !encode_w(&ms->half_wc, w_cond, P, L.c_out, taps * L.c_r, blocks / 2)) return (int)cudaErrorInvalidValue;
     ms->key[0] = x; ms->key[1] = w_base; ms->key[2] = w_cond;
   }
   Tc4Params prm;
@@ -1535,10 +1569,11 @@ int launch_tc4(const LayerDims& L, const Tc4Plan& P, Tc4Maps* maps, const void* 
   prm.residual = static_cast<const __nv_bfloat16*>(residual);
   prm.y = y; prm.mask = mask; prm.counters = counters;
   prm.x = static_cast<const __nv_bfloat16*>(x); prm.w_cond = static_cast<const __nv_bfloat16*>(w_cond);
-  const int which = (P.nt == 128 ? 1 : 0) | (P.i8 ? 2 : 0) | (P.pair ? 4 : 0);
+  const bool half = P.half_job < kNoHalfJob;             // (bf16 pairs of 128 columns)
+  const int which = half ? 7 : (P.nt == 128 ? 1 : 0) | (P.i8 ? 2 : 0) | (P.pair ? 4 : 0);
   static const void* const kernels[8] = {
       instance<64, false, false>(), nullptr, instance<64, true, false>(), nullptr,
-      instance<64, false, true>(), instance<128, false, true>(), instance<64, true, true>(), nullptr};
+      instance<64, false, true>(), instance<128, false, true>(), instance<64, true, true>(), instance<128, false, true, true>()};
   const void* kernel = kernels[which];
   if (!kernel) return (int)cudaErrorInvalidValue;
   static bool attr_set[64][8] = {};   // (the attribute is per device and kernel instance)
@@ -1562,7 +1597,9 @@ int launch_tc4(const LayerDims& L, const Tc4Plan& P, Tc4Maps* maps, const void* 
   attr[1].val.clusterDim.x = P.pair ? 2u : (unsigned)P.split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  void* args[4] = {&ms->x, &ms->wb, &ms->wc, &prm};
+  WeightMaps<true> maps_half = {ms->wb, ms->wc, ms->half_wb, ms->half_wc};
+  WeightMaps<false> maps_all = {ms->wb, ms->wc};
+  void* args[3] = {&ms->x, half ? (void*)&maps_half : (void*)&maps_all, &prm};
   const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, args);
   if (e != cudaSuccess) return (int)e;
   return (int)cudaGetLastError();

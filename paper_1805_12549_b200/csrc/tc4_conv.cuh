@@ -37,6 +37,7 @@ enum : uint8_t {
 
 enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2, kTc4Window2 = 3 };
 constexpr int kTc4MaxTiles = 32;
+constexpr int kNoHalfJob = 1 << 30;
 
 struct Tc4Plan {
   int valid;
@@ -57,6 +58,7 @@ struct Tc4Plan {
   int tiles_first;       // W_cond's tiles come in this order; so many serve the first patch of a stride-2 window
   uint8_t order[kTc4MaxTiles];
   int tiles_m, tiles_n;  // jobs
+  int half_job, half_tiles;   // job of a pair that has half of the columns (kNoHalfJob: none), and how many jobs are halved
   int split;             // 1, 2, 4 or 8
   int grid;
   int rows;              // entries of row[] in use
@@ -72,7 +74,7 @@ struct Tc4Plan {
 
 struct Tc4MapSet {
   const void* key[3];    // x, w_base, w_cond the maps were encoded for
-  CUtensorMap x, wb, wc;
+  CUtensorMap x, wb, wc, half_wb, half_wc;
 };
 
 struct Tc4Maps {

@@ -193,6 +193,13 @@ K_LOOPS = [
     (O.Shape(3000, 2, 2, 128, 256, stride=2, groups=4), "one patch per tap", "streamed", "too much padding for a window"),
     (O.Shape(80, 13, 15, 128, 256, stride=2, groups=4), "one patch per tap", "streamed", "odd extents"),
     (O.Shape(60, 28, 28, 256, 256, stride=2, groups=8), "one patch per tap", "streamed", "too many chunks to pack"),
+    (O.Shape(28, 28, 28, 128, 128, groups=4), "halves", "packed", "18 jobs in halves, packed"),
+    (O.Shape(60, 14, 14, 128, 320, groups=4), "halves", "packed", "halves of a half-empty column tile"),
+    (O.Shape(256, 4, 4, 512, 512, groups=4), "halves", "streamed", "7 jobs in halves, streamed"),
+    (O.Shape(96, 14, 14, 256, 512, stride=2, groups=4), "halves", "streamed", "halves, stride 2"),
+    (O.Shape(60, 28, 28, 128, 256, stride=2, groups=4), "halves", "packed", "halves, stride 2, packed"),
+    (O.Shape(50, 14, 14, 256, 256, groups=8), "halves", "streamed", "halves, two base slices"),
+    (O.Shape(110, 14, 14, 128, 128, 1, 1, 1, 0, groups=1), "halves", "", "halves, 1x1"),
 ]
 
 
