@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_pool_kernel(const __grid_con
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
               if (out && l > 0 && ((cols >> (2 * odd + h)) & 1u))
-                *(uint4*)(y0 + (long long)ab * P.wo * 64 + (14 * h + odd) * 64) = make_uint4(act[h][0], act[h][1], act[h][2], act[h][3]);
+                __stcs((uint4*)(y0 + (long long)ab * P.wo * 64 + (14 * h + odd) * 64), make_uint4(act[h][0], act[h][1], act[h][2], act[h][3]));
               if (edge && !((cols >> (2 * odd + h)) & 1u)) {
 #pragma unroll
                 for (int o = 0; o < 4; ++o) act[h][o] = ninf;

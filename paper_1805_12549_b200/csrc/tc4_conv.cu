@@ -551,7 +551,7 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
     if (ptx::elect_one()) {
       Cursor c{0, 0};
       bool ok = true, seen = false;
-      const int ip = P.wp * P.hp, st = P.mode == kTc4Taps ? L.stride : 1;
+      const int ip = P.wp * P.hp, st = P.mode == kTc4Window ? 1 : L.stride;
       for (int j = 0; j < jobs && ok; ++j) {
         const int pos = job_pos(j);
         const int n0 = pos / ip, rem = pos - n0 * ip, h0 = rem / P.wp, w0 = rem - h0 * P.wp;
@@ -598,7 +598,7 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
                                             (uint16_t)k, (uint16_t)(s.tap_row & 15));
           } else {
             for (int k = 0; k < tiles; ++k)
-              ptx::tma_load_im2col_4d<PAIR>(dst + k * 128 * 128, &map_x, bar, ch + k * (I8 ? 128 : 64), w0, h0, n0, 0, 0);
+              ptx::tma_load_im2col_4d<PAIR>(dst + k * 128 * 128, &map_x, bar, ch + k * (I8 ? 128 : 64), w0 * st, h0 * st, n0, 0, 0);
           }
         }
       }
@@ -1209,7 +1209,7 @@ bool encode_x(CUtensorMap* map, const void* base, const LayerDims& L, const Tc4P
   // window mode: the box ends at the image's last column and row; else at the last filter position
   const int up = P.mode == kTc4Window || P.mode == kTc4Window2 ? 0 : L.pad - (L.kw - 1);
   const int upper[2] = {up, up};
-  const cuuint32_t st = P.mode == kTc4Taps || P.mode == kTc4Window2 ? (cuuint32_t)L.stride : 1u;
+  const cuuint32_t st = P.mode == kTc4Window ? 1u : (cuuint32_t)L.stride;
   const cuuint32_t es[4] = {1, st, st, 1};
   return fn(map, P.i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
             str, lower, upper, (cuuint32_t)(128 / eb), (cuuint32_t)P.patch_rows, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -1361,9 +1361,9 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   const int eb = P.i8 ? 1 : 2, ck = 128 / eb, slice = 32 / eb;
   if (cond_mode == CG_COND_SKIP_TILES || cond_mode == CG_COND_COMPACT) return false;   // R is computed everywhere
   if (L.channel_tau > 0.f || (L.grouping && L.groups > 1)) return false;
-  // 3x3 with pad 1, any stride up to 8; 1x1 without gating of its input
+  // 3x3 with pad 1 and 1x1 without gating of its input, any stride up to 8
   const bool k3 = L.kh == 3 && L.kw == 3 && L.pad == 1 && L.stride <= 8;
-  const bool k1 = L.kh == 1 && L.kw == 1 && L.pad == 0 && L.stride == 1 && L.c_r == 0;
+  const bool k1 = L.kh == 1 && L.kw == 1 && L.pad == 0 && L.stride <= 8 && L.c_r == 0;
   if (!k3 && !k1) return false;
   if (L.c_in % ck != 0 || L.c_in / ck > 255 || L.c_out % 32 != 0) return false;
   // base channels: whole chunks, or one or two K slices (a weight tile then holds whole taps)

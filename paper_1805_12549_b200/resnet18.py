@@ -217,11 +217,17 @@ class Instance:
         self._patches = None
         self.stem_ws = torch.empty(B.cg_stem_workspace_bytes(), dtype=torch.uint8, device="cuda")
         self.convs, self.out, self.mask = {}, {}, {}
+        # large batches: the 1x1 stride-2 shortcuts read every other pixel of their block's input themselves (a launch less
+        # each, and the input not written and read again)
+        self.strided = {}
+        if net.algo == B.CG_ALGO_AUTO and B.cg_stem_pool_pays(n, net.image, net.image):
+            self.strided = {short.name: (c1.h, st) for short, c1, _, st in net.blocks if short is not None and st != 1}
         for s in net.specs:
             algo = net.algo
             if s.c_out % 32 or s.c_in % 64:
                 algo = B.CG_ALGO_AUTO
-            conv = B.GatedConv(n, s.h, s.h, s.c_in, s.c_out, k=s.k, stride=s.stride, pad=s.pad,
+            h, stride = self.strided.get(s.name, (s.h, s.stride))
+            conv = B.GatedConv(n, h, h, s.c_in, s.c_out, k=s.k, stride=stride, pad=s.pad,
                                groups=s.groups, dtype=B.CG_BF16, relu=s.relu, has_residual=s.has_residual,
                                algo=algo, cond_mode=net.cond_mode)
             self.convs[s.name] = conv
@@ -230,7 +236,7 @@ class Instance:
             self.mask[s.name] = mask if s.gated else None
         hp = (net.stem_hw + 2 - 3) // 2 + 1
         self.pooled = torch.empty((n, hp, hp, 64), **bf)
-        self.sub = {sh.name: torch.empty((n, sh.h, sh.h, sh.c_in), **bf) for sh, _, _, _ in net.blocks if sh}
+        self._sub = {}
         self.avg = torch.empty((n, 1, 1, net.fc.c_in), **bf)
         self.launches = None
         self.stem_pools = self.convs["stem"].uses_tensor_cores and B.cg_stem_pool_pays(n, net.image, net.image)
@@ -243,6 +249,13 @@ class Instance:
             self._patches = torch.empty((self.n, hw, hw, STEM_KPAD), dtype=torch.bfloat16, device="cuda")
         return self._patches
 
+    def _subsampled(self, short, x, stride):
+        """Every stride-th pixel of a block's input, where a shortcut (or who looks at its input) takes that."""
+        if short.name not in self._sub:
+            self._sub[short.name] = torch.empty((self.n, short.h, short.h, short.c_in), dtype=torch.bfloat16, device="cuda")
+        B.cg_subsample_bf16(x, self._sub[short.name], stride)
+        return self._sub[short.name]
+
     def _fused_stem(self, x):
         """The stem and, where one kernel does both, the pooling behind it."""
         s = self.net.specs[0]
@@ -253,11 +266,12 @@ class Instance:
             B.cg_stem_forward(self.convs[s.name].handle, x, s.wb, s.bn, s.delta, y, self.stem_ws)
         return y
 
-    def _conv(self, s, x, residual, before_conv, density, record):
+    def _conv(self, s, x, residual, before_conv, density, record, given=None):
+        """`given`: the tensor that the layer's handle reads, where that is not the layer's input x itself."""
         if before_conv is not None:
             before_conv(s, x, self.n, density)
         y = self.out[s.name]
-        self.convs[s.name].forward(x, s.wb, s.wc, s.bn, s.delta, y, self.mask[s.name], residual)
+        self.convs[s.name].forward(x if given is None else given, s.wb, s.wc, s.bn, s.delta, y, self.mask[s.name], residual)
         if record is not None:
             record.append((s, x.clone(), None if residual is None else residual.clone(), y.clone(),
                            None if self.mask[s.name] is None else self.mask[s.name].clone()))
@@ -281,7 +295,7 @@ class Instance:
             events.append((name, e0, e1))
             return out
 
-        go = lambda s, a, r=None: timed(s.name, lambda: self._conv(s, a, r, before_conv, density, record))
+        go = lambda s, a, r=None, given=None: timed(s.name, lambda: self._conv(s, a, r, before_conv, density, record, given))
         patch = lambda: B.cg_im2col_bf16(x, self.patches, STEM_K, STEM_STRIDE, STEM_PAD)   # noqa: E731
         stem = net.specs[0]
         fused = before_conv is None and self.convs[stem.name].uses_tensor_cores
@@ -299,11 +313,13 @@ class Instance:
         for short, c1, c2, st in net.blocks:
             identity = a
             if short is not None:
-                src = a
-                if st != 1:
-                    timed(short.name + ".subsample", lambda: B.cg_subsample_bf16(a, self.sub[short.name], st))
-                    src = self.sub[short.name]
-                identity = go(short, src)
+                src = given = a
+                if short.name not in self.strided:
+                    if st != 1:
+                        src = given = timed(short.name + ".subsample", lambda: self._subsampled(short, a, st))
+                elif before_conv is not None or record is not None:
+                    src = self._subsampled(short, a, st)   # (what the layer is a convolution of)
+                identity = go(short, src, given=given)
             t = go(c1, a)
             a = go(c2, t, identity)
         timed("avgpool", lambda: B.cg_avgpool_bf16(a, self.avg))
@@ -333,9 +349,8 @@ class Instance:
             identity = a
             if short is not None:
                 src = a
-                if st != 1:
-                    src = self.sub[short.name]
-                    B.cg_subsample_bf16(a, src, st)
+                if st != 1 and short.name not in self.strided:
+                    src = self._subsampled(short, a, st)
                 identity = conv(short, src)
             a = conv(c2, conv(c1, a), identity)
         B.cg_avgpool_bf16(a, self.avg)
@@ -344,7 +359,8 @@ class Instance:
     def launches_per_forward(self):
         """Kernels one forward pass launches: those of every layer plus the glue operators."""
         n = sum(B.cg_conv_launches_per_forward(c.handle) for c in self.convs.values())
-        return n + (1 if self.stem_pools else 3) + sum(1 for sh, _, _, st in self.net.blocks if sh is not None and st != 1)
+        return n + (1 if self.stem_pools else 3) + sum(1 for sh, _, _, st in self.net.blocks
+                                                       if sh is not None and st != 1 and sh.name not in self.strided)
 
     def stats(self):
         """Per-layer counters since the last call, and the network's FLOP summary (multiplications

@@ -51,6 +51,9 @@ SHAPES = [
     (O.Shape(1, 7, 5, 192, 64, 1, 1, 1, 0, groups=1), "1x1, three chunks, part of a job"),
     (O.Shape(1, 17, 16, 256, 64, 1, 1, 1, 0, groups=1), "1x1, four chunks, K loop over a cluster"),
     (O.Shape(3, 10, 10, 512, 64, groups=8), "G = 8"),
+    (O.Shape(70, 14, 14, 64, 128, 1, 1, 2, 0, groups=1), "1x1, stride 2, pairs"),
+    (O.Shape(1, 13, 9, 256, 64, 1, 1, 2, 0, groups=1), "1x1, stride 2, odd extents, K loop over a cluster"),
+    (O.Shape(40, 10, 11, 128, 96, 1, 1, 3, 0, groups=1), "1x1, stride 3"),
 ]
 
 
