@@ -230,10 +230,19 @@ __device__ __forceinline__ uint32_t relu_bf16x2(uint32_t v) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// int8 layers: requantised in 64-bit integers, rounded half up, clamped.
-__device__ __forceinline__ int finish_q(int mul, long long off, int acc, int shift, int lo) {
-  const long long q = ((long long)acc * mul + off + (1ll << (shift - 1))) >> shift;
-  return (int)(q < lo ? lo : (q > 127 ? 127 : q));
+// int8 layers: requantised in 64-bit integers, rounded half up (the half is in `off`: add_half), clamped to 32 bits.
+__device__ __forceinline__ long long add_half(long long off, int shift) { return (long long)((unsigned long long)off + (1ull << (shift - 1))); }
+__device__ __forceinline__ int requantise(int mul, long long off, int acc, int shift) {
+  const long long z = (long long)((unsigned long long)((long long)acc * mul) + (unsigned long long)off);
+  const int top = (int)(z >> 32), lo = (int)__funnelshift_r((uint32_t)z, (uint32_t)top, (uint32_t)shift);
+  return (top >> shift) == (lo >> 31) ? lo : (top >> 31) ^ 0x7fffffff;
+}
+// Four of them, clamped to [lo, 127], as bytes.
+__device__ __forceinline__ uint32_t pack_s8(const int* v, int lo) {
+  uint32_t d;
+  asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, 0;" : "=r"(d) : "r"(max(v[3], lo)), "r"(max(v[2], lo)));
+  asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(max(v[1], lo)), "r"(max(v[0], lo)), "r"(d));
+  return d;
 }
 
 // Whether no gate of the column tile can fire: thresholds of +inf (or not a number); int8: beyond every sum.  (Finite
@@ -766,7 +775,7 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
       if (ch < L.c_out) {
         if (I8) {
           s_q[c] = make_int4(prm.bn.q_gate_thr[ch], prm.bn.q_mul_base[ch], prm.bn.q_mul_full[ch], 0);
-          s_o[c] = make_longlong2(prm.bn.q_off_base[ch], prm.bn.q_off_full[ch]);
+          s_o[c] = make_longlong2(add_half(prm.bn.q_off_base[ch], L.shift), add_half(prm.bn.q_off_full[ch], L.shift));
         } else {
           const ChannelConsts k = fold_channel(prm.bn, prm.delta, L.eps, ch);
           s_t[c] = k.t; s_t2[c] = k.t2; s_k[c] = make_float4(k.a1, k.b1, k.a2, k.b2);
@@ -860,15 +869,15 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 if constexpr (I8) {
-                  out[h][g] = 0;
+                  int q[4];
 #pragma unroll
                   for (int e = 0; e < 4; ++e) {
                     const int v = 4 * (e >> 1) + 2 * h + (e & 1), k = 4 * g + e;
                     const bool d = (int)p[v] >= qt[k];
                     if (d) bits |= 1u << (k + 8 * (2 * i + h));
-                    const int y = finish_q(d ? qm2[k] : qm1[k], d ? qo2[k] : qo1[k], (int)p[v] + (d ? (int)r[v] : 0), L.shift, lo_q);
-                    out[h][g] |= ((uint32_t)y & 255u) << (8 * e);
+                    q[e] = requantise(d ? qm2[k] : qm1[k], d ? qo2[k] : qo1[k], (int)p[v] + (d ? (int)r[v] : 0), L.shift);
                   }
+                  out[h][g] = pack_s8(q, lo_q);
                 } else {
 #pragma unroll
                   for (int w = 0; w < 2; ++w) {
@@ -1012,16 +1021,16 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
         if (u + kEpiThreads < rows * kLanes) next = item(u + kEpiThreads);
         if (t.valid) {
           if (I8) {
-            uint32_t v = 0;
+            int q[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int4 k = s_q[cc + e];
               const bool d = pi[e] >= k.x;
               if (d) w |= 1u << e;
               const longlong2 o = s_o[cc + e];
-              v |= ((uint32_t)finish_q(d ? k.z : k.y, d ? o.y : o.x, pi[e] + (d ? ri[e] : 0), L.shift, lo_q) & 255u) << (8 * e);
+              q[e] = requantise(d ? k.z : k.y, d ? o.y : o.x, pi[e] + (d ? ri[e] : 0), L.shift);
             }
-            *(uint32_t*)((uint8_t*)prm.y + t.at) = v;
+            *(uint32_t*)((uint8_t*)prm.y + t.at) = pack_s8(q, lo_q);
           } else {
             float v[4];
 #pragma unroll
