@@ -830,6 +830,8 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
         const uint32_t h0 = P.div_wp.div(rem), w0 = rem - h0 * (uint32_t)P.wp;
         // pixel of this lane's row, or -1 (a padding position); the rows of the pieces take it from there
         const int own = (int)n0 < L.n && (int)h0 < L.ho && (int)w0 < L.wo ? (int)((n0 * L.ho + h0) * L.wo + w0) : -1;
+        // (the residual comes to L2 while the sums are waited for)
+        if (has_res && own >= 0 && ch < L.c_out) ptx::prefetch_l2(prm.residual + (long long)own * L.c_out + ch);
         ok = wait4(sh, prm.counters, &sh->acc_full[stage], (j / kAcc) & 1, 6);
         if (!ok) break;
         ptx::tc_fence_after();
