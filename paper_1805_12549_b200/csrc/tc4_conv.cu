@@ -10,8 +10,10 @@
 //       its filter tap (r, s) is the position r*(w+1) + s further on: a patch of 128 + 2*(w+2) positions
 //       serves all nine taps, each as another start row of the same shared-memory operand.  Positions in the
 //       padding are computed and dropped: (w/(w+1))*(h/(h+1)) of the rows are pixels, whatever the image size.
-//   tap mode (stride > 1, wide images)  one copy per filter tap and chunk, of 128 output pixels; no row is
-//       dropped.  1x1 layers: one copy per chunk.
+//   stride-2 windows (pairs, even extents)  the pixels of odd or even rows and columns are four lattices of pitch
+//       w' + 1 and h' + 1, and a window over each serves four, two, two or one of the taps.
+//   tap mode (other strides, wide images)  one copy per filter tap and chunk, of 128 output pixels; no row is
+//       dropped.  1x1 layers of any stride: one copy per chunk.
 // The partial sum P and the conditional sum R have separate TMEM accumulators, two (N = 128) or four
 // (N = 64) jobs deep, and both are computed for every pixel: a block of 128 pixels and 64 channels always
 // holds a firing gate at the densities in use, and waiting for the gate costs more than it saves.  So the
@@ -34,18 +36,18 @@
 // 16-byte pieces, four lanes to a 64-byte run.  The K loop goes by filter rows (three taps, up to 12 MMAs, one weight
 // stage), written out for the kinds of rows a layer has (issue_jobs): a row then costs its issuer 170 cycles beside its MMAs.
 // As a table of row kinds it took 570 to 1,000, two issuers in turns, more than the MMAs: 128@16x16 b256 23.6 us for 20.0
-// now, 128@28x28 b128 31.8 for 26.1, 64@56x56 b128 37.8 for 35.2 (graphs of 20 calls).  The copies of a pair's second CTA count on its leader's barriers without an arrival of their own: with
-// one per slot, and copies issued from divergent code, every streamed layer waited for its weights (512 channels,
-// 4x4, batch 256: 67 us).
+// now, 128@28x28 b128 31.8 for 26.1, 64@56x56 b128 37.8 for 35.2 (graphs of 20 calls).  The copies of a pair's second CTA
+// count on its leader's barriers without an arrival of their own: with one per slot, and copies issued from divergent
+// code, every streamed layer waited for its weights (512 channels, 4x4, batch 256: 67 us).
 //
-// Measured (us per pass among others, batch as named, G = 4; in brackets the other kernels' best, timed alike):
-// 128@16x16 b256 24.3 (34.2), 256@8x8 b256 23.8 (34.0), 512@4x4 b256 28.1 (43.7), 64@56x56 b64 with residual 26.6 (50.1),
-// 128->256 stride 2 at 28x28 b64 16.3 (27.4), int8 128@28x28 b64 17.5 (32.6); on the device, one image: 128@28x28 8.2
-// (19.5), 512@7x7 8.1 (23.2).  What bounds it now (cycles that its roles wait, per launch, in a copy with clock reads):
-// nobody waits for copies.  512@4x4 takes what its MMAs take in two rounds of jobs (36,900 cycles), 256@8x8 27,600 of
-// 32,400; elsewhere the issuers' rows are the longer chain: 930 to 1,490 cycles of a row's issue, table entry, barriers
-// and commits beside 9 or 12 MMAs of 64, 33,000 of 38,500 cycles at 128@16x16.  Neither resident weights nor fewer,
-// larger copies made it faster.
+// Measured (graphs of 20 calls, us; in brackets with two issuers that walked a table, before the steps that the comments
+// below describe): 128@16x16 b256 17.4 (23.0), 256@8x8 b256 20.4 (23.7), 512@4x4 b256 23.8 (27.8), 64@56x56 b64 with residual
+// 22.4 (23.4), b128 39 (43), 128->256 stride 2 at 28x28 b64 12.7 (16.0), int8 128@28x28 b64 15.8 (17.6), 128@28x28 b128 22.8 (30.7),
+// 64->128 stride 2 b128 17.0 (26.4); one image: 64@56x56 7.0 (7.4), 512@7x7 7.7 (8.1).  What bounds it now: 256 and 512
+// channels their MMAs in whole rounds of jobs (9,000 cycles a job of 256 channels, 9,200 of MMAs); 128 channels the same behind a
+// start of 4,000 cycles and a tail of 4,000; 64 channels operand reads, 2,100 cycles a job of 1,550 of MMAs at 43 each beside
+// the patches' writes to shared memory; int8 its epilogue; one image the chain of first copies (2,500 cycles), MMAs, exchange
+// and epilogue.  Neither a fixed order of first copies (patch, weights, patches) nor two small CTAs to an SM made it faster.
 // Every mbarrier wait is bounded; on expiry the CTA records CG_ERR_DEVICE_TIMEOUT with the id of the wait
 // and leaves.
 #include <cstring>
@@ -1349,7 +1351,7 @@ bool plan_window2(const LayerDims& L, Tc4Plan* P) {
   if (L.c_p % ck != 0) {
     // a base path of less than a chunk: with packed weights that stay in shared memory
     const int tiles = (9 * L.c_p + ck - 1) / ck + (9 * L.c_r + ck - 1) / ck;
-    if (L.c_in > 2 * ck || (int)(kSmemBytes - 1024 - kOffStages) - tiles * (L.c_out <= 64 || P->i8 ? 4096 : 8192) < 3 * rows * 128) return false;
+    if (L.c_in > 2 * ck || (int)(kSmemBytes - 1024 - kOffStages) - tiles * (L.c_out <= 64 || (P->i8 && L.c_in <= ck) ? 4096 : 8192) < 3 * rows * 128) return false;
   }
   P->mode = kTc4Window2;
   P->wp = L.wo + 1; P->hp = L.ho + 1;
@@ -1439,7 +1441,9 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   } else {
     // CTA pairs: each SM then fetches and holds half of the weights.  128 channels per job unless the layer
     // has fewer or the rounds of jobs come out shorter with 64: such a job takes about 0.85 of the time (512@4x4
-    // b256: 3 rounds of 64 36.1 us, 2 rounds of 128 27.6; 128->256 stride 2: 19.0 and 15.7).  int8: 64 (the requantisation constants of 128 do not fit the epilogue's registers).
+    // b256: 3 rounds of 64 36.1 us, 2 rounds of 128 27.6; 128->256 stride 2: 19.0 and 15.7).  int8 layers of one chunk, whose epilogue is the longer
+    // part: 64 (128@28x28 b64 15.6 and 15.8 us with 128, b20 9.7 and 10.0); with more chunks 128 is faster (256@14x14 b128
+    // 20.4 and 19.3, 512@7x7 b128 21.1 and 18.8).
     P.pair = 1;
     const int pairs = sms / 2;
     int tiles256 = (int)((positions + 255) / 256);
@@ -1456,7 +1460,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
       }
       P.div_ip.set((uint32_t)(P.wp * P.hp)); P.div_wp.set((uint32_t)P.wp);
     }
-    P.nt = (P.i8 || L.c_out <= 64 || rounds(tn64) * 0.85 < rounds(tn128)) ? 64 : 128;
+    P.nt = ((P.i8 && L.c_in <= ck) || L.c_out <= 64 || rounds(tn64) * 0.85 < rounds(tn128)) ? 64 : 128;
     P.tiles_m = tiles256; P.tiles_n = P.nt == 64 ? tn64 : tn128;
     if (P.tiles_n > pairs) return false;
     if (P.mode == kTc4Window2) P.rows = 0;                     // (walked without a table)
@@ -1580,14 +1584,14 @@ int launch_tc4(const LayerDims& L, const Tc4Plan& P, Tc4Maps* maps, const void* 
   prm.residual = static_cast<const __nv_bfloat16*>(residual);
   prm.y = y; prm.mask = mask; prm.counters = counters;
   prm.x = static_cast<const __nv_bfloat16*>(x); prm.w_cond = static_cast<const __nv_bfloat16*>(w_cond);
-  const bool half = P.half_job < kNoHalfJob;             // (bf16 pairs of 128 columns)
-  const int which = half ? 7 : (P.nt == 128 ? 1 : 0) | (P.i8 ? 2 : 0) | (P.pair ? 4 : 0);
-  static const void* const kernels[8] = {
+  const bool half = P.half_job < kNoHalfJob;             // (pairs of 128 columns)
+  const int which = half ? (P.i8 ? 9 : 8) : (P.nt == 128 ? 1 : 0) | (P.i8 ? 2 : 0) | (P.pair ? 4 : 0);
+  static const void* const kernels[10] = {
       instance<64, false, false>(), nullptr, instance<64, true, false>(), nullptr,
-      instance<64, false, true>(), instance<128, false, true>(), instance<64, true, true>(), instance<128, false, true, true>()};
+      instance<64, false, true>(), instance<128, false, true>(), instance<64, true, true>(), instance<128, true, true>(), instance<128, false, true, true>(), instance<128, true, true, true>()};
   const void* kernel = kernels[which];
   if (!kernel) return (int)cudaErrorInvalidValue;
-  static bool attr_set[64][8] = {};   // (the attribute is per device and kernel instance)
+  static bool attr_set[64][10] = {};   // (the attribute is per device and kernel instance)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
   if (!attr_set[dev][which]) {
