@@ -90,6 +90,12 @@ struct Tc4Params {
 template <bool HALF> struct WeightMaps { CUtensorMap wb, wc; };
 template <> struct WeightMaps<true> { CUtensorMap wb, wc, half_wb, half_wc; };
 
+// Rows of a cluster's job that each of its CTAs finishes: the positions that there are, in even shares.
+__device__ __forceinline__ int split_rows(const Tc4Plan& P, int group) {
+  const int there = min(128, P.positions - group * 128);
+  return ((there + P.split - 1) / P.split + 1) & ~1;
+}
+
 struct Shared4 {
   uint64_t a_full[kMaxNA], a_empty[kMaxNA];
   uint64_t b_full[kMaxNB], b_empty[kMaxNB];
@@ -951,7 +957,7 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
     if constexpr (SPLIT) {
       // rows [part * rows, (part + 1) * rows) of the job are this CTA's to finish: four channels per thread
       constexpr int kLanes = NT / 4;                           // threads per row
-      const int rows = 128 / P.split;
+      const int rows = split_rows(P, group);
       const uint32_t block = (uint32_t)rows * kSumPitch;       // a CTA's sums of those rows, of one path
       struct Item { long long at; int m; uint2 res; bool valid; };
       auto item = [&](int u) {
@@ -992,9 +998,9 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
       if (P.sums_late) ptx::cluster_sync();                    // (their room is part of the rings: no MMA reads those any more)
       const int turn = warp - kEpiWarp0 + 1;                   // (one destination a warp, another one first in every CTA: all
       if (ok && turn <= P.split && lane < 2) {                 // sending to the first and then to the second took three times as long)
-        const int to = (part + turn) & (P.split - 1), mine = lane ? P.r_mask : P.p_mask;
-        if ((mine >> part) & 1) {
-          const int slot = (lane ? __popc(P.p_mask) : 0) + __popc(mine & ((1 << part) - 1));
+        const int to = (part + turn) & (P.split - 1), mine = lane ? P.r_mask : P.p_mask, others = ~(1 << to);
+        if (to != part && ((mine >> part) & 1)) {
+          const int slot = (lane ? __popc(P.p_mask & others) : 0) + __popc(mine & others & ((1 << part) - 1));
           ptx::bulk_copy_cluster(ptx::map_cluster(ptx::smem_u32(smem) + P.off_sums + (uint32_t)slot * block, (uint32_t)to),
                                  ptx::smem_u32(smem) + kOffStages + (uint32_t)lane * 128u * kSumPitch + (uint32_t)to * block, block,
                                  ptx::map_cluster(ptx::smem_u32(&sh->sums), (uint32_t)to));
@@ -1003,23 +1009,29 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
       }
       __syncwarp();
       ok = ok && wait4(sh, prm.counters, &sh->sums, 0, 9);
-      const int p_slots = __popc(P.p_mask), slots = p_slots + __popc(P.r_mask);
       for (int u = et; ok && u < rows * kLanes; u += kEpiThreads) {
         const Item t = next;
         const int lr = u / kLanes, cc = (u % kLanes) * 4, ch = tile_n * NT + cc;
         uint32_t w = 0;
         float pf[4] = {0.f, 0.f, 0.f, 0.f}, rf[4] = {0.f, 0.f, 0.f, 0.f};
         int pi[4] = {0, 0, 0, 0}, ri[4] = {0, 0, 0, 0};
-        const uint32_t off = ptx::smem_u32(smem) + P.off_sums + (uint32_t)lr * kSumPitch + (uint32_t)cc * 4u;
-        // the partial sums of the CTAs in order
-        for (int k = 0; k < slots; ++k) {
-          const uint4 v = ptx::ld_shared_16(off + (uint32_t)k * block);
-          if (k < p_slots) {
-            if (I8) { pi[0] += (int)v.x; pi[1] += (int)v.y; pi[2] += (int)v.z; pi[3] += (int)v.w; }
-            else { pf[0] += __uint_as_float(v.x); pf[1] += __uint_as_float(v.y); pf[2] += __uint_as_float(v.z); pf[3] += __uint_as_float(v.w); }
-          } else {
-            if (I8) { ri[0] += (int)v.x; ri[1] += (int)v.y; ri[2] += (int)v.z; ri[3] += (int)v.w; }
-            else { rf[0] += __uint_as_float(v.x); rf[1] += __uint_as_float(v.y); rf[2] += __uint_as_float(v.z); rf[3] += __uint_as_float(v.w); }
+        // the partial sums of the CTAs in order; this CTA's own are where it left them
+        const uint32_t base = ptx::smem_u32(smem), in_row = (uint32_t)lr * kSumPitch + (uint32_t)cc * 4u;
+        uint32_t from = base + P.off_sums + in_row, own = base + kOffStages + (uint32_t)part * block + in_row;
+#pragma unroll
+        for (int path = 0; path < 2; ++path, own += 128u * kSumPitch) {
+          const int mask = path ? P.r_mask : P.p_mask;
+          for (int peer = 0; peer < P.split; ++peer) {
+            if (!((mask >> peer) & 1)) continue;
+            const uint4 v = ptx::ld_shared_16(peer == part ? own : from);
+            if (peer != part) from += block;
+            if (path == 0) {
+              if (I8) { pi[0] += (int)v.x; pi[1] += (int)v.y; pi[2] += (int)v.z; pi[3] += (int)v.w; }
+              else { pf[0] += __uint_as_float(v.x); pf[1] += __uint_as_float(v.y); pf[2] += __uint_as_float(v.z); pf[3] += __uint_as_float(v.w); }
+            } else {
+              if (I8) { ri[0] += (int)v.x; ri[1] += (int)v.y; ri[2] += (int)v.z; ri[3] += (int)v.w; }
+              else { rf[0] += __uint_as_float(v.x); rf[1] += __uint_as_float(v.y); rf[2] += __uint_as_float(v.z); rf[3] += __uint_as_float(v.w); }
+            }
           }
         }
         if (u + kEpiThreads < rows * kLanes) next = item(u + kEpiThreads);
@@ -1117,7 +1129,8 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     if (SPLIT && lane == 0) {
       // what the cluster sends here: P and R of this CTA's rows from every CTA that has some
       ptx::mbar_init(&sh->sums, 1);
-      ptx::mbar_expect_tx(&sh->sums, (uint32_t)(__popc(P.p_mask) + __popc(P.r_mask)) * (128u / (unsigned)P.split) * kSumPitch);
+      const int others = ~(1 << part);
+      ptx::mbar_expect_tx(&sh->sums, (uint32_t)((__popc(P.p_mask & others) + __popc(P.r_mask & others)) * split_rows(P, group)) * kSumPitch);
     }
     if (lane == 0) { sh->abort_flag = 0; sh->active = 0; sh->rows_active = 0; sh->epi_done = 0; }
     ptx::fence_mbar_init();
@@ -1546,6 +1559,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   for (int i = 0; i < P.rows; ++i) {
     P.row[i] = raw[i].r;
   }
+  P.positions = (int)((long long)L.n * P.wp * P.hp);
   P.off_b = kOffStages;
   P.off_a = kOffStages + (unsigned)(P.packed ? weights : P.nb * P.stage_bytes);
   P.smem_bytes = kSmemBytes;

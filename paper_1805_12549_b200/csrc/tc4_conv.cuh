@@ -47,6 +47,7 @@ struct Tc4Plan {
   int mode;              // kTc4Window, kTc4Taps, kTc4Chunks, kTc4Window2: what a patch slot holds
   int wp, hp;            // pitch of the stacked pixel space: window mode w + pad, h + pad; else w', h'
   FastDiv div_ip, div_wp;   // by wp * hp and by wp
+  int positions;         // n * wp * hp
   int patch_rows;        // pixels per patch load
   int slot_bytes;        // patch slot: one or two loads of a window, or up to three loads of 128 pixels
   int loads;             // window mode: loads per slot
