@@ -1424,19 +1424,30 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   // (1x1 layers of up to three chunks have one row and nothing to share: as pairs they end without the exchange of
   // sums, 28x28 x 64 -> 128, one image, 8.5 and 5.0 us)
   const bool one_row = P.mode == kTc4Chunks && L.c_in <= 3 * ck;
-  if (!one_row && (long long)tiles128 * tn64 * 2 <= sms) {
+  // Where a job's K loop is short, or only two CTAs could share it, pairs end sooner: they have no exchange of sums, but
+  // their epilogue of 256 pixels waits longer for a residual.  us shared / as pairs (and with a residual), by MMAs a job:
+  //   up to 36: 56x56 x 64 7.0 / 5.9, 28x28 x 64 6.3 / 6.0 (6.3 / 6.4), 56x56 x 64->128 stride 2 7.9 / 6.0, 14x14 x 256->512
+  //     1x1 6.9 / 5.2; the pixels of a single job are shared sooner, 5x5 x 64 5.4 / 5.9 (5.2 / 6.1);
+  //   up to 72: 2 x 28x28 x 128 8.5 / 7.5, one image (14 jobs) 7.9 / 7.5 (7.9 / 8.1), 28x28 x 128->256 stride 2 8.1 / 6.5;
+  //     eight CTAs to a job are faster, 3 x 14x14 x 128 (10 jobs) 6.9 / 7.4 (6.9 / 8.1);
+  //   two CTAs: 8 x 14x14 x 256 10.7 / 8.5, 5 x 14x14 x 256 10.6 / 8.1 (10.6 / 8.7), 51 x 5x8 x 512->192 14.3 / 12.0;
+  //   else shared: 14x14 x 256 7.5 / 8.1 (7.5 / 8.4), 7x7 x 512 7.3 / 11.5.
+  const long long small = (long long)tiles128 * tn64, mmas = (long long)L.kh * L.kw * L.c_in / slice;
+  const bool as_pairs = small * 4 > sms * 7 / 8 ||
+                        (mmas <= 72 && small >= (L.has_residual ? 16 : 14)) ||
+                        (mmas <= 72 && !L.has_residual && (mmas <= 36 ? tiles128 >= 2 : L.stride == 2));
+  if (!one_row && !as_pairs && small * 2 <= sms) {
     // Fewer jobs of 128 pixels and 64 channels than half the SMs: their K loops are shared, as far as all clusters
     // are on the chip at once.  Measured with 148 SMs: 32 clusters of 4 are, 15 of 8 are and 16 are not (9.2 against
     // 16.5 us for 4 x 7x7 x 512).  14 and 15 clusters of 8 gain nothing over 4 (4 x 7x7 x 512 -> 448 9.2 and 9.4 us, 6 x 7x7
     // x 512 -> 320 9.4 and 9.3), so the line of 8 lies at 13, clear of the edge.
     // Eight CTAs need sixteen rows, or exactly eight: with 9 or 12 the exchange costs what the shorter loops save (14x14 x
-    // 256 7.5 us with 4 and 8; 28x28 x 128, 8 rows, 8.0 and 7.8; 9x9 x 128 7.0 and 6.5; 56x56 x 64, 4 rows, 7.7 with 2
-    // CTAs and 7.2 with 4).
+    // 256 7.5 us with 4 and 8; 28x28 x 128, 8 rows, 8.0 and 7.8; 9x9 x 128 7.0 and 6.5).
     P.nt = 64; P.tiles_m = tiles128; P.tiles_n = tn64;
     P.rows = raw_rows(L, P, raw);
     if (P.rows > kTc4MaxRows) return false;
     for (int s = 2; s <= kTc4MaxSplit; s *= 2)
-      if ((long long)tiles128 * tn64 * s <= (s == 8 ? sms * 3 / 4 : (s == 4 ? sms * 7 / 8 : sms)) &&
+      if (small * s <= (s == 8 ? sms * 3 / 4 : (s == 4 ? sms * 7 / 8 : sms)) &&
           (P.rows >= (s == 8 ? 16 : s) || P.rows == s))
         P.split = s;
     int total = 0, done = 0, s = 1;

@@ -225,3 +225,29 @@ def test_k_loops_of_pairs(s, patch, weights, why, how):
                          ids=["one chunk", "two base slices", "one base slice", "a base chunk"])
 def test_int8_stride_2_windows(s):
     _run(K.make_int8_case("wini8s2", s, density=0.3))
+
+
+# Layers of few jobs, on either side of each line between K loops shared by a cluster and CTA pairs.
+FEW_JOBS = [
+    (O.Shape(2, 5, 5, 64, 64, groups=4), False, 4, "36 MMAs, one job"),
+    (O.Shape(1, 14, 14, 64, 64, groups=4), False, 1, "36 MMAs, two pixel tiles"),
+    (O.Shape(1, 28, 28, 64, 64, groups=4), True, 4, "36 MMAs, residual, 7 jobs"),
+    (O.Shape(1, 56, 56, 64, 64, groups=4), True, 1, "36 MMAs, residual, 28 jobs"),
+    (O.Shape(3, 14, 14, 128, 128, groups=4), False, 8, "72 MMAs, 12 jobs"),
+    (O.Shape(1, 28, 28, 128, 128, groups=4), False, 1, "72 MMAs, 16 jobs"),
+    (O.Shape(1, 28, 28, 128, 128, groups=4), True, 4, "72 MMAs, residual, 14 jobs"),
+    (O.Shape(2, 28, 28, 128, 128, groups=4), True, 1, "72 MMAs, residual, 28 jobs"),
+    (O.Shape(1, 28, 28, 128, 256, stride=2, groups=4), False, 1, "72 MMAs, stride 2"),
+    (O.Shape(3, 14, 14, 256, 256, groups=4), False, 4, "144 MMAs, room for four CTAs a job"),
+    (O.Shape(5, 14, 14, 256, 256, groups=4), False, 1, "144 MMAs, room for two"),
+]
+
+
+@pytest.mark.parametrize("s,residual,ctas,why", FEW_JOBS, ids=[f[3] for f in FEW_JOBS])
+def test_layers_of_few_jobs(s, residual, ctas, why):
+    c = K.make_float_case("winfew", s, "bf16", density=0.3, residual=residual)
+    _run(c)
+    g = K.GpuCase(c, algo=0)
+    plan = g.conv.plan
+    g.close()
+    assert f"over {ctas} CTA(s)" in plan, plan
