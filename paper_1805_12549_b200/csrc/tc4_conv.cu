@@ -26,8 +26,8 @@
 //
 // Jobs are 256 pixels of a CTA pair (cta_group::2): each SM holds half of a job's pixels and half of its
 // weights, which halves what an SM has to fetch from L2 and what an MMA reads of shared memory (one CTA's
-// 128 x 128 MMA takes the whole 128 bytes per clock).  Layers with fewer jobs than SMs instead split the K
-// loop of a 128-pixel job over the 2, 4 or 8 CTAs of a cluster: every CTA finishes 1/split of the rows, and is sent the
+// 128 x 128 MMA takes the whole 128 bytes per clock).  Layers of few jobs with long K loops (tc4_plan has
+// the lines) instead split the K loop of a 128-pixel job over the 2, 4 or 8 CTAs of a cluster: every CTA finishes 1/split of the rows, and is sent the
 // others' sums of those by bulk copies between the CTAs' shared memories.
 //
 // Warp roles (640 threads): 0 = patch producer, 2 = weight producer, 1 = MMA issuer, 4-19 = epilogue (TMEM
