@@ -10,8 +10,11 @@
 //       its filter tap (r, s) is the position r*(w+1) + s further on: a patch of 128 + 2*(w+2) positions
 //       serves all nine taps, each as another start row of the same shared-memory operand.  Positions in the
 //       padding are computed and dropped: (w/(w+1))*(h/(h+1)) of the rows are pixels, whatever the image size.
-//   stride-2 windows (pairs, even extents)  the pixels of odd or even rows and columns are four lattices of pitch
-//       w' + 1 and h' + 1, and a window over each serves four, two, two or one of the taps.
+//   stride-2 windows (pairs, even extents)  the pixels of odd or even rows and columns are four lattices, and a filter row
+//       reads two of them: the odd columns serve its first and last tap, one position apart, the even ones its middle tap.
+//       The taps come in the order 0..8, as everywhere: with one patch for all taps of a lattice (four to a chunk for six) they
+//       came as 0 2 6 8 1 7 3 5 4, and a gate whose partial sum lies within an fp32 rounding of its threshold could decide
+//       otherwise than in the same layer tap by tap.
 //   tap mode (other strides, wide images)  one copy per filter tap and chunk, of 128 output pixels; no row is
 //       dropped.  1x1 layers of any stride: one copy per chunk.
 // The partial sum P and the conditional sum R have separate TMEM accumulators, two (N = 128) or four
@@ -69,7 +72,7 @@ constexpr int kSpinLimit = 1 << 21;
 constexpr long long kWaitCycles = 2000000000ll;
 constexpr unsigned kOffConsts = 1024;                  // behind the barriers; 32 bytes per channel
 constexpr unsigned kOffRows = kOffConsts + 128 * 32;   // the row table
-constexpr unsigned kOffStages = 7 * 1024;              // weight stages, then patch slots
+constexpr unsigned kOffStages = 6 * 1024;              // weight stages, then patch slots
 static_assert(kOffRows + kTc4MaxRows * sizeof(Tc4Row) <= kOffStages, "row table");
 constexpr unsigned kSmemBytes = 227 * 1024;
 
@@ -162,14 +165,22 @@ __device__ __forceinline__ void issue_row(int tiles, uint32_t d, uint32_t hi, ui
   }
 }
 
+// From a filter row's first tap to its tap s, in 16-byte units of the patch: `step` each, or, for kTwoPatches (stride-2
+// windows), the odd columns' next position (s = 2) and the patch of the even columns behind them (s = 1).
+constexpr int kLatticeRows = 136;                              // positions per patch: 129, in whole swizzle atoms
+constexpr uint32_t kTwoPatches = ~0u;
+__device__ __forceinline__ uint32_t tap_step(uint32_t s, uint32_t step) {
+  return step != kTwoPatches ? s * step : s == 1 ? kLatticeRows * 8u : s * 4u;
+}
+
 // The taps [T0, T1) of a chunk, K slices [K0, K0 + NK) of each: PER taps of NK slices share a weight tile, B0 is the first
-// tile of the stage.  Tap t reads the patch at (t / 3 - R0) * row_lo + (t % 3) * step.
+// tile of the stage.  Tap t reads the patch at (t / 3 - R0) * row_lo + tap_step(t % 3).
 template <bool PAIR, bool I8, int T0, int T1, int R0, int K0, int NK, int PER, int B0>
 __device__ __forceinline__ void issue_taps(uint32_t d, uint32_t hi, uint32_t a, uint32_t row_lo, uint32_t step, uint32_t b,
                                            uint32_t tile, uint32_t idesc, uint32_t acc) {
 #pragma unroll
   for (int t = T0; t < T1; ++t) {
-    const uint32_t a_t = a + (uint32_t)(t / 3 - R0) * row_lo + (uint32_t)(t % 3) * step + 2u * K0;
+    const uint32_t a_t = a + (uint32_t)(t / 3 - R0) * row_lo + tap_step((uint32_t)(t % 3), step) + 2u * K0;
     const uint32_t b_t = b + (uint32_t)(t / PER - B0) * tile + (uint32_t)((t % PER) * NK) * 2u;
 #pragma unroll
     for (int k = 0; k < NK; ++k)
@@ -181,39 +192,16 @@ __device__ __forceinline__ void issue_taps(uint32_t d, uint32_t hi, uint32_t a, 
 // The same with the weights' K slices packed (Tc4Plan::packed): a tap has PT conditional slices, of which the patch's chunk takes
 // NK from FIRST on, beside its own slices from K0 on.  Filter row R; `a` is its first tap.
 template <bool I8, int R, int PT, int FIRST, int K0, int NK>
-__device__ __forceinline__ void issue_packed(uint32_t d, uint32_t hi, uint32_t a, uint32_t b, uint32_t tile, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void issue_packed(uint32_t d, uint32_t hi, uint32_t a, uint32_t step, uint32_t b, uint32_t tile, uint32_t idesc,
+                                             uint32_t acc) {
 #pragma unroll
   for (int t = 0; t < 3; ++t)
 #pragma unroll
     for (int k = 0; k < NK; ++k) {
       const int s = (3 * R + t) * PT + FIRST + k;
-      ptx::umma<true, I8>(d, ((uint64_t)hi << 32) | (a + 8u * t + 2u * (K0 + k)),
+      ptx::umma<true, I8>(d, ((uint64_t)hi << 32) | (a + tap_step((uint32_t)t, step) + 2u * (K0 + k)),
                           ((uint64_t)hi << 32) | (b + (uint32_t)(s / 4) * tile + (uint32_t)(s % 4) * 2u), idesc, t == 0 && k == 0 ? acc : 1u);
     }
-}
-
-// Stride-2 windows: the filter taps by parity patch (kTc4Window2): patch 0 serves taps 0, 2, 6, 8, patch 1 taps 1, 7, patch 2
-// taps 3, 5, patch 3 tap 4.
-constexpr unsigned long long kTapOrder = 0x453718620ull;       // a nibble each
-__host__ __device__ constexpr int tap_at(int i) { return (int)((kTapOrder >> (4 * i)) & 15); }
-constexpr int kParityTaps[5] = {0, 4, 6, 8, 9};                // where the taps of patch p start in that order
-
-// The taps [I0, I1) of that order, all of patch PP: NK slices of each from K0 on.  Their weights: PT slices a tap from FIRST on,
-// packed (PT > 0), or a stage of three tiles in the same order (PT = 0).
-template <bool I8, int PP, int I0, int I1, int PT, int FIRST, int K0, int NK>
-__device__ __forceinline__ void issue_parity(uint32_t d, uint32_t hi, uint32_t a, uint32_t row_lo, uint32_t b, uint32_t tile,
-                                             uint32_t idesc, uint32_t acc) {
-#pragma unroll
-  for (int i = I0; i < I1; ++i) {
-    const int j = i - kParityTaps[PP];                         // (the patch's second column, row: one position further)
-    const uint32_t a_t = a + (PP == 0 ? (j & 1) * 8u + (j >> 1) * row_lo : PP == 1 ? j * row_lo : PP == 2 ? j * 8u : 0u);
-#pragma unroll
-    for (int k = 0; k < NK; ++k) {
-      const int s = tap_at(i) * PT + FIRST + k;
-      const uint32_t b_t = PT > 0 ? b + (uint32_t)(s / 4) * tile + (uint32_t)(s % 4) * 2u : b + (uint32_t)(i % 3) * tile + 2u * k;
-      ptx::umma<true, I8>(d, ((uint64_t)hi << 32) | (a_t + 2u * (K0 + k)), ((uint64_t)hi << 32) | b_t, idesc, i == I0 && k == 0 ? acc : 1u);
-    }
-  }
 }
 
 // One row of the table in shared memory.
@@ -314,13 +302,13 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
                                            int jobs) {
   constexpr int kAcc = 512 / (2 * NT);
   constexpr uint32_t kTileU = (uint32_t)(NT / 2) * 8u;         // a weight tile, 16-byte units
-  constexpr bool kWin = MODE == kTc4Window || MODE == kTc4Window2;
+  constexpr bool kWin = MODE == kTc4Window;
   const Tc4Plan& P = prm.P;
   uint32_t idesc = I8 ? ptx::idesc_s8(256, NT) : ptx::idesc_bf16(256, NT);
   const uint32_t hi = (uint32_t)(ptx::smem_desc(0, 1024, 2) >> 32);
   const uint32_t a_size = (uint32_t)P.slot_bytes >> 4, b_size = (uint32_t)P.stage_bytes >> 4;
   const uint32_t row_lo = kWin ? (uint32_t)P.wp * 8u : 0u;
-  constexpr uint32_t kStep = kWin ? 8u : 1024u;                // from tap to tap of a filter row
+  constexpr uint32_t kStep = kWin ? 8u : MODE == kTc4Window2 ? kTwoPatches : 1024u;   // from tap to tap of a filter row
   const int na = P.na, nb = P.nb;
   const bool resident = P.resident != 0;
   const int ck = I8 ? 128 : 64;
@@ -363,59 +351,27 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
     }
     if (resident) { b = IssueRing{0, 0u, b0}; new_b = j == 0; b_seen = false; }
     if constexpr (MODE == kTc4Window2 && CH > 0) {
+      // a patch per chunk and filter row
       constexpr int PT = 4 * CH - KP;                          // conditional slices of a tap
       const uint32_t bc = b0 + (uint32_t)P.tiles_base * kTileU;
-      auto chunk = [&](auto second) {
-        constexpr int Q = decltype(second)::value, FIRST = Q ? 4 - KP : 0, K0 = Q ? 0 : KP, NK = Q ? 4 : 4 - KP;
-        auto patch = [&](auto which) {
-          constexpr int PP = decltype(which)::value, I0 = kParityTaps[PP], I1 = kParityTaps[PP + 1];
-          take_a();
-          if (Q == 0) need_tile(BASE ? P.tiles_base - 1 : P.tiles_base - 1 + (PP == 0 ? P.tiles_first : P.tiles_cond));
-          if (!ok) return;
-          look_a();
-          if (Q == 0) issue_parity<I8, PP, I0, I1, KP, 0, 0, KP>(d_p, hi, a_at, row_lo, b0, kTileU, idesc, PP ? 1u : 0u);
-          if (!BASE) issue_parity<I8, PP, I0, I1, PT, FIRST, K0, NK>(d_r, hi, a_at, row_lo, bc, kTileU, idesc, Q || PP ? 1u : 0u);
-          free_a();
-        };
-        patch(std::integral_constant<int, 0>{});
-        if (ok) patch(std::integral_constant<int, 1>{});
-        if (ok) patch(std::integral_constant<int, 2>{});
-        if (ok) patch(std::integral_constant<int, 3>{});
+      auto filter_row = [&](auto chunk, auto row) {
+        constexpr int Q = decltype(chunk)::value, R = decltype(row)::value, FIRST = Q ? 4 - KP : 0, K0 = Q ? 0 : KP, NK = Q ? 4 : 4 - KP;
+        take_a();
+        need_tile(BASE ? ((3 * R + 3) * KP - 1) / 4 : P.tiles_base + ((3 * R + 2) * PT + FIRST + NK - 1) / 4);
+        if (!ok) return;
+        look_a();
+        if (Q == 0) issue_taps<true, I8, 3 * R, 3 * R + 3, R, 0, KP, 4 / KP, 0>(d_p, hi, a_at, 0, kStep, b0, kTileU, idesc, R ? 1u : 0u);
+        if (!BASE) issue_packed<I8, R, PT, FIRST, K0, NK>(d_r, hi, a_at, kStep, bc, kTileU, idesc, Q || R ? 1u : 0u);
+        free_a();
+      };
+      auto chunk = [&](auto q) {
+        filter_row(q, std::integral_constant<int, 0>{});
+        if (ok) filter_row(q, std::integral_constant<int, 1>{});
+        if (ok) filter_row(q, std::integral_constant<int, 2>{});
       };
       chunk(std::integral_constant<int, 0>{});
       if (ok && CH == 2 && !BASE) chunk(std::integral_constant<int, 1>{});
       if (!ok) return;
-    } else if constexpr (MODE == kTc4Window2) {
-#pragma unroll 1
-      for (int q = 0; q < chunks; ++q) {
-        const uint32_t d = q < base_chunks ? d_p : d_r, acc = q == 0 || q == base_chunks ? 0u : 1u;
-        take_a(); take_b();
-        if (!ok) return;
-        issue_parity<I8, 0, 0, 3, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, acc);
-        free_b(b_slot);
-        take_b();
-        if (!ok) return;
-        look_a();
-        issue_parity<I8, 0, 3, 4, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
-        free_a();
-        take_a();
-        if (!ok) return;
-        look_a();
-        issue_parity<I8, 1, 4, 6, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
-        free_b(b_slot);
-        free_a();
-        take_a(); take_b();
-        if (!ok) return;
-        look_a();
-        issue_parity<I8, 2, 6, 8, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
-        free_a();
-        take_a();
-        if (!ok) return;
-        look_a();
-        issue_parity<I8, 3, 8, 9, 0, 0, 0, 4>(d, hi, a_at, row_lo, b_at, kTileU, idesc, 1u);
-        free_b(b_slot);
-        free_a();
-      }
     } else if constexpr (CH > 0) {
       static_assert(CH == 0 || CH == 2, "two chunks");
       constexpr int PT = 8 - KP;                               // conditional slices of a tap
@@ -427,19 +383,19 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
       if (!BASE) {
         auto upto = [&](int last) { need_tile(P.tiles_base + last / 4); return ok; };
         if (!upto(2 * PT + 3 - KP)) return;
-        issue_packed<I8, 0, PT, 0, KP, 4 - KP>(d_r, hi, a_at, bc, kTileU, idesc, 0u);
+        issue_packed<I8, 0, PT, 0, KP, 4 - KP>(d_r, hi, a_at, kStep, bc, kTileU, idesc, 0u);
         if (!upto(5 * PT + 3 - KP)) return;
-        issue_packed<I8, 1, PT, 0, KP, 4 - KP>(d_r, hi, a_at + row_lo, bc, kTileU, idesc, 1u);
+        issue_packed<I8, 1, PT, 0, KP, 4 - KP>(d_r, hi, a_at + row_lo, kStep, bc, kTileU, idesc, 1u);
         if (!upto(8 * PT + 3 - KP)) return;
         look_a();
-        issue_packed<I8, 2, PT, 0, KP, 4 - KP>(d_r, hi, a_at + 2u * row_lo, bc, kTileU, idesc, 1u);
+        issue_packed<I8, 2, PT, 0, KP, 4 - KP>(d_r, hi, a_at + 2u * row_lo, kStep, bc, kTileU, idesc, 1u);
         free_a();
         take_a();
         if (!upto(9 * PT - 1)) return;
-        issue_packed<I8, 0, PT, 4 - KP, 0, 4>(d_r, hi, a_at, bc, kTileU, idesc, 1u);
-        issue_packed<I8, 1, PT, 4 - KP, 0, 4>(d_r, hi, a_at + row_lo, bc, kTileU, idesc, 1u);
+        issue_packed<I8, 0, PT, 4 - KP, 0, 4>(d_r, hi, a_at, kStep, bc, kTileU, idesc, 1u);
+        issue_packed<I8, 1, PT, 4 - KP, 0, 4>(d_r, hi, a_at + row_lo, kStep, bc, kTileU, idesc, 1u);
         look_a();
-        issue_packed<I8, 2, PT, 4 - KP, 0, 4>(d_r, hi, a_at + 2u * row_lo, bc, kTileU, idesc, 1u);
+        issue_packed<I8, 2, PT, 4 - KP, 0, 4>(d_r, hi, a_at + 2u * row_lo, kStep, bc, kTileU, idesc, 1u);
       }
       free_a();
     } else for (int q = 0; q < chunks; ++q) {
@@ -574,23 +530,6 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
         const int n0 = pos / ip, rem = pos - n0 * ip, h0 = rem / P.wp, w0 = rem - h0 * P.wp;
         const int pos1 = pos + P.patch_rows;                   // start of a window's second load
         const int n1 = pos1 / ip, rem1 = pos1 - n1 * ip, h1 = rem1 / P.wp, w1 = rem1 - h1 * P.wp;
-        if (PAIR && P.mode == kTc4Window2) {
-          // four patches per chunk, the pixels of odd or even rows and columns
-          const int ck = I8 ? 128 : 64, patches = 4 * (BASE ? (L.c_p + ck - 1) / ck : L.c_in / ck);
-          for (int i = 0; i < patches && ok; ++i) {
-            if (!seen) ok = wait4_one(sh, prm.counters, &sh->a_empty[c.slot], c.par ^ 1u, 1);
-            if (!ok) break;
-            uint8_t* dst = s_a + (size_t)c.slot * P.slot_bytes;
-            uint64_t* full = &sh->a_full[c.slot];
-            c.next(P.na);
-            seen = ptx::mbar_test_wait(&sh->a_empty[c.slot], c.par ^ 1u);
-            const uint32_t bar = leader(full);
-            expect(full, (uint32_t)P.patch_rows * 128u);
-            ptx::tma_load_im2col_4d<PAIR>(dst, &map_x, bar, (i >> 2) * ck, w0 * 2 - 1, h0 * 2 - 1, n0, (uint16_t)(i & 1),
-                                          (uint16_t)((i >> 1) & 1));
-          }
-          continue;
-        }
         Tc4Row next = row_at(table, lo);
         for (int i = lo; i < hi; ++i) {
           const Tc4Row s = next;
@@ -603,12 +542,17 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
           c.next(P.na);
           seen = ptx::mbar_test_wait(&sh->a_empty[c.slot], c.par ^ 1u);
           const uint32_t bar = leader(full);
-          const int ch = (int)s.chunk * (I8 ? 128 : 64), tiles = P.mode == kTc4Window ? P.loads : ((s.kind >> 4) & 3) + 1;
+          const int ch = (int)s.chunk * (I8 ? 128 : 64);
+          const int tiles = P.mode == kTc4Window || P.mode == kTc4Window2 ? P.loads : ((s.kind >> 4) & 3) + 1;
           expect(full, (uint32_t)(tiles * P.patch_rows) * 128u);
           if (P.mode == kTc4Window) {
             ptx::tma_load_im2col_4d<PAIR>(dst, &map_x, bar, ch, w0 - L.pad, h0 - L.pad, n0, 0, 0);
             if (tiles == 2)
               ptx::tma_load_im2col_4d<PAIR>(dst + (size_t)P.patch_rows * 128, &map_x, bar, ch, w1 - L.pad, h1 - L.pad, n1, 0, 0);
+          } else if (P.mode == kTc4Window2) {
+            for (int k = 0; k < 2; ++k)
+              ptx::tma_load_im2col_4d<PAIR>(dst + k * kLatticeRows * 128, &map_x, bar, ch, w0 * 2 - 1, h0 * 2 - 1, n0, (uint16_t)k,
+                                            (uint16_t)(s.tap_row & 15));
           } else if (P.mode == kTc4Taps) {
             for (int k = 0; k < 3; ++k)
               ptx::tma_load_im2col_4d<PAIR>(dst + k * 128 * 128, &map_x, bar, ch, w0 * st - L.pad, h0 * st - L.pad, n0,
@@ -633,37 +577,9 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
           expect(&sh->b_full[t / 3], (uint32_t)tiles * kTile);
           for (int k = t; k < t + tiles; ++k) {
             const bool cond = k >= P.tiles_base;
-            const int tile = cond ? (int)P.order[k - P.tiles_base] : k;
-            ptx::tma_load_5d<PAIR>(s_b + (size_t)(tile + (cond ? P.tiles_base : 0)) * kTile, cond ? &map_wc : &map_wb, bar,
+            const int tile = cond ? k - P.tiles_base : k;
+            ptx::tma_load_5d<PAIR>(s_b + (size_t)k * kTile, cond ? &map_wc : &map_wb, bar,
                                    tile * (I8 ? 128 : 64), 0, 0, 0, row0);
-          }
-        }
-      }
-    } else if (PAIR && P.mode == kTc4Window2) {
-      // stages of three taps in the order of the parity patches
-      if (ptx::elect_one()) {
-        Cursor c{0, 0};
-        bool ok = true, seen = false;
-        const int ck = I8 ? 128 : 64, base_chunks = L.c_p / ck, stages = 3 * (BASE ? base_chunks : L.c_in / ck);
-        const int rounds = P.resident ? (jobs > 0 ? 1 : 0) : jobs;
-        for (int j = 0; j < rounds && ok; ++j) {
-          for (int i = 0; i < stages; ++i) {
-            if (!seen) ok = wait4_one(sh, prm.counters, &sh->b_empty[c.slot], c.par ^ 1u, 2);
-            if (!ok) break;
-            uint8_t* dst = s_b + (size_t)c.slot * P.stage_bytes;
-            uint64_t* full = &sh->b_full[c.slot];
-            c.next(P.nb);
-            seen = ptx::mbar_test_wait(&sh->b_empty[c.slot], c.par ^ 1u);
-            const uint32_t bar = leader(full);
-            const int q = i / 3, first = (i - 3 * q) * 3;
-            const bool cond = q >= base_chunks;
-            const int per_tap = cond ? L.c_r : L.c_p, k0 = (cond ? q - base_chunks : q) * ck;
-            const bool half = HALF && j == P.half_job && !P.resident;
-            const CUtensorMap* map = cond ? &map_wc : &map_wb;
-            if constexpr (HALF) map = half ? (cond ? &maps.half_wc : &maps.half_wb) : map;
-            expect(full, half ? 3u * kTile / 2u : 3u * kTile);
-            for (int k = 0; k < 3; ++k)
-              ptx::tma_load_5d<PAIR>(dst + k * kTile, map, bar, tap_at(first + k) * per_tap + k0, 0, 0, 0, row0 + (half ? group & 1 : 0));
           }
         }
       }
@@ -1232,9 +1148,10 @@ bool encode_x(CUtensorMap* map, const void* base, const LayerDims& L, const Tc4P
   const cuuint64_t dims[4] = {(cuuint64_t)L.c_in, (cuuint64_t)L.w, (cuuint64_t)L.h, (cuuint64_t)L.n};
   const cuuint64_t str[3] = {L.c_in * eb, (cuuint64_t)L.w * L.c_in * eb, (cuuint64_t)L.h * L.w * L.c_in * eb};
   const int lower[2] = {-L.pad, -L.pad};
-  // window mode: the box ends at the image's last column and row; else at the last filter position
-  const int up = P.mode == kTc4Window || P.mode == kTc4Window2 ? 0 : L.pad - (L.kw - 1);
-  const int upper[2] = {up, up};
+  // window mode: the box ends at the image's last column and row; else at the last filter position.  Stride-2 windows: at
+  // the last column (a position more than there are outputs) and the last filter position of a column.
+  const int last = L.pad - (L.kw - 1);
+  const int upper[2] = {P.mode == kTc4Window || P.mode == kTc4Window2 ? 0 : last, P.mode == kTc4Window ? 0 : last};
   const cuuint32_t st = P.mode == kTc4Window ? 1u : (cuuint32_t)L.stride;
   const cuuint32_t es[4] = {1, st, st, 1};
   return fn(map, P.i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
@@ -1281,7 +1198,7 @@ int raw_rows(const LayerDims& L, const Tc4Plan& P, RawRow* out) {
     o.r.kind = (uint8_t)((nks - 1) | ks0 << 2 | (tiles - 1) << 4);
     o.r.chunk = (uint8_t)q;
     o.r.tap_row = (uint8_t)(r | stage_tiles << 4);
-    o.a_key = P.mode == kTc4Taps ? q * 16 + r : q;
+    o.a_key = P.mode == kTc4Taps || P.mode == kTc4Window2 ? q * 16 + r : q;
     o.b_key = b_key;
     return &o;
   };
@@ -1353,22 +1270,22 @@ void plan_base(RawRow* raw, Tc4Plan* P) {
   }
 }
 
-// Stride-2 layers of pairs: windows over the four lattices of odd and even rows and columns, of pitch w' + 1 and h' + 1 (an odd
-// lattice starts in the padding; an even one ends there).  Tap by tap the pixels of a job were copied nine times: 128->256
+// Stride-2 layers of pairs: windows over the lattices of odd and even columns, of pitch w' + 1, two to a filter row (an odd one
+// starts in the padding; an even one ends there).  Tap by tap the pixels of a job were copied nine times a chunk: 128->256
 // channels at 28x28, 650 KB a job and CTA, 9,000 cycles of copies for 4,600 of MMAs.
 bool plan_window2(const LayerDims& L, Tc4Plan* P) {
-  const int eb = P->i8 ? 1 : 2, ck = 128 / eb;
-  const int rows = (128 + L.wo + 2 + 7) / 8 * 8;
-  if (L.w % 2 || L.h % 2 || rows > 256) return false;
-  if ((long long)L.n * (L.wo + 1) * (L.ho + 1) > 0x7fffffffll - 65536) return false;
+  const int eb = P->i8 ? 1 : 2, ck = 128 / eb, slot = 2 * kLatticeRows * 128;
+  if (L.w % 2 || L.h % 2) return false;
+  if (L.wo < 2) return false;                                  // (half of the positions would be padding)
+  if ((long long)L.n * (L.wo + 1) * L.ho > 0x7fffffffll - 65536) return false;
   if (L.c_p % ck != 0) {
     // a base path of less than a chunk: with packed weights that stay in shared memory
     const int tiles = (9 * L.c_p + ck - 1) / ck + (9 * L.c_r + ck - 1) / ck;
-    if (L.c_in > 2 * ck || (int)(kSmemBytes - 1024 - kOffStages) - tiles * (L.c_out <= 64 || (P->i8 && L.c_in <= ck) ? 4096 : 8192) < 3 * rows * 128) return false;
+    if (L.c_in > 2 * ck || (int)(kSmemBytes - 1024 - kOffStages) - tiles * (L.c_out <= 64 || (P->i8 && L.c_in <= ck) ? 4096 : 8192) < 2 * slot) return false;
   }
   P->mode = kTc4Window2;
-  P->wp = L.wo + 1; P->hp = L.ho + 1;
-  P->loads = 1; P->patch_rows = rows; P->slot_bytes = (rows * 128 + 1023) / 1024 * 1024; P->a_step = 8;
+  P->wp = L.wo + 1; P->hp = L.ho;
+  P->loads = 2; P->patch_rows = kLatticeRows; P->slot_bytes = slot; P->a_step = 8;
   return true;
 }
 
@@ -1473,22 +1390,21 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     int tiles256 = (int)((positions + 255) / 256);
     auto rounds = [&](int tn) { return tn > pairs ? 1e30 : (double)((tiles256 + pairs / tn - 1) / (pairs / tn)); };
     if (k3 && L.stride == 2 && plan_window2(L, &P)) {
-      // a third of the patch bytes, and up to a third more positions: not where that makes more than half as many rounds again
+      // two thirds of the patch bytes, and up to half as many positions again: not where that makes more than half as many rounds again
       const double taps = rounds(tn128);
       const long long padded = (long long)L.n * P.wp * P.hp;
       const int before = tiles256;
       tiles256 = (int)((padded + 255) / 256);
       if (rounds(tn128) > 1.5 * taps) {
         tiles256 = before;
-        P.mode = kTc4Taps; P.wp = L.wo; P.hp = L.ho; P.patch_rows = 128; P.slot_bytes = 3 * 128 * 128; P.a_step = 1024;
+        P.mode = kTc4Taps; P.wp = L.wo; P.hp = L.ho; P.loads = 1; P.patch_rows = 128; P.slot_bytes = 3 * 128 * 128; P.a_step = 1024;
       }
       P.div_ip.set((uint32_t)(P.wp * P.hp)); P.div_wp.set((uint32_t)P.wp);
     }
     P.nt = ((P.i8 && L.c_in <= ck) || L.c_out <= 64 || rounds(tn64) * 0.85 < rounds(tn128)) ? 64 : 128;
     P.tiles_m = tiles256; P.tiles_n = P.nt == 64 ? tn64 : tn128;
     if (P.tiles_n > pairs) return false;
-    if (P.mode == kTc4Window2) P.rows = 0;                     // (walked without a table)
-    else P.rows = raw_rows(L, P, raw);
+    P.rows = raw_rows(L, P, raw);
     if (P.rows > kTc4MaxRows) return false;
     const int groups = pairs / P.tiles_n;
     // A last round that less than half of the pairs take part in: its jobs as two of 64 columns each, which take two thirds
@@ -1519,8 +1435,6 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.sums_late = !P.pair && P.mode == kTc4Taps && room - (int)sums_bytes < slots_wanted * P.slot_bytes + stages_wanted * P.stage_bytes;
   if (!P.sums_late) room -= (int)sums_bytes;
 
-  if (P.mode == kTc4Window2) { max_a = 4 * (L.c_in / ck); max_b = 3 * (L.c_in / ck); }
-
   // shared memory: resident weights if they leave room for three patch slots, else rings of both
   const int clusters = P.grid / (P.pair ? 2 : P.split);
   const int jobs = P.pair ? (P.tiles_m + clusters / P.tiles_n - 1) / (clusters / P.tiles_n) : 1;
@@ -1533,24 +1447,14 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
                             : P.pair && P.mode == kTc4Window && P.nt == 128 && L.c_in == 2 * ck && L.c_p < ck && L.c_r > 0 &&
                                   room - (tb + tc) * tile_bytes >= 2 * P.slot_bytes) {
     P.packed = 1; P.resident = 1;
-    P.tiles_base = tb; P.tiles_cond = tc; P.tiles_first = tc;
+    P.tiles_base = tb; P.tiles_cond = tc;
     P.nb = (tb + tc + 2) / 3;
-    // the conditional tiles in the order in which the taps take them
-    const int per_tap = L.c_r / slice;
-    bool in[kTc4MaxTiles] = {};
-    int n = 0;
-    for (int i = 0; i < 9; ++i) {
-      const int t = P.mode == kTc4Window2 ? tap_at(i) : i;
-      for (int k = t * per_tap; k < (t + 1) * per_tap; ++k)
-        if (!in[k / 4]) { in[k / 4] = true; P.order[n++] = (uint8_t)(k / 4); }
-      if (i == 3 && P.mode == kTc4Window2) P.tiles_first = n;
-    }
   } else if (max_b <= kMaxNB && jobs > 1 && room - max_b * P.stage_bytes >= 3 * P.slot_bytes) {
     P.resident = 1;
     P.nb = max_b;
   } else {
     // (three weight stages at least: a base stage stays while conditional ones pass)
-    int na = P.mode == kTc4Window || P.mode == kTc4Window2 ? 3 : 2;
+    int na = P.mode == kTc4Window ? 3 : 2;
     if (na > max_a * jobs) na = max_a * jobs;
     while (na > 2 && room - na * P.slot_bytes < 4 * P.stage_bytes) --na;
     if (!P.pair && na > 1 && room - na * P.slot_bytes < 3 * P.stage_bytes) --na;
@@ -1563,10 +1467,7 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   P.na = (room - weights) / P.slot_bytes;                      // what is left goes to patches
   if (P.na > kMaxNA) P.na = kMaxNA;
   if (P.na < 1 || (P.pair && P.na < 2 && max_a * jobs > 1)) return false;
-  if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) {
-    if (P.mode == kTc4Window2) P.base_rows = 1;
-    else plan_base(raw, &P);
-  }
+  if (P.pair && L.c_r > 0 && cond_mode == CG_COND_AUTO) plan_base(raw, &P);
   for (int i = 0; i < P.rows; ++i) {
     P.row[i] = raw[i].r;
   }

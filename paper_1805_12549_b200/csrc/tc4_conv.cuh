@@ -36,7 +36,6 @@ enum : uint8_t {
 };
 
 enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2, kTc4Window2 = 3 };
-constexpr int kTc4MaxTiles = 32;
 constexpr int kNoHalfJob = 1 << 30;
 
 struct Tc4Plan {
@@ -45,19 +44,17 @@ struct Tc4Plan {
   int pair;              // 1: CTA pairs (256 pixels per job); 0: `split` CTAs share the K loop of a 128-pixel job
   int nt;                // output channels per job: 64 or 128
   int mode;              // kTc4Window, kTc4Taps, kTc4Chunks, kTc4Window2: what a patch slot holds
-  int wp, hp;            // pitch of the stacked pixel space: window mode w + pad, h + pad; else w', h'
+  int wp, hp;            // pitch of the stacked pixel space: window mode w + pad, h + pad; stride-2 windows w' + 1, h'; else w', h'
   FastDiv div_ip, div_wp;   // by wp * hp and by wp
   int positions;         // n * wp * hp
   int patch_rows;        // pixels per patch load
-  int slot_bytes;        // patch slot: one or two loads of a window, or up to three loads of 128 pixels
-  int loads;             // window mode: loads per slot
+  int slot_bytes;        // patch slot: one or two loads of a window, two of a stride-2 window's filter row, or up to three of 128 pixels
+  int loads;             // window modes: loads per slot
   int a_step;            // distance of a row's pixel operands, 16-byte units
   int na, nb;            // ring depths: patch slots, weight stages
   int stage_bytes;       // weight stage of one CTA
   int resident;          // the weights of a column tile stay in shared memory
   int packed, tiles_base, tiles_cond;   // ... as tiles of consecutive K elements of W_base and of W_cond, three to a barrier
-  int tiles_first;       // W_cond's tiles come in this order; so many serve the first patch of a stride-2 window
-  uint8_t order[kTc4MaxTiles];
   int tiles_m, tiles_n;  // jobs
   int half_job, half_tiles;   // job of a pair that has half of the columns (kNoHalfJob: none), and how many jobs are halved
   int split;             // 1, 2, 4 or 8

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from oracle import oracle as O
+from paper_1805_12549_b200 import binding as B
 from tests import cases as K
 
 pytestmark = pytest.mark.gpu
@@ -225,6 +226,29 @@ def test_k_loops_of_pairs(s, patch, weights, why, how):
                          ids=["one chunk", "two base slices", "one base slice", "a base chunk"])
 def test_int8_stride_2_windows(s):
     _run(K.make_int8_case("wini8s2", s, density=0.3))
+
+
+STRIDE_2 = [k for k in K_LOOPS if k[0].stride == 2 and k[0].h > 4]
+
+
+@pytest.mark.parametrize("s", [k[0] for k in STRIDE_2], ids=[k[3] for k in STRIDE_2])
+def test_a_stride_2_layer_sums_as_every_other_pixel_of_the_dense_one(s):
+    """The same taps in the same order, whatever copies bring the pixels: bit for bit, gates included."""
+    import torch
+    c = K.make_float_case("winorder", s, "bf16", density=0.3, calib_images=4)
+    g = K.GpuCase(c, algo=0)
+    y2, mask2, _ = g.run()
+    dense = B.GatedConv(s.n, s.h, s.w, s.c_in, s.c_out, groups=s.groups, dtype=B.CG_BF16)
+    assert dense.kernel_id == WINDOW and "over 1 CTA(s)" in dense.plan and "over 1 CTA(s)" in g.conv.plan
+    y1, mask1 = dense.alloc_outputs()
+    dense.forward(g.x, g.wb, g.wc, g.bn, g.delta, y1, mask1)
+    torch.cuda.synchronize()
+    y1 = y1[:, ::2, ::2].float().cpu().numpy()
+    mask1 = mask1.view(s.n, s.h, s.w, s.words)[:, ::2, ::2].cpu().numpy().view(np.uint32)
+    np.testing.assert_array_equal(mask2, mask1.reshape(-1, s.words))
+    np.testing.assert_array_equal(y2, y1)
+    dense.close()
+    g.close()
 
 
 # Layers of few jobs, on either side of each line between K loops shared by a cluster and CTA pairs.
