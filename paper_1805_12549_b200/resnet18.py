@@ -218,18 +218,28 @@ class Instance:
         self.stem_ws = torch.empty(B.cg_stem_workspace_bytes(), dtype=torch.uint8, device="cuda")
         self.convs, self.out, self.mask = {}, {}, {}
         # large batches: the 1x1 stride-2 shortcuts read every other pixel of their block's input themselves (a launch less
-        # each, and the input not written and read again)
-        self.strided = {}
-        if net.algo == B.CG_ALGO_AUTO and B.cg_stem_pool_pays(n, net.image, net.image):
-            self.strided = {short.name: (c1.h, st) for short, c1, _, st in net.blocks if short is not None and st != 1}
+        # each, and the input not written and read again), where the layer gets the window kernel: no other kernel on tensor
+        # cores has a stride for 1x1 layers, and whether that one runs it depends on the conditional path's mode
+        large = net.algo == B.CG_ALGO_AUTO and B.cg_stem_pool_pays(n, net.image, net.image)
+        wanted = {short.name: (c1.h, st) for short, c1, _, st in net.blocks if large and short is not None and st != 1}
+        self.strided = set()
         for s in net.specs:
             algo = net.algo
             if s.c_out % 32 or s.c_in % 64:
                 algo = B.CG_ALGO_AUTO
-            h, stride = self.strided.get(s.name, (s.h, s.stride))
-            conv = B.GatedConv(n, h, h, s.c_in, s.c_out, k=s.k, stride=stride, pad=s.pad,
-                               groups=s.groups, dtype=B.CG_BF16, relu=s.relu, has_residual=s.has_residual,
-                               algo=algo, cond_mode=net.cond_mode)
+
+            def handle(h, stride):
+                return B.GatedConv(n, h, h, s.c_in, s.c_out, k=s.k, stride=stride, pad=s.pad,
+                                   groups=s.groups, dtype=B.CG_BF16, relu=s.relu, has_residual=s.has_residual,
+                                   algo=algo, cond_mode=net.cond_mode)
+
+            conv = handle(*wanted[s.name]) if s.name in wanted else None
+            if conv is not None and conv.kernel_id == B.CG_KERNEL_TENSOR_WINDOW:
+                self.strided.add(s.name)
+            else:
+                if conv is not None:
+                    conv.close()
+                conv = handle(s.h, s.stride)
             self.convs[s.name] = conv
             y, mask = conv.alloc_outputs()
             self.out[s.name] = y

@@ -152,6 +152,31 @@ def test_every_layer_matches_the_oracle_on_two_images(network):
     inst.close()
 
 
+@pytest.mark.parametrize("cond_mode", [0, 1, 2, 3], ids=["auto", "dense", "skip tiles", "compact"])
+def test_shortcuts_of_a_large_batch_stay_on_tensor_cores(cond_mode):
+    """Whatever the conditional path's mode; where their handles read every other pixel themselves, the result is that
+    of the subsampled input, bit for bit."""
+    import torch
+    from paper_1805_12549_b200 import binding as B, resnet18 as R
+    net = R.CgResNet18(image=64, cond_mode=cond_mode)
+    x = R.synthetic_images("test_shortcuts", 24, 64)
+    net.calibrate(x[:2].contiguous(), 0.3)
+    inst = net.instance(24)
+    assert len(inst.strided) == (3 if cond_mode < 2 else 0)
+    record = []
+    inst.forward(x, record=record)
+    for s, xin, _, y, _ in record:
+        if not s.name.endswith("shortcut"):
+            continue
+        assert inst.convs[s.name].uses_tensor_cores, (s.name, inst.convs[s.name].plan)
+        alone = B.GatedConv(24, s.h, s.h, s.c_in, s.c_out, k=1, pad=0, groups=1, relu=s.relu, cond_mode=cond_mode)
+        out, _ = alone.alloc_outputs()
+        alone.forward(xin, s.wb, None, s.bn, s.delta, out)
+        assert torch.equal(out, y), s.name
+        alone.close()
+    inst.close()
+
+
 def test_flop_reduction_and_density_one_twin(network):
     import torch
     net, x, tau = network
