@@ -246,7 +246,11 @@ class Instance:
             self.mask[s.name] = mask if s.gated else None
         hp = (net.stem_hw + 2 - 3) // 2 + 1
         self.pooled = torch.empty((n, hp, hp, 64), **bf)
+        # every stride-th pixel of a block's input, where the shortcut's handle takes that (else for who looks at its input)
         self._sub = {}
+        for short, _, _, st in net.blocks:
+            if short is not None and st != 1 and short.name not in self.strided:
+                self._sub_buffer(short)
         self.avg = torch.empty((n, 1, 1, net.fc.c_in), **bf)
         self.launches = None
         self.stem_pools = self.convs["stem"].uses_tensor_cores and B.cg_stem_pool_pays(n, net.image, net.image)
@@ -259,11 +263,14 @@ class Instance:
             self._patches = torch.empty((self.n, hw, hw, STEM_KPAD), dtype=torch.bfloat16, device="cuda")
         return self._patches
 
-    def _subsampled(self, short, x, stride):
-        """Every stride-th pixel of a block's input, where a shortcut (or who looks at its input) takes that."""
+    def _sub_buffer(self, short):
         if short.name not in self._sub:
             self._sub[short.name] = torch.empty((self.n, short.h, short.h, short.c_in), dtype=torch.bfloat16, device="cuda")
-        B.cg_subsample_bf16(x, self._sub[short.name], stride)
+        return self._sub[short.name]
+
+    def _subsampled(self, short, x, stride):
+        """Every stride-th pixel of a block's input, where a shortcut (or who looks at its input) takes that."""
+        B.cg_subsample_bf16(x, self._sub_buffer(short), stride)
         return self._sub[short.name]
 
     def _fused_stem(self, x):

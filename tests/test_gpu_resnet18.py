@@ -177,6 +177,22 @@ def test_shortcuts_of_a_large_batch_stay_on_tensor_cores(cond_mode):
     inst.close()
 
 
+@pytest.mark.parametrize("n", [1, 24])
+def test_a_pass_allocates_nothing(n):
+    import torch
+    from paper_1805_12549_b200 import resnet18 as R
+    net = R.CgResNet18(image=64)
+    x = R.synthetic_images("test_alloc", n, 64)
+    inst = net.instance(n)
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_stats()["allocation.all.allocated"]
+    inst.forward(x)
+    inst.forward(x)
+    torch.cuda.synchronize()
+    assert torch.cuda.memory_stats()["allocation.all.allocated"] == before
+    inst.close()
+
+
 def test_flop_reduction_and_density_one_twin(network):
     import torch
     net, x, tau = network
