@@ -262,10 +262,12 @@ TapBox tap_box(const LayerDims& L) {
   return b;
 }
 
+// (Ordinary loads, and no __restrict__ on what they read: the kernel in front, whose end this one's launch does not wait for,
+// may still be writing it.)
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
-template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
 template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
-  const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+  const uint2 v = *reinterpret_cast<const uint2*>(p);
   return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
                      __uint_as_float(v.y & 0xffff0000u));
 }
@@ -291,8 +293,8 @@ struct DirectTile {
 // BOX: the taps of tap_box() only (an instance of its own: the index arithmetic of its weights costs the others 4 %)
 template <typename T, int NTH, int TC, int PXT, int CH, bool BOX>
 __global__ void __launch_bounds__(NTH, PXT == 4 ? 2 : 3)
-direct_tile_kernel(LayerDims L, const T* __restrict__ x, const T* __restrict__ w_base, const T* __restrict__ w_cond,
-                   cg_bn_params bn, const float* __restrict__ delta, const T* __restrict__ residual, T* __restrict__ y,
+direct_tile_kernel(LayerDims L, const T* x, const T* w_base, const T* w_cond,
+                   cg_bn_params bn, const float* delta, const T* residual, T* __restrict__ y,
                    uint32_t* __restrict__ mask, float* __restrict__ p_out, int base_only,
                    unsigned long long* __restrict__ counters, FastDiv div_base, FastDiv div_cond, FastDiv div_kw, TapBox box, uint64_t minus_zero) {
   using D = DirectTile<NTH, TC, PXT, CH>;

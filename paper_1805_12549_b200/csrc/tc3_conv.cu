@@ -227,7 +227,7 @@ tc3_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
       const int tap = 3 * r + (n >> 6), c = n & 63, ch = p * 8;
       const __nv_bfloat16* src = ch < L.c_p ? prm.w_base + ((size_t)c * 9 + tap) * L.c_p + ch
                                             : prm.w_cond + ((size_t)c * 9 + tap) * L.c_r + (ch - L.c_p);
-      v[k] = __ldg((const uint4*)src);
+      v[k] = ptx::ld_global_16(src);
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -401,7 +401,7 @@ tc3_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
       const bool has_res = prm.residual != nullptr && valid;
       if (has_res) {
         const uint4* rp = (const uint4*)(prm.residual + m * 64 + cb);
-        res[0] = __ldg(rp); res[1] = __ldg(rp + 1);
+        res[0] = ptx::ld_global_16(rp); res[1] = ptx::ld_global_16(rp + 1);   // (the kernel in front may have written them)
       }
       ok = wait3(sh, prm.counters, &sh->rawp_full, j & 1, 7);
       if (!ok) break;

@@ -93,6 +93,36 @@ def test_maxpool_over_filters_and_sizes(k, stride, pad, n, h, w, c):
     assert bool((buf[:64] == 7).all()) and bool((buf[-64:] == 7).all())
 
 
+@pytest.mark.parametrize("algo,h", [(0, 32), (5, 28), (1, 28)], ids=["tap-stacked", "tap-stacked, edges exchanged", "direct"])
+def test_a_layer_reads_what_the_operator_in_front_of_it_wrote(algo, h):
+    """Operators and layers are dependent launches: a layer's blocks are there while the pooling in front of it still writes
+    its input and residual.  The same buffers with other values each time, nothing waited for in between."""
+    import torch
+    from paper_1805_12549_b200 import binding as B
+    n, c = 24, 64
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    images = [torch.randn((n, 2 * h, 2 * h, c), device="cuda", generator=gen).bfloat16() for _ in range(6)]
+    wb = (torch.randn((c, 3, 3, c // 4), device="cuda", generator=gen) * 0.06).bfloat16()
+    wc = (torch.randn((c, 3, 3, c - c // 4), device="cuda", generator=gen) * 0.06).bfloat16()
+    one, zero = torch.ones(c, device="cuda"), torch.zeros(c, device="cuda")
+    bn = B.make_bn(dict(gamma=one, beta=zero, mean_base=zero, var_base=one, mean_full=zero, var_full=one))
+    conv = B.GatedConv(n, h, h, c, c, algo=algo, has_residual=True)
+    assert conv.kernel_id == (0 if algo == 1 else 3), conv.plan
+    pooled = torch.empty((n, h, h, c), dtype=torch.bfloat16, device="cuda")
+    outs = {wait: [conv.alloc_outputs() for _ in images] for wait in (False, True)}
+    for wait in (False, True):
+        torch.cuda.synchronize()
+        for x, (y, mask) in zip(images, outs[wait]):
+            B.cg_maxpool_bf16(x, pooled, 3, 2, 1)
+            if wait:
+                torch.cuda.synchronize()
+            conv.forward(pooled, wb, wc, bn, one, y, mask, pooled)
+    torch.cuda.synchronize()
+    for (y, mask), (u, v) in zip(outs[False], outs[True]):
+        assert torch.equal(y, u) and torch.equal(mask, v)
+    conv.close()
+
+
 @pytest.fixture(scope="module")
 def network():
     import torch
