@@ -1076,13 +1076,10 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
   if (shut) {
     if constexpr (PAIR) {
-      // the base rows move together; another row may now be the last of its patch
+      // the base rows move together
       const int i = (int)threadIdx.x;
-      if (i < P.rows && ((P.base_mask >> i) & 1ull)) {
-        uint4 row = ((const uint4*)P.row)[i];
-        row.w = (row.w & ~(uint32_t)kRowAFree) | ((row.w & kRowAFreeBase) ? (uint32_t)kRowAFree : 0u);
-        ((uint4*)(smem + kOffRows))[__popcll(P.base_mask & ((1ull << i) - 1ull))] = row;
-      }
+      if (i < P.rows && ((P.base_mask >> i) & 1ull))
+        ((uint4*)(smem + kOffRows))[__popcll(P.base_mask & ((1ull << i) - 1ull))] = ((const uint4*)P.row)[i];
       __syncthreads();
       run_roles<NT, I8, PAIR, HALF, true>(map_x, maps, prm, smem, warp, lane, part, tile_n, group, groups, jobs, tmem);
     }
@@ -1258,13 +1255,9 @@ void flag_rows(RawRow* st, int lo, int hi, int* a_count, int* b_count) {
 }
 
 // The base rows of a pair's jobs, as the jobs of a column tile whose gates cannot fire run them.
-void plan_base(RawRow* raw, Tc4Plan* P) {
+void plan_base(const RawRow* raw, Tc4Plan* P) {
   for (int i = 0; i < P->rows; ++i) {
-    Tc4Row& r = raw[i].r;
-    if (r.flags & kRowCond) continue;
-    int k = i + 1;
-    while (k < P->rows && (raw[k].r.flags & kRowCond)) ++k;
-    if (k == P->rows || raw[k].a_key != raw[i].a_key) r.flags |= kRowAFreeBase;
+    if (raw[i].r.flags & kRowCond) continue;
     P->base_mask |= 1ull << i;
     ++P->base_rows;
   }

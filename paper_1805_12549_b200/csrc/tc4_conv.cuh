@@ -26,13 +26,13 @@ struct alignas(16) Tc4Row {
 static_assert(sizeof(Tc4Row) == 16, "row table");
 
 enum : uint8_t {
+  // (the producers read kRowANew, kRowBNew and kRowCond; the others are for the issuer of a cluster's CTA: a pair's has no table)
   kRowR = 1,        // accumulates into R (else P)
   kRowInit = 2,     // first row into its accumulator: overwrites it
   kRowANew = 4, kRowAFree = 8,     // takes the next patch slot / is the last to read its slot
   kRowBNew = 16, kRowBFree = 32,   // the same for the weight stage
   kKindTaps = 64,   // (in `kind`) the first taps of the base path of a window, several per weight tile
-  kRowCond = 64,    // the weights come from W_cond (else W_base)
-  kRowAFreeBase = 128              // kRowAFree of a job that runs the base rows only
+  kRowCond = 64     // the weights come from W_cond (else W_base)
 };
 
 enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2, kTc4Window2 = 3 };
