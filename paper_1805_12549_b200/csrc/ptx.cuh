@@ -539,9 +539,6 @@ __device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, ui
                "r"(bytes), "r"(bar)
                : "memory");
 }
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// Waits until this thread's copies have read their source.
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t ld_cluster_4(uint32_t addr, uint32_t rank) {
   uint32_t v;

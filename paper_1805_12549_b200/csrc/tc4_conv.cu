@@ -920,7 +920,6 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
           ptx::bulk_copy_cluster(ptx::map_cluster(ptx::smem_u32(smem) + P.off_sums + (uint32_t)slot * block, (uint32_t)to),
                                  ptx::smem_u32(smem) + kOffStages + (uint32_t)lane * 128u * kSumPitch + (uint32_t)to * block, block,
                                  ptx::map_cluster(ptx::smem_u32(&sh->sums), (uint32_t)to));
-          ptx::bulk_commit();
         }
       }
       __syncwarp();
@@ -993,7 +992,6 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
           if (prm.mask) prm.mask[(long long)t.m * L.words + (ch >> 5)] = w;
         }
       }
-      if (warp - kEpiWarp0 < P.split) ptx::bulk_wait_read();   // (the copies have left this CTA's shared memory)
     }
     active = __reduce_add_sync(0xffffffffu, active);
     rows_active = __reduce_add_sync(0xffffffffu, rows_active);
@@ -1097,8 +1095,9 @@ tc4_gated_conv_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
   __syncwarp();
   ptx::tc_fence_before();
-  // No CTA leaves while a peer may still use its shared memory or TMEM.  (A CTA has waited for all that is sent to it and that
-  // it sends, and its stores to global memory need not be waited for.)
+  // No CTA leaves while a peer may still use its shared memory or TMEM.  (Every CTA has waited on its barrier `sums` for all
+  // that is sent to it before it arrives here, so what a CTA sends has left its shared memory once all have arrived; stores to
+  // global memory need not be waited for.  Where a CTA gave up waiting, the copies have the drain time above.)
   ptx::cluster_sync_relaxed();
   ptx::tc_fence_after();
   if (threadIdx.x == 0 && !*(volatile uint32_t*)&sh->abort_flag) {
