@@ -200,13 +200,14 @@ __global__ void __launch_bounds__(kAvgBlock) avgpool_kernel(const uint4* x, uint
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    for (int p = 0; p < hw; p += kAvgLoads) {
+    const unsigned pixels = (unsigned)hw;                        // (p runs up to seven past them)
+    for (unsigned p = 0; p < pixels; p += kAvgLoads) {
       uint4 t[kAvgLoads];
 #pragma unroll
-      for (int k = 0; k < kAvgLoads; ++k) t[k] = p + k < hw ? src[(long long)(p + k) * cv] : make_uint4(0u, 0u, 0u, 0u);
+      for (int k = 0; k < kAvgLoads; ++k) t[k] = p + k < pixels ? src[(long long)(p + k) * cv] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
       for (int k = 0; k < kAvgLoads; ++k) {
-        if (p + k >= hw) break;
+        if (p + k >= pixels) break;
         const __nv_bfloat16* tb = reinterpret_cast<const __nv_bfloat16*>(&t[k]);
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[e] += __bfloat162float(tb[e]);
