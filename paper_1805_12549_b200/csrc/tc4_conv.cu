@@ -1478,23 +1478,31 @@ int launch_tc4(const LayerDims& L, const Tc4Plan& P, Tc4Maps* maps, const void* 
                uint32_t* mask, unsigned long long* counters, cudaStream_t stream) {
   if (!P.valid) return (int)cudaErrorInvalidValue;
   Tc4MapSet* ms = nullptr;
+  const Tc4MapSet* same_weights = nullptr;                     // (x alone is new: the weights' maps, up to four, are there)
   for (int i = 0; i < Tc4Maps::kEntries; ++i) {
     Tc4MapSet* c = &maps->set[i];
-    if (c->key[0] == x && c->key[1] == w_base && c->key[2] == w_cond) { ms = c; break; }
+    if (!c->key[0] || c->key[1] != w_base || c->key[2] != w_cond) continue;
+    same_weights = c;
+    if (c->key[0] == x) { ms = c; break; }
   }
   if (!ms) {
     ms = &maps->set[maps->next];
     maps->next = (maps->next + 1) % Tc4Maps::kEntries;
     ms->key[0] = nullptr;
-    const int taps = L.kh * L.kw;
     if (!encode_x(&ms->x, x, L, P)) return (int)cudaErrorInvalidValue;
-    const int blocks = P.pair ? P.nt / 64 : P.nt / 32;
-    const bool halves = P.half_job < kNoHalfJob;
-    if (!encode_w(&ms->wb, w_base, P, L.c_out, taps * L.c_p, blocks)) return (int)cudaErrorInvalidValue;
-    ms->wc = ms->half_wb = ms->half_wc = ms->wb;
-    if (L.c_r > 0 && !encode_w(&ms->wc, w_cond, P, L.c_out, taps * L.c_r, blocks)) return (int)cudaErrorInvalidValue;
-    if (halves && !encode_w(&ms->half_wb, w_base, P, L.c_out, taps * L.c_p, blocks / 2)) return (int)cudaErrorInvalidValue;
-    if (halves && L.c_r > 0 && !encode_w(&ms->half_wc, w_cond, P, L.c_out, taps * L.c_r, blocks / 2)) return (int)cudaErrorInvalidValue;
+    if (same_weights) {
+      ms->wb = same_weights->wb; ms->wc = same_weights->wc;
+      ms->half_wb = same_weights->half_wb; ms->half_wc = same_weights->half_wc;
+    } else {
+      const int taps = L.kh * L.kw;
+      const int blocks = P.pair ? P.nt / 64 : P.nt / 32;
+      const bool halves = P.half_job < kNoHalfJob;
+      if (!encode_w(&ms->wb, w_base, P, L.c_out, taps * L.c_p, blocks)) return (int)cudaErrorInvalidValue;
+      ms->wc = ms->half_wb = ms->half_wc = ms->wb;
+      if (L.c_r > 0 && !encode_w(&ms->wc, w_cond, P, L.c_out, taps * L.c_r, blocks)) return (int)cudaErrorInvalidValue;
+      if (halves && !encode_w(&ms->half_wb, w_base, P, L.c_out, taps * L.c_p, blocks / 2)) return (int)cudaErrorInvalidValue;
+      if (halves && L.c_r > 0 && !encode_w(&ms->half_wc, w_cond, P, L.c_out, taps * L.c_r, blocks / 2)) return (int)cudaErrorInvalidValue;
+    }
     ms->key[0] = x; ms->key[1] = w_base; ms->key[2] = w_cond;
   }
   Tc4Params prm;

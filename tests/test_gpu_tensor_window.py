@@ -228,6 +228,27 @@ def test_int8_stride_2_windows(s):
     _run(K.make_int8_case("wini8s2", s, density=0.3))
 
 
+def test_new_inputs_and_new_weights_of_one_handle():
+    """More pointers than a handle keeps tensor maps of, in an order in which the input, the weights or both are new."""
+    import torch
+    c = K.make_float_case("winmaps", O.Shape(28, 28, 28, 128, 128, groups=4), "bf16", density=0.3, calib_images=1)
+    g = K.GpuCase(c, algo=0)
+    assert "halves" in g.conv.plan
+    xs = [g.x.roll(i, 0) for i in range(6)]
+    weights = [(g.wb, g.wc), (g.wb.flip(0), g.wc.flip(0)), (g.wb, g.wc.flip(0))]
+    order = [(i, j) for j in (0, 1, 2, 0) for i in range(6)] + [(i % 6, i % 3) for i in range(12)]
+    first = {}
+    for i, j in order:
+        g.conv.forward(xs[i], *weights[j], g.bn, g.delta, g.y, g.mask)
+        if (i, j) not in first:
+            fresh = K.GpuCase(c, algo=0)
+            fresh.conv.forward(xs[i], *weights[j], g.bn, g.delta, fresh.y, fresh.mask)
+            first[i, j] = fresh.y.clone(), fresh.mask.clone()
+            fresh.close()
+        assert torch.equal(g.y, first[i, j][0]) and torch.equal(g.mask, first[i, j][1]), (i, j)
+    g.close()
+
+
 STRIDE_2 = [k for k in K_LOOPS if k[0].stride == 2 and k[0].h > 4]
 
 
