@@ -29,6 +29,7 @@ struct cg_conv_s {
   int use_tc4;                    // window tensor-core kernel (tc4_conv.cu)
   cg::Tc4Plan plan4;
   cg::Tc4Maps maps4;
+  cg::StemPoolPlan stem_pool;     // of cg_stem_pool_forward's last extents
 };
 
 namespace {
@@ -145,6 +146,7 @@ cg_status cg_conv_create(cg_conv_t* out, const cg_conv_desc* desc) {
   std::memset(&h->maps2, 0, sizeof(h->maps2));
   std::memset(&h->maps3, 0, sizeof(h->maps3));
   std::memset(&h->maps4, 0, sizeof(h->maps4));
+  std::memset(&h->stem_pool, 0, sizeof(h->stem_pool));
   // (which kernels apply is decided before the device is needed, so that an ineligible layer is
   // reported as such on any machine)
   const bool have_device = cudaGetDevice(&h->device) == cudaSuccess;
@@ -337,7 +339,7 @@ cg_status cg_stem_pool_forward(cg_conv_t h, const void* x, int n, int image_h, i
   const cg_status st = check_stem(h, x, n, image_h, image_w, c, w_base, bn, delta, y, pooled);
   if (st != CG_OK) return st;
   const cg::LayerDims& L = h->L;
-  const int err = cg::launch_stem_pool(x, n, image_h, image_w, w_base, L.c_in, *bn, delta, L.eps, L.relu, y, pooled,
+  const int err = cg::launch_stem_pool(&h->stem_pool, x, n, image_h, image_w, w_base, L.c_in, *bn, delta, L.eps, L.relu, y, pooled,
                                        h->counters, reinterpret_cast<cudaStream_t>(cuda_stream));
   return err == 0 ? CG_OK : CG_ERR_CUDA;
 }

@@ -13,9 +13,14 @@ int launch_stem(const void* x, int n, int h, int w, const void* w_base, int k_pa
                 const float* delta, float eps, int relu, void* y, void* ws, unsigned long long* counters,
                 cudaStream_t stream);
 
+// How launch_stem_pool cuts n images into strips: worked out by its first call for these extents, kept by the handle.
+struct StemPoolPlan {
+  int n, h, w;             // 0: none yet
+  int sms, segs, per;      // a column of an image in `segs` strips of `per` pooled rows
+};
 // The stem and the 3x3 stride-2 max pooling behind it in one launch (stem_pool.cu): y as above, pooled [n,hp,wp,64].
 // Even image widths only.
-int launch_stem_pool(const void* x, int n, int h, int w, const void* w_base, int k_pad, const cg_bn_params& bn,
+int launch_stem_pool(StemPoolPlan* plan, const void* x, int n, int h, int w, const void* w_base, int k_pad, const cg_bn_params& bn,
                      const float* delta, float eps, int relu, void* y, void* pooled, unsigned long long* counters,
                      cudaStream_t stream);
 // Whether that is faster than launch_stem and a pooling kernel.

@@ -447,13 +447,15 @@ __global__ void __launch_bounds__(kThreads, 1) stem_pool_kernel(const __grid_con
 }
 
 // Strips of an image: as many segments as make the longest CTA shortest (every segment repeats one unit and fills a ring).
-void split_strips(long long columns, int hp, int sms, StemPoolParams* P) {
+// More than 1024 of them, seven to an SM, are not looked at.
+void split_strips(long long columns, int hp, StemPoolPlan* plan) {
   double best = 0.0;
-  for (int s = 1; s <= hp; ++s) {
+  plan->per = 0;
+  for (int s = 1; s <= hp && s <= 1024; ++s) {
     const int per = (hp + s - 1) / s, segs = (hp + per - 1) / per;
     const long long items = (columns * segs + 1) / 2;
-    const double cost = (double)((items + sms - 1) / sms) * (per + 1.7);
-    if (P->per == 0 || cost < best) { best = cost; P->per = per; P->segs = segs; }
+    const double cost = (double)((items + plan->sms - 1) / plan->sms) * (per + 1.7);
+    if (plan->per == 0 || cost < best) { best = cost; plan->per = per; plan->segs = segs; }
   }
 }
 
@@ -469,12 +471,11 @@ bool stem_pool_pays(int n, int h, int w) {
   return n * ho >= 148 * 4 && 4 * wo >= 2 * kCols * cols;
 }
 
-int launch_stem_pool(const void* x, int n, int h, int w, const void* w_base, int k_pad, const cg_bn_params& bn,
+int launch_stem_pool(StemPoolPlan* plan, const void* x, int n, int h, int w, const void* w_base, int k_pad, const cg_bn_params& bn,
                      const float* delta, float eps, int relu, void* y, void* pooled, unsigned long long* counters,
                      cudaStream_t stream) {
-  int dev = 0, sms = 0;
+  int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 148;
   StemPoolParams P;
   std::memset(&P, 0, sizeof(P));
   P.x = static_cast<const uint32_t*>(x); P.w = static_cast<const __nv_bfloat16*>(w_base);
@@ -483,7 +484,13 @@ int launch_stem_pool(const void* x, int n, int h, int w, const void* w_base, int
   P.h = h; P.w2 = w / 2 * 3; P.ho = (h - 1) / 2 + 1; P.wo = (w - 1) / 2 + 1;
   P.hp = (P.ho - 1) / 2 + 1; P.wp = (P.wo - 1) / 2 + 1;
   P.col_tiles = (P.wp + kCols - 1) / kCols;
-  split_strips((long long)n * P.col_tiles, P.hp, sms, &P);
+  if (plan->n != n || plan->h != h || plan->w != w) {
+    if (cudaDeviceGetAttribute(&plan->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || plan->sms <= 0) plan->sms = 148;
+    split_strips((long long)n * P.col_tiles, P.hp, plan);
+    plan->n = n; plan->h = h; plan->w = w;
+  }
+  const int sms = plan->sms;
+  P.segs = plan->segs; P.per = plan->per;
   const long long strips = (long long)n * P.col_tiles * P.segs;
   if (w % 2 || strips > 0x3fffffffll) return (int)cudaErrorInvalidValue;
   P.strips = (int)strips;
