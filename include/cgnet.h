@@ -41,7 +41,7 @@ cg_status cg_stem_forward(cg_conv_t h, const void* x, int n, int image_h, int im
                           const cg_bn_params* bn, const float* delta, void* y, void* workspace, void* cuda_stream);
 
 /* cg_stem_forward and cg_maxpool_bf16 (k = 3, stride 2, pad 1) behind it in one kernel: y as there, pooled
- * [n,(h' - 1)/2 + 1,(w' - 1)/2 + 1,64].  Even image widths (else CG_ERR_INVALID_ARG); no workspace.
+ * [n,(h' - 1)/2 + 1,(w' - 1)/2 + 1,64].  Even image widths, extents up to 2^30 (else CG_ERR_INVALID_ARG); no workspace.
  * cg_stem_pool_pays: 1 where it is the faster way for n images of these extents, else 0. */
 int cg_stem_pool_pays(int n, int image_h, int image_w);
 cg_status cg_stem_pool_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,

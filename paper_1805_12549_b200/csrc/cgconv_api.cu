@@ -335,7 +335,7 @@ int cg_stem_pool_pays(int n, int image_h, int image_w) {
 
 cg_status cg_stem_pool_forward(cg_conv_t h, const void* x, int n, int image_h, int image_w, int c, const void* w_base,
                                const cg_bn_params* bn, const float* delta, void* y, void* pooled, void* cuda_stream) {
-  if (!pooled || (image_w & 1)) return CG_ERR_INVALID_ARG;
+  if (!pooled || (image_w & 1) || image_w > cg::kStemPoolMaxExtent || image_h > cg::kStemPoolMaxExtent) return CG_ERR_INVALID_ARG;
   const cg_status st = check_stem(h, x, n, image_h, image_w, c, w_base, bn, delta, y, pooled);
   if (st != CG_OK) return st;
   const cg::LayerDims& L = h->L;

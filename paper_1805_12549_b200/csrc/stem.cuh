@@ -19,7 +19,8 @@ struct StemPoolPlan {
   int sms, segs, per;      // a column of an image in `segs` strips of `per` pooled rows
 };
 // The stem and the 3x3 stride-2 max pooling behind it in one launch (stem_pool.cu): y as above, pooled [n,hp,wp,64].
-// Even image widths only.
+// Even image widths only, extents up to kStemPoolMaxExtent (words of an image row are counted in 32 bits).
+constexpr int kStemPoolMaxExtent = 1 << 30;
 int launch_stem_pool(StemPoolPlan* plan, const void* x, int n, int h, int w, const void* w_base, int k_pad, const cg_bn_params& bn,
                      const float* delta, float eps, int relu, void* y, void* pooled, unsigned long long* counters,
                      cudaStream_t stream);
