@@ -272,6 +272,31 @@ def test_a_stride_2_layer_sums_as_every_other_pixel_of_the_dense_one(s):
     g.close()
 
 
+# int8 jobs of 128 columns, with gates that fire: what the plan says of patches, weights and the last round.
+INT8_K_LOOPS = [
+    (O.Shape(60, 14, 14, 256, 256, groups=4), "one patch for all taps", "packed", True, "two base slices"),
+    (O.Shape(48, 14, 14, 256, 256, groups=8), "one patch for all taps", "packed", True, "one base slice"),
+    (O.Shape(60, 14, 14, 256, 256, groups=2), "one patch for all taps", "resident", True, "a base chunk"),
+    (O.Shape(64, 7, 7, 512, 512, groups=4), "one patch for all taps", "streamed", False, "a base chunk, streamed"),
+    (O.Shape(96, 14, 14, 256, 512, stride=2, groups=4), "four patches", "packed", True, "stride 2, two base slices"),
+    (O.Shape(96, 14, 14, 256, 512, stride=2, groups=8), "four patches", "packed", True, "stride 2, one base slice"),
+    (O.Shape(96, 14, 14, 256, 512, stride=2, groups=2), "four patches", "resident", True, "stride 2, a base chunk"),
+    (O.Shape(40, 28, 28, 256, 512, stride=2, groups=4), "four patches", "packed", False, "stride 2, whole rounds"),
+    (O.Shape(96, 14, 14, 512, 512, stride=2, groups=4), "four patches", "streamed", True, "stride 2, streamed"),
+]
+
+
+@pytest.mark.parametrize("s,patch,weights,halves,why", INT8_K_LOOPS, ids=[k[4] for k in INT8_K_LOOPS])
+def test_int8_jobs_of_128_columns(s, patch, weights, halves, why):
+    c = K.make_int8_case("wini8k", s, density=0.3)
+    g = K.GpuCase(c, algo=0)
+    plan = g.conv.plan
+    g.close()
+    assert "channel tiles of 128" in plan and patch in plan and weights in plan and ("halves" in plan) == halves, plan
+    _, st, _ = _run(c)
+    assert 0.2 < st.active / st.outputs < 0.4
+
+
 # Layers of few jobs, on either side of each line between K loops shared by a cluster and CTA pairs.
 FEW_JOBS = [
     (O.Shape(2, 5, 5, 64, 64, groups=4), False, 4, "36 MMAs, one job"),
