@@ -248,7 +248,8 @@ int cg_conv_plan_string(cg_conv_t h, char* buf, size_t len) {
                          "window tcgen05: %d pixel tiles of %d x %d channel tiles of %d, %s, K loop of %d rows over %d CTA(s), %s "
                          "weights (%d stages), %d patch slots of %d bytes, grid %d%s",
                          P.tiles_m, P.pair ? 256 : 128, P.tiles_n, P.nt,
-                         P.mode == cg::kTc4Window ? "one patch for all taps" : P.mode == cg::kTc4Window2 ? "two of the four patches of a stride-2 lattice per filter row"
+                         P.mode == cg::kTc4Window ? "one patch for all taps" : P.mode == cg::kTc4Lattice ? "four patches of a stride-2 lattice"
+                         : P.mode == cg::kTc4Rows2 ? "two of the four patches of a stride-2 lattice per filter row"
                          : P.mode == cg::kTc4Taps ? "one patch per tap" : "1x1",
                          P.rows, P.split, P.packed ? "packed" : P.resident ? "resident" : "streamed", P.nb, P.na, P.slot_bytes,
                          P.grid, P.half_job < cg::kNoHalfJob ? ", last round in halves" : "");

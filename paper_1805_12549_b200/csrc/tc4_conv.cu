@@ -10,11 +10,12 @@
 //       its filter tap (r, s) is the position r*(w+1) + s further on: a patch of 128 + 2*(w+2) positions
 //       serves all nine taps, each as another start row of the same shared-memory operand.  Positions in the
 //       padding are computed and dropped: (w/(w+1))*(h/(h+1)) of the rows are pixels, whatever the image size.
-//   stride-2 windows (pairs, even extents)  the pixels of odd or even rows and columns are four lattices, and a filter row
-//       reads two of them: the odd columns serve its first and last tap, one position apart, the even ones its middle tap.
-//       The taps come in the order 0..8, as everywhere: with one patch for all taps of a lattice (four to a chunk for six) they
-//       came as 0 2 6 8 1 7 3 5 4, and a gate whose partial sum lies within an fp32 rounding of its threshold could decide
-//       otherwise than in the same layer tap by tap.
+//   stride-2 windows (pairs, even extents)  the pixels of odd or even rows and columns are four lattices of pitch
+//       w' + 1 and h' + 1, and a window over each serves four, two, two or one of the taps.  The taps come in the order 0..8 all
+//       the same, so that all four patches of a chunk are there at a time: in the order 0 2 6 8 1 7 3 5 4, which needs one, a
+//       gate whose partial sum lies within an fp32 rounding of its threshold could decide otherwise than tap by tap.  (int8 sums
+//       have no rounding: they take that order where the weights leave no room.)  bf16 layers whose weights leave no room have a
+//       patch per filter row: of its two lattices the odd columns serve the first and last tap, the even ones the middle tap.
 //   tap mode (other strides, wide images)  one copy per filter tap and chunk, of 128 output pixels; no row is
 //       dropped.  1x1 layers of any stride: one copy per chunk.
 // The partial sum P and the conditional sum R have separate TMEM accumulators, two (N = 128) or four
@@ -45,8 +46,8 @@
 //
 // Measured (graphs of 20 calls, us; in brackets with two issuers that walked a table, before the steps that the comments
 // below describe): 128@16x16 b256 17.4 (23.0), 256@8x8 b256 20.4 (23.7), 512@4x4 b256 23.8 (27.8), 64@56x56 b64 with residual
-// 22.4 (23.4), b128 39 (43), 128->256 stride 2 at 28x28 b64 12.7 (16.0), int8 128@28x28 b64 15.8 (17.6), 128@28x28 b128 22.8 (30.7),
-// 64->128 stride 2 b128 17.0 (26.4); one image: 64@56x56 7.0 (7.4), 512@7x7 7.7 (8.1).  What bounds it now: 256 and 512
+// 22.4 (23.4), b128 39 (43), 128->256 stride 2 at 28x28 b64 13.6 (16.0), int8 128@28x28 b64 15.8 (17.6), 128@28x28 b128 22.8 (30.7),
+// 64->128 stride 2 b128 18.5 (26.4); one image: 64@56x56 5.9 (7.4), 512@7x7 7.3 (8.1).  What bounds it now: 256 and 512
 // channels their MMAs in whole rounds of jobs (9,000 cycles a job of 256 channels, 9,200 of MMAs); 128 channels the same behind a
 // start of 4,000 cycles and a tail of 4,000; 64 channels operand reads, 2,100 cycles a job of 1,550 of MMAs at 43 each beside
 // the patches' writes to shared memory; int8 its epilogue; one image the chain of first copies (2,500 cycles), MMAs, exchange
@@ -165,8 +166,9 @@ __device__ __forceinline__ void issue_row(int tiles, uint32_t d, uint32_t hi, ui
   }
 }
 
-// From a filter row's first tap to its tap s, in 16-byte units of the patch: `step` each, or, for kTwoPatches (stride-2
-// windows), the odd columns' next position (s = 2) and the patch of the even columns behind them (s = 1).
+// From a filter row's first tap to its tap s, in 16-byte units of the patch: `step` each, or, for kTwoPatches (a patch per
+// filter row at stride 2), the odd columns' next position (s = 2) and the patch of the even columns behind them (s = 1).
+constexpr int kLatticeSlots = 8;                              // patches of a lattice at most, where weights stream
 constexpr int kLatticeRows = 136;                              // positions per patch: 129, in whole swizzle atoms
 constexpr uint32_t kTwoPatches = ~0u;
 __device__ __forceinline__ uint32_t tap_step(uint32_t s, uint32_t step) {
@@ -202,6 +204,33 @@ __device__ __forceinline__ void issue_packed(uint32_t d, uint32_t hi, uint32_t a
       ptx::umma<true, I8>(d, ((uint64_t)hi << 32) | (a + tap_step((uint32_t)t, step) + 2u * (K0 + k)),
                           ((uint64_t)hi << 32) | (b + (uint32_t)(s / 4) * tile + (uint32_t)(s % 4) * 2u), idesc, t == 0 && k == 0 ? acc : 1u);
     }
+}
+
+// Stride-2 windows: patch of tap t (bit 0: even columns, bit 1: even rows), the taps in the order of the sums or (BY_PATCH) by
+// patches, and in which places of that order a patch is taken first and last.
+__host__ __device__ constexpr int lattice_of(int t) { return (t / 3 == 1 ? 2 : 0) + (t % 3 == 1 ? 1 : 0); }
+template <bool BY_PATCH> __host__ __device__ constexpr int lattice_tap(int i) { return BY_PATCH ? (int)((0x453718620ull >> (4 * i)) & 15) : i; }
+template <bool BY_PATCH> __host__ __device__ constexpr bool lattice_first(int i) {
+  for (int k = 0; k < i; ++k)
+    if (lattice_of(lattice_tap<BY_PATCH>(k)) == lattice_of(lattice_tap<BY_PATCH>(i))) return false;
+  return true;
+}
+template <bool BY_PATCH> __host__ __device__ constexpr bool lattice_last(int i) {
+  for (int k = i + 1; k < 9; ++k)
+    if (lattice_of(lattice_tap<BY_PATCH>(k)) == lattice_of(lattice_tap<BY_PATCH>(i))) return false;
+  return true;
+}
+// Tap t of such a patch: NK slices from K0 on.  Its weights: PT slices a tap from FIRST on, packed (PT > 0), or tile t % 3 of a stage.
+template <bool I8, int PT, int FIRST, int K0, int NK>
+__device__ __forceinline__ void issue_lattice_tap(int t, uint32_t d, uint32_t hi, uint32_t a, uint32_t row_lo, uint32_t b, uint32_t tile,
+                                                  uint32_t idesc, uint32_t acc) {
+  const uint32_t a_t = a + (t / 3 == 2 ? row_lo : 0u) + (t % 3 == 2 ? 8u : 0u);
+#pragma unroll
+  for (int k = 0; k < NK; ++k) {
+    const int s = t * PT + FIRST + k;
+    const uint32_t b_t = PT > 0 ? b + (uint32_t)(s / 4) * tile + (uint32_t)(s % 4) * 2u : b + (uint32_t)(t % 3) * tile + 2u * k;
+    ptx::umma<true, I8>(d, ((uint64_t)hi << 32) | (a_t + 2u * (K0 + k)), ((uint64_t)hi << 32) | b_t, idesc, k == 0 ? acc : 1u);
+  }
 }
 
 // One row of the table in shared memory.
@@ -307,8 +336,8 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
   uint32_t idesc = I8 ? ptx::idesc_s8(256, NT) : ptx::idesc_bf16(256, NT);
   const uint32_t hi = (uint32_t)(ptx::smem_desc(0, 1024, 2) >> 32);
   const uint32_t a_size = (uint32_t)P.slot_bytes >> 4, b_size = (uint32_t)P.stage_bytes >> 4;
-  const uint32_t row_lo = kWin ? (uint32_t)P.wp * 8u : 0u;
-  constexpr uint32_t kStep = kWin ? 8u : MODE == kTc4Window2 ? kTwoPatches : 1024u;   // from tap to tap of a filter row
+  const uint32_t row_lo = kWin || MODE == kTc4Lattice ? (uint32_t)P.wp * 8u : 0u;
+  constexpr uint32_t kStep = kWin ? 8u : MODE == kTc4Rows2 ? kTwoPatches : 1024u;   // from tap to tap of a filter row
   const int na = P.na, nb = P.nb;
   const bool resident = P.resident != 0;
   const int ck = I8 ? 128 : 64;
@@ -350,7 +379,44 @@ __device__ __forceinline__ void issue_jobs(const Tc4Params& prm, Shared4* sh, ui
       if (resident) b0 += (uint32_t)(group & 1) * (kTileU / 2u);
     }
     if (resident) { b = IssueRing{0, 0u, b0}; new_b = j == 0; b_seen = false; }
-    if constexpr (MODE == kTc4Window2 && CH > 0) {
+    if constexpr (MODE == kTc4Lattice) {
+      // four patches a chunk; packed weights (CH > 0) or a stage per filter row
+      constexpr bool kByPatch = I8 && CH == 2;
+      constexpr int KB = CH > 0 ? KP : 4, PT = CH > 0 ? 4 * CH - KP : 0;
+      const uint32_t bc = b0 + (uint32_t)P.tiles_base * kTileU;
+      auto chunk = [&](auto second, int q) {
+        constexpr int Q = decltype(second)::value, FIRST = Q ? 4 - KB : 0, K0 = Q ? 0 : KB, NK = Q ? 4 : 4 - KB;
+        uint32_t at[4] = {0u, 0u, 0u, 0u};
+        int slot[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          const int t = lattice_tap<kByPatch>(i), p = lattice_of(t);
+          if (lattice_first<kByPatch>(i)) { take_a(); at[p] = a_at; slot[p] = a_slot; }
+          if (CH == 0 && t % 3 == 0) take_b();
+          if (CH > 0 && Q == 0) need_tile((t * KB + KB - 1) / 4);
+          if (CH > 0 && !BASE) need_tile(P.tiles_base + (t * PT + FIRST + NK - 1) / 4);
+          if (!ok) return;
+          if (i < 8 && lattice_first<kByPatch>(i + 1)) look_a();
+          if (CH == 0) {
+            issue_lattice_tap<I8, 0, 0, 0, 4>(t, q < base_chunks ? d_p : d_r, hi, at[p], row_lo, b_at, kTileU, idesc,
+                                              i == 0 && (q == 0 || q == base_chunks) ? 0u : 1u);
+          } else {
+            if (Q == 0) issue_lattice_tap<I8, KB, 0, 0, KB>(t, d_p, hi, at[p], row_lo, b0, kTileU, idesc, i ? 1u : 0u);
+            if (!BASE) issue_lattice_tap<I8, PT, FIRST, K0, NK>(t, d_r, hi, at[p], row_lo, bc, kTileU, idesc, Q || i ? 1u : 0u);
+          }
+          if (lattice_last<kByPatch>(i)) ptx::umma_commit_pair(&sh->a_empty[slot[p]]);
+          if (CH == 0 && t % 3 == 2) free_b(b_slot);
+        }
+      };
+      if constexpr (CH > 0) {
+        chunk(std::integral_constant<int, 0>{}, 0);
+        if (ok && CH == 2 && !BASE) chunk(std::integral_constant<int, 1>{}, 1);
+      } else {
+#pragma unroll 1
+        for (int q = 0; q < chunks && ok; ++q) chunk(std::integral_constant<int, 0>{}, q);
+      }
+      if (!ok) return;
+    } else if constexpr (MODE == kTc4Rows2 && CH > 0) {
       // a patch per chunk and filter row
       constexpr int PT = 4 * CH - KP;                          // conditional slices of a tap
       const uint32_t bc = b0 + (uint32_t)P.tiles_base * kTileU;
@@ -530,6 +596,23 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
         const int n0 = pos / ip, rem = pos - n0 * ip, h0 = rem / P.wp, w0 = rem - h0 * P.wp;
         const int pos1 = pos + P.patch_rows;                   // start of a window's second load
         const int n1 = pos1 / ip, rem1 = pos1 - n1 * ip, h1 = rem1 / P.wp, w1 = rem1 - h1 * P.wp;
+        if (PAIR && P.mode == kTc4Lattice) {
+          // the patches of a chunk in the order in which they are taken: odd or even rows and columns
+          const int ck = I8 ? 128 : 64, patches = 4 * (BASE ? (L.c_p + ck - 1) / ck : L.c_in / ck);
+          for (int i = 0; i < patches && ok; ++i) {
+            if (!seen) ok = wait4_one(sh, prm.counters, &sh->a_empty[c.slot], c.par ^ 1u, 1);
+            if (!ok) break;
+            uint8_t* dst = s_a + (size_t)c.slot * P.slot_bytes;
+            uint64_t* full = &sh->a_full[c.slot];
+            c.next(P.na);
+            seen = ptx::mbar_test_wait(&sh->a_empty[c.slot], c.par ^ 1u);
+            const uint32_t bar = leader(full);
+            expect(full, (uint32_t)P.patch_rows * 128u);
+            ptx::tma_load_im2col_4d<PAIR>(dst, &map_x, bar, (i >> 2) * ck, w0 * 2 - 1, h0 * 2 - 1, n0, (uint16_t)(i & 1),
+                                          (uint16_t)((i >> 1) & 1));
+          }
+          continue;
+        }
         Tc4Row next = row_at(table, lo);
         for (int i = lo; i < hi; ++i) {
           const Tc4Row s = next;
@@ -543,13 +626,13 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
           seen = ptx::mbar_test_wait(&sh->a_empty[c.slot], c.par ^ 1u);
           const uint32_t bar = leader(full);
           const int ch = (int)s.chunk * (I8 ? 128 : 64);
-          const int tiles = P.mode == kTc4Window || P.mode == kTc4Window2 ? P.loads : ((s.kind >> 4) & 3) + 1;
+          const int tiles = P.mode == kTc4Window || P.mode == kTc4Rows2 ? P.loads : ((s.kind >> 4) & 3) + 1;
           expect(full, (uint32_t)(tiles * P.patch_rows) * 128u);
           if (P.mode == kTc4Window) {
             ptx::tma_load_im2col_4d<PAIR>(dst, &map_x, bar, ch, w0 - L.pad, h0 - L.pad, n0, 0, 0);
             if (tiles == 2)
               ptx::tma_load_im2col_4d<PAIR>(dst + (size_t)P.patch_rows * 128, &map_x, bar, ch, w1 - L.pad, h1 - L.pad, n1, 0, 0);
-          } else if (P.mode == kTc4Window2) {
+          } else if (P.mode == kTc4Rows2) {
             for (int k = 0; k < 2; ++k)
               ptx::tma_load_im2col_4d<PAIR>(dst + k * kLatticeRows * 128, &map_x, bar, ch, w0 * 2 - 1, h0 * 2 - 1, n0, (uint16_t)k,
                                             (uint16_t)(s.tap_row & 15));
@@ -628,14 +711,23 @@ __device__ __forceinline__ void run_roles(const CUtensorMap& map_x, const Weight
           } else if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Window, 4>(prm, sh, a0, b0, tmem, group, jobs);
           else if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Window, 2>(prm, sh, a0, b0, tmem, group, jobs);
           else issue_jobs<NT, I8, BASE, HALF, kTc4Window, 1>(prm, sh, a0, b0, tmem, group, jobs);
-        } else if (P.mode == kTc4Window2) {
-          if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 4>(prm, sh, a0, b0, tmem, group, jobs);
+        } else if (P.mode == kTc4Lattice) {
+          if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Lattice, 4>(prm, sh, a0, b0, tmem, group, jobs);
           else if (L.c_in == (I8 ? 256 : 128)) {
-            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 2, 2>(prm, sh, a0, b0, tmem, group, jobs);
-            else issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 1, 2>(prm, sh, a0, b0, tmem, group, jobs);
+            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Lattice, 2, 2>(prm, sh, a0, b0, tmem, group, jobs);
+            else issue_jobs<NT, I8, BASE, HALF, kTc4Lattice, 1, 2>(prm, sh, a0, b0, tmem, group, jobs);
           } else {
-            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 2, 1>(prm, sh, a0, b0, tmem, group, jobs);
-            else issue_jobs<NT, I8, BASE, HALF, kTc4Window2, 1, 1>(prm, sh, a0, b0, tmem, group, jobs);
+            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Lattice, 2, 1>(prm, sh, a0, b0, tmem, group, jobs);
+            else issue_jobs<NT, I8, BASE, HALF, kTc4Lattice, 1, 1>(prm, sh, a0, b0, tmem, group, jobs);
+          }
+        } else if (P.mode == kTc4Rows2) {
+          if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Rows2, 4>(prm, sh, a0, b0, tmem, group, jobs);
+          else if (L.c_in == (I8 ? 256 : 128)) {
+            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Rows2, 2, 2>(prm, sh, a0, b0, tmem, group, jobs);
+            else issue_jobs<NT, I8, BASE, HALF, kTc4Rows2, 1, 2>(prm, sh, a0, b0, tmem, group, jobs);
+          } else {
+            if (kp == 2) issue_jobs<NT, I8, BASE, HALF, kTc4Rows2, 2, 1>(prm, sh, a0, b0, tmem, group, jobs);
+            else issue_jobs<NT, I8, BASE, HALF, kTc4Rows2, 1, 1>(prm, sh, a0, b0, tmem, group, jobs);
           }
         } else if (P.mode == kTc4Taps) {
           if (kp == 4) issue_jobs<NT, I8, BASE, HALF, kTc4Taps, 4>(prm, sh, a0, b0, tmem, group, jobs);
@@ -1144,10 +1236,11 @@ bool encode_x(CUtensorMap* map, const void* base, const LayerDims& L, const Tc4P
   const cuuint64_t dims[4] = {(cuuint64_t)L.c_in, (cuuint64_t)L.w, (cuuint64_t)L.h, (cuuint64_t)L.n};
   const cuuint64_t str[3] = {L.c_in * eb, (cuuint64_t)L.w * L.c_in * eb, (cuuint64_t)L.h * L.w * L.c_in * eb};
   const int lower[2] = {-L.pad, -L.pad};
-  // window mode: the box ends at the image's last column and row; else at the last filter position.  Stride-2 windows: at
-  // the last column (a position more than there are outputs) and the last filter position of a column.
+  // window modes: the box ends at the image's last column and row (at stride 2 a position more than there are outputs); else at
+  // the last filter position.  A patch per filter row at stride 2: the last column, and the last filter position of a column.
   const int last = L.pad - (L.kw - 1);
-  const int upper[2] = {P.mode == kTc4Window || P.mode == kTc4Window2 ? 0 : last, P.mode == kTc4Window ? 0 : last};
+  const bool window = P.mode == kTc4Window || P.mode == kTc4Lattice;
+  const int upper[2] = {window || P.mode == kTc4Rows2 ? 0 : last, window ? 0 : last};
   const cuuint32_t st = P.mode == kTc4Window ? 1u : (cuuint32_t)L.stride;
   const cuuint32_t es[4] = {1, st, st, 1};
   return fn(map, P.i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
@@ -1194,7 +1287,7 @@ int raw_rows(const LayerDims& L, const Tc4Plan& P, RawRow* out) {
     o.r.kind = (uint8_t)((nks - 1) | ks0 << 2 | (tiles - 1) << 4);
     o.r.chunk = (uint8_t)q;
     o.r.tap_row = (uint8_t)(r | stage_tiles << 4);
-    o.a_key = P.mode == kTc4Taps || P.mode == kTc4Window2 ? q * 16 + r : q;
+    o.a_key = P.mode == kTc4Taps || P.mode == kTc4Rows2 ? q * 16 + r : q;
     o.b_key = b_key;
     return &o;
   };
@@ -1262,22 +1355,34 @@ void plan_base(const RawRow* raw, Tc4Plan* P) {
   }
 }
 
-// Stride-2 layers of pairs: windows over the lattices of odd and even columns, of pitch w' + 1, two to a filter row (an odd one
-// starts in the padding; an even one ends there).  Tap by tap the pixels of a job were copied nine times a chunk: 128->256
-// channels at 28x28, 650 KB a job and CTA, 9,000 cycles of copies for 4,600 of MMAs.
-bool plan_window2(const LayerDims& L, Tc4Plan* P) {
-  const int eb = P->i8 ? 1 : 2, ck = 128 / eb, slot = 2 * kLatticeRows * 128;
+// Stride-2 layers of pairs: windows over the four lattices of odd and even rows and columns, of pitch w' + 1 and h' + 1 (an odd
+// lattice starts in the padding; an even one ends there).  Tap by tap the pixels of a job were copied nine times: 128->256
+// channels at 28x28, 650 KB a job and CTA, 9,000 cycles of copies for 4,600 of MMAs.  Four of its patches are in use at a time
+// (one by one for int8 with two packed chunks) and two more on their way, or a patch per filter row serves, of two lattices of
+// pitch w' + 1 and h': six copies a chunk for four.  us a
+// patch per filter row / per lattice (per lattice and one by one): 256->512 at 14x14 b128 21.6 / 17.6 (17.6), b64 13.0 / 12.0 (11.7),
+// 128->256 at 28x28 b64 with G = 2 12.7 / 12.4 (11.7), with G = 4 13.6 / no room (12.7), 64->128 at 56x56 b128 18.2 / 18.5 (17.0).
+bool plan_stride2(const LayerDims& L, Tc4Plan* P) {
+  const int eb = P->i8 ? 1 : 2, ck = 128 / eb, tile = L.c_out <= 64 || (P->i8 && L.c_in <= ck) ? 4096 : 8192;
   if (L.w % 2 || L.h % 2) return false;
-  if (L.wo < 2) return false;                                  // (half of the positions would be padding)
-  if ((long long)L.n * (L.wo + 1) * L.ho > 0x7fffffffll - 65536) return false;
-  if (L.c_p % ck != 0) {
-    // a base path of less than a chunk: with packed weights that stay in shared memory
-    const int tiles = (9 * L.c_p + ck - 1) / ck + (9 * L.c_r + ck - 1) / ck;
-    if (L.c_in > 2 * ck || (int)(kSmemBytes - 1024 - kOffStages) - tiles * (L.c_out <= 64 || (P->i8 && L.c_in <= ck) ? 4096 : 8192) < 2 * slot) return false;
+  if ((long long)L.n * (L.wo + 1) * (L.ho + 1) > 0x7fffffffll - 65536) return false;
+  // a base path of less than a chunk: with packed weights that stay in shared memory
+  const bool packed = L.c_p % ck != 0;
+  if (packed && L.c_in > 2 * ck) return false;
+  const int weights = (packed ? (9 * L.c_p + ck - 1) / ck + (9 * L.c_r + ck - 1) / ck : 9) * tile;
+  const int room = (int)(kSmemBytes - 1024 - kOffStages) - weights, rows = (128 + L.wo + 2 + 7) / 8 * 8, slot = (rows * 128 + 1023) / 1024 * 1024;
+  if (rows <= 256 && room >= (P->i8 && packed && L.c_in == 2 * ck ? 3 : 6) * slot) {
+    P->mode = kTc4Lattice;
+    P->wp = L.wo + 1; P->hp = L.ho + 1;
+    P->loads = 1; P->patch_rows = rows; P->slot_bytes = slot;
+  } else {
+    const int slot2 = 2 * kLatticeRows * 128;
+    if (L.wo < 2 || room < 2 * slot2) return false;            // (one pixel a row: half of the positions would be padding)
+    P->mode = kTc4Rows2;
+    P->wp = L.wo + 1; P->hp = L.ho;
+    P->loads = 2; P->patch_rows = kLatticeRows; P->slot_bytes = slot2;
   }
-  P->mode = kTc4Window2;
-  P->wp = L.wo + 1; P->hp = L.ho;
-  P->loads = 2; P->patch_rows = kLatticeRows; P->slot_bytes = slot; P->a_step = 8;
+  P->a_step = 8;
   return true;
 }
 
@@ -1336,7 +1441,8 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   // Where a job's K loop is short, or only two CTAs could share it, pairs end sooner: they have no exchange of sums, but
   // their epilogue of 256 pixels waits longer for a residual.  us shared / as pairs (and with a residual), by MMAs a job:
   //   up to 36: 56x56 x 64 7.0 / 5.9, 28x28 x 64 6.3 / 6.0 (6.3 / 6.4), 56x56 x 64->128 stride 2 7.9 / 6.0, 14x14 x 256->512
-  //     1x1 6.9 / 5.2; the pixels of a single job are shared sooner, 5x5 x 64 5.4 / 5.9 (5.2 / 6.1);
+  //     1x1 6.9 / 5.2; the pixels of a single job are shared sooner, 5x5 x 64 5.4 / 5.9 (5.2 / 6.1), but not with many columns:
+  //     a classifier, 128 x 512->1024, 7.6 / 5.6, 10x10 x 64->1024 6.5 / 5.7;
   //   up to 72: 2 x 28x28 x 128 8.5 / 7.5, one image (14 jobs) 7.9 / 7.5 (7.9 / 8.1), 28x28 x 128->256 stride 2 8.1 / 6.5;
   //     eight CTAs to a job are faster, 3 x 14x14 x 128 (10 jobs) 6.9 / 7.4 (6.9 / 8.1);
   //   two CTAs: 8 x 14x14 x 256 10.7 / 8.5, 5 x 14x14 x 256 10.6 / 8.1 (10.6 / 8.7), 51 x 5x8 x 512->192 14.3 / 12.0;
@@ -1381,8 +1487,8 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     const int pairs = sms / 2;
     int tiles256 = (int)((positions + 255) / 256);
     auto rounds = [&](int tn) { return tn > pairs ? 1e30 : (double)((tiles256 + pairs / tn - 1) / (pairs / tn)); };
-    if (k3 && L.stride == 2 && plan_window2(L, &P)) {
-      // two thirds of the patch bytes, and up to half as many positions again: not where that makes more than half as many rounds again
+    if (k3 && L.stride == 2 && plan_stride2(L, &P)) {
+      // a third or two of the patch bytes, and more positions: not where that makes more than half as many rounds again
       const double taps = rounds(tn128);
       const long long padded = (long long)L.n * P.wp * P.hp;
       const int before = tiles256;
@@ -1418,6 +1524,8 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
     }
   }
 
+  if (P.mode == kTc4Lattice) max_a = 4 * (L.c_in / ck);        // (not in the table)
+
   P.stage_bytes = 3 * (P.pair ? P.nt / 2 : P.nt) * 128;
   // a cluster's CTA: room for the sums that are sent to it, and for its own behind the rings' start
   const unsigned sums_bytes = P.pair ? 0u : (unsigned)(__builtin_popcount(P.p_mask) + __builtin_popcount(P.r_mask)) * (128u / (unsigned)P.split) * kSumPitch;
@@ -1435,20 +1543,20 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   // pair's MMAs fetch of each other's weights: 5,300 cycles a job, 4,600 of MMAs.
   const int tile_bytes = (P.pair ? P.nt / 2 : P.nt) * 128;
   const int tb = (9 * L.c_p + ck - 1) / ck, tc = (9 * L.c_r + ck - 1) / ck;
-  if (P.mode == kTc4Window2 ? L.c_p % ck != 0
+  if (P.mode == kTc4Lattice || P.mode == kTc4Rows2 ? L.c_p % ck != 0
                             : P.pair && P.mode == kTc4Window && P.nt == 128 && L.c_in == 2 * ck && L.c_p < ck && L.c_r > 0 &&
                                   room - (tb + tc) * tile_bytes >= 2 * P.slot_bytes) {
     P.packed = 1; P.resident = 1;
     P.tiles_base = tb; P.tiles_cond = tc;
     P.nb = (tb + tc + 2) / 3;
-  } else if (max_b <= kMaxNB && jobs > 1 && room - max_b * P.stage_bytes >= 3 * P.slot_bytes) {
+  } else if (max_b <= kMaxNB && jobs > 1 && room - max_b * P.stage_bytes >= (P.mode == kTc4Lattice ? 6 : P.mode == kTc4Rows2 ? 2 : 3) * P.slot_bytes) {
     P.resident = 1;
     P.nb = max_b;
   } else {
     // (three weight stages at least: a base stage stays while conditional ones pass)
-    int na = P.mode == kTc4Window ? 3 : 2;
+    int na = P.mode == kTc4Lattice ? kLatticeSlots : P.mode == kTc4Window ? 3 : 2;
     if (na > max_a * jobs) na = max_a * jobs;
-    while (na > 2 && room - na * P.slot_bytes < 4 * P.stage_bytes) --na;
+    while (na > (P.mode == kTc4Lattice ? 6 : 2) && room - na * P.slot_bytes < (P.mode == kTc4Lattice ? 3 : 4) * P.stage_bytes) --na;
     if (!P.pair && na > 1 && room - na * P.slot_bytes < 3 * P.stage_bytes) --na;
     P.nb = (room - na * P.slot_bytes) / P.stage_bytes;
     if (P.nb < 3) return false;

@@ -35,7 +35,7 @@ enum : uint8_t {
   kRowCond = 64     // the weights come from W_cond (else W_base)
 };
 
-enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2, kTc4Window2 = 3 };
+enum { kTc4Window = 0, kTc4Taps = 1, kTc4Chunks = 2, kTc4Lattice = 3, kTc4Rows2 = 4 };
 constexpr int kNoHalfJob = 1 << 30;
 
 struct Tc4Plan {
@@ -43,12 +43,12 @@ struct Tc4Plan {
   int i8;
   int pair;              // 1: CTA pairs (256 pixels per job); 0: `split` CTAs share the K loop of a 128-pixel job
   int nt;                // output channels per job: 64 or 128
-  int mode;              // kTc4Window, kTc4Taps, kTc4Chunks, kTc4Window2: what a patch slot holds
-  int wp, hp;            // pitch of the stacked pixel space: window mode w + pad, h + pad; stride-2 windows w' + 1, h'; else w', h'
+  int mode;              // kTc4Window, kTc4Taps, kTc4Chunks, kTc4Lattice, kTc4Rows2: what a patch slot holds
+  int wp, hp;            // pitch of the stacked pixel space: window mode w + pad, h + pad; stride-2 windows w' + 1 and h' + 1 or h'; else w', h'
   FastDiv div_ip, div_wp;   // by wp * hp and by wp
   int positions;         // n * wp * hp
   int patch_rows;        // pixels per patch load
-  int slot_bytes;        // patch slot: one or two loads of a window, two of a stride-2 window's filter row, or up to three of 128 pixels
+  int slot_bytes;        // patch slot: one or two loads of a window, two of a filter row (kTc4Rows2), or up to three of 128 pixels
   int loads;             // window modes: loads per slot
   int a_step;            // distance of a row's pixel operands, 16-byte units
   int na, nb;            // ring depths: patch slots, weight stages

@@ -280,7 +280,7 @@ INT8_K_LOOPS = [
     (O.Shape(64, 7, 7, 512, 512, groups=4), "one patch for all taps", "streamed", False, "a base chunk, streamed"),
     (O.Shape(96, 14, 14, 256, 512, stride=2, groups=4), "four patches", "packed", True, "stride 2, two base slices"),
     (O.Shape(96, 14, 14, 256, 512, stride=2, groups=8), "four patches", "packed", True, "stride 2, one base slice"),
-    (O.Shape(96, 14, 14, 256, 512, stride=2, groups=2), "four patches", "resident", True, "stride 2, a base chunk"),
+    (O.Shape(96, 14, 14, 256, 512, stride=2, groups=2), "four patches", "streamed", True, "stride 2, a base chunk"),
     (O.Shape(40, 28, 28, 256, 512, stride=2, groups=4), "four patches", "packed", False, "stride 2, whole rounds"),
     (O.Shape(96, 14, 14, 512, 512, stride=2, groups=4), "four patches", "streamed", True, "stride 2, streamed"),
 ]
@@ -310,6 +310,8 @@ FEW_JOBS = [
     (O.Shape(1, 28, 28, 128, 256, stride=2, groups=4), False, 1, "72 MMAs, stride 2"),
     (O.Shape(3, 14, 14, 256, 256, groups=4), False, 4, "144 MMAs, room for four CTAs a job"),
     (O.Shape(5, 14, 14, 256, 256, groups=4), False, 1, "144 MMAs, room for two"),
+    (O.Shape(128, 1, 1, 512, 1024, 1, 1, 1, 0, groups=1), False, 1, "a classifier: 32 MMAs, one pixel tile, 16 jobs"),
+    (O.Shape(1, 10, 10, 64, 1024, groups=4), False, 1, "36 MMAs, one pixel tile, 16 jobs"),
 ]
 
 
