@@ -65,6 +65,22 @@ def test_subsample_maxpool_avgpool_match_their_definitions():
     assert np.abs(got - mean).max() <= 2.0 ** -8 * np.abs(mean).max() + 1e-6   # one bf16 rounding of an fp32 sum
 
 
+@pytest.mark.parametrize("h", [1, 3])
+def test_average_pooling_of_many_images_is_that_of_few(h):
+    """The kernels for batches that fill the device and for those that do not: the same sums in the same order."""
+    import torch
+    from paper_1805_12549_b200 import binding as B
+    n, c = 5000, 512
+    x = torch.randn((n, h, h, c), device="cuda", generator=torch.Generator(device="cuda").manual_seed(2)).bfloat16()
+    y = torch.full((n, 1, 1, c), 7.0, dtype=torch.bfloat16, device="cuda")
+    B.cg_avgpool_bf16(x, y)
+    for first in (0, n - 33):
+        few = torch.empty((33, 1, 1, c), dtype=torch.bfloat16, device="cuda")
+        B.cg_avgpool_bf16(x[first:first + 33].contiguous(), few)
+        assert torch.equal(y[first:first + 33], few)
+    assert (y.float() - x.float().mean((1, 2), keepdim=True)).abs().max() <= 2.0 ** -8 * y.float().abs().max()
+
+
 @pytest.mark.parametrize("k,stride,pad", [(2, 2, 0), (3, 1, 1), (3, 2, 1), (3, 2, 0), (3, 3, 1), (5, 2, 2)])
 @pytest.mark.parametrize("n,h,w,c", [(1, 1, 1, 8), (2, 1, 13, 16), (1, 9, 1, 8), (2, 2, 2, 8), (3, 7, 10, 40), (1, 33, 31, 64)])
 def test_maxpool_over_filters_and_sizes(k, stride, pad, n, h, w, c):
