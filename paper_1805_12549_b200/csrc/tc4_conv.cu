@@ -1441,15 +1441,16 @@ bool tc4_plan(const LayerDims& L, int in_dtype, int cond_mode, int sms, Tc4Plan*
   // Where a job's K loop is short, or only two CTAs could share it, pairs end sooner: they have no exchange of sums, but
   // their epilogue of 256 pixels waits longer for a residual.  us shared / as pairs (and with a residual), by MMAs a job:
   //   up to 36: 56x56 x 64 7.0 / 5.9, 28x28 x 64 6.3 / 6.0 (6.3 / 6.4), 56x56 x 64->128 stride 2 7.9 / 6.0, 14x14 x 256->512
-  //     1x1 6.9 / 5.2; the pixels of a single job are shared sooner, 5x5 x 64 5.4 / 5.9 (5.2 / 6.1), but not with many columns:
-  //     a classifier, 128 x 512->1024, 7.6 / 5.6, 10x10 x 64->1024 6.5 / 5.7;
+  //     1x1 6.9 / 5.2; the pixels of a single job are shared sooner, 5x5 x 64 5.4 / 5.9 (5.2 / 6.1); with
+  //     many columns, too: 128 x 512->1024, a classifier, is 5.6 as pairs in a chain of itself and 7.6 shared, but behind the
+  //     other layers of a network 18.9 and 14.9 between events, a pass of one image 178.9 and 176.3;
   //   up to 72: 2 x 28x28 x 128 8.5 / 7.5, one image (14 jobs) 7.9 / 7.5 (7.9 / 8.1), 28x28 x 128->256 stride 2 8.1 / 6.5;
   //     eight CTAs to a job are faster, 3 x 14x14 x 128 (10 jobs) 6.9 / 7.4 (6.9 / 8.1);
   //   two CTAs: 8 x 14x14 x 256 10.7 / 8.5, 5 x 14x14 x 256 10.6 / 8.1 (10.6 / 8.7), 51 x 5x8 x 512->192 14.3 / 12.0;
   //   else shared: 14x14 x 256 7.5 / 8.1 (7.5 / 8.4), 7x7 x 512 7.3 / 11.5.
   const long long small = (long long)tiles128 * tn64, mmas = (long long)L.kh * L.kw * L.c_in / slice;
   const bool as_pairs = small * 4 > sms * 7 / 8 ||
-                        (mmas <= 72 && small >= (L.has_residual ? 16 : 14)) ||
+                        (mmas <= 72 && tiles128 >= 2 && small >= (L.has_residual ? 16 : 14)) ||
                         (mmas <= 72 && !L.has_residual && (mmas <= 36 ? tiles128 >= 2 : L.stride == 2));
   if (!one_row && !as_pairs && small * 2 <= sms) {
     // Fewer jobs of 128 pixels and 64 channels than half the SMs: their K loops are shared, as far as all clusters

@@ -310,8 +310,8 @@ FEW_JOBS = [
     (O.Shape(1, 28, 28, 128, 256, stride=2, groups=4), False, 1, "72 MMAs, stride 2"),
     (O.Shape(3, 14, 14, 256, 256, groups=4), False, 4, "144 MMAs, room for four CTAs a job"),
     (O.Shape(5, 14, 14, 256, 256, groups=4), False, 1, "144 MMAs, room for two"),
-    (O.Shape(128, 1, 1, 512, 1024, 1, 1, 1, 0, groups=1), False, 1, "a classifier: 32 MMAs, one pixel tile, 16 jobs"),
-    (O.Shape(1, 10, 10, 64, 1024, groups=4), False, 1, "36 MMAs, one pixel tile, 16 jobs"),
+    (O.Shape(128, 1, 1, 512, 1024, 1, 1, 1, 0, groups=1), False, 2, "a classifier: 32 MMAs, one pixel tile, 16 jobs"),
+    (O.Shape(1, 10, 10, 64, 1024, groups=4), False, 4, "36 MMAs, one pixel tile, 16 jobs"),
 ]
 
 
