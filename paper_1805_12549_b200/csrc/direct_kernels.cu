@@ -243,7 +243,7 @@ direct_gated_conv_i8_kernel(LayerDims L, const int8_t* __restrict__ x,
 // x CH channels.  A run of kStage K elements (tap-major, then channel) is gathered per stage: four consecutive
 // channels of a tap per load, converted to fp32, two stages in flight.  The warp-per-output kernel above waits
 // for one pair of global loads per product: 156 us for the partial sums of four images of 56x56 (64 channels,
-// c_p = 16), here 18.7; counters there: shared-memory reads 58 % of their rate, issue slots 48 %, DRAM 1 %.  It remains for channel counts that are not multiples of four, channel
+// c_p = 16), here 19.1; counters there: shared-memory reads 58 % of their rate, issue slots 48 %, DRAM 1 %.  It remains for channel counts that are not multiples of four, channel
 // grouping and the channel-wise gate.
 // Products and sums are rounded separately, for bf16 operands too: their products are exact in fp32 only inside its
 // normal range, so a fused multiply-add is another sum where one is below 2^-126 or beyond 2^128.
