@@ -243,7 +243,7 @@ direct_gated_conv_i8_kernel(LayerDims L, const int8_t* __restrict__ x,
 // x CH channels.  A run of kStage K elements (tap-major, then channel) is gathered per stage: four consecutive
 // channels of a tap per load, converted to fp32, two stages in flight.  The warp-per-output kernel above waits
 // for one pair of global loads per product: 156 us for the partial sums of four images of 56x56 (64 channels,
-// c_p = 16), here 19.1; counters there: shared-memory reads 58 % of their rate, issue slots 48 %, DRAM 1 %.  It remains for channel counts that are not multiples of four, channel
+// c_p = 16), here 19.2; counters there: shared-memory reads 58 % of their rate, issue slots 48 %, DRAM 1 %.  It remains for channel counts that are not multiples of four, channel
 // grouping and the channel-wise gate.
 // Products and sums are rounded separately, for bf16 operands too: their products are exact in fp32 only inside its
 // normal range, so a fused multiply-add is another sum where one is below 2^-126 or beyond 2^128.
@@ -262,19 +262,22 @@ TapBox tap_box(const LayerDims& L) {
   return b;
 }
 
-// Pixels by ordinary loads, and no __restrict__ on what they read: the kernel in front, whose end this one's launch does not
-// wait for, may still be writing them.  (us with all loads on the read-only path / weights on it / none: 16 channels of 8x8, two
-// images, fp32 5.9 / 6.05 / 6.15, partial sums of four images of 56x56 18.65 / 19.1 / 19.1.  Inline loads that the compiler may
-// move are no way out: it may also move them out of the test that keeps them in bounds.)
-template <bool READ_ONLY> __device__ __forceinline__ float4 load4(const float* p) {
-  const float4* q = reinterpret_cast<const float4*>(p);
-  return READ_ONLY ? __ldg(q) : *q;
-}
-template <bool READ_ONLY> __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
-  const uint2* q = reinterpret_cast<const uint2*>(p);
-  const uint2 v = READ_ONLY ? __ldg(q) : *q;
+// Four channels as they lie in memory; they become fp32 on their way to shared memory.
+template <typename T> struct Four { using Raw = float4; };
+template <> struct Four<__nv_bfloat16> { using Raw = uint2; };
+__device__ __forceinline__ float4 widen(float4 v) { return v; }
+__device__ __forceinline__ float4 widen(uint2 v) {
   return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
                      __uint_as_float(v.y & 0xffff0000u));
+}
+// Pixels by ordinary loads, and no __restrict__ on what they read: the kernel in front, whose end this one's launch does not
+// wait for, may still be writing them.  Weights by the read-only path.  (us with all loads on the read-only path / this, with the
+// loads of a stage in front of the barrier and widened behind it: 16 channels of 8x8, two images, fp32 5.1 / 5.1 in a chain; 64
+// channels of 28x28, 64 images, fp32 240 / 231; partial sums of four images of 28x28 x 128 33.8 / 32.0, of 56x56 x 64 18.3 / 18.9.)
+// Inline loads that the compiler may move are no way out: it may also move them out of the test that keeps them in bounds.
+template <bool READ_ONLY, typename T> __device__ __forceinline__ typename Four<T>::Raw load4(const T* p) {
+  const typename Four<T>::Raw* q = reinterpret_cast<const typename Four<T>::Raw*>(p);
+  return READ_ONLY ? __ldg(q) : *q;
 }
 __device__ __forceinline__ float mul_add(float a, float b, float c) { return __fadd_rn(c, __fmul_rn(a, b)); }
 
@@ -330,7 +333,7 @@ direct_tile_kernel(LayerDims L, const T* x, const T* __restrict__ w_base, const 
     w0 = (int)(mi - ho * (unsigned)L.wo) * L.stride - L.pad;
     x_off = (((long long)n * L.h + h0) * L.w + w0) * L.c_in;
   }
-  float4 xr[kXUnits], wr[kWUnits];
+  typename Four<T>::Raw xr[kXUnits], wr[kWUnits];
   uint32_t okr = 0;
 
   // stage of the sums over `cw` channels from c_lo on: K elements [k0, k0 + kStage) into registers ...
@@ -340,7 +343,7 @@ direct_tile_kernel(LayerDims L, const T* x, const T* __restrict__ w_base, const 
 #pragma unroll
     for (int i = 0; i < kXUnits; ++i) {
       const int u = tid + NTH * i, k = k0 + u / D::TM * 4;
-      xr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      xr[i] = {};
       if (have_pixel && u < kXTotal && k < kt) {
         const int tap = (int)div.div(k), ci = k - tap * cw, rr = (int)div_kw.div(tap), r = taps.r0 + rr, s = taps.s0 + tap - rr * taps.kw;
         if (h0 + r >= 0 && h0 + r < L.h && w0 + s >= 0 && w0 + s < L.w) {
@@ -352,7 +355,7 @@ direct_tile_kernel(LayerDims L, const T* x, const T* __restrict__ w_base, const 
 #pragma unroll
     for (int i = 0; i < kWUnits; ++i) {
       const int u = tid + NTH * i, c = u % TC, k = k0 + u / TC * 4;
-      wr[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      wr[i] = {};
       if (u < kWTotal && k < kt && c0 + c < L.c_out) {
         int at = k;                                        // element of the channel's filter
         if (BOX) {
@@ -369,16 +372,17 @@ direct_tile_kernel(LayerDims L, const T* x, const T* __restrict__ w_base, const 
     for (int i = 0; i < kXUnits; ++i) {
       const int u = tid + NTH * i, g = u / D::TM;
       if (u >= kXTotal) break;
-      *reinterpret_cast<float4*>(&S.x[b][gx * D::kXPitch + g * 4]) = xr[i];
+      *reinterpret_cast<float4*>(&S.x[b][gx * D::kXPitch + g * 4]) = widen(xr[i]);
       S.ok[b][g * D::TM + gx] = (uint8_t)((okr >> i) & 1u);
     }
 #pragma unroll
     for (int i = 0; i < kWUnits; ++i) {
       const int u = tid + NTH * i, c = u % TC, g = u / TC;
       if (u >= kWTotal) break;
-      if (CH == 1) { *reinterpret_cast<float4*>(&S.w[b][c * D::kWPitch + g * 4]) = wr[i]; continue; }
+      const float4 v = widen(wr[i]);
+      if (CH == 1) { *reinterpret_cast<float4*>(&S.w[b][c * D::kWPitch + g * 4]) = v; continue; }
       float* d = &S.w[b][g * 4 * D::kWPitch + c];
-      d[0] = wr[i].x; d[D::kWPitch] = wr[i].y; d[2 * D::kWPitch] = wr[i].z; d[3 * D::kWPitch] = wr[i].w;
+      d[0] = v.x; d[D::kWPitch] = v.y; d[2 * D::kWPitch] = v.z; d[3 * D::kWPitch] = v.w;
     }
   };
   int b = 0;                                               // buffer of the current stage
@@ -392,10 +396,15 @@ direct_tile_kernel(LayerDims L, const T* x, const T* __restrict__ w_base, const 
 #pragma unroll
     for (int i = 0; i < PXT; ++i) a2[i][0] = a2[i][1] = 0;
     const int kt = taps.kh * taps.kw * cw, stages = (kt + kStage - 1) / kStage;
+    // (the next loads are issued in front of the barrier: ordinary loads that come behind it in the program stay behind it)
+    auto next = [&](int st) {
+      if (st < stages) fetch(w, div, c_lo, cw, st * kStage);
+      else if (st == stages) then();
+    };
     put(b);
+    next(1);
     __syncthreads();
     for (int st = 0; st < stages; ++st) {
-      if (st + 1 < stages) fetch(w, div, c_lo, cw, (st + 1) * kStage); else then();
       const int groups = min(kStage / 4, (kt - st * kStage) / 4);
       // operands of four K elements, read one group ahead where few warps share an SM
       float4 xv[2][PXT], wv[2][CH];                           // (of the weights: K elements x channels, or the reverse)
@@ -447,7 +456,7 @@ direct_tile_kernel(LayerDims L, const T* x, const T* __restrict__ w_base, const 
         add(1);
       }
       b ^= 1;
-      if (st + 1 < stages) put(b);
+      if (st + 1 < stages) { put(b); next(st + 2); }
       __syncthreads();
     }
     if constexpr (CH == 4) {
